@@ -95,7 +95,7 @@ DynGeom geom(sox_handle h, int n, int N, int T, int S, int nO) {
 size_t fixed_bytes(const DynGeom &g) {
   const int n = g.n, N = g.N, T = g.T, nO = g.nO;
   size_t b = aligned_bytes((size_t)N * g.Kp * g.Kp, 4) + 2 * aligned_bytes((size_t)n * g.NR * g.Kp, 2) +
-             aligned_bytes(N, 4);                                                     // U mixed, U2 split
+             aligned_bytes(N, 4) + aligned_bytes(rows_f32_bytes(N, n), 1);            // U mixed, U2 split, X in FP32
   b += 2 * aligned_bytes((size_t)nO * N * g.Np, 2);                                   // W_d split
   b += 2 * aligned_bytes((size_t)2 * nO * g.KpT, 2) + 2 * aligned_bytes((size_t)T * g.KpO, 2);   // transforms
   b += 3 * aligned_bytes((size_t)T * N * n, 8);                                       // GR, GWt, GG
@@ -122,7 +122,7 @@ size_t chunk_bytes(const DynGeom &g) {
 
 size_t dynamic_tc_bytes(sox_handle h, int n, int N, int T, int S, int n_omega) {
   const DynGeom g = geom(h, n, N, T, S, n_omega);
-  return fixed_bytes(g) + chunk_bytes(g) + (1 << 20);
+  return fixed_bytes(g) + std::max(chunk_bytes(g), aligned_bytes(mixed_f32_scratch(N, n), 1)) + (1 << 20);
 }
 
 Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omega, const double *G, const double *X,
@@ -153,13 +153,16 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
   DynScalars *sc = ar.take<DynScalars>(1);
   const int mT = std::max(T, N);
   float *ones = ar.take<float>(mT), *sAv = ar.take<float>(mT), *tmp1 = ar.take<float>(mT), *tmp2 = ar.take<float>(mT);
+  float *Xf = reinterpret_cast<float *>(ar.take<char>(rows_f32_bytes(N, n)));
+  Arena scr = ar;   // the mixed tensor's scratch, where the chunk buffers will lie
+  void *mix_scratch = scr.take<char>(mixed_f32_scratch(N, n));
   const int tcn = g.tc;
   float *Af = ar.take<float>((size_t)tcn * n * g.Nn4);
   __half *Ah = ar.take<__half>((size_t)tcn * n * NR * Kp), *Al = ar.take<__half>((size_t)tcn * n * NR * Kp);
   float *rowf = ar.take<float>((size_t)tcn * N), *colf = ar.take<float>((size_t)tcn * N);
   float *Dt = ar.take<float>((size_t)tcn * N * N), *Tm = ar.take<float>((size_t)tcn * N * n);
   double *Sd = ar.take<double>((size_t)tcn * nn);
-  if (!Sd) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+  if (!Sd || !mix_scratch) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
   (void)tmp1;
   (void)tmp2;
   ProfScope ps(h, "sosex_dynamic_tc", s, 0);
@@ -171,9 +174,8 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
 
   // ---- set-up: U2 = mixed tensor of V (per-P scale), W_d and the transforms (per tensor)
   SOX_CUDA_TRY(cudaMemsetAsync(sc, 0, sizeof(DynScalars), s));
-  SOX_CUDA_TRY(cudaMemsetAsync(U2h, 0, 2 * (size_t)n * NR * Kp, s));
-  SOX_CUDA_TRY(cudaMemsetAsync(U2l, 0, 2 * (size_t)n * NR * Kp, s));
-  launch_mixed_f32(V, X, N, n, Kp, Um, s);
+  launch_rows_f32(X, N, n, Xf, s);
+  launch_mixed_f32(V, X, N, n, Kp, Um, mix_scratch, s);
   launch_split_mixed(Um, N, NR, n, Kp, nullptr, nullptr, U2h, U2l, inv_u2, s);
   launch_absmax(Wd, false, N, nO * N, 0, 1, 1, N, &sc->mx[kWd], s);
   launch_split_tensor(Wd, false, N, nO * N, 0, 1, 1, N, g.Np, 0, 1.f, &sc->mx[kWd], nullptr, Wh, Wl, &sc->sc[kWd], s);
@@ -190,7 +192,7 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
   // X in the G_Rq slot, one copy per tau point (the fused kernel reads it at batch b)
   launch_split_rows_f64(X, n, 0, N, NR, n, Kp, Xh, Xl, inv_x, T, s);
   k_fill1<<<(mT + 255) / 256, 256, 0, s>>>(ones, mT, 1.f);
-  launches += 13;
+  launches += 16;
 
   // ---- tensor maps (fixed addresses)
   CUtensorMap mft[5], mwd[5], mbcd[8];
@@ -313,7 +315,7 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
         SOX_CUDA_TRY(launch_sox_bcd_tc(m, ba, grid, s, Kp <= 128 ? kBcdResident : kBcdStreamed));
       }
       // Sigma_d = -X^T D^T X (FP32 half transform, FP64 final sum), added to Sigma
-      launch_backproject_T(Dt, N, X, N, n, ic, Tm, s);
+      launch_backproject_T(Dt, N, Xf, N, n, ic, Tm, s);
       launch_backproject_sigma(X, Tm, N, n, ic, Sd, nn, s, nullptr);
       double *Sout = Sigma + ((long long)sp * T + i0) * nn;
       launch_add_f64(Sout, Sd, Sout, (long long)ic * nn, s);

@@ -1386,33 +1386,58 @@ __device__ float block_max(float v) {
   return red[0];
 }
 
-// Mixed tensor U[P][q][s] (FP32, Kp x Kp per P) -> split with one scale per P, written as
+// Mixed tensor U[P][q][s] (FP32, n x n valid of Kp x Kp per P, the rest not read and taken as
+// zero) -> split with one scale per P, written as
 //   U1 layout [P][q][s]     (if u1_hi)   and/or   U2 layout [v][R][w] = U[R][v][w] (if u2_hi, v < n,
 //   R-stride NR rows)
-__global__ void k_split_mixed(const float *U, int N, int NR, int n, int Kp, __half *u1_hi, __half *u1_lo,
-                              __half *u2_hi, __half *u2_lo, float *inv_scale) {
+// One block per P, rows P >= N of the padded operands zero: every element of U1 and U2 is
+// written here, so neither needs a memset.  Bound by HBM (4 bytes read, 8 written per
+// element); four elements per thread and pass, 16-byte loads and 8-byte stores.
+__global__ void __launch_bounds__(256) k_split_mixed(const float *U, int N, int NR, int n, int Kp, __half *u1_hi,
+                                                     __half *u1_lo, __half *u2_hi, __half *u2_lo, float *inv_scale) {
   const int P = blockIdx.x;
-  const long long blk = (long long)Kp * Kp;
-  const float *u = U + (long long)P * blk;
-  float m = 0.f;
-  for (long long e = threadIdx.x; e < blk; e += blockDim.x) m = fmaxf(m, fabsf(u[e]));
-  m = block_max(m);
-  const float s = tc::pow2_floor_inv(m);
-  for (long long e = threadIdx.x; e < blk; e += blockDim.x) {
-    __half hi, lo;
-    tc::split_f16(u[e] * s, hi, lo);
-    if (u1_hi) {
-      u1_hi[(long long)P * blk + e] = hi;
-      u1_lo[(long long)P * blk + e] = lo;
+  const int k4 = Kp / 4;
+  const bool live = P < N;
+  const float *u = U + (long long)P * Kp * Kp;
+  auto load = [&](int q, int w) {
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live && q < n && w < n) {
+      x = *reinterpret_cast<const float4 *>(u + (long long)q * Kp + w);
+      if (w + 1 >= n) x.y = 0.f;
+      if (w + 2 >= n) x.z = 0.f;
+      if (w + 3 >= n) x.w = 0.f;
     }
-    const int v = (int)(e / Kp), w = (int)(e % Kp);
-    if (u2_hi && v < n) {
-      const long long o = ((long long)v * NR + P) * Kp + w;
-      u2_hi[o] = hi;
-      u2_lo[o] = lo;
+    return x;
+  };
+  float s = 1.f;
+  if (live) {
+    float m = 0.f;
+    for (int e = threadIdx.x; e < n * k4; e += blockDim.x) {
+      const float4 x = load(e / k4, (e % k4) * 4);
+      m = fmaxf(fmaxf(fmaxf(m, fabsf(x.x)), fmaxf(fabsf(x.y), fabsf(x.z))), fabsf(x.w));
+    }
+    m = block_max(m);
+    s = tc::pow2_floor_inv(m);
+    if (threadIdx.x == 0) inv_scale[P] = 1.f / s;
+  }
+  const int rows = u1_hi ? Kp : n;   // U2 has rows v < n only
+  for (int e = threadIdx.x; e < rows * k4; e += blockDim.x) {
+    const int q = e / k4, w = (e % k4) * 4;
+    const float4 x = load(q, w);
+    uint2 hi, lo;
+    tc::split_f16x2(x.x * s, x.y * s, hi.x, lo.x);
+    tc::split_f16x2(x.z * s, x.w * s, hi.y, lo.y);
+    if (u1_hi) {
+      const long long o = ((long long)P * Kp + q) * Kp + w;
+      *reinterpret_cast<uint2 *>(u1_hi + o) = hi;
+      *reinterpret_cast<uint2 *>(u1_lo + o) = lo;
+    }
+    if (u2_hi && q < n) {
+      const long long o = ((long long)q * NR + P) * Kp + w;
+      *reinterpret_cast<uint2 *>(u2_hi + o) = hi;
+      *reinterpret_cast<uint2 *>(u2_lo + o) = lo;
     }
   }
-  if (threadIdx.x == 0) inv_scale[P] = 1.f / s;
 }
 
 // Per batch b (spin, tau): Gm = G(-tau) = -G[T-1-j] as Gm^T[v][s] split with one scale
@@ -1477,109 +1502,6 @@ __global__ void k_bcd_scales(const float *inv_u1, const float *gsc, const float 
   }
 }
 
-// Mixed THC tensor U[P][q][s] = sum_Q V[P][Q] X[Q][q] X[Q][s] (Eq. U_contraction at k = 0),
-// FP32 round-to-nearest accumulation over Q on CUDA cores; columns (q, s) run over
-// the padded Kp x Kp block and are zero outside [0, n)^2.  64 x 64 tile, 4 x 4 per thread.
-__global__ void __launch_bounds__(256) k_mixed_f32(const double *V, const double *X, int N, int n, int Kp,
-                                                   float *U) {
-  __shared__ float sa[16][65];
-  __shared__ float sb[16][65];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int P0 = blockIdx.y * 64;
-  const long long c0 = (long long)blockIdx.x * 64;
-  const long long ncol = (long long)Kp * Kp;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < N; k0 += 16) {
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int e = tid + it * 256;
-      const int rr = e / 16, kk = e % 16;
-      const int P = P0 + rr, Q = k0 + kk;
-      sa[kk][rr] = (P < N && Q < N) ? (float)V[(long long)P * N + Q] : 0.f;
-      const int kb = e / 64, cc = e % 64;
-      const int Qb = k0 + kb;
-      const long long col = c0 + cc;
-      const int q = (int)(col / Kp), sidx = (int)(col % Kp);
-      sb[kb][cc] = (Qb < N && col < ncol && q < n && sidx < n)
-                       ? (float)(X[(long long)Qb * n + q] * X[(long long)Qb * n + sidx])
-                       : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float av[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = sa[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = sb[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int P = P0 + ty + 16 * i;
-    if (P >= N) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long long col = c0 + tx + 16 * j;
-      if (col < ncol) U[(long long)P * ncol + col] = acc[i][j];
-    }
-  }
-}
-
-// T[b][R][r] = sum_P Dt[b][R][P] X[P][r]   (FP32 accumulate; D carries FP32 accuracy)
-// 64 x 64 tile of (R, r) per block, 256 threads, 4 x 4 per thread.
-__global__ void __launch_bounds__(256) k_backproject_T(const float *Dt, long long ldD, const double *X, int N,
-                                                       int n, float *T) {
-  __shared__ float sa[16][65];
-  __shared__ float sb[16][65];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int R0 = blockIdx.y * 64, r0 = blockIdx.x * 64;
-  const int b = blockIdx.z;
-  const float *D = Dt + (long long)b * N * ldD;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < N; k0 += 16) {
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int e = tid + it * 256;
-      const int rr = e / 16, kk = e % 16;
-      const int R = R0 + rr, P = k0 + kk;
-      sa[kk][rr] = (R < N && P < N) ? D[(long long)R * ldD + P] : 0.f;
-      const int kb = e / 64, cc = e % 64;
-      const int Pb = k0 + kb, c = r0 + cc;
-      sb[kb][cc] = (Pb < N && c < n) ? (float)X[(long long)Pb * n + c] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float av[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = sa[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = sb[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int R = R0 + ty + 16 * i;
-    if (R >= N) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = r0 + tx + 16 * j;
-      if (c < n) T[((long long)b * N + R) * n + c] = acc[i][j];
-    }
-  }
-}
-
 // Sigma[b][t][r] = -sum_R X[R][t] T[b][R][r]   (FP64 accumulate: the final orbital-basis sum)
 __global__ void __launch_bounds__(256) k_backproject_sigma(const double *X, const float *T, int N, int n,
                                                            double *Sigma, long long sstride, const int *sym) {
@@ -1632,18 +1554,6 @@ __global__ void __launch_bounds__(256) k_backproject_sigma(const double *X, cons
 }  // namespace
 
 // ------------------------------ launchers ----------------------------------
-
-void launch_mixed_f32(const double *V, const double *X, int N, int n, int Kp, float *U, cudaStream_t s) {
-  const long long ncol = (long long)Kp * Kp;
-  dim3 grid((unsigned)((ncol + 63) / 64), (N + 63) / 64);
-  k_mixed_f32<<<grid, 256, 0, s>>>(V, X, N, n, Kp, U);
-}
-
-void launch_backproject_T(const float *Dt, long long ldD, const double *X, int N, int n, int batch, float *T,
-                          cudaStream_t s) {
-  dim3 grid((n + 63) / 64, (N + 63) / 64, batch);
-  k_backproject_T<<<grid, 256, 0, s>>>(Dt, ldD, X, N, n, T);
-}
 
 void launch_backproject_sigma(const double *X, const float *T, int N, int n, int batch, double *Sigma,
                               long long sstride, cudaStream_t s, const int *sym) {
@@ -1804,7 +1714,7 @@ void launch_split_rows_f64(const double *src, long long ld, long long bstride, i
 
 void launch_split_mixed(const float *U, int N, int NR, int n, int Kp, __half *u1_hi, __half *u1_lo,
                         __half *u2_hi, __half *u2_lo, float *inv_scale, cudaStream_t s) {
-  k_split_mixed<<<N, 256, 0, s>>>(U, N, NR, n, Kp, u1_hi, u1_lo, u2_hi, u2_lo, inv_scale);
+  k_split_mixed<<<NR, 256, 0, s>>>(U, N, NR, n, Kp, u1_hi, u1_lo, u2_hi, u2_lo, inv_scale);
 }
 
 void launch_prep_gminus(const double *G, int n, int T, int nbatch, int Kp, __half *hi, __half *lo,

@@ -104,7 +104,12 @@ cudaError_t launch_gemm_f16x2(const CUtensorMap *maps, const GemmTcArgs &a, int 
 void launch_split_rows_f64(const double *src, long long ld, long long bstride, int rows_valid, int rows_out,
                            int L, int Kp, __half *hi, __half *lo, float *inv_scale, int batch, cudaStream_t s,
                            const double *alt_src = nullptr, const int *use_alt = nullptr);
-void launch_mixed_f32(const double *V, const double *X, int N, int n, int Kp, float *U, cudaStream_t s);
+// U[P][q][s] = sum_Q V[P][Q] X[Q][q] X[Q][s] for q, s < n (rows of Kp, Kp x Kp per P; the padding is
+// not written).  scratch: mixed_f32_scratch bytes, 256-byte aligned, free again after the call
+// on the stream (mixed.cu).
+size_t mixed_f32_scratch(int N, int n);
+void launch_mixed_f32(const double *V, const double *X, int N, int n, int Kp, float *U, void *scratch,
+                      cudaStream_t s);
 void launch_split_mixed(const float *U, int N, int NR, int n, int Kp, __half *u1_hi, __half *u1_lo,
                         __half *u2_hi, __half *u2_lo, float *inv_scale, cudaStream_t s);
 void launch_prep_gminus(const double *G, int n, int T, int nbatch, int Kp, __half *hi, __half *lo,
@@ -113,8 +118,13 @@ void launch_bcd_scales(const float *inv_u1, const float *gsc, const float *osc, 
                        const float *inv_gw, const float *inv_gr, const float *inv_u2, int N, int batch,
                        float *row, float *col, cudaStream_t s);
 
-// SIMT back-projection helpers (FP32 / FP64 accumulate), tc_kernels.cu
-void launch_backproject_T(const float *Dt, long long ldD, const double *X, int N, int n, int batch, float *T,
+// FP32 copy of X [N][n] with rows padded to a multiple of 4 (rows_f32_bytes), for
+// launch_backproject_T
+size_t rows_f32_bytes(int N, int n);
+void launch_rows_f32(const double *X, int N, int n, float *Xf, cudaStream_t s);
+// Back-projection helpers: the half transform T = Dt X (FP32, mixed.cu) and the final sum
+// (FP64, tc_kernels.cu)
+void launch_backproject_T(const float *Dt, long long ldD, const float *Xf, int N, int n, int batch, float *T,
                           cudaStream_t s);
 // sym (optional, per batch): when set, Sigma[b] is symmetric and only the upper
 // block triangle is computed, then mirrored

@@ -28,7 +28,9 @@ struct Geometry {
   int NR;   // rows allocated along P / R (>= 128, rows >= N are zero)
   int RG;   // rows allocated for G(-tau)^T (>= 128)
   int Bc;   // (spin, tau) batches per chunk
-  size_t fixed_bytes, per_b_bytes;
+  size_t fixed_bytes, per_b_bytes, scratch_bytes;
+  // the chunk buffers of Bc batches; the mixed tensor's scratch lies in them before the first chunk
+  size_t chunk_bytes(int bc) const { return std::max(per_b_bytes * (size_t)bc, scratch_bytes); }
 };
 
 size_t hb(size_t count) { return aligned_bytes(count, 2); }   // FP16 buffer
@@ -45,7 +47,9 @@ Geometry geometry(sox_handle h, int n, int N, int T, int S, bool two) {
   const size_t Kp2 = (size_t)g.Kp * g.Kp;
   g.fixed_bytes = fb((size_t)g.N * Kp2)                             // FP32 mixed tensor
                   + 2 * hb((size_t)g.NR * Kp2) + fb(g.N)              // U1 split
-                  + 2 * hb((size_t)g.n * g.NR * g.Kp) + fb(g.N);      // U2 split
+                  + 2 * hb((size_t)g.n * g.NR * g.Kp) + fb(g.N)       // U2 split
+                  + aligned_bytes(rows_f32_bytes(N, n), 1);           // X in FP32
+  g.scratch_bytes = aligned_bytes(mixed_f32_scratch(N, n), 1);
   g.per_b_bytes = 2 * db((size_t)N * n)                                // FP64 projections
                   + 4 * hb((size_t)g.NR * g.Kp) + 2 * fb(N)           // GR / GW splits
                   + 2 * hb((size_t)g.RG * g.Kp) + 2 * fb(1)           // G(-tau)^T split, scales
@@ -117,7 +121,7 @@ Status tune_bcd(sox_handle h, const CUtensorMap *maps, const BcdArgs &a, int gri
 
 size_t tc_sigma_bytes(sox_handle h, int n, int N, int T, int S, bool two) {
   Geometry g = geometry(h, n, N, T, S, two);
-  return g.fixed_bytes + g.per_b_bytes * g.Bc + 64 * 1024;
+  return g.fixed_bytes + g.chunk_bytes(g.Bc) + 64 * 1024;
 }
 
 void tc_release(sox_handle) {}
@@ -135,7 +139,10 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
   __half *U1h = ar.take<__half>((size_t)NR * Kp2), *U1l = ar.take<__half>((size_t)NR * Kp2);
   float *inv_u1 = ar.take<float>(N);
   __half *U2h = ar.take<__half>((size_t)n * NR * Kp), *U2l = ar.take<__half>((size_t)n * NR * Kp);
-  float *inv_u2 = ar.take<float>(N);
+  float *inv_u2 = two ? ar.take<float>(N) : inv_u1;   // one split serves both slots
+  float *Xf = reinterpret_cast<float *>(ar.take<char>(rows_f32_bytes(N, n)));
+  Arena scr = ar;   // the mixed tensor's scratch, where the chunk buffers will lie
+  void *mix_scratch = scr.take<char>(g.scratch_bytes);
   // ---- per-chunk buffers ----
   double *GR64 = ar.take<double>((size_t)Bc * N * n), *GW64 = ar.take<double>((size_t)Bc * N * n);
   __half *GRh = ar.take<__half>((size_t)Bc * NR * Kp), *GRl = ar.take<__half>((size_t)Bc * NR * Kp);
@@ -149,25 +156,21 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
   float *Dt = ar.take<float>((size_t)Bc * N * N);
   float *Tm = ar.take<float>((size_t)Bc * N * n);
   int *symf = ar.take<int>((size_t)Bc);
-  if (!symf) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+  if (!symf || !mix_scratch) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
 
   const long long limit = h->spin_limit;
   auto grid_for = [&](long long tiles) { return (int)std::max<long long>(1, std::min<long long>(tiles, h->sm_count)); };
 
   // ---- mixed tensors (Eq. U_contraction at k = 0) ----
   {
-    ProfScope ps(h, "mixed_f32", s, two ? 4 : 2);
-    SOX_CUDA_TRY(cudaMemsetAsync(U1h, 0, hb((size_t)NR * Kp2), s));
-    SOX_CUDA_TRY(cudaMemsetAsync(U1l, 0, hb((size_t)NR * Kp2), s));
-    SOX_CUDA_TRY(cudaMemsetAsync(U2h, 0, hb((size_t)n * NR * Kp), s));
-    SOX_CUDA_TRY(cudaMemsetAsync(U2l, 0, hb((size_t)n * NR * Kp), s));
+    ProfScope ps(h, "mixed_f32", s, two ? 9 : 5);
+    launch_rows_f32(X, N, n, Xf, s);
     const double *src[2] = {U1, U2};
     for (int k = 0; k < (two ? 2 : 1); ++k) {
-      launch_mixed_f32(src[k], X, N, n, Kp, Uf, s);
+      launch_mixed_f32(src[k], X, N, n, Kp, Uf, mix_scratch, s);
       const bool slot1 = (k == 0), slot2 = two ? (k == 1) : true;
       launch_split_mixed(Uf, N, NR, n, Kp, slot1 ? U1h : nullptr, slot1 ? U1l : nullptr, slot2 ? U2h : nullptr,
                          slot2 ? U2l : nullptr, slot1 ? inv_u1 : inv_u2, s);
-      if (!two) SOX_CUDA_TRY(cudaMemcpyAsync(inv_u2, inv_u1, 4 * (size_t)N, cudaMemcpyDeviceToDevice, s));
     }
   }
 
@@ -249,7 +252,7 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
     }
     {  // back-projection to orbitals
       ProfScope ps(h, "backproject", s, 2);
-      launch_backproject_T(Dt, N, X, N, n, bc, Tm, s);
+      launch_backproject_T(Dt, N, Xf, N, n, bc, Tm, s);
       // bare SOX with a symmetric G(tau) has a symmetric Sigma(tau)
       // (a partial v range breaks that symmetry: then every block is computed)
       launch_backproject_sigma(X, Tm, N, n, bc, Sigma + (long long)b0 * n * n, (long long)n * n, s,
@@ -293,7 +296,7 @@ BatchGeo batch_geometry(sox_handle h, int count, const int *n, const int *N, con
     bg.Bc[i] = (int)B[i];
     fixed += g[i].fixed_bytes + 64 * 1024;
   }
-  auto chunk_mem = [&](int i) { return g[i].per_b_bytes * (size_t)bg.Bc[i]; };
+  auto chunk_mem = [&](int i) { return g[i].chunk_bytes(bg.Bc[i]); };
   for (;;) {
     size_t total = fixed;
     int hog = -1;
@@ -316,7 +319,8 @@ struct Inst {
   int n, N, T, S, Kp, NR, RG, Bc;
   const double *G, *X, *V;
   double *Sigma;
-  float *Uf, *inv_u1, *inv_u2;
+  float *Uf, *inv_u1, *inv_u2, *Xf;
+  void *mix_scratch;
   __half *U1h, *U1l, *U2h, *U2l;
   double *GR64, *GW64;
   __half *GRh, *GRl, *GWh, *GWl, *Gmh, *Gml, *Ah, *Al;
@@ -350,7 +354,10 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
     c.U1h = ar.take<__half>((size_t)NR * Kp2); c.U1l = ar.take<__half>((size_t)NR * Kp2);
     c.inv_u1 = ar.take<float>(NN);
     c.U2h = ar.take<__half>((size_t)nn * NR * Kp); c.U2l = ar.take<__half>((size_t)nn * NR * Kp);
-    c.inv_u2 = ar.take<float>(NN);
+    c.inv_u2 = c.inv_u1;   // one split serves both slots
+    c.Xf = reinterpret_cast<float *>(ar.take<char>(rows_f32_bytes(NN, nn)));
+    Arena scr = ar;   // the mixed tensor's scratch, where the chunk buffers will lie
+    c.mix_scratch = scr.take<char>(g.scratch_bytes);
     c.GR64 = ar.take<double>((size_t)Bc * NN * nn); c.GW64 = ar.take<double>((size_t)Bc * NN * nn);
     c.GRh = ar.take<__half>((size_t)Bc * NR * Kp); c.GRl = ar.take<__half>((size_t)Bc * NR * Kp);
     c.GWh = ar.take<__half>((size_t)Bc * NR * Kp); c.GWl = ar.take<__half>((size_t)Bc * NR * Kp);
@@ -363,7 +370,8 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
     c.Dt = ar.take<float>((size_t)Bc * NN * NN);
     c.Tm = ar.take<float>((size_t)Bc * NN * nn);
     c.symf = ar.take<int>((size_t)Bc);
-    if (!c.symf) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+    if (!c.symf || !c.mix_scratch) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+    ar.off = std::max(ar.off, scr.off);
     if (!make_tmap_f16_3d(&c.bcd[0], c.Ah, Kp, NR, (uint64_t)Bc * nn, 64, 128, &err) ||
         !make_tmap_f16_3d(&c.bcd[1], c.Al, Kp, NR, (uint64_t)Bc * nn, 64, 128, &err) ||
         !make_tmap_f16_3d(&c.bcd[2], c.GRh, Kp, NR, Bc, 64, 128, &err) ||
@@ -384,16 +392,11 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
   auto grid_for = [&](long long tiles) { return (int)std::max<long long>(1, std::min<long long>(tiles, h->sm_count)); };
   // mixed tensors of every instance (Eq. U_contraction at k = 0; one interaction in both slots)
   {
-    ProfScope ps(h, "mixed_f32", s, 2 * count);
+    ProfScope ps(h, "mixed_f32", s, 5 * count);
     for (Inst &c : in) {
-      const size_t Kp2 = (size_t)c.Kp * c.Kp;
-      SOX_CUDA_TRY(cudaMemsetAsync(c.U1h, 0, hb((size_t)c.NR * Kp2), s));
-      SOX_CUDA_TRY(cudaMemsetAsync(c.U1l, 0, hb((size_t)c.NR * Kp2), s));
-      SOX_CUDA_TRY(cudaMemsetAsync(c.U2h, 0, hb((size_t)c.n * c.NR * c.Kp), s));
-      SOX_CUDA_TRY(cudaMemsetAsync(c.U2l, 0, hb((size_t)c.n * c.NR * c.Kp), s));
-      launch_mixed_f32(c.V, c.X, c.N, c.n, c.Kp, c.Uf, s);
+      launch_rows_f32(c.X, c.N, c.n, c.Xf, s);
+      launch_mixed_f32(c.V, c.X, c.N, c.n, c.Kp, c.Uf, c.mix_scratch, s);
       launch_split_mixed(c.Uf, c.N, c.NR, c.n, c.Kp, c.U1h, c.U1l, c.U2h, c.U2l, c.inv_u1, s);
-      SOX_CUDA_TRY(cudaMemcpyAsync(c.inv_u2, c.inv_u1, 4 * (size_t)c.N, cudaMemcpyDeviceToDevice, s));
     }
   }
   // instances by cost per tile (n Kp), largest first: the persistent grid ends on cheap tiles
@@ -482,7 +485,7 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
       const int B = c.S * c.T, b0 = k * c.Bc, bc = std::min(c.Bc, B - b0);
       if (bc <= 0) continue;
       ProfScope ps(h, "backproject", s, 2);
-      launch_backproject_T(c.Dt, c.N, c.X, c.N, c.n, bc, c.Tm, s);
+      launch_backproject_T(c.Dt, c.N, c.Xf, c.N, c.n, bc, c.Tm, s);
       launch_backproject_sigma(c.X, c.Tm, c.N, c.n, bc, c.Sigma + (long long)b0 * c.n * c.n, (long long)c.n * c.n, s,
                                v_range_is_full(h, c.n) ? c.symf : nullptr);
     }
