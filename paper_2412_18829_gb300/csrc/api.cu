@@ -1287,10 +1287,14 @@ int sox_iw_to_tau(sox_handle h, const sox_problem *p, int n_w, const double *ome
     SOX_TRY(call.input(tails, 3 * S * nn, &sT));
     SOX_TRY(call.input(tau, (size_t)n_t, &st_));
     SOX_TRY(call.output(G_tau, S * n_t * nn, &oG));
+    const size_t scratch = sox::iw_to_tau_bytes(n_w, n_t);
     Arena ar;
-    SOX_TRY(call.begin(0, &ar));
-    sox::ProfScope ps(h, "iw_to_tau", call.stream());
-    sox::launch_iw_to_tau(sG.in, sw.in, n_w, sT.in, st_.in, n_t, p->n, p->n_spin, p->beta, oG.out, call.stream());
+    SOX_TRY(call.begin(scratch, &ar));
+    void *phases = ar.take<char>(scratch);
+    if (!phases) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+    sox::ProfScope ps(h, "iw_to_tau", call.stream(), 2);
+    sox::launch_iw_to_tau(sG.in, sw.in, n_w, sT.in, st_.in, n_t, p->n, p->n_spin, p->beta, phases, oG.out,
+                          call.stream());
     SOX_CUDA_TRY(cudaGetLastError());
     return call.end();
   }();
@@ -1339,6 +1343,13 @@ int sox_find_mu(sox_handle h, const sox_problem *p, int n_w, const double *omega
     SOX_TRY(call.input(Sigma_iw, 2 * S * n_w * nn, &sSi));
     SOX_TRY(call.input(Sigma_tau, S * p->n_tau * nn, &sSt));
     Arena ar;
+    if (sox::mu_on_device(p->n)) {
+      SOX_TRY(call.begin(sox::mu_bytes(n_w, p->n_spin), &ar));
+      SOX_TRY(sox::mu_bisect(h, p->n, p->n_tau, n_w, p->n_spin, sw.in, p->beta, target, sF.in, sSi.in, sSt.in, &lo, &hi,
+                             tol, max_iter, ar, call.stream()));
+      *mu = 0.5 * (lo + hi);
+      return call.end();
+    }
     const size_t extra = sox::aligned_bytes(2 * S * n_w * nn, 8) + sox::aligned_bytes(3 * S * nn, 8) + 4096;
     SOX_TRY(call.begin(sox::dyson_bytes(p->n, n_w, p->n_spin) + extra, &ar));
     cudaStream_t s = call.stream();
@@ -1351,7 +1362,6 @@ int sox_find_mu(sox_handle h, const sox_problem *p, int n_w, const double *omega
       Arena a2 = ar;
       SOX_TRY(sox::dyson(h, p->n, n_w, p->n_spin, sw.in, mid, sF.in, sSi.in, Giw, a2, s));
       sox::launch_green_tails(sF.in, mid, sSt.in, p->n, p->n_tau, p->n_spin, tails, s);
-      SOX_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(double), s));
       sox::launch_trace_gamma(Giw, sw.in, n_w, tails, p->n, p->n_spin, p->beta, count, s);
       h->launches += 3;
       double c = 0.0;
@@ -1389,7 +1399,7 @@ int sox_sigma_hf(sox_handle h, const sox_problem *p, const double *X, const doub
     SOX_TRY(call.begin(sox::aligned_bytes(N + S * N * p->n, 8) + sox::aligned_bytes(S * N * N, 8), &ar));
     double *d = ar.take<double>(N + S * N * p->n), *Gam = ar.take<double>(S * N * N);
     if (!Gam) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-    sox::ProfScope ps(h, "sigma_hf", call.stream(), 2 + 2 * p->n_spin);
+    sox::ProfScope ps(h, "sigma_hf", call.stream(), 3 + 2 * p->n_spin);
     sox::launch_sigma_hf(sX.in, sV.in, sg.in, p->N, p->n, p->n_spin, d, Gam, oS.out, call.stream());
     for (int sp = 0; oF.out && sp < p->n_spin; ++sp)   // F[s] = H0 + Sigma_HF[s]
       sox::launch_add_f64(sH.in, oS.out + sp * nn, oF.out + sp * nn, (long long)nn, call.stream());

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import synth
-from oracle import sox as osox
+from oracle import scloop, sox as osox
 from gpu_common import check, pkg_built, to_dev, torch_cuda
 
 pytestmark = pytest.mark.gpu
@@ -33,3 +33,53 @@ def test_mixed_tensor_and_half_transform_tiles(env, n, N):
     pkg.sox_sigma(hs["f16x2"], p, G, X, V, S)
     pkg.sox_check_device(hs["f16x2"])
     check(S.cpu().numpy(), osox.sox_sigma(w.X, w.V, w.G).real, "f16x2", f"n={n} N={N}", n=n, N=N)
+
+
+@pytest.mark.parametrize("n,n_spin", [(1, 1), (2, 2), (31, 1), (33, 2), (110, 1), (111, 1)])
+def test_dyson_and_mu_on_both_sides_of_the_shared_memory_rule(env, n, n_spin):
+    """Systems inverted in shared memory (n <= 110) and through the augmented elimination:
+    G(i w) against numpy's inverse with a condition-scaled bound, mu against the oracle's bisection."""
+    torch, pkg, hs = env
+    h = hs["fp64"]
+    rng = np.random.default_rng(n)
+    n_tau, beta, n_max, mu0 = 5, 4.0, 6 if n > 40 else 40, 0.1
+    F = rng.standard_normal((n_spin, n, n)) / np.sqrt(n)
+    F = 0.5 * (F + np.swapaxes(F, 1, 2))
+    om = scloop.fermionic_frequencies(beta, n_max)
+    S_tau = 0.05 * rng.standard_normal((n_spin, n_tau, n, n)) / np.sqrt(n)
+    S_iw = 0.05 * (rng.standard_normal((n_spin, om.size, n, n)) + 1j * rng.standard_normal((n_spin, om.size, n, n)))
+    S_iw /= np.sqrt(n)
+    p = pkg.problem(n, 8, n_tau, n_spin, beta)
+    Fd, Swd, Std, omd = to_dev(torch, F, S_iw, S_tau, om)
+    out = torch.empty(n_spin, om.size, n, n, dtype=torch.complex128, device="cuda")
+    pkg.sox_dyson(h, p, omd, mu0, Fd, Swd, out)
+    for s in range(n_spin):
+        ref = scloop.dyson(om, mu0, F[s], S_iw[s])
+        A = (1j * om + mu0)[:, None, None] * np.eye(n) - F[s] - S_iw[s]
+        # the forward error of an inverse with partial pivoting: n eps cond(A), a factor 8 to spare
+        bound = 8 * n * 2.0 ** -53 * np.linalg.cond(A).max() * np.abs(ref).max()
+        assert np.abs(out[s].cpu().numpy() - ref).max() <= bound
+    target = 0.5 * n * n_spin
+    got = pkg.sox_find_mu(h, p, omd, target, Fd, Swd, Std)
+    ref_mu = scloop.find_mu(om, beta, target, list(F), list(S_iw), list(S_tau))
+    assert abs(got - ref_mu) < 1e-9
+
+
+def test_find_mu_limits(env):
+    """max_iter ends the bisection early (the midpoint after that many halvings), and a
+    singular system is reported."""
+    torch, pkg, hs = env
+    h = hs["fp64"]
+    n, beta = 3, 4.0
+    om = scloop.fermionic_frequencies(beta, 8)
+    F = np.diag([-0.5, 0.1, 0.7])[None]
+    p = pkg.problem(n, 4, 3, 1, beta)
+    Fd, omd = to_dev(torch, F, om)
+    zt, zw = np.zeros((3, n, n)), np.zeros((om.size, n, n), complex)
+    for it in (1, 2, 7):
+        got = pkg.sox_find_mu(h, p, omd, 1.5, Fd, lo=-8.0, hi=8.0, max_iter=it)
+        ref = scloop.find_mu(om, beta, 1.5, [F[0]], [zw], [zt], lo=-8.0, hi=8.0, iters=it)
+        assert abs(got - ref) < 1e-12
+    zero, = to_dev(torch, np.zeros(2))
+    with pytest.raises(pkg.SoxError):
+        pkg.sox_find_mu(h, p, zero, 1.5, to_dev(torch, np.zeros((1, n, n)))[0], lo=-1.0, hi=1.0)
