@@ -8,6 +8,7 @@
 
 #include "adjoint.h"
 #include "dynamic.h"
+#include "f64_slices.h"
 #include "internal.h"
 #include "ctc.h"
 #include "kpoint.h"
@@ -553,32 +554,40 @@ int thc_project_G(sox_handle h, const sox_problem *p, const double *G, const dou
     SOX_TRY(call.output(G_Rq, nb * d.N * d.n, &oR));
     SOX_TRY(call.output(G_wP, nb * d.N * d.n, &oW));
     SOX_TRY(call.output(G_PQ, nb * d.N * d.N, &oP));
-    Arena ar;
-    SOX_TRY(call.begin(G_PQ && !G_Rq ? sox::aligned_bytes(nb * d.N * d.n, 8) : 0, &ar));
-    double *gr = oR.out ? oR.out : (G_PQ ? ar.take<double>(nb * d.N * d.n) : nullptr);
-    cudaStream_t s = call.stream();
     GemmF64 g;  // GR[b][R][q] = sum_u X[R][u] G[b][u][q]
     g.M = d.N; g.Nc = d.n; g.K = d.n; g.batch = (int)nb;
-    g.A = sX.in; g.ai = d.n; g.ak = 1;
-    g.B = sG.in; g.sB = d.nn(); g.bk = d.n; g.bj = 1;
-    g.C = gr; g.sC = (long long)d.N * d.n; g.ci = d.n; g.cj = 1;
+    g.ai = d.n; g.ak = 1;
+    g.sB = d.nn(); g.bk = d.n; g.bj = 1;
+    g.sC = (long long)d.N * d.n; g.ci = d.n; g.cj = 1;
+    GemmF64 w;  // G_wP[b][w][P] = sum_p G[b][w][p] X[P][p]
+    w.M = d.n; w.Nc = d.N; w.K = d.n; w.batch = (int)nb;
+    w.sA = d.nn(); w.ai = d.n; w.ak = 1;
+    w.bk = 1; w.bj = d.n;
+    w.sC = (long long)d.N * d.n; w.ci = d.N; w.cj = 1;
+    GemmF64 q;  // G_PQ[b][P][Q] = sum_q GR[b][P][q] X[Q][q]
+    q.M = d.N; q.Nc = d.N; q.K = d.n; q.batch = (int)nb;
+    q.sA = (long long)d.N * d.n; q.ai = d.n; q.ak = 1;
+    q.bk = 1; q.bj = d.n;
+    q.sC = (long long)d.N * d.N; q.ci = d.N; q.cj = 1;
+    size_t scratch = sox::gemm_f64_bytes(g);
+    if (G_wP) scratch = std::max(scratch, sox::gemm_f64_bytes(w));
+    if (G_PQ) scratch = std::max(scratch, sox::gemm_f64_bytes(q));
+    Arena ar;
+    SOX_TRY(call.begin((G_PQ && !G_Rq ? sox::aligned_bytes(nb * d.N * d.n, 8) : 0) + scratch, &ar));
+    double *gr = oR.out ? oR.out : (G_PQ ? ar.take<double>(nb * d.N * d.n) : nullptr);
+    cudaStream_t s = call.stream();
     sox::ProfScope ps(h, "project_f64", s, (gr ? 1 : 0) + (oW.out ? 1 : 0) + (oP.out ? 1 : 0));
-    if (gr) sox::launch_gemm_f64(g, s);
-    if (oW.out) {  // G_wP[b][w][P] = sum_p G[b][w][p] X[P][p]
-      GemmF64 w;
-      w.M = d.n; w.Nc = d.N; w.K = d.n; w.batch = (int)nb;
-      w.A = sG.in; w.sA = d.nn(); w.ai = d.n; w.ak = 1;
-      w.B = sX.in; w.bk = 1; w.bj = d.n;
-      w.C = oW.out; w.sC = (long long)d.N * d.n; w.ci = d.N; w.cj = 1;
-      sox::launch_gemm_f64(w, s);
+    if (gr) {
+      g.A = sX.in; g.B = sG.in; g.C = gr;
+      SOX_TRY(sox::gemm_f64(h, g, ar, s));
     }
-    if (oP.out) {  // G_PQ[b][P][Q] = sum_q GR[b][P][q] X[Q][q]
-      GemmF64 q;
-      q.M = d.N; q.Nc = d.N; q.K = d.n; q.batch = (int)nb;
-      q.A = gr; q.sA = (long long)d.N * d.n; q.ai = d.n; q.ak = 1;
-      q.B = sX.in; q.bk = 1; q.bj = d.n;
-      q.C = oP.out; q.sC = (long long)d.N * d.N; q.ci = d.N; q.cj = 1;
-      sox::launch_gemm_f64(q, s);
+    if (oW.out) {
+      w.A = sG.in; w.B = sX.in; w.C = oW.out;
+      SOX_TRY(sox::gemm_f64(h, w, ar, s));
+    }
+    if (oP.out) {
+      q.A = gr; q.B = sX.in; q.C = oP.out;
+      SOX_TRY(sox::gemm_f64(h, q, ar, s));
     }
     return call.end();
   }();
@@ -693,26 +702,29 @@ int sox_pi0(sox_handle h, const sox_problem *p, const double *G, const double *X
     SOX_TRY(call.input(w, (size_t)d.T, &sw));
     SOX_TRY(call.output(Pi0, (size_t)d.S * d.N * d.N, &oP));
     const size_t gpq = (size_t)d.T * d.N * d.N, gr = (size_t)d.T * d.N * d.n;
+    GemmF64 g;  // GR[j][P][q] = sum_p X[P][p] G[j][p][q]
+    g.M = d.N; g.Nc = d.n; g.K = d.n; g.batch = d.T;
+    g.ai = d.n; g.ak = 1;
+    g.sB = d.nn(); g.bk = d.n; g.bj = 1;
+    g.sC = (long long)d.N * d.n; g.ci = d.n; g.cj = 1;
+    GemmF64 q;  // GPQ[j][P][Q] = sum_q GR[j][P][q] X[Q][q]
+    q.M = d.N; q.Nc = d.N; q.K = d.n; q.batch = d.T;
+    q.sA = (long long)d.N * d.n; q.ai = d.n; q.ak = 1;
+    q.bk = 1; q.bj = d.n;
+    q.sC = (long long)d.N * d.N; q.ci = d.N; q.cj = 1;
     Arena ar;
-    SOX_TRY(call.begin(sox::aligned_bytes(gpq, 8) + sox::aligned_bytes(gr, 8), &ar));
+    SOX_TRY(call.begin(sox::aligned_bytes(gpq, 8) + sox::aligned_bytes(gr, 8) +
+                           std::max(sox::gemm_f64_bytes(g), sox::gemm_f64_bytes(q)), &ar));
     double *GPQ = ar.take<double>(gpq);
     double *GR = ar.take<double>(gr);
     cudaStream_t s = call.stream();
     for (int sp = 0; sp < d.S; ++sp) {
       const double *Gs = sG.in + (long long)sp * d.T * d.nn();
-      GemmF64 g;
-      g.M = d.N; g.Nc = d.n; g.K = d.n; g.batch = d.T;
-      g.A = sX.in; g.ai = d.n; g.ak = 1;
-      g.B = Gs; g.sB = d.nn(); g.bk = d.n; g.bj = 1;
-      g.C = GR; g.sC = (long long)d.N * d.n; g.ci = d.n; g.cj = 1;
       sox::ProfScope ps0(h, "project_f64", s, 2);
-      sox::launch_gemm_f64(g, s);
-      GemmF64 q;
-      q.M = d.N; q.Nc = d.N; q.K = d.n; q.batch = d.T;
-      q.A = GR; q.sA = (long long)d.N * d.n; q.ai = d.n; q.ak = 1;
-      q.B = sX.in; q.bk = 1; q.bj = d.n;
-      q.C = GPQ; q.sC = (long long)d.N * d.N; q.ci = d.N; q.cj = 1;
-      sox::launch_gemm_f64(q, s);
+      g.A = sX.in; g.B = Gs; g.C = GR;
+      SOX_TRY(sox::gemm_f64(h, g, ar, s));
+      q.A = GR; q.B = sX.in; q.C = GPQ;
+      SOX_TRY(sox::gemm_f64(h, q, ar, s));
       sox::ProfScope ps1(h, "pi0_reduce", s);
       sox::launch_pi0_reduce(GPQ, sw.in, d.N, d.T, oP.out + (long long)sp * d.N * d.N, s);
     }

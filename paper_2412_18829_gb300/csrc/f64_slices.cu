@@ -1,0 +1,576 @@
+#include "f64_slices.h"
+
+#include <algorithm>
+#include <string>
+
+#include "smem_attr.h"
+#include "tc_common.cuh"
+
+namespace sox {
+namespace {
+
+constexpr int kNonFinite = 1 << 20;
+
+// ------------------------------------------------------------------ slicing
+// Exponent field of x, subnormals counted with the smallest normal exponent.
+__device__ __forceinline__ int exp_field(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e == 0 ? 1 : e;
+}
+// x scaled by the row's exponent as an integer: x = X 2^-55 2^(E - 1022), |X| <= 2^55,
+// rounded to nearest (ties up)
+__device__ __forceinline__ long long fixed55(double x, int E) {
+  const long long bits = __double_as_longlong(x);
+  const int ef = (int)((bits >> 52) & 0x7ff);
+  long long m = bits & 0xfffffffffffffll;
+  if (ef) m |= 1ll << 52;
+  const int sh = E - (ef ? ef : 1) - 2;   // m 2^-sh
+  if (sh <= 0)
+    m <<= -sh;
+  else
+    m = sh > 60 ? 0 : (m + (1ll << (sh - 1))) >> sh;
+  return bits < 0 ? -m : m;
+}
+// Balanced base-256 digits of eight values, one 16-byte word of FP16 integers per digit.
+// An integer v in [0, 1023] is the FP16 number 1024 + v with v in its low bits.
+__device__ __forceinline__ void digits8(long long (&X)[8], uint4 (&w)[kSlices]) {
+#pragma unroll
+  for (int s = kSlices - 1; s >= 0; --s) {
+    uint32_t u[4];
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) {
+      int d[2];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (s > 0) {
+          d[t] = (int)(signed char)(X[e + t] & 0xff);
+          X[e + t] = (X[e + t] + 128) >> 8;
+        } else {
+          d[t] = (int)X[e + t];
+        }
+      }
+      const uint32_t v = 0x64006400u + (uint32_t)(d[0] + 128) + ((uint32_t)(d[1] + 128) << 16);
+      const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), __floats2half2_rn(1152.f, 1152.f));
+      u[e / 2] = *reinterpret_cast<const uint32_t *>(&h);
+    }
+    w[s] = make_uint4(u[0], u[1], u[2], u[3]);
+  }
+}
+
+// Rows with contiguous elements (sk == 1): `lpr` lanes per row.
+template <class T>
+__global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, long long sr, int rows, int batch,
+                                                    int batch_all, int K, int K8, int lpr, __half *p, int *ex) {
+  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long row = g / lpr;
+  const int l = (int)(g % lpr);
+  const bool live = row < (long long)rows * batch;
+  const T *x = live ? src + (row / rows) * sb + (row % rows) * sr : src;
+  int E = 1;
+  if (live)
+    for (int k = l; k < K; k += lpr) E = max(E, exp_field((double)x[k]));
+  for (int o = lpr / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+  if (!live) return;
+  const bool fin = E < 0x7ff;
+  if (l == 0) ex[row] = fin ? E : kNonFinite;
+  const long long plane = (long long)batch_all * rows * K8;
+  for (int c = l; c < K8 / 8; c += lpr) {
+    long long X[8];
+    uint4 w[kSlices];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int k = c * 8 + e;
+      X[e] = (fin && k < K) ? fixed55((double)x[k], E) : 0;
+    }
+    digits8(X, w);
+#pragma unroll
+    for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint4 *>(p + s * plane + row * K8 + c * 8) = w[s];
+  }
+}
+
+// Rows whose elements lie apart: 32 rows per block, transposed through shared memory.
+template <class T>
+__global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, long long sr, long long sk, int rows,
+                                                    int batch_all, int K, int K8, __half *p, int *ex) {
+  __shared__ long long sx[64][33];
+  __shared__ int se[8][32];
+  const int b = blockIdx.y, r0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const T *x = src + b * sb + (long long)(r0 + tx) * sr;
+  const bool in = r0 + tx < rows;
+  int E = 1;
+  if (in)
+    for (int k = ty; k < K; k += 8) E = max(E, exp_field((double)x[k * sk]));
+  se[ty][tx] = E;
+  __syncthreads();
+  E = 1;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) E = max(E, se[i][tx]);
+  const bool fin = E < 0x7ff;
+  if (ty == 0 && in) ex[(long long)b * rows + r0 + tx] = fin ? E : kNonFinite;
+  const long long plane = (long long)batch_all * rows * K8;
+  const int row = threadIdx.x / 8, c8 = threadIdx.x % 8;
+  for (int k0 = 0; k0 < K8; k0 += 64) {
+    __syncthreads();
+    for (int k = ty; k < 64; k += 8)
+      sx[k][tx] = (in && fin && k0 + k < K) ? fixed55((double)x[(k0 + k) * sk], E) : 0;
+    __syncthreads();
+    if (r0 + row < rows && k0 + c8 * 8 < K8) {
+      long long X[8];
+      uint4 w[kSlices];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) X[e] = sx[c8 * 8 + e][row];
+      digits8(X, w);
+      const long long o = ((long long)b * rows + r0 + row) * K8 + k0 + c8 * 8;
+#pragma unroll
+      for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint4 *>(p + s * plane + o) = w[s];
+    }
+  }
+}
+
+// ------------------------------------------------------------------ product
+// 128 (lane side, TMEM lanes) x 64 output tiles: the eight FP32 sums of a tile fill the 512
+// TMEM columns.  K goes in chunks of 32 (64-byte swizzled rows, seven digit tiles of both
+// operands, 84 KB a stage, two stages) and in windows of 128, after which the sums are
+// read out; each sum's columns are handed back as soon as they are read, so the next window's
+// first products run while the later sums are still being read.
+// Bound by the MMAs (34 of 128 x 64 x 16 per 16 of K) and, at K <= 128, by reading the sums
+// out in equal parts; the FP64 pipe (1.6 FMA a clock and SM) sees no instruction of it.
+// n = 120, N = 600, 160 batches: projections 2.84 ms on the FP64 pipe, 0.35 ms here with the
+// slicing; final sum (K = 600) 1.74 -> 0.43 ms.  n = 250, N = 2000, 12 times: X G X^T 27.9 -> 1.7 ms.
+constexpr int kL = 128, kW = 64, kKc = 32, kWin = 4;   // kWin chunks per window
+constexpr int kLBytes = kL * kKc * 2, kWBytes = kW * kKc * 2;
+constexpr int kStageBytes = kSlices * (kLBytes + kWBytes);
+constexpr int kStages = 2;
+constexpr int kThreads = 320;   // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
+constexpr int kGroups = 8;
+
+struct Bars {
+  uint64_t full[kStages], empty[kStages];
+  uint64_t acc_full, acc_empty[kGroups];
+  uint64_t drain;
+  uint32_t tmem_base;
+  int abort;
+};
+
+struct Args {
+  int nL, nW, K, batch, tL, tW;
+  int bL, bW;                // batches of the operands (1: shared)
+  const int *eL, *eW;
+  double *C;
+  long long sC, cl, cw;
+  double alpha, beta;
+  const int *skip, *mirror;
+  int lane_is_row;           // lane index is C's row index i (else its column index j)
+  // sources, for rows with infinities or NaNs
+  const void *xL, *xW;
+  int f32L, f32W;
+  long long sbL, srL, skL, sbW, srW, skW;
+  long long spin_limit;
+  int *status;
+};
+
+__device__ __forceinline__ uint64_t desc_kmajor_sw64(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(512 >> 4) << 32;   // next 8-row group
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;            // 64-byte swizzle
+  return d;
+}
+
+__device__ __forceinline__ long long wind_down(long long cap) { return cap > (1LL << 20) ? cap : (1LL << 20); }
+
+// All products of one chunk with KS 16-wide steps, sums in ascending order; on the window's
+// first chunk each sum waits until the epilogue has read its columns.
+template <int KS>
+__device__ __forceinline__ bool issue_chunk(uint32_t tmem, uint32_t st, bool first, Bars *bar, uint32_t ph,
+                                            long long limit, volatile int *abort, int *status) {
+  constexpr uint32_t idesc = tc::idesc_f16_f32(kL, kW);
+  const uint32_t w0 = st + kSlices * kLBytes;
+#pragma unroll 1
+  for (int g = 0; g < kGroups; ++g) {
+    if (first) {
+      if (!tc::mbar_wait(&bar->acc_empty[g], ph, limit, abort, status, 2)) return false;
+      tc::tc_fence_after();
+    }
+    const int i0 = g < kSlices ? 0 : g - (kSlices - 1), i1 = g < kSlices ? g : kSlices - 1;
+    for (int i = i0; i <= i1; ++i) {
+      const uint32_t a = st + i * kLBytes, w = w0 + (g - i) * kWBytes;
+#pragma unroll
+      for (int k = 0; k < KS; ++k)
+        tc::mma_f16(tmem + g * kW, desc_kmajor_sw64(a + k * 32), desc_kmajor_sw64(w + k * 32), idesc,
+                    (first && i == i0 && k == 0) ? 0u : 1u);
+    }
+  }
+  return true;
+}
+
+__device__ __forceinline__ double plain_at(const void *x, int f32, long long o) {
+  return f32 ? (double)static_cast<const float *>(x)[o] : static_cast<const double *>(x)[o];
+}
+// the element as a chain of FP64 FMAs from the sources (rows with infinities or NaNs)
+__device__ __noinline__ double plain_element(const Args &a, int b, int l, int w) {
+  const long long oL = (a.bL == 1 ? 0LL : b * a.sbL) + l * a.srL, oW = (a.bW == 1 ? 0LL : b * a.sbW) + w * a.srW;
+  double acc = 0.0;
+  for (int k = 0; k < a.K; ++k)
+    acc = fma(plain_at(a.xL, a.f32L, oL + k * a.skL), plain_at(a.xW, a.f32W, oW + k * a.skW), acc);
+  return acc;
+}
+
+__device__ __noinline__ double slow_scale(long long I, int x) { return scalbn((double)I, x); }
+
+// I 2^(x) rounded to nearest even, from integer instructions (a 64-bit conversion and a
+// scaling would cost the FP64 pipe more than all products of the element did)
+__device__ __forceinline__ double scaled_double(long long I, int x) {
+  if (I == 0) return 0.0;
+  const unsigned long long u = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << lz;
+  unsigned long long r = m >> 11;
+  const unsigned rem = (unsigned)(m & 0x7ff);
+  r += (rem > 0x400u || (rem == 0x400u && (r & 1))) ? 1u : 0u;
+  const int eb = 63 - lz + x + 1023;   // biased exponent of the leading bit
+  if (eb < 1 || eb > 2045) return slow_scale(I, x);   // subnormal or beyond FP64
+  const unsigned long long b =
+      ((unsigned long long)(eb - 1) << 52) + r + (I < 0 ? 0x8000000000000000ull : 0ull);
+  return __longlong_as_double((long long)b);
+}
+
+// LK: the sums of a tile stay below 2^LK (K <= 2^LK), kept as integers of 2^-(62 - LK)
+template <int LK>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_slice_gemm(const __grid_constant__ CUtensorMap tmL, const __grid_constant__ CUtensorMap tmW, const Args a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  Bars *bar = reinterpret_cast<Bars *>(smem + kStages * kStageBytes);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const long long per_b = (long long)a.tL * a.tW, total = per_b * a.batch;
+  const int nkc = (a.K + kKc - 1) / kKc, nwin = (nkc + kWin - 1) / kWin;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      tc::mbar_init(&bar->full[s], 1);
+      tc::mbar_init(&bar->empty[s], 1);
+    }
+    tc::mbar_init(&bar->acc_full, 1);
+    for (int g = 0; g < kGroups; ++g) tc::mbar_init(&bar->acc_empty[g], 8);
+    tc::mbar_init(&bar->drain, 1);
+    bar->abort = 0;
+    tc::fence_barrier_init();
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(&bar->tmem_base, 512);
+    tc::tmem_relinquish();
+  }
+  if (warp == 0 && lane == 0) {
+    tc::prefetch_tmap(&tmL);
+    tc::prefetch_tmap(&tmW);
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+  volatile int *abort = &bar->abort;
+  const long long limit = a.spin_limit;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      long long it = 0;
+      for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+        const int b = (int)(t / per_b), r = (int)(t % per_b);
+        if (a.skip && a.skip[b]) continue;
+        const int l0 = (r % a.tL) * kL, w0 = (r / a.tL) * kW;
+        const int zl = a.bL == 1 ? 0 : b, zw = a.bW == 1 ? 0 : b;
+        for (int kc = 0; kc < nkc; ++kc, ++it) {
+          const int s = (int)(it % kStages);
+          if (!tc::mbar_wait(&bar->empty[s], (uint32_t)((it / kStages) & 1) ^ 1u, limit, abort, a.status, 1)) break;
+          tc::mbar_arrive_expect_tx(&bar->full[s], kStageBytes);
+          uint8_t *st = smem + (size_t)s * kStageBytes;
+          for (int d = 0; d < kSlices; ++d) {
+            tc::tma_load_3d(st + d * kLBytes, &tmL, &bar->full[s], kc * kKc, l0, d * a.bL + zl);
+            tc::tma_load_3d(st + kSlices * kLBytes + d * kWBytes, &tmW, &bar->full[s], kc * kKc, w0, d * a.bW + zw);
+          }
+        }
+      }
+      // every stage issued has landed before the CTA exits
+      for (int s = 0; s < kStages; ++s) {
+        const long long n = it / kStages + ((it % kStages) > s ? 1 : 0);   // phases issued on stage s
+        if (n > 0)
+          for (long long i = 0; i < wind_down(limit) && !tc::mbar_try_wait(&bar->full[s], (uint32_t)((n - 1) & 1)); ++i) {
+          }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      long long it = 0, win = 0;
+      bool ok = true;
+      for (long long t = blockIdx.x; t < total && ok && !*abort; t += gridDim.x) {
+        if (a.skip && a.skip[(int)(t / per_b)]) continue;
+        for (int w = 0; w < nwin && ok; ++w, ++win) {
+          const int c1 = min(nkc, (w + 1) * kWin);
+          for (int kc = w * kWin; kc < c1; ++kc, ++it) {
+            const int s = (int)(it % kStages);
+            ok = tc::mbar_wait(&bar->full[s], (uint32_t)((it / kStages) & 1), limit, abort, a.status, 4);
+            if (!ok) break;
+            tc::tc_fence_after();
+            const uint32_t st = tc::smem_u32(smem + (size_t)s * kStageBytes);
+            const bool first = kc == w * kWin;
+            const uint32_t ph = (uint32_t)(win & 1) ^ 1u;
+            ok = (a.K - kc * kKc > 16) ? issue_chunk<2>(tmem, st, first, bar, ph, limit, abort, a.status)
+                                       : issue_chunk<1>(tmem, st, first, bar, ph, limit, abort, a.status);
+            if (!ok) break;
+            tc::mma_commit(&bar->empty[s]);
+          }
+          if (ok) tc::mma_commit(&bar->acc_full);
+        }
+      }
+      tc::mma_commit(&bar->drain);
+      for (long long i = 0; i < wind_down(limit) && !tc::mbar_try_wait(&bar->drain, 0); ++i) {
+      }
+    }
+  } else {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const int lr = q * 32 + lane;
+    long long win = 0;
+    for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+      const int b = (int)(t / per_b), r = (int)(t % per_b);
+      if (a.skip && a.skip[b]) continue;
+      const int l = (r % a.tL) * kL + lr, w0 = (r / a.tL) * kW + half * 32;
+      long long acc[32];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) acc[j] = 0;
+      bool ok = true;
+      for (int w = 0; w < nwin; ++w, ++win) {
+        ok = tc::mbar_wait(&bar->acc_full, (uint32_t)(win & 1), limit, abort, a.status, 8);
+        if (!ok) break;
+        tc::tc_fence_after();
+        const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + half * 32;
+        float low[32];
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) {
+          float v[32];
+          tc::tmem_ld_32x32b_x32(base + g * kW, v);
+          tc::tmem_ld_wait();
+          tc::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&bar->acc_empty[g]);
+          // sum g has the unit 2^-(8 g + 14); those with bits below the integer's unit are
+          // added in FP32 first and rounded once
+          constexpr int top = 62 - LK - 14, kLow = top / 8 + 1;   // first sum with such bits
+          const int sh = top - 8 * g;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            if (g < kLow)
+              acc[j] += (long long)__float2int_rn(v[j]) << (g < kLow ? sh : 0);
+            else if (g == kLow)
+              low[j] = v[j];
+            else
+              low[j] = fmaf(v[j], 1.f / (float)(1 << (8 * (g - kLow))), low[j]);
+            if (g == kGroups - 1)
+              acc[j] += (long long)__float2int_rn(low[j] * (1.f / (float)(1 << (8 * kLow - top))));
+          }
+        }
+      }
+      if (!ok) break;
+      if (l >= a.nL) continue;
+      const int eL = a.eL[(a.bL == 1 ? 0LL : (long long)b * a.nL) + l];
+      double *C = a.C + b * a.sC + l * a.cl;
+      const bool mir = a.mirror && a.mirror[b];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const int w = w0 + j;
+        if (w < a.nW) {
+          const int eW = a.eW[(a.bW == 1 ? 0LL : (long long)b * a.nW) + w];
+          double v;
+          if (eL == kNonFinite || eW == kNonFinite)
+            v = plain_element(a, b, l, w);
+          else
+            v = scaled_double(acc[j], eL + eW - 2044 - (62 - LK));
+          if (a.alpha != 1.0) v = a.alpha == -1.0 ? -v : a.alpha * v;
+          double *c = C + w * a.cw;
+          if (a.beta != 0.0) v = fma(a.beta, *c, v);
+          const int ib = (a.lane_is_row ? l : w) / 32, jb = (a.lane_is_row ? w : l) / 32;
+          if (!mir || ib <= jb) *c = v;
+          if (mir && ib < jb) a.C[b * a.sC + w * a.cl + l * a.cw] = v;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, 512);
+  }
+}
+
+size_t smem_bytes() { return (size_t)kStages * kStageBytes + sizeof(Bars) + 1024; }
+
+bool make_map(CUtensorMap *map, const SliceOp &op, int box_rows, std::string *err) {
+  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  if (!encode) {
+    cudaDriverEntryPointQueryResult q;
+    void *fn = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess || !fn) {
+      *err = "cuTensorMapEncodeTiled entry point not available";
+      return false;
+    }
+    encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+  }
+  cuuint64_t dims[3] = {(cuuint64_t)op.K8, (cuuint64_t)op.rows, (cuuint64_t)kSlices * op.batch};
+  cuuint64_t strides[2] = {(cuuint64_t)op.K8 * 2, (cuuint64_t)op.K8 * op.rows * 2};
+  cuuint32_t box[3] = {kKc, (cuuint32_t)box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, op.p, dims, strides, box, estr,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    *err = "cuTensorMapEncodeTiled (slices) failed with CUresult " + std::to_string((int)r);
+    return false;
+  }
+  return true;
+}
+
+inline int round8(int x) { return (x + 7) & ~7; }
+inline size_t al(size_t b) { return (b + 255) & ~size_t(255); }
+
+}  // namespace
+
+size_t slice_bytes(long long batch, int rows, int K) {
+  return al((size_t)kSlices * batch * rows * round8(K) * 2) + al((size_t)batch * rows * 4);
+}
+
+SliceOp slice_take(Arena &ar, int batch, int rows, int K) {
+  SliceOp op;
+  op.batch = batch;
+  op.rows = rows;
+  op.K = K;
+  op.K8 = round8(K);
+  op.p = ar.take<__half>((size_t)kSlices * batch * rows * op.K8);
+  op.ex = ar.take<int>((size_t)batch * rows);
+  if (!op.ex) op.p = nullptr;
+  return op;
+}
+
+void slice_rows(const void *src, bool f32, long long sb, long long sr, long long sk, int batch, SliceOp &op,
+                cudaStream_t s) {
+  op.src = src;
+  op.f32 = f32;
+  op.sb = sb;
+  op.sr = sr;
+  op.sk = sk;
+  if (batch <= 0 || op.rows <= 0) return;
+  if (sk == 1) {
+    int lpr = 4;
+    while (lpr < 32 && lpr * 8 < op.K8) lpr *= 2;
+    const long long blocks = ((long long)batch * op.rows * lpr + 255) / 256;
+    if (f32)
+      k_slice_rows<float><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const float *>(src), sb, sr, op.rows, batch,
+                                                         op.batch, op.K, op.K8, lpr, op.p, op.ex);
+    else
+      k_slice_rows<double><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const double *>(src), sb, sr, op.rows, batch,
+                                                          op.batch, op.K, op.K8, lpr, op.p, op.ex);
+  } else {
+    const dim3 grid((op.rows + 31) / 32, batch);
+    if (f32)
+      k_slice_cols<float><<<grid, 256, 0, s>>>(static_cast<const float *>(src), sb, sr, sk, op.rows, op.batch, op.K,
+                                               op.K8, op.p, op.ex);
+    else
+      k_slice_cols<double><<<grid, 256, 0, s>>>(static_cast<const double *>(src), sb, sr, sk, op.rows, op.batch, op.K,
+                                                op.K8, op.p, op.ex);
+  }
+}
+
+Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceGemm &g, cudaStream_t s) {
+  if (g.batch <= 0 || A.rows <= 0 || B.rows <= 0) return Status::ok();
+  // TMEM lanes along the index that leaves less padding in the 128 x 64 tiles; equal: along
+  // the one that is contiguous in C
+  auto area = [](int l, int w) { return (long long)((l + kL - 1) / kL) * kL * ((w + kW - 1) / kW) * kW; };
+  const long long ab = area(A.rows, B.rows), ba = area(B.rows, A.rows);
+  const bool lane_a = ab != ba ? ab < ba : g.ci == 1;
+  const SliceOp &L = lane_a ? A : B, &W = lane_a ? B : A;
+  CUtensorMap mL, mW;
+  std::string err;
+  if (!make_map(&mL, L, kL, &err) || !make_map(&mW, W, kW, &err)) return {SOX_ERR_CUDA, err};
+  Args a;
+  a.nL = L.rows; a.nW = W.rows; a.K = A.K; a.batch = g.batch;
+  a.tL = (L.rows + kL - 1) / kL;
+  a.tW = (W.rows + kW - 1) / kW;
+  a.bL = L.batch; a.bW = W.batch;
+  a.eL = L.ex; a.eW = W.ex;
+  a.C = g.C; a.sC = g.sC;
+  a.cl = lane_a ? g.ci : g.cj;
+  a.cw = lane_a ? g.cj : g.ci;
+  a.alpha = g.alpha; a.beta = g.beta;
+  a.skip = g.skip; a.mirror = g.mirror;
+  a.lane_is_row = lane_a ? 1 : 0;
+  a.xL = L.src; a.xW = W.src;
+  a.f32L = L.f32; a.f32W = W.f32;
+  a.sbL = L.sb; a.srL = L.sr; a.skL = L.sk;
+  a.sbW = W.sb; a.srW = W.sr; a.skW = W.sk;
+  a.spin_limit = h->spin_limit;
+  a.status = h->d_status;
+  const long long tiles = (long long)a.tL * a.tW * a.batch;
+  const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, h->sm_count));
+  static std::atomic<unsigned long long> attr7{0}, attr10{0};
+  if (a.K <= 128) {
+    SOX_CUDA_TRY(set_smem_once(k_slice_gemm<7>, (int)smem_bytes(), attr7));
+    k_slice_gemm<7><<<grid, kThreads, smem_bytes(), s>>>(mL, mW, a);
+  } else {
+    SOX_CUDA_TRY(set_smem_once(k_slice_gemm<10>, (int)smem_bytes(), attr10));
+    k_slice_gemm<10><<<grid, kThreads, smem_bytes(), s>>>(mL, mW, a);
+  }
+  SOX_CUDA_TRY(cudaGetLastError());
+  return Status::ok();
+}
+
+// The FP64 pipe makes 0.48e12 multiply-adds a second on a full grid: 31 us at the line, where
+// slicing both operands and the product take about 20 us in three launches.
+bool slices_pay(long long M, long long N, long long K, long long batch) {
+  return (double)M * (double)N * (double)K * (double)batch >= 1.5e7;
+}
+
+namespace {
+// the operands of g as (batch, rows) with one block where the stride is 0 or the batch is 1
+struct Ops {
+  int bA, bB;
+};
+Ops ops_of(const GemmF64 &g) {
+  return {(g.batch == 1 || g.sA == 0) ? 1 : g.batch, (g.batch == 1 || g.sB == 0) ? 1 : g.batch};
+}
+}  // namespace
+
+size_t gemm_f64_bytes(const GemmF64 &g) {
+  if (!slices_pay(g.M, g.Nc, g.K, g.batch)) return 0;
+  const Ops o = ops_of(g);
+  const int k = std::min(g.K, kSliceMaxK);
+  return slice_bytes(o.bA, g.M, k) + slice_bytes(o.bB, g.Nc, k);
+}
+
+Status gemm_f64(sox_handle h, const GemmF64 &g, Arena scratch, cudaStream_t s) {
+  if (g.M <= 0 || g.Nc <= 0 || g.batch <= 0) return Status::ok();
+  if (!h || !slices_pay(g.M, g.Nc, g.K, g.batch)) {
+    launch_gemm_f64(g, s);
+    return Status::ok();
+  }
+  const Ops o = ops_of(g);
+  for (int k0 = 0; k0 < g.K; k0 += kSliceMaxK) {
+    const int k = std::min(kSliceMaxK, g.K - k0);
+    Arena ar = scratch;
+    SliceOp A = slice_take(ar, o.bA, g.M, k), B = slice_take(ar, o.bB, g.Nc, k);
+    if (!A.p || !B.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+    slice_rows(g.A + k0 * g.ak, false, g.sA, g.ai, g.ak, o.bA, A, s);
+    slice_rows(g.B + k0 * g.bk, false, g.sB, g.bj, g.bk, o.bB, B, s);
+    SliceGemm sg;
+    sg.C = g.C; sg.sC = g.sC; sg.ci = g.ci; sg.cj = g.cj;
+    sg.alpha = g.alpha;
+    sg.beta = k0 == 0 ? g.beta : 1.0;
+    sg.batch = g.batch;
+    sg.skip = g.skip;
+    SOX_TRY(slice_gemm(h, A, B, sg, s));
+    h->launches += 2;   // the two slicings; callers count the product
+  }
+  return Status::ok();
+}
+
+}  // namespace sox

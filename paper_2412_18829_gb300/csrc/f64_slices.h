@@ -1,0 +1,64 @@
+// FP64 matrix products on the FP16 tensor cores (f64_slices.cu).
+//
+// Each row of an operand (its K elements) is scaled by a power of two and written as seven
+// 8-bit signed digits, x = 2^e sum_i d_i 2^-(8 i + 7), |d_i| <= 128, each digit an FP16
+// integer.  Digit products d_i d_j are exact in the tensor core, and so are their FP32 sums
+// over 128 elements (at most 7 * 128 * 2^14 < 2^24).  Products with equal i + j share one
+// accumulator; i + j <= 7 are kept (34 of 49).  The eight sums are added as 64-bit integers
+// and rounded to FP64 once.  What is dropped lies below 2^-63 of (row maximum x column
+// maximum) per term, so the result is closer to the exact sum than a chain of FP64 FMAs.
+// This is the Ozaki splitting (error-free transformation of a matrix product into exact
+// lower-precision ones; Ozaki, Ogita, Oishi and Rump, 2012), with the digits on the K-major
+// operand layout of tcgen05.
+#pragma once
+#include <cuda_fp16.h>
+
+#include "internal.h"
+
+namespace sox {
+
+constexpr int kSlices = 7;
+
+// A sliced operand: `batch` blocks of `rows` rows of K elements, digit s of (b, r, k) at
+// p[((s * batch + b) * rows + r) * K8 + k]; ex[b * rows + r] the row's exponent (kNonFinite:
+// the row holds an infinity or a NaN).  src and its strides stay readable until the products
+// that use the operand are done.
+struct SliceOp {
+  __half *p = nullptr;
+  int *ex = nullptr;
+  int batch = 0, rows = 0, K = 0, K8 = 0;
+  const void *src = nullptr;
+  bool f32 = false;
+  long long sb = 0, sr = 0, sk = 0;
+};
+size_t slice_bytes(long long batch, int rows, int K);
+SliceOp slice_take(Arena &ar, int batch, int rows, int K);
+// digits of element (b, r, k) = src[b * sb + r * sr + k * sk], FP64 or FP32; `batch` blocks
+// (at most op's)
+void slice_rows(const void *src, bool f32, long long sb, long long sr, long long sk, int batch, SliceOp &op,
+                cudaStream_t s);
+
+// C[b](i, j) = alpha sum_k A(b, i, k) B(b, j, k) + beta C[b](i, j); an operand of batch 1 is
+// shared.  Element (i, j) at C + b * sC + i * ci + j * cj.
+struct SliceGemm {
+  double *C = nullptr;
+  long long sC = 0, ci = 0, cj = 0;
+  double alpha = 1.0, beta = 0.0;
+  int batch = 1;
+  const int *skip = nullptr;     // batch b is left out when skip[b] != 0
+  const int *mirror = nullptr;   // mirror[b] != 0: square C, only the 32 x 32 blocks with i / 32 <= j / 32
+                                 // are computed and the others are their mirror images
+};
+// K <= kSliceMaxK per call
+constexpr int kSliceMaxK = 1024;
+Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceGemm &g, cudaStream_t s);
+
+// Whether a product of these sizes is faster through slices than on the FP64 pipe.
+bool slices_pay(long long M, long long N, long long K, long long batch);
+
+// Any GemmF64 through slices (operands sliced into `scratch`, K in blocks of kSliceMaxK), or
+// on the FP64 pipe where slices_pay says so.  gemm_f64_bytes: the scratch it needs (0 without).
+size_t gemm_f64_bytes(const GemmF64 &g);
+Status gemm_f64(sox_handle h, const GemmF64 &g, Arena scratch, cudaStream_t s);
+
+}  // namespace sox

@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "f64_slices.h"
 #include "tc_kernels.h"
 #include "tc_path.h"
 
@@ -29,6 +30,7 @@ struct Geometry {
   int RG;   // rows allocated for G(-tau)^T (>= 128)
   int Bc;   // (spin, tau) batches per chunk
   size_t fixed_bytes, per_b_bytes, scratch_bytes;
+  bool slices;   // the FP64 products run as digit slices on the tensor cores
   // the chunk buffers of Bc batches; the mixed tensor's scratch lies in them before the first chunk
   size_t chunk_bytes(int bc) const { return std::max(per_b_bytes * (size_t)bc, scratch_bytes); }
 };
@@ -36,6 +38,12 @@ struct Geometry {
 size_t hb(size_t count) { return aligned_bytes(count, 2); }   // FP16 buffer
 size_t fb(size_t count) { return aligned_bytes(count, 4); }   // FP32 buffer
 size_t db(size_t count) { return aligned_bytes(count, 8); }   // FP64 buffer
+
+size_t xt_slice_bytes(int N, int n) {
+  size_t b = 0;
+  for (int k0 = 0; k0 < N; k0 += kSliceMaxK) b += slice_bytes(1, n, std::min(kSliceMaxK, N - k0));
+  return b;
+}
 
 Geometry geometry(sox_handle h, int n, int N, int T, int S, bool two) {
   Geometry g{};
@@ -48,7 +56,8 @@ Geometry geometry(sox_handle h, int n, int N, int T, int S, bool two) {
   g.fixed_bytes = fb((size_t)g.N * Kp2)                             // FP32 mixed tensor
                   + 2 * hb((size_t)g.NR * Kp2) + fb(g.N)              // U1 split
                   + 2 * hb((size_t)g.n * g.NR * g.Kp) + fb(g.N)       // U2 split
-                  + aligned_bytes(rows_f32_bytes(N, n), 1);           // X in FP32
+                  + aligned_bytes(rows_f32_bytes(N, n), 1)            // X in FP32
+                  + slice_bytes(1, N, n) + xt_slice_bytes(N, n);      // digits of X, X^T
   g.scratch_bytes = aligned_bytes(mixed_f32_scratch(N, n), 1);
   g.per_b_bytes = 2 * db((size_t)N * n)                                // FP64 projections
                   + 4 * hb((size_t)g.NR * g.Kp) + 2 * fb(N)           // GR / GW splits
@@ -57,11 +66,94 @@ Geometry geometry(sox_handle h, int n, int N, int T, int S, bool two) {
                   + 2 * hb((size_t)n * g.NR * g.Kp)                   // A split
                   + 2 * fb(N)                                         // row/col factors
                   + fb((size_t)N * N) + fb((size_t)N * n) + 4096      // Dt, T
-                  + fb(1);                                            // symmetry flag
+                  + fb(1)                                             // symmetry flag
+                  + std::max(2 * slice_bytes(1, n, n),                // digits of G, or of T
+                             slice_bytes(1, n, std::min(N, kSliceMaxK)));
   long long c = (long long)(chunk_budget(h, kChunkBudget) / std::max<size_t>(g.per_b_bytes, 1));
   c = std::max<long long>(1, std::min<long long>(c, (long long)T * S));
   g.Bc = (int)c;
+  g.slices = slices_pay(N, n, n, (long long)T * S);
   return g;
+}
+
+// ---- the FP64 products of the chain (projections, final sum), on the FP64 pipe or as slices
+struct F64Ops {
+  bool on = false;
+  SliceOp X;                  // rows R, K = orbitals
+  std::vector<SliceOp> XT;    // rows t, K = R in blocks of kSliceMaxK
+};
+
+F64Ops f64_take(Arena &ar, const Geometry &g) {
+  F64Ops f;
+  f.on = g.slices;
+  f.X = slice_take(ar, 1, g.N, g.n);
+  for (int k0 = 0; k0 < g.N; k0 += kSliceMaxK) f.XT.push_back(slice_take(ar, 1, g.n, std::min(kSliceMaxK, g.N - k0)));
+  return f;
+}
+
+void f64_slice_x(sox_handle h, F64Ops &f, const double *X, int n, cudaStream_t s) {
+  if (!f.on) return;
+  slice_rows(X, false, 0, n, 1, 1, f.X, s);
+  for (size_t i = 0; i < f.XT.size(); ++i) slice_rows(X + (long long)i * kSliceMaxK * n, false, 0, 1, n, 1, f.XT[i], s);
+  h->launches += 1 + (long long)f.XT.size();
+}
+
+// FP64 projections G_Rq = X G, G_wP^T = X G^T of bc batches.  For a symmetric G(tau) (real
+// molecular orbitals) G_wP^T = G_Rq: batches flagged in symf leave the second product out.
+Status project_f64(sox_handle h, const F64Ops &f, const double *Gc, const double *X, int N, int n, int bc,
+                   const int *symf, double *GR64, double *GW64, Arena scratch, cudaStream_t s) {
+  const long long nn = (long long)n * n;
+  if (f.on) {
+    SliceOp Gq = slice_take(scratch, bc, n, n), Gw = slice_take(scratch, bc, n, n);
+    if (!Gq.p || !Gw.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+    slice_rows(Gc, false, nn, 1, n, bc, Gq, s);
+    slice_rows(Gc, false, nn, n, 1, bc, Gw, s);
+    h->launches += 2;
+    SliceGemm g;
+    g.batch = bc;
+    g.C = GR64; g.sC = (long long)N * n; g.ci = n; g.cj = 1;
+    SOX_TRY(slice_gemm(h, f.X, Gq, g, s));
+    g.C = GW64;
+    g.skip = symf;
+    return slice_gemm(h, f.X, Gw, g, s);
+  }
+  GemmF64 gp;
+  gp.M = N; gp.Nc = n; gp.K = n; gp.batch = bc;
+  gp.A = X; gp.ai = n; gp.ak = 1;
+  gp.B = Gc; gp.sB = nn; gp.bk = n; gp.bj = 1;
+  gp.C = GR64; gp.sC = (long long)N * n; gp.ci = n; gp.cj = 1;
+  launch_gemm_f64(gp, s);
+  GemmF64 gw = gp;
+  gw.bk = 1; gw.bj = n;
+  gw.C = GW64;
+  gw.skip = symf;
+  launch_gemm_f64(gw, s);
+  return Status::ok();
+}
+
+// Sigma[b] = -X^T T[b], FP64 (sym: as launch_backproject_sigma)
+Status final_sum_f64(sox_handle h, const F64Ops &f, const double *X, const float *Tm, int N, int n, int bc,
+                     double *Sigma, const int *sym, Arena scratch, cudaStream_t s) {
+  const long long nn = (long long)n * n;
+  if (!f.on) {
+    launch_backproject_sigma(X, Tm, N, n, bc, Sigma, nn, s, sym);
+    return Status::ok();
+  }
+  for (size_t i = 0; i < f.XT.size(); ++i) {
+    Arena ar = scratch;
+    SliceOp Ts = slice_take(ar, bc, n, f.XT[i].K);
+    if (!Ts.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+    slice_rows(Tm + (long long)i * kSliceMaxK * n, true, (long long)N * n, 1, n, bc, Ts, s);
+    SliceGemm g;
+    g.batch = bc;
+    g.C = Sigma; g.sC = nn; g.ci = n; g.cj = 1;
+    g.alpha = -1.0;
+    g.beta = i == 0 ? 0.0 : 1.0;
+    g.mirror = sym;
+    SOX_TRY(slice_gemm(h, f.XT[i], Ts, g, s));
+    h->launches += 2;
+  }
+  return Status::ok();
 }
 
 
@@ -141,6 +233,7 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
   __half *U2h = ar.take<__half>((size_t)n * NR * Kp), *U2l = ar.take<__half>((size_t)n * NR * Kp);
   float *inv_u2 = two ? ar.take<float>(N) : inv_u1;   // one split serves both slots
   float *Xf = reinterpret_cast<float *>(ar.take<char>(rows_f32_bytes(N, n)));
+  F64Ops f64 = f64_take(ar, g);
   Arena scr = ar;   // the mixed tensor's scratch, where the chunk buffers will lie
   void *mix_scratch = scr.take<char>(g.scratch_bytes);
   // ---- per-chunk buffers ----
@@ -165,6 +258,7 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
   {
     ProfScope ps(h, "mixed_f32", s, two ? 9 : 5);
     launch_rows_f32(X, N, n, Xf, s);
+    f64_slice_x(h, f64, X, n, s);
     const double *src[2] = {U1, U2};
     for (int k = 0; k < (two ? 2 : 1); ++k) {
       launch_mixed_f32(src[k], X, N, n, Kp, Uf, mix_scratch, s);
@@ -201,22 +295,10 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
   for (int b0 = 0; b0 < B; b0 += Bc) {
     const int bc = std::min(Bc, B - b0);
     const double *Gc = G + (long long)b0 * n * n;
-    {  // FP64 projections G_Rq = X G, G_wP^T = X G^T, then row splits.  For a symmetric
-       // G(tau) (real molecular orbitals) G_wP^T = G_Rq: a device flag per (spin, tau)
-       // lets the second GEMM skip its blocks and the split read G_Rq instead.
+    {  // FP64 projections, then row splits (a symmetric G(tau)'s second split reads G_Rq)
       ProfScope ps(h, "project_f64", s, 5);
       launch_symmetry_flags(Gc, n, bc, symf, s);
-      GemmF64 gp;
-      gp.M = N; gp.Nc = n; gp.K = n; gp.batch = bc;
-      gp.A = X; gp.ai = n; gp.ak = 1;
-      gp.B = Gc; gp.sB = (long long)n * n; gp.bk = n; gp.bj = 1;
-      gp.C = GR64; gp.sC = (long long)N * n; gp.ci = n; gp.cj = 1;
-      launch_gemm_f64(gp, s);
-      GemmF64 gw = gp;
-      gw.bk = 1; gw.bj = n;
-      gw.C = GW64;
-      gw.skip = symf;
-      launch_gemm_f64(gw, s);
+      SOX_TRY(project_f64(h, f64, Gc, X, N, n, bc, symf, GR64, GW64, ar, s));
       launch_split_rows_f64(GR64, n, (long long)N * n, N, NR, n, Kp, GRh, GRl, inv_gr, bc, s);
       launch_split_rows_f64(GW64, n, (long long)N * n, N, NR, n, Kp, GWh, GWl, inv_gw, bc, s, GR64, symf);
     }
@@ -255,8 +337,8 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
       launch_backproject_T(Dt, N, Xf, N, n, bc, Tm, s);
       // bare SOX with a symmetric G(tau) has a symmetric Sigma(tau)
       // (a partial v range breaks that symmetry: then every block is computed)
-      launch_backproject_sigma(X, Tm, N, n, bc, Sigma + (long long)b0 * n * n, (long long)n * n, s,
-                               (two || !v_range_is_full(h, n)) ? nullptr : symf);
+      SOX_TRY(final_sum_f64(h, f64, X, Tm, N, n, bc, Sigma + (long long)b0 * n * n,
+                            (two || !v_range_is_full(h, n)) ? nullptr : symf, ar, s));
     }
   }
   SOX_CUDA_TRY(cudaGetLastError());
@@ -326,6 +408,8 @@ struct Inst {
   __half *GRh, *GRl, *GWh, *GWl, *Gmh, *Gml, *Ah, *Al;
   float *inv_gr, *inv_gw, *gsc, *osc, *asc, *rowf, *colf, *Dt, *Tm;
   int *symf;
+  F64Ops f64;
+  Arena scratch;   // digits of G or T
   CUtensorMap bcd[8], agemm[6];
 };
 
@@ -356,6 +440,7 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
     c.U2h = ar.take<__half>((size_t)nn * NR * Kp); c.U2l = ar.take<__half>((size_t)nn * NR * Kp);
     c.inv_u2 = c.inv_u1;   // one split serves both slots
     c.Xf = reinterpret_cast<float *>(ar.take<char>(rows_f32_bytes(NN, nn)));
+    c.f64 = f64_take(ar, g);
     Arena scr = ar;   // the mixed tensor's scratch, where the chunk buffers will lie
     c.mix_scratch = scr.take<char>(g.scratch_bytes);
     c.GR64 = ar.take<double>((size_t)Bc * NN * nn); c.GW64 = ar.take<double>((size_t)Bc * NN * nn);
@@ -370,7 +455,10 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
     c.Dt = ar.take<float>((size_t)Bc * NN * NN);
     c.Tm = ar.take<float>((size_t)Bc * NN * nn);
     c.symf = ar.take<int>((size_t)Bc);
-    if (!c.symf || !c.mix_scratch) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+    const size_t per_b = std::max(2 * slice_bytes(1, nn, nn), slice_bytes(1, nn, std::min(NN, kSliceMaxK)));
+    c.scratch = ar;
+    if (!c.symf || !c.mix_scratch || !ar.take<char>(per_b * Bc))
+      return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
     ar.off = std::max(ar.off, scr.off);
     if (!make_tmap_f16_3d(&c.bcd[0], c.Ah, Kp, NR, (uint64_t)Bc * nn, 64, 128, &err) ||
         !make_tmap_f16_3d(&c.bcd[1], c.Al, Kp, NR, (uint64_t)Bc * nn, 64, 128, &err) ||
@@ -395,6 +483,7 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
     ProfScope ps(h, "mixed_f32", s, 5 * count);
     for (Inst &c : in) {
       launch_rows_f32(c.X, c.N, c.n, c.Xf, s);
+      f64_slice_x(h, c.f64, c.X, c.n, s);
       launch_mixed_f32(c.V, c.X, c.N, c.n, c.Kp, c.Uf, c.mix_scratch, s);
       launch_split_mixed(c.Uf, c.N, c.NR, c.n, c.Kp, c.U1h, c.U1l, c.U2h, c.U2l, c.inv_u1, s);
     }
@@ -414,17 +503,7 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
       {
         ProfScope ps(h, "project_f64", s, 5);
         launch_symmetry_flags(Gc, c.n, bc, c.symf, s);
-        GemmF64 gp;
-        gp.M = c.N; gp.Nc = c.n; gp.K = c.n; gp.batch = bc;
-        gp.A = c.X; gp.ai = c.n; gp.ak = 1;
-        gp.B = Gc; gp.sB = (long long)c.n * c.n; gp.bk = c.n; gp.bj = 1;
-        gp.C = c.GR64; gp.sC = (long long)c.N * c.n; gp.ci = c.n; gp.cj = 1;
-        launch_gemm_f64(gp, s);
-        GemmF64 gw = gp;
-        gw.bk = 1; gw.bj = c.n;
-        gw.C = c.GW64;
-        gw.skip = c.symf;
-        launch_gemm_f64(gw, s);
+        SOX_TRY(project_f64(h, c.f64, Gc, c.X, c.N, c.n, bc, c.symf, c.GR64, c.GW64, c.scratch, s));
         launch_split_rows_f64(c.GR64, c.n, (long long)c.N * c.n, c.N, c.NR, c.n, c.Kp, c.GRh, c.GRl, c.inv_gr, bc, s);
         launch_split_rows_f64(c.GW64, c.n, (long long)c.N * c.n, c.N, c.NR, c.n, c.Kp, c.GWh, c.GWl, c.inv_gw, bc, s,
                               c.GR64, c.symf);
@@ -486,8 +565,8 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
       if (bc <= 0) continue;
       ProfScope ps(h, "backproject", s, 2);
       launch_backproject_T(c.Dt, c.N, c.Xf, c.N, c.n, bc, c.Tm, s);
-      launch_backproject_sigma(c.X, c.Tm, c.N, c.n, bc, c.Sigma + (long long)b0 * c.n * c.n, (long long)c.n * c.n, s,
-                               v_range_is_full(h, c.n) ? c.symf : nullptr);
+      SOX_TRY(final_sum_f64(h, c.f64, c.X, c.Tm, c.N, c.n, bc, c.Sigma + (long long)b0 * c.n * c.n,
+                            v_range_is_full(h, c.n) ? c.symf : nullptr, c.scratch, s));
     }
   }
   SOX_CUDA_TRY(cudaGetLastError());

@@ -83,3 +83,75 @@ def test_find_mu_limits(env):
     zero, = to_dev(torch, np.zeros(2))
     with pytest.raises(pkg.SoxError):
         pkg.sox_find_mu(h, p, zero, 1.5, to_dev(torch, np.zeros((1, n, n)))[0], lo=-1.0, hi=1.0)
+
+
+def _exact_projections(X, G):
+    """X G, (X G^T), X G X^T in extended precision (rounded to FP64 only at the end)."""
+    Xl, Gl = X.astype(np.longdouble), G.astype(np.longdouble)
+    gr = np.stack([Xl @ g for g in Gl])
+    gw = np.stack([g @ Xl.T for g in Gl])
+    return gr, gw, np.stack([r @ Xl.T for r in gr])
+
+
+# (n, N, batches): K = n at the ends of a 16-wide step, a 32-wide chunk, a 128-wide window
+# (the 2^-55 and 2^-52 forms of the sums); rows at the ends of the 128 x 64 tiles; the last
+# two stay on the FP64 pipe
+@pytest.mark.parametrize("n,N,nb", [(15, 129, 600), (16, 64, 1000), (17, 128, 500), (33, 127, 120), (64, 65, 64),
+                                    (127, 130, 10), (128, 128, 10), (129, 191, 6), (260, 70, 6), (5, 40, 4), (1, 7, 2)])
+def test_fp64_products_from_digit_slices(env, n, N, nb):
+    """thc_project_G against extended precision.  Bound per element: K terms whose factors are
+    rounded at 2^-56 of twice the row maximum (2^-54 a term together), the final rounding and the
+    dropped digit products below one more unit: (K + 4) 2^-53 of the maxima's product."""
+    torch, pkg, hs = env
+    rng = np.random.default_rng(1000 * n + N)
+    G = rng.standard_normal((1, 1, nb, n, n)) * np.exp2(rng.integers(-40, 40, size=(1, 1, nb, 1, 1)).astype(float))
+    X = rng.standard_normal((1, N, n))
+    p = pkg.problem(n, N, nb, 1, 10.0)
+    Gd, Xd = to_dev(torch, G, X)
+    out = [torch.full(s, float("nan"), dtype=torch.float64, device="cuda")
+           for s in ((1, 1, nb, N, n), (1, 1, nb, n, N), (1, 1, nb, N, N))]
+    pkg.thc_project_G(hs["fp64"], p, Gd, Xd, *out)
+    pkg.sox_check_device(hs["fp64"])
+    ref = _exact_projections(X[0], G[0, 0])
+    eps = (n + 4) * 2.0 ** -53
+    gmax = np.abs(G[0, 0]).max(axis=(1, 2))[:, None, None]
+    xmax = np.abs(X).max()
+    got = [o.cpu().numpy()[0, 0] for o in out]
+    assert (np.abs(got[0] - ref[0]) <= eps * xmax * gmax).all()
+    assert (np.abs(got[1] - ref[1]) <= eps * xmax * gmax).all()
+    # the second product's factor G_Rq carries the first one's error: K more times its bound
+    rmax = np.abs(ref[0]).max(axis=(1, 2))[:, None, None].astype(float)
+    assert (np.abs(got[2] - ref[2]) <= eps * xmax * rmax + n * xmax * eps * xmax * gmax).all()
+    # not further from the exact product than FP64 arithmetic is
+    f64 = np.stack([X[0] @ g for g in G[0, 0]])
+    err = lambda a: float(np.sqrt((((a - ref[0]) / gmax) ** 2).sum()))  # noqa: E731
+    assert err(got[0]) <= 1.5 * err(f64) + n * 2.0 ** -54
+
+
+def test_fp64_products_with_zeros_infinities_and_nans(env):
+    """Zero rows, subnormals, infinities and NaNs through the sliced product as through FP64."""
+    torch, pkg, hs = env
+    n, N, nb = 24, 96, 400
+    rng = np.random.default_rng(3)
+    G, X = rng.standard_normal((1, 1, nb, n, n)), rng.standard_normal((1, N, n))
+    X[0, 5] = 0.0
+    G[0, 0, 1] = 0.0
+    G[0, 0, 2] *= 1e-310
+    G[0, 0, 3, 2, 7] = np.inf
+    G[0, 0, 4, 2, 7], G[0, 0, 4, 9, 7] = np.inf, -np.inf
+    G[0, 0, 5, 0, 0] = np.nan
+    G[0, 0, 6] *= 1e300
+    p = pkg.problem(n, N, nb, 1, 10.0)
+    Gd, Xd = to_dev(torch, G, X)
+    gr = torch.zeros(1, 1, nb, N, n, dtype=torch.float64, device="cuda")
+    pkg.thc_project_G(hs["fp64"], p, Gd, Xd, gr)
+    got = gr.cpu().numpy()[0, 0]
+    with np.errstate(all="ignore"):
+        ref = np.stack([np.einsum("Ru,uq->Rq", X[0], g) for g in G[0, 0]])
+    assert (np.isnan(got) == np.isnan(ref)).all()
+    assert (np.isinf(got) == np.isinf(ref)).all() and (np.sign(got[np.isinf(ref)]) == np.sign(ref[np.isinf(ref)])).all()
+    fin = np.isfinite(ref)
+    cmax = np.where(np.isfinite(G[0, 0]), np.abs(G[0, 0]), 0.0).max(axis=1)[:, None, :]
+    bound = (n + 4) * 2.0 ** -52 * np.abs(X).max() * np.broadcast_to(cmax, ref.shape) + 1e-320
+    assert (np.abs(got - np.where(fin, ref, 0.0))[fin] <= bound[fin]).all()
+    assert (got[:, 5][np.isfinite(G[0, 0]).all(axis=(1, 2))] == 0.0).all() and (got[1] == 0.0).all()
