@@ -157,33 +157,43 @@ struct Dims {
   long long nn() const { return (long long)n * n; }
 };
 
-// Projections for cc tau points starting at t0 of one spin block (FP64).
-void project_chunk(sox_handle H, const double *Gs, const double *X, const Dims &d, int t0, int cc,
-                   double *GR, double *GWt, cudaStream_t s) {
-  GemmF64 g;  // GR[b][R][q] = sum_u X[R][u] G[t0+b][u][q]
-  g.M = d.N; g.Nc = d.n; g.K = d.n; g.batch = cc;
-  g.A = X; g.ai = d.n; g.ak = 1;
-  g.B = Gs + (long long)t0 * d.nn(); g.sB = d.nn(); g.bk = d.n; g.bj = 1;
-  g.C = GR; g.sC = (long long)d.N * d.n; g.ci = d.n; g.cj = 1;
-  GemmF64 h = g;  // GWt[b][P][w] = sum_p X[P][p] G[t0+b][w][p]
-  h.bk = 1; h.bj = d.n;
-  h.C = GWt;
-  sox::ProfScope ps(H, "project_f64", s, 2);
-  sox::launch_gemm_f64(g, s);
-  sox::launch_gemm_f64(h, s);
-}
-
-// Um[P][q][s] = sum_Q U[P][Q] X[Q][q] X[Q][s]   (Eq. U_contraction at k = 0)
-void mixed_tensor_f64(sox_handle H, const double *U, const double *X, const Dims &d, double *Y,
-                      double *Um, cudaStream_t s) {
-  GemmF64 g;
-  g.M = d.N; g.Nc = (int)d.nn(); g.K = d.N;
-  g.A = U; g.ai = d.N; g.ak = 1;
-  g.B = Y; g.bk = d.nn(); g.bj = 1;
-  g.C = Um; g.ci = d.nn(); g.cj = 1;
-  sox::ProfScope ps(H, "mixed_f64", s, 2);
-  sox::launch_pair_products_f64(X, Y, d.N, d.n, s);
-  sox::launch_gemm_f64(g, s);
+// The products of the FP64 chain for cc tau points (operands and outputs set by the caller).
+struct Fp64Gemms {
+  GemmF64 mix, gr, gw, A, T, S;
+};
+Fp64Gemms fp64_gemms(const Dims &d, int cc) {
+  Fp64Gemms f;
+  const long long nn = d.nn(), Nn = (long long)d.N * d.n, NN = (long long)d.N * d.N;
+  // Um[P][(q,s)] = sum_Q U[P][Q] Y[Q][(q,s)],  Y = X[Q][q] X[Q][s]   (Eq. U_contraction at k = 0)
+  f.mix.M = d.N; f.mix.Nc = (int)nn; f.mix.K = d.N;
+  f.mix.ai = d.N; f.mix.ak = 1;
+  f.mix.bk = nn; f.mix.bj = 1;
+  f.mix.ci = nn; f.mix.cj = 1;
+  // GR[b][R][q] = sum_u X[R][u] G[b][u][q],  GWt[b][P][w] = sum_p X[P][p] G[b][w][p]
+  f.gr.M = d.N; f.gr.Nc = d.n; f.gr.K = d.n; f.gr.batch = cc;
+  f.gr.ai = d.n; f.gr.ak = 1;
+  f.gr.sB = nn; f.gr.bk = d.n; f.gr.bj = 1;
+  f.gr.sC = Nn; f.gr.ci = d.n; f.gr.cj = 1;
+  f.gw = f.gr;
+  f.gw.bk = 1; f.gw.bj = d.n;
+  // A[b][v][(P,q)] = sum_s G(-tau)[s][v] Um1[(P,q)][s],  G(-tau_j) = -G(tau_{T-1-j})
+  f.A.M = d.n; f.A.Nc = d.N * d.n; f.A.K = d.n; f.A.batch = cc;
+  f.A.sA = -nn; f.A.ai = 1; f.A.ak = d.n;
+  f.A.bk = 1; f.A.bj = d.n;
+  f.A.sC = Nn * d.n; f.A.ci = Nn; f.A.cj = 1;
+  f.A.alpha = -1.0;
+  // T[b][R][r] = sum_P D[b][P][R] X[P][r]
+  f.T.M = d.N; f.T.Nc = d.n; f.T.K = d.N; f.T.batch = cc;
+  f.T.sA = NN; f.T.ai = 1; f.T.ak = d.N;
+  f.T.bk = d.n; f.T.bj = 1;
+  f.T.sC = Nn; f.T.ci = d.n; f.T.cj = 1;
+  // Sigma[t][r] = -sum_R X[R][t] T[R][r]
+  f.S.M = d.n; f.S.Nc = d.n; f.S.K = d.N; f.S.batch = cc;
+  f.S.ai = 1; f.S.ak = d.n;
+  f.S.sB = Nn; f.S.bk = d.n; f.S.bj = 1;
+  f.S.sC = nn; f.S.ci = d.n; f.S.cj = 1;
+  f.S.alpha = -1.0;
+  return f;
 }
 
 int tau_chunk(sox_handle h, const Dims &d, size_t per_tau_bytes, size_t fixed_bytes) {
@@ -195,23 +205,41 @@ int tau_chunk(sox_handle h, const Dims &d, size_t per_tau_bytes, size_t fixed_by
   return (int)c;
 }
 
-size_t sigma_fp64_bytes(sox_handle h, const Dims &d, bool two_slots, int *chunk) {
-  size_t Nn2 = (size_t)d.N * d.nn();
+// Sizes of the FP64 chain.  slices: B, C and D through digit slices on the tensor cores; a
+// chain whose B and C are small products (slices_pay) stays on the FP64 pipe.
+struct Fp64Plan {
+  bool slices = false;
+  int c = 1;
+  size_t bytes = 0;
+};
+Fp64Plan fp64_plan(sox_handle h, const Dims &d, bool two_slots) {
+  Fp64Plan p;
+  p.slices = sox::slices_pay(d.N, d.N, 2 * d.nn(), d.T);
+  const size_t Nn2 = (size_t)d.N * d.nn();
   size_t fixed = sox::aligned_bytes(Nn2, 8) * (two_slots ? 2 : 1);
   size_t per_tau = 8 * (Nn2 + 3 * (size_t)d.N * d.n + (size_t)d.N * d.N) + 1024;
-  int c = tau_chunk(h, d, per_tau, fixed);
-  if (chunk) *chunk = c;
-  return fixed + sox::aligned_bytes(std::max<size_t>(Nn2 * c, Nn2), 8) +
-         4 * sox::aligned_bytes((size_t)c * d.N * std::max(d.n, d.N), 8);
+  if (p.slices) {
+    fixed += sox::slice_bytes(d.n, d.N, d.n);                                    // digits of U2
+    per_tau += sox::slice_bytes(d.n, d.N, d.n) + 2 * sox::slice_bytes(1, d.N, d.n);   // of A, GR, GWt
+  }
+  p.c = tau_chunk(h, d, per_tau, fixed);
+  const Fp64Gemms f = fp64_gemms(d, p.c);
+  size_t scratch = 0;
+  for (const GemmF64 *g : {&f.mix, &f.gr, &f.gw, &f.A, &f.T, &f.S}) scratch = std::max(scratch, sox::gemm_f64_bytes(*g));
+  p.bytes = fixed + sox::aligned_bytes(std::max<size_t>(Nn2 * p.c, Nn2), 8) +
+            4 * sox::aligned_bytes((size_t)p.c * d.N * std::max(d.n, d.N), 8) + scratch;
+  if (p.slices) p.bytes += sox::slice_bytes((long long)d.n * p.c, d.N, d.n) + 2 * sox::slice_bytes(p.c, d.N, d.n);
+  return p;
 }
 
 // Sigma for every spin and tau point; U1 == U2 allowed (bare SOX).
 Status sigma_fp64(sox_handle H, const Dims &d, const double *G, const double *X, const double *U1,
                   const double *U2, double *Sigma, Arena &ar, cudaStream_t s) {
   const bool two = (U1 != U2);
-  int c = 1;
-  sigma_fp64_bytes(H, d, two, &c);
+  const Fp64Plan pl = fp64_plan(H, d, two);
+  const int c = pl.c;
   const size_t Nn2 = (size_t)d.N * d.nn();
+  const long long Nn = (long long)d.N * d.n;
   double *Um1 = ar.take<double>(Nn2);
   double *Um2 = two ? ar.take<double>(Nn2) : Um1;
   double *big = ar.take<double>(std::max<size_t>(Nn2 * c, Nn2));
@@ -219,49 +247,68 @@ Status sigma_fp64(sox_handle H, const Dims &d, const double *G, const double *X,
   double *GWt = ar.take<double>((size_t)c * d.N * d.n);
   double *Dm = ar.take<double>((size_t)c * d.N * d.N);
   double *Tm = ar.take<double>((size_t)c * d.N * d.n);
-  if (!Tm) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-  mixed_tensor_f64(H, U1, X, d, big, Um1, s);
-  if (two) mixed_tensor_f64(H, U2, X, d, big, Um2, s);
+  sox::SliceOp U2s;
+  if (pl.slices) U2s = sox::slice_take(ar, d.n, d.N, d.n);
+  if (!Tm || (pl.slices && !U2s.p)) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+  {
+    sox::ProfScope ps(H, "mixed_f64", s, two ? 3 : 2);
+    sox::launch_pair_products_f64(X, big, d.N, d.n, s);
+    GemmF64 m = fp64_gemms(d, c).mix;
+    m.A = U1; m.B = big; m.C = Um1;
+    SOX_TRY(sox::gemm_f64(H, m, ar, s));
+    if (two) {
+      m.A = U2; m.C = Um2;
+      SOX_TRY(sox::gemm_f64(H, m, ar, s));
+    }
+  }
+  if (pl.slices) {   // rows (v, R) of U2[R][v][w]
+    sox::slice_rows(Um2, false, d.n, d.nn(), 1, d.n, U2s, s);
+    ++H->launches;
+  }
   for (int sp = 0; sp < d.S; ++sp) {
     const double *Gs = G + (long long)sp * d.T * d.nn();
     double *Ss = Sigma + (long long)sp * d.T * d.nn();
     for (int t0 = 0; t0 < d.T; t0 += c) {
-      int cc = std::min(c, d.T - t0);
-      project_chunk(H, Gs, X, d, t0, cc, GR, GWt, s);
-      // A[b][v][(P,q)] = sum_s G(-tau)[s][v] Um1[(P,q)][s],  G(-tau_j) = -G(tau_{T-1-j})
-      GemmF64 a;
-      a.M = d.n; a.Nc = d.N * d.n; a.K = d.n; a.batch = cc;
-      a.A = Gs + (long long)(d.T - 1 - t0) * d.nn(); a.sA = -d.nn(); a.ai = 1; a.ak = d.n;
-      a.B = Um1; a.bk = 1; a.bj = d.n;
-      a.C = big; a.sC = (long long)Nn2; a.ci = (long long)d.N * d.n; a.cj = 1;
-      a.alpha = -1.0;
+      const int cc = std::min(c, d.T - t0);
+      Fp64Gemms f = fp64_gemms(d, cc);
+      {
+        sox::ProfScope ps(H, "project_f64", s, 2);
+        f.gr.A = f.gw.A = X;
+        f.gr.B = f.gw.B = Gs + (long long)t0 * d.nn();
+        f.gr.C = GR;
+        f.gw.C = GWt;
+        SOX_TRY(sox::gemm_f64(H, f.gr, ar, s));
+        SOX_TRY(sox::gemm_f64(H, f.gw, ar, s));
+      }
       {
         sox::ProfScope ps(H, "A_f64", s);
-        sox::launch_gemm_f64(a, s);
+        f.A.A = Gs + (long long)(d.T - 1 - t0) * d.nn();
+        f.A.B = Um1;
+        f.A.C = big;
+        SOX_TRY(sox::gemm_f64(H, f.A, ar, s));
       }
       {  // D[b][P][R] = sum_v B o C
-        sox::ProfScope ps(H, "sox_bcd", s);
-        sox::launch_sox_bcd_f64(big, (long long)Nn2, GR, (long long)d.N * d.n, GWt,
-                                (long long)d.N * d.n, Um2, Dm, (long long)d.N * d.N, d.n, d.N, cc, s,
-                                H ? H->v0 : 0, H ? H->v1 : 0);
+        sox::ProfScope ps(H, "sox_bcd", s, pl.slices ? 4 : 1);
+        if (pl.slices) {
+          Arena a2 = ar;
+          sox::SliceOp As = sox::slice_take(a2, cc * d.n, d.N, d.n), GRs = sox::slice_take(a2, cc, d.N, d.n),
+                       GWs = sox::slice_take(a2, cc, d.N, d.n);
+          if (!As.p || !GRs.p || !GWs.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+          sox::slice_rows(big, false, Nn, d.n, 1, cc * d.n, As, s);
+          sox::slice_rows(GR, false, Nn, d.n, 1, cc, GRs, s);
+          sox::slice_rows(GWt, false, Nn, d.n, 1, cc, GWs, s);
+          SOX_TRY(sox::slice_bcd(H, As, GRs, GWs, U2s, d.n, d.N, cc, H->v0, H->v1, Dm, (long long)d.N * d.N, s));
+        } else {
+          sox::launch_sox_bcd_f64(big, (long long)Nn2, GR, Nn, GWt, Nn, Um2, Dm, (long long)d.N * d.N, d.n, d.N, cc, s,
+                                  H->v0, H->v1);
+        }
       }
-      // T[b][R][r] = sum_P D[b][P][R] X[P][r]
-      GemmF64 t;
-      t.M = d.N; t.Nc = d.n; t.K = d.N; t.batch = cc;
-      t.A = Dm; t.sA = (long long)d.N * d.N; t.ai = 1; t.ak = d.N;
-      t.B = X; t.bk = d.n; t.bj = 1;
-      t.C = Tm; t.sC = (long long)d.N * d.n; t.ci = d.n; t.cj = 1;
-      // Sigma[t][r] = -sum_R X[R][t] T[R][r]
-      GemmF64 b;
-      b.M = d.n; b.Nc = d.n; b.K = d.N; b.batch = cc;
-      b.A = X; b.ai = 1; b.ak = d.n;
-      b.B = Tm; b.sB = (long long)d.N * d.n; b.bk = d.n; b.bj = 1;
-      b.C = Ss + (long long)t0 * d.nn(); b.sC = d.nn(); b.ci = d.n; b.cj = 1;
-      b.alpha = -1.0;
       {
         sox::ProfScope ps(H, "backproject_f64", s, 2);
-        sox::launch_gemm_f64(t, s);
-        sox::launch_gemm_f64(b, s);
+        f.T.A = Dm; f.T.B = X; f.T.C = Tm;
+        SOX_TRY(sox::gemm_f64(H, f.T, ar, s));
+        f.S.A = X; f.S.B = Tm; f.S.C = Ss + (long long)t0 * d.nn();
+        SOX_TRY(sox::gemm_f64(H, f.S, ar, s));
       }
     }
   }
@@ -273,7 +320,7 @@ Dims dims_of(const sox_problem *p) { return Dims{p->n, p->N, p->n_tau, p->n_spin
 
 size_t sigma_bytes(sox_handle h, const Dims &d, bool two) {
   if (h->precision == SOX_PREC_F16X2) return sox::tc_sigma_bytes(h, d.n, d.N, d.T, d.S, two);
-  return sigma_fp64_bytes(h, d, two, nullptr);
+  return fp64_plan(h, d, two).bytes;
 }
 
 Status sigma_any(sox_handle h, const Dims &d, const double *G, const double *X, const double *U1,

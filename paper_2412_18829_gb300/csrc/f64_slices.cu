@@ -135,13 +135,16 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
 // first products run while the later sums are still being read.
 // Bound by the MMAs (34 of 128 x 64 x 16 per 16 of K) and, at K <= 128, by reading the sums
 // out in equal parts; the FP64 pipe (1.6 FMA a clock and SM) sees no instruction of it.
-// n = 120, N = 600, 160 batches: projections 2.84 ms on the FP64 pipe, 0.35 ms here with the
-// slicing; final sum (K = 600) 1.74 -> 0.43 ms.  n = 250, N = 2000, 12 times: X G X^T 27.9 -> 1.7 ms.
+// n = 120, N = 600, 160 batches: projections 2.84 ms on the FP64 pipe, 0.22 ms here with the
+// slicing; final sum (K = 600) 1.74 -> 0.29 ms.  n = 250, N = 2000, 12 times: X G X^T 27.9 -> 1.7 ms.
 constexpr int kL = 128, kW = 64, kKc = 32, kWin = 4;   // kWin chunks per window
 constexpr int kLBytes = kL * kKc * 2, kWBytes = kW * kKc * 2;
 constexpr int kStageBytes = kSlices * (kLBytes + kWBytes);
 constexpr int kStages = 2;
-constexpr int kThreads = 320;   // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
+// warp 0 TMA, warp 1 MMA, warps 2-17 epilogue: reading a sum out is a chain of dependent
+// integer instructions, so four warps per scheduler take half the time of two
+constexpr int kEpiWarps = 16;
+constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kGroups = 8;
 
 struct Bars {
@@ -181,29 +184,104 @@ __device__ __forceinline__ uint64_t desc_kmajor_sw64(uint32_t saddr) {
 
 __device__ __forceinline__ long long wind_down(long long cap) { return cap > (1LL << 20) ? cap : (1LL << 20); }
 
-// All products of one chunk with KS 16-wide steps, sums in ascending order; on the window's
-// first chunk each sum waits until the epilogue has read its columns.
-template <int KS>
-__device__ __forceinline__ bool issue_chunk(uint32_t tmem, uint32_t st, bool first, Bars *bar, uint32_t ph,
+// All products of one chunk with KS 16-wide steps; sum g lies at TMEM column g W.  The
+// digit tiles of the W side follow one another in shared memory, and digit i of the lane side
+// times digits j, j + 1, ... lands in the neighbouring sums i + j, i + j + 1, ...: one MMA takes
+// as many digits as fit in N = 256 (an MMA below that width costs nearly as much as at it: with
+// one MMA per pair of digits the fused kernel took 16.2 ms instead of 8.7 at n = 80).  On a window's first chunk a sum is
+// overwritten by its first product, and waited for until the epilogue has read its columns.
+template <int W, int KS>
+__device__ __forceinline__ bool issue_chunk(uint32_t tmem, uint32_t st, bool first, uint64_t *acc_empty, uint32_t ph,
                                             long long limit, volatile int *abort, int *status) {
-  constexpr uint32_t idesc = tc::idesc_f16_f32(kL, kW);
-  const uint32_t w0 = st + kSlices * kLBytes;
-#pragma unroll 1
-  for (int g = 0; g < kGroups; ++g) {
-    if (first) {
-      if (!tc::mbar_wait(&bar->acc_empty[g], ph, limit, abort, status, 2)) return false;
-      tc::tc_fence_after();
-    }
-    const int i0 = g < kSlices ? 0 : g - (kSlices - 1), i1 = g < kSlices ? g : kSlices - 1;
-    for (int i = i0; i <= i1; ++i) {
-      const uint32_t a = st + i * kLBytes, w = w0 + (g - i) * kWBytes;
+  constexpr int kPer = 256 / W < kSlices ? 256 / W : kSlices;   // digits per MMA
+  constexpr uint32_t kWB = W * kKc * 2;
+  const uint64_t dl = desc_kmajor_sw64(st), dw = desc_kmajor_sw64(st + kSlices * kLBytes);
+  auto ready = [&](int g0, int g1) {   // sums g0 .. g1 - 1 may be overwritten
+    for (int g = g0; g < g1; ++g)
+      if (!tc::mbar_wait(&acc_empty[g], ph, limit, abort, status, 2)) return false;
+    tc::tc_fence_after();
+    return true;
+  };
+  auto mma = [&](int i, int j, int nj, int k, uint32_t acc) {
+    tc::mma_f16(tmem + (i + j) * W, dl + (uint64_t)((i * kLBytes + k * 32) >> 4),
+                dw + (uint64_t)((j * (int)kWB + k * 32) >> 4), tc::idesc_f16_f32(kL, nj * W), acc);
+  };
 #pragma unroll
-      for (int k = 0; k < KS; ++k)
-        tc::mma_f16(tmem + g * kW, desc_kmajor_sw64(a + k * 32), desc_kmajor_sw64(w + k * 32), idesc,
-                    (first && i == i0 && k == 0) ? 0u : 1u);
+  for (int k = 0; k < KS; ++k)
+#pragma unroll
+    for (int i = 0; i < kSlices; ++i) {
+      const int J = i == 0 ? kSlices : kGroups - i;   // digits j < J
+#pragma unroll
+      for (int j = 0; j < J; j += kPer) {
+        const int nj = J - j < kPer ? J - j : kPer;
+        if (k == 0 && i == 0) {          // the first product of sums j .. j + nj - 1
+          if (first && !ready(j, j + nj)) return false;
+          mma(i, j, nj, k, first ? 0u : 1u);
+        } else if (k == 0 && i == 1 && j + nj == J) {   // the last digit starts the last sum
+          if (first) {
+            if (!ready(kGroups - 1, kGroups)) return false;
+            if (nj > 1) mma(i, j, nj - 1, k, 1u);
+            mma(i, J - 1, 1, k, 0u);
+          } else {
+            mma(i, j, nj, k, 1u);
+          }
+        } else {
+          mma(i, j, nj, k, 1u);
+        }
+      }
+    }
+  return true;
+}
+
+template <int C>
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[C]) {
+  if constexpr (C == 16) tc::tmem_ld_32x32b_x16(taddr, v);
+  else tc::tmem_ld_32x32b_x8(taddr, v);
+}
+// waits for the loads issued so far; v passes through, so nothing reads it before
+template <int C>
+__device__ __forceinline__ void tmem_ld_wait_for(float (&v)[C]) {
+  tc::tmem_ld_wait();
+#pragma unroll
+  for (int i = 0; i < C; i += 8)
+    asm volatile("" : "+f"(v[i]), "+f"(v[i + 1]), "+f"(v[i + 2]), "+f"(v[i + 3]), "+f"(v[i + 4]), "+f"(v[i + 5]),
+                 "+f"(v[i + 6]), "+f"(v[i + 7]));
+}
+
+// Adds the eight sums of C columns of a window to the integers acc (unit 2^-(62 - LK)) and
+// hands each sum's columns back once they are read.
+template <int LK, int C, int W>
+__device__ __forceinline__ void read_window(uint32_t base, uint64_t *acc_empty, int lane, long long (&acc)[C]) {
+  // sum g has the unit 2^-(8 g + 14); those with bits below the integer's unit are added
+  // in FP32 first and rounded once
+  constexpr int top = 62 - LK - 14, kLow = top / 8 + 1;   // first sum with such bits
+  float low[C], buf[2][C];
+  tmem_ld_cols(base, buf[0]);
+#pragma unroll
+  for (int g = 0; g < kGroups; ++g) {
+    float (&v)[C] = buf[g & 1];
+    tmem_ld_wait_for(v);
+    if (g + 1 < kGroups) tmem_ld_cols(base + (g + 1) * W, buf[(g + 1) & 1]);   // in flight during the sums of g
+    tc::tc_fence_before();
+    __syncwarp();
+    if (lane == 0) tc::mbar_arrive(&acc_empty[g]);
+    const int sh = top - 8 * g;
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+      if (g < kLow) {
+        const int i = __float2int_rn(v[j]);
+        if (sh >= 32)   // the high word alone
+          acc[j] += (long long)((unsigned long long)((unsigned)i << (sh >= 32 ? sh - 32 : 0)) << 32);
+        else
+          acc[j] += (long long)i * (long long)(1u << (sh >= 0 && sh < 32 ? sh : 0));
+      } else if (g == kLow) {
+        low[j] = v[j];
+      } else {
+        low[j] = fmaf(v[j], 1.f / (float)(1 << (8 * (g - kLow))), low[j]);
+      }
+      if (g == kGroups - 1) acc[j] += (long long)__float2int_rn(low[j] * (1.f / (float)(1 << (8 * kLow - top))));
     }
   }
-  return true;
 }
 
 __device__ __forceinline__ double plain_at(const void *x, int f32, long long o) {
@@ -218,23 +296,22 @@ __device__ __noinline__ double plain_element(const Args &a, int b, int l, int w)
   return acc;
 }
 
-__device__ __noinline__ double slow_scale(long long I, int x) { return scalbn((double)I, x); }
-
-// I 2^(x) rounded to nearest even, from integer instructions (a 64-bit conversion and a
-// scaling would cost the FP64 pipe more than all products of the element did)
-__device__ __forceinline__ double scaled_double(long long I, int x) {
-  if (I == 0) return 0.0;
+// I 2^x rounded to nearest even, from integer instructions (a 64-bit conversion and a
+// scaling would cost the FP64 pipe more than all products of the element did).  False, and no
+// value, for a row with infinities or NaNs (x then lies beyond any exponent) and for results
+// outside the normal range: those elements are recomputed from the sources.
+__device__ __forceinline__ bool scaled_double(long long I, int x, double &v) {
   const unsigned long long u = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
-  const int lz = __clzll((long long)u);
+  const int lz = __clzll((long long)(u | 1));
   const unsigned long long m = u << lz;
   unsigned long long r = m >> 11;
-  const unsigned rem = (unsigned)(m & 0x7ff);
-  r += (rem > 0x400u || (rem == 0x400u && (r & 1))) ? 1u : 0u;
+  const unsigned rem = (unsigned)m & 0x7ffu;
+  r += (rem + (unsigned)(r & 1)) > 0x400u ? 1u : 0u;
   const int eb = 63 - lz + x + 1023;   // biased exponent of the leading bit
-  if (eb < 1 || eb > 2045) return slow_scale(I, x);   // subnormal or beyond FP64
   const unsigned long long b =
       ((unsigned long long)(eb - 1) << 52) + r + (I < 0 ? 0x8000000000000000ull : 0ull);
-  return __longlong_as_double((long long)b);
+  v = I == 0 ? 0.0 : __longlong_as_double((long long)b);
+  return I == 0 ? x < kNonFinite / 2 : (unsigned)(eb - 1) <= 2044u;
 }
 
 // LK: the sums of a tile stay below 2^LK (K <= 2^LK), kept as integers of 2^-(62 - LK)
@@ -253,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(&bar->empty[s], 1);
     }
     tc::mbar_init(&bar->acc_full, 1);
-    for (int g = 0; g < kGroups; ++g) tc::mbar_init(&bar->acc_empty[g], 8);
+    for (int g = 0; g < kGroups; ++g) tc::mbar_init(&bar->acc_empty[g], kEpiWarps);
     tc::mbar_init(&bar->drain, 1);
     bar->abort = 0;
     tc::fence_barrier_init();
@@ -316,8 +393,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t st = tc::smem_u32(smem + (size_t)s * kStageBytes);
             const bool first = kc == w * kWin;
             const uint32_t ph = (uint32_t)(win & 1) ^ 1u;
-            ok = (a.K - kc * kKc > 16) ? issue_chunk<2>(tmem, st, first, bar, ph, limit, abort, a.status)
-                                       : issue_chunk<1>(tmem, st, first, bar, ph, limit, abort, a.status);
+            ok = (a.K - kc * kKc > 16)
+                     ? issue_chunk<kW, 2>(tmem, st, first, bar->acc_empty, ph, limit, abort, a.status)
+                     : issue_chunk<kW, 1>(tmem, st, first, bar->acc_empty, ph, limit, abort, a.status);
             if (!ok) break;
             tc::mma_commit(&bar->empty[s]);
           }
@@ -329,70 +407,62 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else {
-    const int q = warp & 3, half = (warp - 2) >> 2;
+    constexpr int kC = 4 * kW / kEpiWarps;   // columns per warp
+    const int q = warp & 3, part = (warp - 2) >> 2;
     const int lr = q * 32 + lane;
     long long win = 0;
     for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
       const int b = (int)(t / per_b), r = (int)(t % per_b);
       if (a.skip && a.skip[b]) continue;
-      const int l = (r % a.tL) * kL + lr, w0 = (r / a.tL) * kW + half * 32;
-      long long acc[32];
+      const int l = (r % a.tL) * kL + lr, w0 = (r / a.tL) * kW + part * kC;
+      // exponents of this lane's row and of column w0 + lane (handed round by shuffles)
+      const int eL = l < a.nL ? a.eL[(a.bL == 1 ? 0LL : (long long)b * a.nL) + l] : 0;
+      const int eWl = lane < kC && w0 + lane < a.nW ? a.eW[(a.bW == 1 ? 0LL : (long long)b * a.nW) + w0 + lane] : 0;
+      long long acc[kC];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = 0;
+      for (int j = 0; j < kC; ++j) acc[j] = 0;
       bool ok = true;
       for (int w = 0; w < nwin; ++w, ++win) {
         ok = tc::mbar_wait(&bar->acc_full, (uint32_t)(win & 1), limit, abort, a.status, 8);
         if (!ok) break;
         tc::tc_fence_after();
-        const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + half * 32;
-        float low[32];
+        read_window<LK, kC, kW>(tmem + ((uint32_t)(q * 32) << 16) + part * kC, bar->acc_empty, lane, acc);
+      }
+      if (!ok) break;
+      double *C = a.C + b * a.sC + l * a.cl + w0 * a.cw;
+      double *Cm = a.C + b * a.sC + w0 * a.cl + l * a.cw;   // mirror image
+      const bool mir = a.mirror && a.mirror[b];
+      unsigned odd = 0u;   // columns to recompute from the sources
 #pragma unroll
-        for (int g = 0; g < kGroups; ++g) {
-          float v[32];
-          tc::tmem_ld_32x32b_x32(base + g * kW, v);
-          tc::tmem_ld_wait();
-          tc::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&bar->acc_empty[g]);
-          // sum g has the unit 2^-(8 g + 14); those with bits below the integer's unit are
-          // added in FP32 first and rounded once
-          constexpr int top = 62 - LK - 14, kLow = top / 8 + 1;   // first sum with such bits
-          const int sh = top - 8 * g;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (g < kLow)
-              acc[j] += (long long)__float2int_rn(v[j]) << (g < kLow ? sh : 0);
-            else if (g == kLow)
-              low[j] = v[j];
-            else
-              low[j] = fmaf(v[j], 1.f / (float)(1 << (8 * (g - kLow))), low[j]);
-            if (g == kGroups - 1)
-              acc[j] += (long long)__float2int_rn(low[j] * (1.f / (float)(1 << (8 * kLow - top))));
+      for (int j = 0; j < kC; ++j) {
+        const int w = w0 + j;
+        const int eW = __shfl_sync(0xffffffffu, eWl, j);
+        double v;
+        const bool fine = scaled_double(acc[j], eL + eW - 2044 - (62 - LK), v);
+        if (l < a.nL && w < a.nW) {
+          if (fine) {
+            v = a.alpha == 1.0 ? v : (a.alpha == -1.0 ? -v : a.alpha * v);
+            if (a.beta != 0.0) v = fma(a.beta, C[j * a.cw], v);
+            if (!mir) {
+              C[j * a.cw] = v;
+            } else {
+              const int ib = (a.lane_is_row ? l : w) / 32, jb = (a.lane_is_row ? w : l) / 32;
+              if (ib <= jb) C[j * a.cw] = v;
+              if (ib < jb) Cm[j * a.cl] = v;
+            }
+          } else {
+            odd |= 1u << j;
           }
         }
       }
-      if (!ok) break;
-      if (l >= a.nL) continue;
-      const int eL = a.eL[(a.bL == 1 ? 0LL : (long long)b * a.nL) + l];
-      double *C = a.C + b * a.sC + l * a.cl;
-      const bool mir = a.mirror && a.mirror[b];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const int w = w0 + j;
-        if (w < a.nW) {
-          const int eW = a.eW[(a.bW == 1 ? 0LL : (long long)b * a.nW) + w];
-          double v;
-          if (eL == kNonFinite || eW == kNonFinite)
-            v = plain_element(a, b, l, w);
-          else
-            v = scaled_double(acc[j], eL + eW - 2044 - (62 - LK));
-          if (a.alpha != 1.0) v = a.alpha == -1.0 ? -v : a.alpha * v;
-          double *c = C + w * a.cw;
-          if (a.beta != 0.0) v = fma(a.beta, *c, v);
-          const int ib = (a.lane_is_row ? l : w) / 32, jb = (a.lane_is_row ? w : l) / 32;
-          if (!mir || ib <= jb) *c = v;
-          if (mir && ib < jb) a.C[b * a.sC + w * a.cl + l * a.cw] = v;
-        }
+      while (odd) {
+        const int j = __ffs((int)odd) - 1, w = w0 + j;
+        odd &= odd - 1;
+        double v = a.alpha * plain_element(a, b, l, w);
+        if (a.beta != 0.0) v = fma(a.beta, C[j * a.cw], v);
+        const int ib = (a.lane_is_row ? l : w) / 32, jb = (a.lane_is_row ? w : l) / 32;
+        if (!mir || ib <= jb) C[j * a.cw] = v;
+        if (mir && ib < jb) Cm[j * a.cl] = v;
       }
     }
   }
@@ -403,9 +473,226 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
+// ------------------------------------------------------------------ fused B / C / D
+// D[b][P][R] = sum_v B_v C_v with B_v = A_v GR^T and C_v = GW U2_v^T, FP64 (Sec. II C, the B,
+// C and D steps): 128 P (lanes) x 32 R tiles; the eight sums of B_v and of C_v fill the 512
+// TMEM columns, so one is read out while the other accumulates.  The two products become
+// FP64 numbers with their own scales and D sums their product over v in FP64 registers.
+// Per (tile, v) 14 MMAs (34 digit products each for B_v and C_v) per 16 of n; the FP64 pipe
+// sees one FMA per element and v.  n = 80, N = 480, 30 times: 172.9 ms on the FP64 pipe, 7.4 ms
+// here (tensor pipe 41 % busy; the copies of the digits into shared memory set the pace).
+constexpr int kFW = 32;
+constexpr int kFWBytes = kFW * kKc * 2;
+constexpr int kFStageBytes = kSlices * (kLBytes + kFWBytes);
+constexpr int kFStages = 3;
+
+struct FBars {
+  uint64_t full[kFStages], empty[kFStages];
+  uint64_t acc_full[2], acc_empty[2][kGroups];
+  uint64_t drain;
+  uint32_t tmem_base;
+  int abort;
+};
+
+struct FArgs {
+  int n, N, batch, v0, v1, tP, tR;
+  const int *eA, *eGR, *eGW, *eU;   // [b][v][P], [b][R], [b][P], [v][R]
+  double *D;
+  long long sD;
+  // sources, for rows with infinities or NaNs: A[b][v][P][q], GR[b][R][q], GW[b][P][w], U2[R][v][w]
+  const double *xA, *xGR, *xGW, *xU;
+  int nv;   // v slices of A (n)
+  long long spin_limit;
+  int *status;
+};
+
+__device__ __noinline__ double plain_row_dot(const double *x, const double *y, int n) {
+  double acc = 0.0;
+  for (int k = 0; k < n; ++k) acc = fma(x[k], y[k], acc);
+  return acc;
+}
+
+template <int LK>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_slice_bcd(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmGR,
+                const __grid_constant__ CUtensorMap tmGW, const __grid_constant__ CUtensorMap tmU, const FArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  FBars *bar = reinterpret_cast<FBars *>(smem + kFStages * kFStageBytes);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int per_b = a.tP * a.tR;
+  const long long total = (long long)per_b * a.batch;
+  const int nkc = (a.n + kKc - 1) / kKc, nwin = (nkc + kWin - 1) / kWin;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kFStages; ++s) {
+      tc::mbar_init(&bar->full[s], 1);
+      tc::mbar_init(&bar->empty[s], 1);
+    }
+    for (int h = 0; h < 2; ++h) {
+      tc::mbar_init(&bar->acc_full[h], 1);
+      for (int g = 0; g < kGroups; ++g) tc::mbar_init(&bar->acc_empty[h][g], kEpiWarps);
+    }
+    tc::mbar_init(&bar->drain, 1);
+    bar->abort = 0;
+    tc::fence_barrier_init();
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(&bar->tmem_base, 512);
+    tc::tmem_relinquish();
+  }
+  if (warp == 0 && lane == 0) {
+    tc::prefetch_tmap(&tmA); tc::prefetch_tmap(&tmGR); tc::prefetch_tmap(&tmGW); tc::prefetch_tmap(&tmU);
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = bar->tmem_base;
+  volatile int *abort = &bar->abort;
+  const long long limit = a.spin_limit;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      long long it = 0;
+      for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+        const int b = (int)(t / per_b), r = (int)(t % per_b);
+        const int P0 = (r / a.tR) * kL, R0 = (r % a.tR) * kFW;
+        for (int v = a.v0; v < a.v1 && !*abort; ++v) {
+          for (int c = 0; c < 2 * nkc; ++c, ++it) {   // the chunks of B_v, then of C_v
+            const int s = (int)(it % kFStages);
+            if (!tc::mbar_wait(&bar->empty[s], (uint32_t)((it / kFStages) & 1) ^ 1u, limit, abort, a.status, 1)) break;
+            tc::mbar_arrive_expect_tx(&bar->full[s], kFStageBytes);
+            uint8_t *st = smem + (size_t)s * kFStageBytes;
+            const int x = (c % nkc) * kKc;
+            for (int d = 0; d < kSlices; ++d) {
+              uint8_t *sl = st + d * kLBytes, *sw = st + kSlices * kLBytes + d * kFWBytes;
+              if (c < nkc) {
+                tc::tma_load_3d(sl, &tmA, &bar->full[s], x, P0, (d * a.batch + b) * a.nv + v);
+                tc::tma_load_3d(sw, &tmGR, &bar->full[s], x, R0, d * a.batch + b);
+              } else {
+                tc::tma_load_3d(sl, &tmGW, &bar->full[s], x, P0, d * a.batch + b);
+                tc::tma_load_3d(sw, &tmU, &bar->full[s], x, R0, d * a.nv + v);
+              }
+            }
+          }
+        }
+      }
+      for (int s = 0; s < kFStages; ++s) {   // every stage issued has landed before the CTA exits
+        const long long n = it / kFStages + ((it % kFStages) > s ? 1 : 0);
+        if (n > 0)
+          for (long long i = 0; i < wind_down(limit) && !tc::mbar_try_wait(&bar->full[s], (uint32_t)((n - 1) & 1)); ++i) {
+          }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      long long it = 0, win = 0;   // win: windows done per half
+      bool ok = true;
+      for (long long t = blockIdx.x; t < total && ok && !*abort; t += gridDim.x)
+        for (int v = a.v0; v < a.v1 && ok; ++v) {
+          for (int h = 0; h < 2 && ok; ++h)
+            for (int w = 0; w < nwin && ok; ++w) {
+              const int c1 = min(nkc, (w + 1) * kWin);
+              for (int kc = w * kWin; kc < c1; ++kc, ++it) {
+                const int s = (int)(it % kFStages);
+                ok = tc::mbar_wait(&bar->full[s], (uint32_t)((it / kFStages) & 1), limit, abort, a.status, 4);
+                if (!ok) break;
+                tc::tc_fence_after();
+                const uint32_t st = tc::smem_u32(smem + (size_t)s * kFStageBytes);
+                const bool first = kc == w * kWin;
+                const uint32_t ph = (uint32_t)((win + w) & 1) ^ 1u;
+                ok = (a.n - kc * kKc > 16) ? issue_chunk<kFW, 2>(tmem + h * 256, st, first, bar->acc_empty[h], ph, limit,
+                                                                 abort, a.status)
+                                           : issue_chunk<kFW, 1>(tmem + h * 256, st, first, bar->acc_empty[h], ph, limit,
+                                                                 abort, a.status);
+                if (!ok) break;
+                tc::mma_commit(&bar->empty[s]);
+              }
+              if (ok) tc::mma_commit(&bar->acc_full[h]);
+            }
+          win += nwin;
+        }
+      tc::mma_commit(&bar->drain);
+      for (long long i = 0; i < wind_down(limit) && !tc::mbar_try_wait(&bar->drain, 0); ++i) {
+      }
+    }
+  } else {
+    constexpr int kC = 4 * kFW / kEpiWarps;   // columns per warp
+    const int q = warp & 3, part = (warp - 2) >> 2;
+    const int lr = q * 32 + lane;
+    long long win = 0;
+    for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+      const int b = (int)(t / per_b), r = (int)(t % per_b);
+      const int P = (r / a.tR) * kL + lr, R0 = (r % a.tR) * kFW + part * kC;
+      double d[kC];
+#pragma unroll
+      for (int j = 0; j < kC; ++j) d[j] = 0.0;
+      const bool in = P < a.N;
+      const int cols = min(kC, a.N - R0);   // columns of this warp inside the tile (<= 0: none)
+      const int eW = in ? a.eGW[(long long)b * a.N + P] : 0;
+      const int eRl = lane < cols ? a.eGR[(long long)b * a.N + R0 + lane] : 0;
+      bool ok = true;
+      for (int v = a.v0; v < a.v1 && ok; ++v) {
+        long long ib[kC], ic[kC];
+#pragma unroll
+        for (int j = 0; j < kC; ++j) ib[j] = ic[j] = 0;
+        const int eA = in ? a.eA[((long long)b * a.nv + v) * a.N + P] : 0;
+        const int eUl = lane < cols ? a.eU[(long long)v * a.N + R0 + lane] : 0;
+        for (int h = 0; h < 2 && ok; ++h)
+          for (int w = 0; w < nwin; ++w) {
+            ok = tc::mbar_wait(&bar->acc_full[h], (uint32_t)((win + w) & 1), limit, abort, a.status, 8);
+            if (!ok) break;
+            tc::tc_fence_after();
+            const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + h * 256 + part * kC;
+            if (h == 0)
+              read_window<LK, kC, kFW>(base, bar->acc_empty[0], lane, ib);
+            else
+              read_window<LK, kC, kFW>(base, bar->acc_empty[1], lane, ic);
+          }
+        win += nwin;
+        if (!ok) break;
+        unsigned odd = 0u;   // columns to recompute from the sources
+#pragma unroll
+        for (int j = 0; j < kC; ++j) {
+          const int eR = __shfl_sync(0xffffffffu, eRl, j), eU = __shfl_sync(0xffffffffu, eUl, j);
+          double bv, cv;
+          const bool fb = scaled_double(ib[j], eA + eR - 2044 - (62 - LK), bv);
+          const bool fc = scaled_double(ic[j], eW + eU - 2044 - (62 - LK), cv);
+          if (fb && fc)
+            d[j] = fma(bv, cv, d[j]);
+          else
+            odd |= 1u << j;
+        }
+        if (odd && in) {
+#pragma unroll
+          for (int j = 0; j < kC; ++j)
+            if (((odd >> j) & 1u) && j < cols)
+              d[j] = fma(plain_row_dot(a.xA + (((long long)b * a.nv + v) * a.N + P) * a.n,
+                                       a.xGR + ((long long)b * a.N + R0 + j) * a.n, a.n),
+                         plain_row_dot(a.xGW + ((long long)b * a.N + P) * a.n,
+                                       a.xU + ((long long)(R0 + j) * a.nv + v) * a.n, a.n),
+                         d[j]);
+        }
+      }
+      if (!ok) break;
+      if (!in) continue;
+      double *D = a.D + b * a.sD + (long long)P * a.N;
+#pragma unroll
+      for (int j = 0; j < kC; ++j)
+        if (R0 + j < a.N) D[R0 + j] = d[j];
+    }
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem, 512);
+  }
+}
+
+size_t fsmem_bytes() { return (size_t)kFStages * kFStageBytes + sizeof(FBars) + 1024; }
+
 size_t smem_bytes() { return (size_t)kStages * kStageBytes + sizeof(Bars) + 1024; }
 
-bool make_map(CUtensorMap *map, const SliceOp &op, int box_rows, std::string *err) {
+bool make_map(CUtensorMap *map, const SliceOp &op, int box_rows, std::string *err) {   // box kKc x box_rows
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     cudaDriverEntryPointQueryResult q;
@@ -524,6 +811,43 @@ Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceG
   return Status::ok();
 }
 
+Status slice_bcd(sox_handle h, const SliceOp &A, const SliceOp &GR, const SliceOp &GW, const SliceOp &U2, int n, int N,
+                 int batch, int v0, int v1, double *D, long long sD, cudaStream_t s) {
+  if (batch <= 0) return Status::ok();
+  v1 = (v1 <= 0 || v1 > n) ? n : v1;
+  v0 = v0 < 0 ? 0 : (v0 > v1 ? v1 : v0);
+  CUtensorMap mA, mGR, mGW, mU;
+  std::string err;
+  if (!make_map(&mA, A, kL, &err) || !make_map(&mGR, GR, kFW, &err) || !make_map(&mGW, GW, kL, &err) ||
+      !make_map(&mU, U2, kFW, &err))
+    return {SOX_ERR_CUDA, err};
+  FArgs a;
+  a.n = n; a.N = N; a.batch = GR.batch; a.v0 = v0; a.v1 = v1;
+  a.tP = (N + kL - 1) / kL;
+  a.tR = (N + kFW - 1) / kFW;
+  a.eA = A.ex; a.eGR = GR.ex; a.eGW = GW.ex; a.eU = U2.ex;
+  a.D = D; a.sD = sD;
+  a.xA = static_cast<const double *>(A.src);
+  a.xGR = static_cast<const double *>(GR.src);
+  a.xGW = static_cast<const double *>(GW.src);
+  a.xU = static_cast<const double *>(U2.src);
+  a.nv = n;
+  a.spin_limit = h->spin_limit;
+  a.status = h->d_status;
+  const long long tiles = (long long)a.tP * a.tR * a.batch;
+  const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, h->sm_count));
+  static std::atomic<unsigned long long> attr7{0}, attr10{0};
+  if (n <= 128) {
+    SOX_CUDA_TRY(set_smem_once(k_slice_bcd<7>, (int)fsmem_bytes(), attr7));
+    k_slice_bcd<7><<<grid, kThreads, fsmem_bytes(), s>>>(mA, mGR, mGW, mU, a);
+  } else {
+    SOX_CUDA_TRY(set_smem_once(k_slice_bcd<10>, (int)fsmem_bytes(), attr10));
+    k_slice_bcd<10><<<grid, kThreads, fsmem_bytes(), s>>>(mA, mGR, mGW, mU, a);
+  }
+  SOX_CUDA_TRY(cudaGetLastError());
+  return Status::ok();
+}
+
 // The FP64 pipe makes 0.48e12 multiply-adds a second on a full grid: 31 us at the line, where
 // slicing both operands and the product take about 20 us in three launches.
 bool slices_pay(long long M, long long N, long long K, long long batch) {
@@ -531,20 +855,31 @@ bool slices_pay(long long M, long long N, long long K, long long batch) {
 }
 
 namespace {
-// the operands of g as (batch, rows) with one block where the stride is 0 or the batch is 1
-struct Ops {
-  int bA, bB;
+// A product runs in passes whose digits stay below kPassBytes per operand: over batches, and
+// over the columns of a single large one.
+constexpr size_t kPassBytes = size_t(1) << 30;
+struct Passes {
+  bool sharedA, sharedB;   // one block for every batch
+  int k, nb, rows;         // K, batches and columns of a pass
 };
-Ops ops_of(const GemmF64 &g) {
-  return {(g.batch == 1 || g.sA == 0) ? 1 : g.batch, (g.batch == 1 || g.sB == 0) ? 1 : g.batch};
+Passes passes_of(const GemmF64 &g) {
+  Passes p;
+  p.sharedA = g.batch == 1 || g.sA == 0;
+  p.sharedB = g.batch == 1 || g.sB == 0;
+  p.k = std::min(g.K, kSliceMaxK);
+  const size_t per = std::max(p.sharedA ? 0 : slice_bytes(1, g.M, p.k), p.sharedB ? 0 : slice_bytes(1, g.Nc, p.k));
+  p.nb = per == 0 ? g.batch : (int)std::max<size_t>(1, std::min<size_t>(g.batch, kPassBytes / per));
+  const size_t row = slice_bytes(1, 1024, p.k) / 1024 + 1;
+  p.rows = (int)std::max<size_t>(1024, std::min<size_t>(g.Nc, kPassBytes / row / (p.sharedB ? 1 : p.nb)));
+  p.rows = std::min(p.rows, g.Nc);
+  return p;
 }
 }  // namespace
 
 size_t gemm_f64_bytes(const GemmF64 &g) {
   if (!slices_pay(g.M, g.Nc, g.K, g.batch)) return 0;
-  const Ops o = ops_of(g);
-  const int k = std::min(g.K, kSliceMaxK);
-  return slice_bytes(o.bA, g.M, k) + slice_bytes(o.bB, g.Nc, k);
+  const Passes p = passes_of(g);
+  return slice_bytes(p.sharedA ? 1 : p.nb, g.M, p.k) + slice_bytes(p.sharedB ? 1 : p.nb, p.rows, p.k);
 }
 
 Status gemm_f64(sox_handle h, const GemmF64 &g, Arena scratch, cudaStream_t s) {
@@ -553,23 +888,30 @@ Status gemm_f64(sox_handle h, const GemmF64 &g, Arena scratch, cudaStream_t s) {
     launch_gemm_f64(g, s);
     return Status::ok();
   }
-  const Ops o = ops_of(g);
-  for (int k0 = 0; k0 < g.K; k0 += kSliceMaxK) {
-    const int k = std::min(kSliceMaxK, g.K - k0);
-    Arena ar = scratch;
-    SliceOp A = slice_take(ar, o.bA, g.M, k), B = slice_take(ar, o.bB, g.Nc, k);
-    if (!A.p || !B.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-    slice_rows(g.A + k0 * g.ak, false, g.sA, g.ai, g.ak, o.bA, A, s);
-    slice_rows(g.B + k0 * g.bk, false, g.sB, g.bj, g.bk, o.bB, B, s);
-    SliceGemm sg;
-    sg.C = g.C; sg.sC = g.sC; sg.ci = g.ci; sg.cj = g.cj;
-    sg.alpha = g.alpha;
-    sg.beta = k0 == 0 ? g.beta : 1.0;
-    sg.batch = g.batch;
-    sg.skip = g.skip;
-    SOX_TRY(slice_gemm(h, A, B, sg, s));
-    h->launches += 2;   // the two slicings; callers count the product
-  }
+  const Passes p = passes_of(g);
+  for (int k0 = 0; k0 < g.K; k0 += p.k)
+    for (int b0 = 0; b0 < g.batch; b0 += p.nb) {
+      const int k = std::min(p.k, g.K - k0), nb = std::min(p.nb, g.batch - b0);
+      Arena ar = scratch;
+      SliceOp A = slice_take(ar, p.sharedA ? 1 : nb, g.M, k);
+      if (!A.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+      slice_rows(g.A + b0 * g.sA + k0 * g.ak, false, g.sA, g.ai, g.ak, A.batch, A, s);
+      for (int j0 = 0; j0 < g.Nc; j0 += p.rows) {
+        Arena br = ar;
+        SliceOp B = slice_take(br, p.sharedB ? 1 : nb, std::min(p.rows, g.Nc - j0), k);
+        if (!B.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+        slice_rows(g.B + b0 * g.sB + k0 * g.bk + j0 * g.bj, false, g.sB, g.bj, g.bk, B.batch, B, s);
+        SliceGemm sg;
+        sg.C = g.C + b0 * g.sC + j0 * g.cj;
+        sg.sC = g.sC; sg.ci = g.ci; sg.cj = g.cj;
+        sg.alpha = g.alpha;
+        sg.beta = k0 == 0 ? g.beta : 1.0;
+        sg.batch = nb;
+        sg.skip = g.skip ? g.skip + b0 : nullptr;
+        SOX_TRY(slice_gemm(h, A, B, sg, s));
+        h->launches += 2;   // the slicings; callers count the product
+      }
+    }
   return Status::ok();
 }
 

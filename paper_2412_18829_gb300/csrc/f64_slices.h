@@ -53,6 +53,12 @@ struct SliceGemm {
 constexpr int kSliceMaxK = 1024;
 Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceGemm &g, cudaStream_t s);
 
+// D[b][P][R] = sum_{v0 <= v < v1} (sum_q A[b][v][P][q] GR[b][R][q]) (sum_w GW[b][P][w] U2[R][v][w]) (v1 <= 0: all n):
+// A sliced as batch (b, v), rows P; GR and GW as batch b; U2 as batch v, rows R, with src
+// strides of the contiguous arrays named here.  n <= kSliceMaxK.
+Status slice_bcd(sox_handle h, const SliceOp &A, const SliceOp &GR, const SliceOp &GW, const SliceOp &U2, int n, int N,
+                 int batch, int v0, int v1, double *D, long long sD, cudaStream_t s);
+
 // Whether a product of these sizes is faster through slices than on the FP64 pipe.
 bool slices_pay(long long M, long long N, long long K, long long batch);
 

@@ -155,3 +155,28 @@ def test_fp64_products_with_zeros_infinities_and_nans(env):
     bound = (n + 4) * 2.0 ** -52 * np.abs(X).max() * np.broadcast_to(cmax, ref.shape) + 1e-320
     assert (np.abs(got - np.where(fin, ref, 0.0))[fin] <= bound[fin]).all()
     assert (got[:, 5][np.isfinite(G[0, 0]).all(axis=(1, 2))] == 0.0).all() and (got[1] == 0.0).all()
+
+
+# n on both sides of a 16-wide step, a 32-wide chunk and the 128-wide window; N at the ends of
+# the 128 x 32 tiles; the first two shapes stay on the FP64 pipe
+@pytest.mark.parametrize("n,N,n_tau,v", [(3, 9, 4, None), (9, 64, 2, None), (16, 128, 6, None), (17, 129, 5, (3, 11)),
+                                         (33, 160, 4, None), (64, 96, 3, None), (128, 33, 4, None), (130, 161, 2, None)])
+def test_fp64_chain_from_digit_slices(env, n, N, n_tau, v):
+    torch, pkg, hs = env
+    w = synth.molecule(500 + n, n, N, n_tau, 30.0, 1)
+    p = pkg.problem(n, N, n_tau, 1, w.beta)
+    G, X, V = to_dev(torch, w.G, w.X, w.V)
+    S = torch.full_like(G, float("nan"))
+    with pkg.Handle("fp64") as h:
+        if v:   # the two parts of a partition add up to the whole
+            S1 = torch.empty_like(G)
+            pkg.sox_set_v_range(h, 0, v[0])
+            pkg.sox_sigma(h, p, G, X, V, S)
+            for a, b in ((v[0], v[1]), (v[1], n)):
+                pkg.sox_set_v_range(h, a, b)
+                pkg.sox_sigma(h, p, G, X, V, S1)
+                S += S1
+        else:
+            pkg.sox_sigma(h, p, G, X, V, S)
+        pkg.sox_check_device(h)
+    check(S.cpu().numpy(), osox.sox_sigma(w.X, w.V, w.G).real, "fp64", f"n={n} N={N}")
