@@ -2,6 +2,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 
 #include "smem_attr.h"
 #include "tc_common.cuh"
@@ -127,6 +128,86 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
   }
 }
 
+// Complex rows (see SliceOp::kind): 32 rows per block, lanes along the index that is
+// contiguous in memory, a row's eight halves (four complex values) per thread.
+template <int KIND>
+__global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long long sb, long long sr, long long sk,
+                                                       int rows, int batch_all, int K, int K8, int sa, int sc,
+                                                       __half *p, int *ex) {
+  __shared__ long long sx[2][32][33];
+  __shared__ int se[32];
+  const int b = blockIdx.y, r0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const bool along_k = sk == 1;
+  const double2 *x = src + b * sb;
+  if (threadIdx.x < 32) se[threadIdx.x] = 1;
+  __syncthreads();
+  if (along_k) {
+    for (int r = ty; r < 32; r += 8) {
+      int E = 1;
+      if (r0 + r < rows)
+        for (int k = tx; k < K; k += 32) {
+          const double2 v = x[(long long)(r0 + r) * sr + k];
+          E = max(E, max(exp_field(v.x), exp_field(v.y)));
+        }
+      for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+      if (tx == 0) se[r] = E;
+    }
+  } else {
+    int E = 1;
+    if (r0 + tx < rows)
+      for (int k = ty; k < K; k += 8) {
+        const double2 v = x[(long long)(r0 + tx) * sr + k * sk];
+        E = max(E, max(exp_field(v.x), exp_field(v.y)));
+      }
+    atomicMax(&se[tx], E);
+  }
+  __syncthreads();
+  const int nr = KIND == 2 ? 2 : 1;   // real rows per complex row
+  if (threadIdx.x < 32 && r0 + tx < rows) {
+    const int e = se[tx] < 0x7ff ? se[tx] : kNonFinite;
+    for (int i = 0; i < nr; ++i) ex[((long long)b * rows + r0 + tx) * nr + i] = e;
+  }
+  const long long plane = (long long)batch_all * rows * nr * K8;
+  const int row = threadIdx.x / 8, c8 = threadIdx.x % 8;
+  for (int k0 = 0; 2 * k0 < K8; k0 += 32) {
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {
+      const int k = along_k ? tx : i, r = along_k ? i : tx, E = se[r];
+      const bool in = r0 + r < rows && k0 + k < K && E < 0x7ff;
+      double2 v = make_double2(0.0, 0.0);
+      if (in) v = x[(long long)(r0 + r) * sr + (k0 + k) * sk];
+      sx[0][k][r] = in ? fixed55(v.x, E) : 0;
+      sx[1][k][r] = in ? fixed55(v.y, E) : 0;
+    }
+    __syncthreads();
+    if (r0 + row < rows && 2 * k0 + c8 * 8 < K8) {
+      const long long o = ((long long)b * rows + r0 + row) * nr * K8 + 2 * k0 + c8 * 8;
+#pragma unroll
+      for (int i = 0; i < nr; ++i) {
+        long long X[8];
+        uint4 w[kSlices];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const long long re = sx[0][c8 * 4 + e][row], im = sx[1][c8 * 4 + e][row];
+          if (KIND == 1) {
+            X[2 * e] = re;
+            X[2 * e + 1] = im;
+          } else if (i == 0) {
+            X[2 * e] = re;
+            X[2 * e + 1] = sa * sc > 0 ? -im : im;
+          } else {
+            X[2 * e] = sc > 0 ? im : -im;
+            X[2 * e + 1] = sa > 0 ? re : -re;
+          }
+        }
+        digits8(X, w);
+#pragma unroll
+        for (int d = 0; d < kSlices; ++d) *reinterpret_cast<uint4 *>(p + d * plane + o + (long long)i * K8) = w[d];
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------ product
 // 128 (lane side, TMEM lanes) x 64 output tiles: the eight FP32 sums of a tile fill the 512
 // TMEM columns.  K goes in chunks of 32 (64-byte swizzled rows, seven digit tiles of both
@@ -155,6 +236,13 @@ struct Bars {
   int abort;
 };
 
+// Where an operand's elements came from
+struct Plain {
+  const void *x;
+  int f32, kind, sa, sc;
+  long long sb, sr, sk;
+};
+
 struct Args {
   int nL, nW, K, batch, tL, tW;
   int bL, bW;                // batches of the operands (1: shared)
@@ -164,10 +252,7 @@ struct Args {
   double alpha, beta;
   const int *skip, *mirror;
   int lane_is_row;           // lane index is C's row index i (else its column index j)
-  // sources, for rows with infinities or NaNs
-  const void *xL, *xW;
-  int f32L, f32W;
-  long long sbL, srL, skL, sbW, srW, skW;
+  Plain xL, xW;              // sources, for rows with infinities or NaNs
   long long spin_limit;
   int *status;
 };
@@ -284,15 +369,21 @@ __device__ __forceinline__ void read_window(uint32_t base, uint64_t *acc_empty, 
   }
 }
 
-__device__ __forceinline__ double plain_at(const void *x, int f32, long long o) {
-  return f32 ? (double)static_cast<const float *>(x)[o] : static_cast<const double *>(x)[o];
+__device__ double plain_at(const Plain &p, long long b, int r, int k) {
+  if (p.kind == 0) {
+    const long long o = b * p.sb + r * p.sr + k * p.sk;
+    return p.f32 ? (double)static_cast<const float *>(p.x)[o] : static_cast<const double *>(p.x)[o];
+  }
+  const double2 v = static_cast<const double2 *>(p.x)[b * p.sb + (p.kind == 2 ? r / 2 : r) * p.sr + (k / 2) * p.sk];
+  if (p.kind == 1) return (k & 1) ? v.y : v.x;
+  if (!(r & 1)) return (k & 1) ? -p.sa * p.sc * v.y : v.x;
+  return (k & 1) ? p.sa * v.x : p.sc * v.y;
 }
 // the element as a chain of FP64 FMAs from the sources (rows with infinities or NaNs)
 __device__ __noinline__ double plain_element(const Args &a, int b, int l, int w) {
-  const long long oL = (a.bL == 1 ? 0LL : b * a.sbL) + l * a.srL, oW = (a.bW == 1 ? 0LL : b * a.sbW) + w * a.srW;
   double acc = 0.0;
   for (int k = 0; k < a.K; ++k)
-    acc = fma(plain_at(a.xL, a.f32L, oL + k * a.skL), plain_at(a.xW, a.f32W, oW + k * a.skW), acc);
+    acc = fma(plain_at(a.xL, a.bL == 1 ? 0 : b, l, k), plain_at(a.xW, a.bW == 1 ? 0 : b, w, k), acc);
   return acc;
 }
 
@@ -314,8 +405,19 @@ __device__ __forceinline__ bool scaled_double(long long I, int x, double &v) {
   return I == 0 ? x < kNonFinite / 2 : (unsigned)(eb - 1) <= 2044u;
 }
 
+// What happens to an element on its way out: +-v, C +- v, or alpha v + beta C.  A template
+// parameter, because a select between FP64 results computes them all, and each FP64
+// instruction of a tile takes 4300 clocks of the SM's pipe (a third of the tile's time).
+enum { kOutSet = 0, kOutAdd = 1, kOutGeneral = 2 };
+template <int OUT>
+__device__ __forceinline__ double out_value(double v, long long sign, double old, double alpha, double beta) {
+  if (OUT == kOutGeneral) return beta != 0.0 ? fma(beta, old, alpha * v) : alpha * v;
+  v = __longlong_as_double(__double_as_longlong(v) ^ sign);
+  return OUT == kOutAdd ? old + v : v;
+}
+
 // LK: the sums of a tile stay below 2^LK (K <= 2^LK), kept as integers of 2^-(62 - LK)
-template <int LK>
+template <int LK, int OUT>
 __global__ void __launch_bounds__(kThreads, 1)
     k_slice_gemm(const __grid_constant__ CUtensorMap tmL, const __grid_constant__ CUtensorMap tmW, const Args a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -432,26 +534,35 @@ __global__ void __launch_bounds__(kThreads, 1)
       double *C = a.C + b * a.sC + l * a.cl + w0 * a.cw;
       double *Cm = a.C + b * a.sC + w0 * a.cl + l * a.cw;   // mirror image
       const bool mir = a.mirror && a.mirror[b];
+      const long long sign = a.alpha < 0.0 ? (long long)0x8000000000000000ull : 0ll;
       unsigned odd = 0u;   // columns to recompute from the sources
+      constexpr int kH = 8;   // C is read eight columns at a time, all loads before the first store
 #pragma unroll
-      for (int j = 0; j < kC; ++j) {
-        const int w = w0 + j;
-        const int eW = __shfl_sync(0xffffffffu, eWl, j);
-        double v;
-        const bool fine = scaled_double(acc[j], eL + eW - 2044 - (62 - LK), v);
-        if (l < a.nL && w < a.nW) {
-          if (fine) {
-            v = a.alpha == 1.0 ? v : (a.alpha == -1.0 ? -v : a.alpha * v);
-            if (a.beta != 0.0) v = fma(a.beta, C[j * a.cw], v);
-            if (!mir) {
-              C[j * a.cw] = v;
+      for (int j0 = 0; j0 < kC; j0 += kH) {
+        double old[kH];
+        if (OUT != kOutSet && a.beta != 0.0) {
+#pragma unroll
+          for (int i = 0; i < kH; ++i) old[i] = (l < a.nL && w0 + j0 + i < a.nW) ? C[(j0 + i) * a.cw] : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < kH; ++i) {
+          const int j = j0 + i, w = w0 + j;
+          const int eW = __shfl_sync(0xffffffffu, eWl, j);
+          double v;
+          const bool fine = scaled_double(acc[j], eL + eW - 2044 - (62 - LK), v);
+          if (l < a.nL && w < a.nW) {
+            if (fine) {
+              v = out_value<OUT>(v, sign, old[i], a.alpha, a.beta);
+              if (!mir) {
+                C[j * a.cw] = v;
+              } else {
+                const int ib = (a.lane_is_row ? l : w) / 32, jb = (a.lane_is_row ? w : l) / 32;
+                if (ib <= jb) C[j * a.cw] = v;
+                if (ib < jb) Cm[j * a.cl] = v;
+              }
             } else {
-              const int ib = (a.lane_is_row ? l : w) / 32, jb = (a.lane_is_row ? w : l) / 32;
-              if (ib <= jb) C[j * a.cw] = v;
-              if (ib < jb) Cm[j * a.cl] = v;
+              odd |= 1u << j;
             }
-          } else {
-            odd |= 1u << j;
           }
         }
       }
@@ -768,6 +879,28 @@ void slice_rows(const void *src, bool f32, long long sb, long long sr, long long
   }
 }
 
+void slice_complex_a(const double *src, long long sb, long long sr, long long sk, int batch, SliceOp &op, cudaStream_t s) {
+  op.src = src;
+  op.sb = sb; op.sr = sr; op.sk = sk;
+  op.kind = 1;
+  if (batch <= 0 || op.rows <= 0) return;
+  k_slice_complex<1><<<dim3((op.rows + 31) / 32, batch), 256, 0, s>>>(
+      reinterpret_cast<const double2 *>(src), sb, sr, sk, op.rows, op.batch, op.K / 2, op.K8, 1, 1, op.p, op.ex);
+}
+
+void slice_complex_b(const double *src, long long sb, long long sr, long long sk, int batch, bool conjA, bool conjB,
+                     SliceOp &op, cudaStream_t s) {
+  op.src = src;
+  op.sb = sb; op.sr = sr; op.sk = sk;
+  op.kind = 2;
+  op.sa = conjA ? -1 : 1;
+  op.sc = conjB ? -1 : 1;
+  if (batch <= 0 || op.rows <= 0) return;
+  const int rows = op.rows / 2;
+  k_slice_complex<2><<<dim3((rows + 31) / 32, batch), 256, 0, s>>>(
+      reinterpret_cast<const double2 *>(src), sb, sr, sk, rows, op.batch, op.K / 2, op.K8, op.sa, op.sc, op.p, op.ex);
+}
+
 Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceGemm &g, cudaStream_t s) {
   if (g.batch <= 0 || A.rows <= 0 || B.rows <= 0) return Status::ok();
   // TMEM lanes along the index that leaves less padding in the 128 x 64 tiles; equal: along
@@ -791,23 +924,28 @@ Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceG
   a.alpha = g.alpha; a.beta = g.beta;
   a.skip = g.skip; a.mirror = g.mirror;
   a.lane_is_row = lane_a ? 1 : 0;
-  a.xL = L.src; a.xW = W.src;
-  a.f32L = L.f32; a.f32W = W.f32;
-  a.sbL = L.sb; a.srL = L.sr; a.skL = L.sk;
-  a.sbW = W.sb; a.srW = W.sr; a.skW = W.sk;
+  a.xL = {L.src, L.f32 ? 1 : 0, L.kind, L.sa, L.sc, L.sb, L.sr, L.sk};
+  a.xW = {W.src, W.f32 ? 1 : 0, W.kind, W.sa, W.sc, W.sb, W.sr, W.sk};
   a.spin_limit = h->spin_limit;
   a.status = h->d_status;
   const long long tiles = (long long)a.tL * a.tW * a.batch;
   const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, h->sm_count));
-  static std::atomic<unsigned long long> attr7{0}, attr10{0};
-  if (a.K <= 128) {
-    SOX_CUDA_TRY(set_smem_once(k_slice_gemm<7>, (int)smem_bytes(), attr7));
-    k_slice_gemm<7><<<grid, kThreads, smem_bytes(), s>>>(mL, mW, a);
-  } else {
-    SOX_CUDA_TRY(set_smem_once(k_slice_gemm<10>, (int)smem_bytes(), attr10));
-    k_slice_gemm<10><<<grid, kThreads, smem_bytes(), s>>>(mL, mW, a);
-  }
-  SOX_CUDA_TRY(cudaGetLastError());
+  const bool unit = a.alpha == 1.0 || a.alpha == -1.0;
+  const int out = unit && a.beta == 0.0 ? kOutSet : (unit && a.beta == 1.0 ? kOutAdd : kOutGeneral);
+  auto go = [&](auto lk, auto o) -> cudaError_t {
+    static std::atomic<unsigned long long> attr{0};
+    auto *k = k_slice_gemm<decltype(lk)::value, decltype(o)::value>;
+    const cudaError_t e = set_smem_once(k, (int)smem_bytes(), attr);
+    if (e != cudaSuccess) return e;
+    k<<<grid, kThreads, smem_bytes(), s>>>(mL, mW, a);
+    return cudaGetLastError();
+  };
+  auto pick = [&](auto lk) {
+    return out == kOutSet ? go(lk, std::integral_constant<int, kOutSet>{})
+                          : (out == kOutAdd ? go(lk, std::integral_constant<int, kOutAdd>{})
+                                            : go(lk, std::integral_constant<int, kOutGeneral>{}));
+  };
+  SOX_CUDA_TRY(a.K <= 128 ? pick(std::integral_constant<int, 7>{}) : pick(std::integral_constant<int, 10>{}));
   return Status::ok();
 }
 

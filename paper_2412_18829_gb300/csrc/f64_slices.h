@@ -30,6 +30,10 @@ struct SliceOp {
   const void *src = nullptr;
   bool f32 = false;
   long long sb = 0, sr = 0, sk = 0;
+  // complex operands (strides in complex elements): kind 1 is the A side, a complex row as one
+  // row of 2 K interleaved reals; kind 2 the B side, a complex row as the two rows
+  // (b_r, -sa sc b_i) and (sc b_i, sa b_r), sa, sc = -1 for the conjugate of A, of B
+  int kind = 0, sa = 1, sc = 1;
 };
 size_t slice_bytes(long long batch, int rows, int K);
 SliceOp slice_take(Arena &ar, int batch, int rows, int K);
@@ -37,6 +41,11 @@ SliceOp slice_take(Arena &ar, int batch, int rows, int K);
 // (at most op's)
 void slice_rows(const void *src, bool f32, long long sb, long long sr, long long sk, int batch, SliceOp &op,
                 cudaStream_t s);
+
+// The same for complex rows (FP64, interleaved): op taken with rows (A) or 2 rows (B) and 2 K
+void slice_complex_a(const double *src, long long sb, long long sr, long long sk, int batch, SliceOp &op, cudaStream_t s);
+void slice_complex_b(const double *src, long long sb, long long sr, long long sk, int batch, bool conjA, bool conjB,
+                     SliceOp &op, cudaStream_t s);
 
 // C[b](i, j) = alpha sum_k A(b, i, k) B(b, j, k) + beta C[b](i, j); an operand of batch 1 is
 // shared.  Element (i, j) at C + b * sC + i * ci + j * cj.

@@ -419,16 +419,8 @@ void launch_gj_step(double *Aug, int N, int k, int *info, cudaStream_t s) {
   k_gj_elim<<<grid, 256, 0, s>>>(Aug, N, k, info);
 }
 
-void launch_build_gj_system(const double *V, const double *Pi, double *Aug, int N, cudaStream_t s) {
+void launch_gj_init(const double *V, double *Aug, int N, cudaStream_t s) {
   k_build_gj<<<grid_for((long long)N * N), 256, 0, s>>>(V, Aug, N);
-  // left half: I - V Pi
-  GemmF64 g;
-  g.M = N; g.Nc = N; g.K = N;
-  g.A = V; g.ai = N; g.ak = 1;
-  g.B = Pi; g.bk = N; g.bj = 1;
-  g.C = Aug; g.ci = 2LL * N; g.cj = 1;
-  g.alpha = -1.0; g.beta = 1.0;
-  launch_gemm_f64(g, s);
 }
 
 void launch_copy_right_half(const double *Aug, double *W, int N, cudaStream_t s) {

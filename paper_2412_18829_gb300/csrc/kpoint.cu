@@ -16,6 +16,8 @@
 #include <vector>
 
 #include "ctc.h"
+#include "f64_slices.h"
+#include "gj.h"
 #include "kpoint.h"
 
 namespace sox {
@@ -106,6 +108,65 @@ void zgemm(const ZGemm &g, cudaStream_t s) {
   if (g.M <= 0 || g.Nc <= 0 || g.batch <= 0) return;
   dim3 grid((g.Nc + TM - 1) / TM, (g.M + TM - 1) / TM, g.batch);
   k_zgemm<<<grid, NT, 0, s>>>(g);
+}
+
+// The complex product through digit slices (f64_slices.h) as one real one: rows of A
+// interleaved, each row of B as its re-row and its im-row, K doubled.  For contiguous C rows
+// (cj = 1), batches at fixed strides; the digits of a pass stay below a GiB per operand.
+struct ZPasses {
+  bool sharedA, sharedB;
+  int k, nb, rows;   // K, batches and columns (complex) of a pass
+};
+ZPasses zpasses(int M, int Nc, int K, int batch, bool sharedA, bool sharedB) {
+  constexpr size_t kPass = size_t(1) << 30;
+  ZPasses p;
+  p.sharedA = sharedA;
+  p.sharedB = sharedB;
+  p.k = std::min(K, kSliceMaxK / 2);
+  const size_t per = std::max(sharedA ? 0 : slice_bytes(1, M, 2 * p.k), sharedB ? 0 : slice_bytes(1, 2 * Nc, 2 * p.k));
+  p.nb = per == 0 ? batch : (int)std::max<size_t>(1, std::min<size_t>(batch, kPass / per));
+  const size_t row = slice_bytes(1, 1024, 2 * p.k) / 512 + 1;
+  p.rows = (int)std::max<size_t>(1024, std::min<size_t>(Nc, kPass / row / (sharedB ? 1 : p.nb)));
+  p.rows = std::min(p.rows, Nc);
+  return p;
+}
+bool zslices_pay(int M, int Nc, int K, long long batch) { return slices_pay(M, 2LL * Nc, 2LL * K, batch); }
+size_t zgemm_bytes(int M, int Nc, int K, int batch, bool sharedA, bool sharedB) {
+  if (!zslices_pay(M, Nc, K, batch)) return 0;
+  const ZPasses p = zpasses(M, Nc, K, batch, sharedA || batch == 1, sharedB || batch == 1);
+  return slice_bytes(p.sharedA ? 1 : p.nb, M, 2 * p.k) + slice_bytes(p.sharedB ? 1 : p.nb, 2 * p.rows, 2 * p.k);
+}
+Status zgemm_f64(sox_handle h, const ZGemm &g, Arena scratch, cudaStream_t s) {
+  if (g.M <= 0 || g.Nc <= 0 || g.batch <= 0) return Status::ok();
+  if (g.offA || g.offB || g.offC || g.cj != 1 || !zslices_pay(g.M, g.Nc, g.K, g.batch)) {
+    zgemm(g, s);
+    return Status::ok();
+  }
+  const ZPasses p = zpasses(g.M, g.Nc, g.K, g.batch, g.sA == 0 || g.batch == 1, g.sB == 0 || g.batch == 1);
+  auto d = [](const z *x) { return reinterpret_cast<const double *>(x); };
+  for (int k0 = 0; k0 < g.K; k0 += p.k)
+    for (int b0 = 0; b0 < g.batch; b0 += p.nb) {
+      const int k = std::min(p.k, g.K - k0), nb = std::min(p.nb, g.batch - b0);
+      Arena ar = scratch;
+      SliceOp A = slice_take(ar, p.sharedA ? 1 : nb, g.M, 2 * k);
+      if (!A.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+      slice_complex_a(d(g.A + b0 * g.sA + k0 * g.ak), g.sA, g.ai, g.ak, A.batch, A, s);
+      for (int j0 = 0; j0 < g.Nc; j0 += p.rows) {
+        Arena br = ar;
+        SliceOp B = slice_take(br, p.sharedB ? 1 : nb, 2 * std::min(p.rows, g.Nc - j0), 2 * k);
+        if (!B.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+        slice_complex_b(d(g.B + b0 * g.sB + k0 * g.bk + j0 * g.bj), g.sB, g.bj, g.bk, B.batch, g.conjA, g.conjB, B, s);
+        SliceGemm sg;
+        sg.C = reinterpret_cast<double *>(g.C + b0 * g.sC + j0);
+        sg.sC = 2 * g.sC; sg.ci = 2 * g.ci; sg.cj = 1;
+        sg.alpha = g.alpha;
+        sg.beta = k0 == 0 ? g.beta : 1.0;
+        sg.batch = nb;
+        SOX_TRY(slice_gemm(h, A, B, sg, s));
+        h->launches += 2;   // the slicings; callers count the product
+      }
+    }
+  return Status::ok();
 }
 
 ZGemm zg() {
@@ -1092,6 +1153,26 @@ __global__ void __launch_bounds__(256) k_bubble_reduce(const z *Ah, const z *Tf,
   }
 }
 
+// Pr[j][P][Q] = Ah[m][j][P][Q] Ah[-m][T-1-j][Q][P] for one m: 32 x 32 tiles, the transposed
+// partner through shared memory.  The sum over j with the transform is then one product.
+__global__ void __launch_bounds__(256) k_bubble_pairs(const z *Am, const z *Bm, int N, int T, z *Pr) {
+  __shared__ z tb[32][33];
+  const int j = blockIdx.z, P0 = blockIdx.y * 32, Q0 = blockIdx.x * 32;
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  const long long NN = (long long)N * N;
+  const z *Bj = Bm + (long long)(T - 1 - j) * NN;
+  for (int r = ty; r < 32; r += 8)
+    if (Q0 + r < N && P0 + tx < N) tb[r][tx] = Bj[(long long)(Q0 + r) * N + P0 + tx];   // tb[Q][P]
+  __syncthreads();
+  for (int r = ty; r < 32; r += 8) {
+    const int P = P0 + r, Q = Q0 + tx;
+    if (P < N && Q < N) {
+      const long long e = (long long)j * NN + (long long)P * N + Q;
+      Pr[e] = zmul(Am[e], tb[tx][r]);
+    }
+  }
+}
+
 // molecules: Pi(i Omega) <- (Re Pi + Re Pi^T) / 2 in place, per frequency
 __global__ void k_sym_real(z *Pi, int N, int nO) {
   const long long NN = (long long)N * N, total = NN * nO;
@@ -1272,7 +1353,13 @@ size_t w_dynamic_bytes(const sox_problem *p, int n_omega) {
   b += aligned_bytes(nk * n_omega * NN, 16);         // the bubble per (m, o), then per (q, o)
   b += aligned_bytes(nk * n_omega * 2 * NN, 16);     // [1 - V Pi | V] per (q, o)
   b += aligned_bytes(nk, 4) + aligned_bytes(4, 4) + aligned_bytes(2, 8);
-  return b + (1 << 20);
+  const int Ni = p->N, ni = p->n, Ti = p->n_tau;
+  // scratch of the products, the bubble's pairs (one m at a time) and the solve
+  size_t scratch = std::max(zgemm_bytes(Ni, ni, ni, Ti, true, false), zgemm_bytes(Ni, Ni, ni, Ti, false, true));
+  scratch = std::max(scratch, zgemm_bytes(Ni, Ni, Ni, n_omega, true, false));
+  scratch = std::max(scratch, aligned_bytes(T * NN, 16) + zgemm_bytes(n_omega, (int)NN, Ti, 1, true, true));
+  if (gj_pays(Ni)) scratch = std::max(scratch, gj_bytes(Ni, (int)nk * n_omega, true));
+  return b + scratch + (1 << 20);
 }
 
 Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *Gd, const double *Xd,
@@ -1348,19 +1435,39 @@ Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *
       a.A = X + (long long)k * N * n; a.sA = 0; a.ai = n; a.ak = 1;
       a.B = G + ((long long)sp * nk + k) * T * nn; a.sB = nn; a.bk = n; a.bj = 1;
       a.C = GR; a.sC = (long long)N * n; a.ci = n; a.cj = 1;
-      zgemm(a, s);
+      SOX_TRY(zgemm_f64(h, a, ar, s));
       ZGemm b = zg();   // A_k(tau_j) = GR[j] X^k^H
       b.M = N; b.Nc = N; b.K = n; b.batch = T;
       b.A = GR; b.sA = (long long)N * n; b.ai = n; b.ak = 1;
       b.B = X + (long long)k * N * n; b.sB = 0; b.bk = 1; b.bj = n; b.conjB = 1;
       b.C = Ah + (long long)k * T * NN; b.sC = NN; b.ci = N; b.cj = 1;
-      zgemm(b, s);
+      SOX_TRY(zgemm_f64(h, b, ar, s));
       launches += 2;
     }
     mesh_dft(Ah, (long long)T * NN, (long long)T * NN, nk3, -1, s);   // A-hat(m) = sum_k w^{-m.k} A_k
-    dim3 grid((N + 31) / 32, (N + 31) / 32, (unsigned)(nk * n_chunks));
-    k_bubble_reduce<<<grid, 256, 0, s>>>(Ah, Tf, negm, N, T, nO, ns, n_chunks, -1.0 / ((double)nk * nk), H);
-    launches += 4;
+    if (zslices_pay(ns, (int)NN, T, 1)) {
+      // 3 x 3 x 3, N = 300, 60 times, 30 frequencies: pairs, digits and a product per m 15 ms, the
+      // transform on the FP64 pipe inside the reduction 47 ms
+      Arena pa = ar;
+      z *Pr = pa.take<z>((size_t)T * NN);
+      if (!Pr) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+      for (int m = 0; m < nk; ++m) {
+        k_bubble_pairs<<<dim3((N + 31) / 32, (N + 31) / 32, T), 256, 0, s>>>(
+            Ah + (long long)m * T * NN, Ah + (long long)h_neg[m] * T * NN, N, T, Pr);
+        ZGemm f = zg();   // H[m][o] += alpha sum_j T_fwd[o][j] Pr[j]
+        f.M = ns; f.Nc = (int)NN; f.K = T;
+        f.A = Tf; f.ai = T; f.ak = 1;
+        f.B = Pr; f.bk = NN; f.bj = 1;
+        f.C = H + (long long)m * nO * NN; f.ci = NN; f.cj = 1;
+        f.alpha = -1.0 / ((double)nk * nk); f.beta = 1.0;
+        SOX_TRY(zgemm_f64(h, f, pa, s));
+      }
+      launches += 2 * nk + 3;
+    } else {
+      dim3 grid((N + 31) / 32, (N + 31) / 32, (unsigned)(nk * n_chunks));
+      k_bubble_reduce<<<grid, 256, 0, s>>>(Ah, Tf, negm, N, T, nO, ns, n_chunks, -1.0 / ((double)nk * nk), H);
+      launches += 4;
+    }
   }
   mesh_dft(H, (long long)ns * NN, (long long)nO * NN, nk3, 1, s);   // Pi^q = sum_m w^{+m.q} H(m), o < ns
   if (real) k_sym_real<<<grid_of((long long)ns * NN), 256, 0, s>>>(H, N, ns);
@@ -1373,9 +1480,11 @@ Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *
     g.B = H + (long long)q * nO * NN; g.sB = NN; g.bk = N; g.bj = 1;
     g.C = Aug + (long long)q * ns * 2 * NN; g.sC = 2 * NN; g.ci = 2LL * N; g.cj = 1;
     g.alpha = -1.0; g.beta = 1.0;
-    zgemm(g, s);
+    SOX_TRY(zgemm_f64(h, g, ar, s));
   }
-  for (int k = 0; k < N; ++k) {
+  const bool blocked = gj_pays(N);
+  if (blocked) SOX_TRY(gj_solve(h, reinterpret_cast<double *>(Aug), N, batch, true, info, ar, s));
+  for (int k = 0; !blocked && k < N; ++k) {
     k_gj_pivot_c<<<batch, 256, 0, s>>>(Aug, N, k, info);
     const int ncols = 2 * N - (k + 1);
     k_gj_elim_c<<<dim3((ncols + 255) / 256, std::min(N, 64), batch), 256, 0, s>>>(Aug, N, k, info);
@@ -1383,7 +1492,7 @@ Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *
   k_gj_out<<<grid_of((long long)batch * NN), 256, 0, s>>>(Aug, V, N, nO, ns, batch, real ? 1 : 0, Wd);
   if (ns < nO)
     k_w_mirror<<<grid_of((long long)nk * (nO - ns) * NN), 256, 0, s>>>(Wd, N, nO, ns, nk, real ? 1 : 0);
-  h->launches += launches + 2LL * N + 4 + nk;
+  h->launches += launches + (blocked ? 0 : 2LL * N) + 4 + nk;
   SOX_CUDA_TRY(cudaGetLastError());
   int hinfo[4] = {0, 0, 0, 0};
   SOX_CUDA_TRY(cudaMemcpyAsync(hinfo, info, sizeof(hinfo), cudaMemcpyDeviceToHost, s));

@@ -180,3 +180,52 @@ def test_fp64_chain_from_digit_slices(env, n, N, n_tau, v):
             pkg.sox_sigma(h, p, G, X, V, S)
         pkg.sox_check_device(h)
     check(S.cpu().numpy(), osox.sox_sigma(w.X, w.V, w.G).real, "fp64", f"n={n} N={N}")
+
+
+# N on both sides of the blocked solve's rule (64), of a 32-column block, of the 8-column inner
+# blocks of a single large system; the larger ones leave shared memory for part of the way
+@pytest.mark.parametrize("N", [1, 8, 63, 64, 65, 95, 130, 301, 1100])
+def test_w_static_blocks_and_pivots(env, N):
+    """W = (1 - V Pi)^-1 V with a V that forces row exchanges, against numpy's LU: the
+    forward error bound of a solve with partial pivoting, N eps cond times a factor 8."""
+    torch, pkg, hs = env
+    rng = np.random.default_rng(N)
+    V = rng.standard_normal((N, N)) / np.sqrt(N)
+    Pi = rng.standard_normal((N, N)) / np.sqrt(N)
+    K = np.eye(N) - V @ Pi
+    p = pkg.problem(2, N, 2, 1, 10.0)
+    Vd, Pd = to_dev(torch, V, Pi)
+    W = torch.full((N, N), float("nan"), dtype=torch.float64, device="cuda")
+    pkg.sox_w_static(hs["fp64"], p, Vd, Pd, W)
+    pkg.sox_check_device(hs["fp64"])
+    ref = np.linalg.solve(K, V)
+    bound = 8 * N * 2.0 ** -53 * np.linalg.cond(K) * np.abs(ref).max()
+    assert np.abs(W.cpu().numpy() - ref).max() <= bound
+
+
+@pytest.mark.parametrize("N", [40, 96])
+def test_w_static_reports_a_singular_system(env, N):
+    torch, pkg, hs = env
+    V, Pi = np.eye(N), np.eye(N)
+    Pi[3, 3] = 0.5   # 1 - V Pi = diag(0, 0, 0, 1/2, 0, ...)
+    p = pkg.problem(2, N, 2, 1, 10.0)
+    Vd, Pd = to_dev(torch, V, Pi)
+    with pytest.raises(pkg.SoxError):
+        pkg.sox_w_static(hs["fp64"], p, Vd, Pd, torch.empty_like(Vd))
+
+
+@pytest.mark.parametrize("nk,n,N,n_tau,M", [((2, 1, 1), 3, 70, 5, 2), ((1, 2, 2), 5, 97, 12, 4), ((3, 1, 1), 17, 130, 9, 3)])
+def test_w_dynamic_of_solids_through_slices(env, nk, n, N, n_tau, M):
+    """Complex products and the blocked complex solve at ragged sizes against the oracle."""
+    from oracle import kpoints
+
+    torch, pkg, hs = env
+    w = synth.solid(40 + n, nk, n, N, n_tau, 20.0)
+    _, Tf, _ = synth.bosonic_transforms(w.tau, w.beta, M)
+    p = pkg.problem(n, N, n_tau, 1, w.beta, nk=nk, dtype=1)
+    G, X, V, F = to_dev(torch, *(np.asarray(a, dtype=complex) for a in (w.G, w.X, w.V, Tf)))
+    out = torch.full((w.n_k, 2 * M + 1, N, N), complex(float("nan"), 0.0), dtype=torch.complex128, device="cuda")
+    pkg.sox_w_dynamic(hs["fp64"], p, G, X, V, F, 2 * M + 1, out)
+    pkg.sox_check_device(hs["fp64"])
+    ref = kpoints.w_dynamic(w.V, kpoints.pi_omega(w.X, w.G[0], Tf, nk))
+    assert np.abs(out.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
