@@ -704,6 +704,12 @@ size_t tables_bytes(const KTc &g) { return 5 * aligned_bytes(g.nk2, 4); }
 
 long long nnpad_of(const KTc &g) { return g.nn + (g.nn & 1); }
 
+// idx[(pair, il)] = ku[pair] * cc + il
+__global__ void k_pair_tau_index(const int *ku, long long nk2, int cc, int *idx) {
+  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (e < nk2 * cc) idx[e] = ku[e / cc] * cc + (int)(e % cc);
+}
+
 // scratch of mixed_tc (released after the call)
 size_t mixed_tc_scratch(const KTc &g) {
   return csplit_bytes(g.nk, g.N, g.N) + csplit_bytes((int)g.nk2, (int)(2 * g.nn), g.N);
@@ -737,38 +743,103 @@ void split_m2_tc(const float *M, const KTc &g, const std::vector<CSplit> &M2s, c
              g.n, false, false, M2s[v], s);
 }
 
-// Sigma^k(tau_i) (+)= alpha X_k^H D[k]^T X_k for every k (D FP64 [k][N][ldN])
-void backproject_k(const z *D, const z *X, const KTc &g, z *T1, z *Sig_i, long long sS, double alpha, double beta,
-                   cudaStream_t s) {
-  ZGemm t = zg();
-  t.M = g.N; t.Nc = g.n; t.K = g.N; t.batch = g.nk;
-  t.A = D; t.sA = (long long)g.N * g.ldN; t.ai = 1; t.ak = g.ldN;
-  t.B = X; t.sB = g.Nn; t.bk = g.n; t.bj = 1;
-  t.C = T1; t.sC = g.Nn; t.ci = g.n; t.cj = 1;
-  zgemm(t, s);
-  ZGemm o = zg();
-  o.M = g.n; o.Nc = g.n; o.K = g.N; o.batch = g.nk;
-  o.A = X; o.sA = g.Nn; o.ai = 1; o.ak = g.n; o.conjA = 1;
-  o.B = T1; o.sB = g.Nn; o.bk = g.n; o.bj = 1;
-  o.C = Sig_i; o.sC = sS; o.ci = g.n; o.cj = 1;
-  o.alpha = alpha; o.beta = beta;
-  zgemm(o, s);
+// The FP64 products of the chain for cc tau points of one k (operands set by the caller):
+// G_Rq = X G, G_wP^T = conj(X) G^T, the half transform T1 = D^T X and Sigma = X^H T1.
+struct KGemms {
+  ZGemm gr, gw, half, out;
+};
+KGemms k_gemms(const KTc &g, int cc) {
+  KGemms f;
+  f.gr = zg();
+  f.gr.M = g.N; f.gr.Nc = g.n; f.gr.K = g.n; f.gr.batch = cc;
+  f.gr.ai = g.n; f.gr.ak = 1;
+  f.gr.sB = g.nn; f.gr.bk = g.n; f.gr.bj = 1;
+  f.gr.sC = g.Nn; f.gr.ci = g.n; f.gr.cj = 1;
+  f.gw = f.gr;
+  f.gw.conjA = 1; f.gw.bk = 1; f.gw.bj = g.n;
+  f.half = zg();
+  f.half.M = g.N; f.half.Nc = g.n; f.half.K = g.N; f.half.batch = cc;
+  f.half.sA = (long long)g.nk * g.N * g.ldN; f.half.ai = 1; f.half.ak = g.ldN;
+  f.half.bk = g.n; f.half.bj = 1;
+  f.half.sC = g.Nn; f.half.ci = g.n; f.half.cj = 1;
+  f.out = zg();
+  f.out.M = g.n; f.out.Nc = g.n; f.out.K = g.N; f.out.batch = cc;
+  f.out.ai = 1; f.out.ak = g.n; f.out.conjA = 1;
+  f.out.sB = g.Nn; f.out.bk = g.n; f.out.bj = 1;
+  f.out.sC = g.nn; f.out.ci = g.n; f.out.cj = 1;
+  return f;
+}
+size_t k_gemms_bytes(const KTc &g, int cc) {
+  size_t b = zgemm_bytes(g.N, g.n, g.n, cc, true, false);
+  b = std::max(b, zgemm_bytes(g.N, g.n, g.N, cc, false, true));
+  return std::max(b, zgemm_bytes(g.n, g.n, g.N, cc, true, false));
+}
+
+// GR and GWt ([k][cc][N][n]) of tau points t0 .. t0 + cc - 1 for every k
+Status project_k(sox_handle h, const z *Gs, const z *X, const KTc &g, int t0, int cc, z *GR, z *GWt, Arena scratch,
+                 cudaStream_t s) {
+  KGemms f = k_gemms(g, cc);
+  for (int k = 0; k < g.nk; ++k) {
+    f.gr.A = f.gw.A = X + (long long)k * g.Nn;
+    f.gr.B = f.gw.B = Gs + ((long long)k * g.T + t0) * g.nn;
+    f.gr.C = GR + (long long)k * cc * g.Nn;
+    f.gw.C = GWt + (long long)k * cc * g.Nn;
+    SOX_TRY(zgemm_f64(h, f.gr, scratch, s));
+    SOX_TRY(zgemm_f64(h, f.gw, scratch, s));
+  }
+  h->launches += 2 * g.nk;
+  return Status::ok();
+}
+
+// Sigma^k(tau_i) (+)= alpha X_k^H D[i][k]^T X_k for every k and cc tau points (D FP64
+// [cc][k][N][ldN]; T1 [cc][N][n]); Sig at the first tau point of k = 0
+Status backproject_k(sox_handle h, const z *D, const z *X, const KTc &g, int cc, z *T1, z *Sig, double alpha, double beta,
+                     Arena scratch, cudaStream_t s) {
+  KGemms f = k_gemms(g, cc);
+  f.out.alpha = alpha;
+  f.out.beta = beta;
+  for (int k = 0; k < g.nk; ++k) {
+    f.half.A = D + (long long)k * g.N * g.ldN;
+    f.half.B = f.out.A = X + (long long)k * g.Nn;
+    f.half.C = T1;
+    f.out.B = T1;
+    f.out.C = Sig + (long long)k * g.T * g.nn;
+    SOX_TRY(zgemm_f64(h, f.half, scratch, s));
+    SOX_TRY(zgemm_f64(h, f.out, scratch, s));
+  }
+  h->launches += 2 * g.nk;
+  return Status::ok();
+}
+
+// The static chain: tau points per chunk, bytes
+struct KStatTc {
+  int ct = 1;
+  size_t bytes = 0;
+};
+KStatTc kstat_plan(sox_handle h, const KTc &g, bool two) {
+  const long long ldNn = g.Nn + (g.Nn & 1);
+  size_t fixed = tables_bytes(g) + mixed_tc_bytes(g) * (two ? 2 : 1) + mixed_tc_scratch(g);
+  fixed += csplit_bytes((int)g.nk2, (int)(2 * g.Nn), g.n) + (size_t)g.n * csplit_bytes((int)g.nk2, 2 * g.N, g.n);
+  auto per = [&](long long c) {
+    size_t b = 2 * aligned_bytes((size_t)c * g.nk * g.Nn, 16);
+    b += csplit_bytes((int)(c * g.nk), 2 * g.N, g.n) + csplit_bytes(g.nk, (int)(c * g.N), g.n) +
+         csplit_bytes(g.nk, (int)(c * g.n), g.n);
+    b += aligned_bytes((size_t)c * g.nk2 * g.n * ldNn, 8) + csplit_bytes((int)(c * g.nk2), g.N, g.n);
+    b += 2 * aligned_bytes((size_t)c * g.nk2 * g.N * g.ldN, 8);
+    b += aligned_bytes((size_t)c * g.nk * g.N * g.ldN, 16) + aligned_bytes((size_t)c * g.Nn, 16);
+    return b + aligned_bytes((size_t)c * g.nk2, 4);
+  };
+  const size_t budget = chunk_budget(h, size_t(24) << 30), one = per(1);
+  KStatTc p;
+  long long c = budget > fixed ? (long long)((budget - fixed) / one) : 1;
+  p.ct = (int)std::max<long long>(1, std::min<long long>(c, g.T));
+  p.bytes = fixed + per(p.ct) + k_gemms_bytes(g, p.ct) + (1 << 20);
+  return p;
 }
 
 }  // namespace
 
-size_t kpoint_tc_bytes(sox_handle, const sox_problem *p, bool two) {
-  const KTc g = ktc_geom(p);
-  size_t b = tables_bytes(g) + mixed_tc_bytes(g) * (two ? 2 : 1) + mixed_tc_scratch(g);
-  const long long ldNn = g.Nn + (g.Nn & 1);
-  b += csplit_bytes((int)g.nk2, (int)(2 * g.Nn), g.n) + (size_t)g.n * csplit_bytes((int)g.nk2, 2 * g.N, g.n);
-  b += 2 * aligned_bytes(g.nk * g.Nn, 16);
-  b += csplit_bytes(g.nk, 2 * g.N, g.n) + csplit_bytes(g.nk, g.N, g.n) + csplit_bytes(g.nk, g.n, g.n);
-  b += aligned_bytes(g.nk2 * g.n * ldNn, 8) + csplit_bytes((int)g.nk2, g.N, g.n);
-  b += 2 * aligned_bytes(g.nk2 * g.N * g.ldN, 8);
-  b += aligned_bytes((size_t)g.nk * g.N * g.ldN, 16) + aligned_bytes(g.nk * g.Nn, 16);
-  return b + (1 << 20);
-}
+size_t kpoint_tc_bytes(sox_handle h, const sox_problem *p, bool two) { return kstat_plan(h, ktc_geom(p), two).bytes; }
 
 Status kpoint_sigma_tc(sox_handle h, const sox_problem *pr, const double *Gd, const double *Xd, const double *U1d,
                        const double *U2d, double *Sd, Arena &ar, cudaStream_t s) {
@@ -776,6 +847,7 @@ Status kpoint_sigma_tc(sox_handle h, const sox_problem *pr, const double *Gd, co
   v_range(h, pr->n, &v_lo, &v_hi);
   const KTc g = ktc_geom(pr);
   const bool two = (U1d != U2d);
+  const int ct = kstat_plan(h, g, two).ct;
   const z *G = reinterpret_cast<const z *>(Gd);
   const z *X = reinterpret_cast<const z *>(Xd);
   const z *U1 = reinterpret_cast<const z *>(U1d);
@@ -790,68 +862,75 @@ Status kpoint_sigma_tc(sox_handle h, const sox_problem *pr, const double *Gd, co
   CSplit M1s = csplit_take(ar, (int)g.nk2, (int)(2 * g.Nn), g.n);
   std::vector<CSplit> M2s(g.n);
   for (int v = 0; v < g.n; ++v) M2s[v] = csplit_take(ar, (int)g.nk2, 2 * g.N, g.n);
-  z *GR = ar.take<z>(g.nk * g.Nn), *GWt = ar.take<z>(g.nk * g.Nn);
-  CSplit GRs = csplit_take(ar, g.nk, 2 * g.N, g.n), GWts = csplit_take(ar, g.nk, g.N, g.n);
-  CSplit Gms = csplit_take(ar, g.nk, g.n, g.n);
-  float *Aall = ar.take<float>(2 * g.nk2 * g.n * ldNn);
-  CSplit As = csplit_take(ar, (int)g.nk2, g.N, g.n);
-  float *Ball = ar.take<float>(2 * g.nk2 * g.N * g.ldN), *Call = ar.take<float>(2 * g.nk2 * g.N * g.ldN);
-  z *D = ar.take<z>((size_t)g.nk * g.N * g.ldN), *T1 = ar.take<z>(g.nk * g.Nn);
-  if (!T1 || !As.hi || !M1s.hi || !M2s.back().hi || !Gms.hi)
+  // Every tau point of a chunk goes through one launch per step: (tau, P) rows where the other
+  // operand does not depend on tau, (pair, tau) batches where it does.  (2 x 1 x 1, N = 300, 60
+  // times: a launch per tau point, each of about ten blocks, took 370 ms, 313 of them in the
+  // FP64 products.)
+  z *GR = ar.take<z>((size_t)ct * g.nk * g.Nn), *GWt = ar.take<z>((size_t)ct * g.nk * g.Nn);
+  const CSplit GRs_all = csplit_take(ar, ct * g.nk, 2 * g.N, g.n), GWts_all = csplit_take(ar, g.nk, ct * g.N, g.n);
+  const CSplit Gms_all = csplit_take(ar, g.nk, ct * g.n, g.n);
+  float *Aall = ar.take<float>(2 * (size_t)ct * g.nk2 * g.n * ldNn);
+  const CSplit As_all = csplit_take(ar, (int)(ct * g.nk2), g.N, g.n);
+  float *Ball = ar.take<float>(2 * (size_t)ct * g.nk2 * g.N * g.ldN);
+  float *Call = ar.take<float>(2 * (size_t)ct * g.nk2 * g.N * g.ldN);
+  z *D = ar.take<z>((size_t)ct * g.nk * g.N * g.ldN), *T1 = ar.take<z>((size_t)ct * g.Nn);
+  int *idxR = ar.take<int>((size_t)ct * g.nk2);
+  if (!idxR || !As_all.hi || !M1s.hi || !M2s.back().hi || !Gms_all.hi || !GRs_all.hi || !GWts_all.hi)
     return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
   ProfScope ps(h, "kpoint_tc", s, 0);
-  SOX_CUDA_TRY(cudaMemsetAsync(Ball, 0, 8 * g.nk2 * g.N * g.ldN, s));   // pad columns stay zero
-  SOX_CUDA_TRY(cudaMemsetAsync(Call, 0, 8 * g.nk2 * g.N * g.ldN, s));
+  SOX_CUDA_TRY(cudaMemsetAsync(Ball, 0, 8 * (size_t)ct * g.nk2 * g.N * g.ldN, s));   // pad columns stay zero
+  SOX_CUDA_TRY(cudaMemsetAsync(Call, 0, 8 * (size_t)ct * g.nk2 * g.N * g.ldN, s));
   SOX_TRY(mixed_tc(h, X, U1, tb, g, ar, M1, s));
   if (two) SOX_TRY(mixed_tc(h, X, U2, tb, g, ar, M2, s));
   split_m1_tc(M1, g, M1s, s);
   split_m2_tc(M2, g, M2s, s);
   long long launches = 1 + g.n;
   const double inv_nk2 = 1.0 / (double)g.nk2;
+  int idx_cc = 0;   // the chunk length that idxR is made for
   for (int sp = 0; sp < g.S; ++sp) {
     const z *Gs = G + (long long)sp * g.nk * g.T * g.nn;
-    for (int j = 0; j < g.T; ++j) {
-      {  // FP64 projections at tau_j for every k
-        ZGemm p = zg();
-        p.M = g.N; p.Nc = g.n; p.K = g.n; p.batch = g.nk;
-        p.A = X; p.sA = g.Nn; p.ai = g.n; p.ak = 1;
-        p.B = Gs + (long long)j * g.nn; p.sB = (long long)g.T * g.nn; p.bk = g.n; p.bj = 1;
-        p.C = GR; p.sC = g.Nn; p.ci = g.n; p.cj = 1;
-        zgemm(p, s);
-        ZGemm w = p;
-        w.conjA = 1; w.bk = 1; w.bj = g.n; w.C = GWt;
-        zgemm(w, s);
+    for (int t0 = 0; t0 < g.T; t0 += ct) {
+      const int cc = std::min(ct, g.T - t0);
+      if (cc != idx_cc) {   // G_Rq of batch (pair, il): k_u of the pair at tau il
+        k_pair_tau_index<<<(unsigned)((cc * g.nk2 + 255) / 256), 256, 0, s>>>(tb.ku, g.nk2, cc, idxR);
+        ++launches;
+        idx_cc = cc;
       }
-      csplit_b(GR, false, g.Nn, g.n, 0, 0, 1, g.nk, g.N, g.n, false, false, GRs, s);
-      csplit_a(GWt, false, g.Nn, g.n, 0, 0, 1, g.nk, g.N, g.n, GWts, s);
-      // A rows v of G(-tau_j)^T: element (v, s) = G^k(tau_{T-1-j})[s][v]; the sign goes into alpha
-      csplit_a(Gs + (long long)(g.T - 1 - j) * g.nn, false, (long long)g.T * g.nn, 1, 0, 0, g.n, g.nk, g.n, g.n, Gms,
-               s);
-      // A^{q1,ks}[v][(P,q)] = -sum_s G^{ks}(tau_{T-1-j})[s][v] M1[(P,q)][s]   ((P,q) contiguous per v)
-      SOX_TRY(cgemm_tc(h, Gms, M1s, (int)g.nk2, tb.kk, nullptr, -1.f, Aall, 2 * ldNn, 2LL * g.n * ldNn, s));
-      SOX_CUDA_TRY(cudaMemsetAsync(D, 0, 16 * (size_t)g.nk * g.N * g.ldN, s));
-      launches += 5;
-      for (int v = v_lo; v < v_hi; ++v) {   // the handle's v range (sox_set_v_range)
-        csplit_a(reinterpret_cast<const float2 *>(Aall) + (long long)v * ldNn, true, g.n * ldNn, g.n, 0, 0, 1,
-                 (int)g.nk2, g.N, g.n, As, s);
+      CSplit GRs = GRs_all, GWts = GWts_all, Gms = Gms_all, As = As_all;
+      GRs.batch = cc * g.nk;
+      GWts.rows = cc * g.N;
+      Gms.rows = cc * g.n;
+      As.batch = (int)(cc * g.nk2);
+      SOX_TRY(project_k(h, Gs, X, g, t0, cc, GR, GWt, ar, s));   // FP64
+      csplit_b(GR, false, g.Nn, g.n, 0, 0, 1, cc * g.nk, g.N, g.n, false, false, GRs, s);
+      csplit_a(GWt, false, (long long)cc * g.Nn, g.n, 0, 0, 1, g.nk, cc * g.N, g.n, GWts, s);
+      // A rows (il, v) of G(-tau_j)^T: element s = G^k(tau_{T-1-j})[s][v]; the sign goes into alpha
+      csplit_a(Gs + (long long)(g.T - 1 - t0) * g.nn, false, (long long)g.T * g.nn, -g.nn, 1, g.n, g.n, g.nk, cc * g.n,
+               g.n, Gms, s);
+      // A^{q1,ks}[(il,v)][(P,q)] = -sum_s G^{ks}(tau_{T-1-j})[s][v] M1[(P,q)][s]
+      SOX_TRY(cgemm_tc(h, Gms, M1s, (int)g.nk2, tb.kk, nullptr, -1.f, Aall, 2 * ldNn, 2LL * cc * g.n * ldNn, s));
+      SOX_CUDA_TRY(cudaMemsetAsync(D, 0, 16 * (size_t)cc * g.nk * g.N * g.ldN, s));
+      launches += 3;
+      for (int v = v_lo; v < v_hi; ++v) {
+        csplit_a(reinterpret_cast<const float2 *>(Aall) + (long long)v * ldNn, true, (long long)cc * g.n * ldNn,
+                 g.n * ldNn, g.n, g.N, 1, (int)g.nk2, cc * g.N, g.n, As, s);
         {
           ProfScope pb(h, "kpoint_bc", s, 0);
-          // B^{q1,ks}_v[P][R] = sum_q A[v][P][q] GR^{ks-q1}[R][q]
-          SOX_TRY(cgemm_tc(h, As, GRs, (int)g.nk2, nullptr, tb.ku, 1.f, Ball, 2LL * g.ldN, 2LL * g.N * g.ldN, s));
-          // C^{q2,kw}_v[P][R] = sum_w GWt^{kw}[P][w] M2^{q2,kw}[R][v][w]
-          SOX_TRY(
-              cgemm_tc(h, GWts, M2s[v], (int)g.nk2, tb.kk, nullptr, 1.f, Call, 2LL * g.ldN, 2LL * g.N * g.ldN, s));
+          // B^{q1,ks}_v(tau)[P][R] = sum_q A[v][P][q] GR^{ks-q1}(tau)[R][q]
+          SOX_TRY(cgemm_tc(h, As, GRs, (int)(cc * g.nk2), nullptr, idxR, 1.f, Ball, 2LL * g.ldN, 2LL * g.N * g.ldN, s));
+          // C^{q2,kw}_v(tau)[P][R] = sum_w GWt^{kw}(tau)[P][w] M2^{q2,kw}[R][v][w]
+          SOX_TRY(cgemm_tc(h, GWts, M2s[v], (int)g.nk2, tb.kk, nullptr, 1.f, Call, 2LL * g.ldN, 2LL * cc * g.N * g.ldN,
+                           s));
         }
         {
           ProfScope pd(h, "kpoint_D", s, 0);
-          SOX_TRY(kpoint_D_f32(Ball, Call, (long long)g.N * g.ldN, 0, tb.add, tb.sub, pr->nk, (long long)g.N * g.ldN,
-                               1, 0, 0, reinterpret_cast<double *>(D), s));
+          SOX_TRY(kpoint_D_f32(Ball, Call, (long long)cc * g.N * g.ldN, (long long)g.N * g.ldN, tb.add, tb.sub, pr->nk,
+                               (long long)g.N * g.ldN, cc, 0, (long long)g.nk * g.N * g.ldN,
+                               reinterpret_cast<double *>(D), s));
         }
         launches += 2;
       }
-      backproject_k(D, X, g, T1, Sig + ((long long)sp * g.nk * g.T + j) * g.nn, (long long)g.T * g.nn, -inv_nk2, 0.0,
-                    s);
-      launches += 4;
+      SOX_TRY(backproject_k(h, D, X, g, cc, T1, Sig + ((long long)sp * g.nk * g.T + t0) * g.nn, -inv_nk2, 0.0, ar, s));
     }
   }
   h->launches += launches;
@@ -890,7 +969,8 @@ KDynTc kdyn_geom(sox_handle h, const sox_problem *p, int nO, size_t *fixed_out, 
   f += aligned_bytes((size_t)g.nk2 * g.T * d.ldNn, 8);                          // A(tau), all pairs
   f += aligned_bytes((size_t)g.T * g.nk * g.N * g.ldN, 16);                     // D for every tau
   f += aligned_bytes(g.nk * g.Nn, 16) + (1 << 20);
-  const size_t per_t = csplit_bytes((int)g.nk2, g.N, g.n) + 2 * aligned_bytes(g.nk2 * g.N * g.ldN, 8);
+  const size_t per_t = csplit_bytes((int)g.nk2, g.N, g.n) + 2 * aligned_bytes(g.nk2 * g.N * g.ldN, 8) +
+                       aligned_bytes(g.Nn, 16);
   const size_t budget = chunk_budget(h, size_t(24) << 30);
   long long ct = budget > f ? (long long)((budget - f) / per_t) : 1;
   d.ct = (int)std::max<long long>(1, std::min<long long>(ct, g.T));
@@ -904,7 +984,7 @@ KDynTc kdyn_geom(sox_handle h, const sox_problem *p, int nO, size_t *fixed_out, 
 size_t kpoint_dynamic_tc_bytes(sox_handle h, const sox_problem *p, int n_omega) {
   size_t f = 0, per_t = 0;
   const KDynTc d = kdyn_geom(h, p, n_omega, &f, &per_t);
-  return f + per_t * d.ct + (1 << 20);
+  return f + per_t * d.ct + std::max(k_gemms_bytes(d.g, d.ct), k_gemms_bytes(d.g, d.g.T)) + (1 << 20);
 }
 
 Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const double *Gd, const double *Xd,
@@ -937,7 +1017,7 @@ Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const
   float *Aw = ar.take<float>(2 * (size_t)nk * nO * N * d.upad);
   CSplit Aws = csplit_take(ar, nk, (int)(2 * g.Nn), nO);
   float *Adyn = ar.take<float>(2 * (size_t)g.nk2 * T * d.ldNn);
-  z *Dall = ar.take<z>((size_t)T * nk * N * g.ldN), *T1 = ar.take<z>(g.nk * g.Nn);
+  z *Dall = ar.take<z>((size_t)T * nk * N * g.ldN), *T1 = ar.take<z>((size_t)d.ct * g.Nn);
   CSplit As = csplit_take(ar, (int)g.nk2, d.ct * N, n);
   float *Ball = ar.take<float>(2 * (size_t)g.nk2 * d.ct * N * g.ldN);
   float *Call = ar.take<float>(2 * (size_t)g.nk2 * d.ct * N * g.ldN);
@@ -964,18 +1044,7 @@ Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const
   const double inv_nk2 = 1.0 / (double)g.nk2;
   for (int sp = 0; sp < g.S; ++sp) {
     const z *Gs = G + (long long)sp * nk * T * g.nn;
-    for (int k = 0; k < nk; ++k) {  // GWt[k][j][Q][u], GR[k][j][Q][v] for every tau, FP64
-      ZGemm p = zg();
-      p.M = N; p.Nc = n; p.K = n; p.batch = T;
-      p.A = X + (long long)k * g.Nn; p.ai = n; p.ak = 1; p.conjA = 1;
-      p.B = Gs + (long long)k * T * g.nn; p.sB = g.nn; p.bk = 1; p.bj = n;
-      p.C = GWt + (long long)k * T * g.Nn; p.sC = g.Nn; p.ci = n; p.cj = 1;
-      zgemm(p, s);
-      ZGemm r = p;
-      r.conjA = 0; r.bk = n; r.bj = 1; r.C = GR + (long long)k * T * g.Nn;
-      zgemm(r, s);
-      launches += 2;
-    }
+    SOX_TRY(project_k(h, Gs, X, g, 0, T, GR, GWt, ar, s));   // [k][j][Q][u] for every tau, FP64
     // rows (tau_i, P) of GWt^k, K = w
     csplit_a(GWt, false, (long long)T * g.Nn, n, 0, 0, 1, nk, T * N, n, GWts, s);
     SOX_CUDA_TRY(cudaMemsetAsync(Dall, 0, 16 * (size_t)T * nk * N * g.ldN, s));
@@ -1025,10 +1094,10 @@ Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const
         launches += 2;
       }
     }
-    for (int i = 0; i < T; ++i) {
-      backproject_k(Dall + (size_t)i * nk * N * g.ldN, X, g, T1, Sig + ((long long)sp * nk * T + i) * g.nn,
-                    (long long)T * g.nn, -inv_nk2, 1.0, s);
-      launches += 2;
+    for (int t0 = 0; t0 < T; t0 += d.ct) {
+      const int cc = std::min(d.ct, T - t0);
+      SOX_TRY(backproject_k(h, Dall + (size_t)t0 * nk * N * g.ldN, X, g, cc, T1, Sig + ((long long)sp * nk * T + t0) * g.nn,
+                            -inv_nk2, 1.0, ar, s));
     }
   }
   h->launches += launches;

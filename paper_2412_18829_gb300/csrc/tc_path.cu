@@ -30,7 +30,7 @@ struct Geometry {
   int RG;   // rows allocated for G(-tau)^T (>= 128)
   int Bc;   // (spin, tau) batches per chunk
   size_t fixed_bytes, per_b_bytes, scratch_bytes;
-  bool slices;   // the FP64 products run as digit slices on the tensor cores
+  bool slices_p, slices_s;   // projections, final sum as digit slices on the tensor cores
   // the chunk buffers of Bc batches; the mixed tensor's scratch lies in them before the first chunk
   size_t chunk_bytes(int bc) const { return std::max(per_b_bytes * (size_t)bc, scratch_bytes); }
 };
@@ -72,30 +72,32 @@ Geometry geometry(sox_handle h, int n, int N, int T, int S, bool two) {
   long long c = (long long)(chunk_budget(h, kChunkBudget) / std::max<size_t>(g.per_b_bytes, 1));
   c = std::max<long long>(1, std::min<long long>(c, (long long)T * S));
   g.Bc = (int)c;
-  g.slices = slices_pay(N, n, n, (long long)T * S);
+  g.slices_p = slices_pay(N, n, n, (long long)T * S);
+  g.slices_s = slices_pay(n, n, N, (long long)T * S);
   return g;
 }
 
 // ---- the FP64 products of the chain (projections, final sum), on the FP64 pipe or as slices
 struct F64Ops {
-  bool on = false;
+  bool on_p = false, on_s = false;
   SliceOp X;                  // rows R, K = orbitals
   std::vector<SliceOp> XT;    // rows t, K = R in blocks of kSliceMaxK
 };
 
 F64Ops f64_take(Arena &ar, const Geometry &g) {
   F64Ops f;
-  f.on = g.slices;
+  f.on_p = g.slices_p;
+  f.on_s = g.slices_s;
   f.X = slice_take(ar, 1, g.N, g.n);
   for (int k0 = 0; k0 < g.N; k0 += kSliceMaxK) f.XT.push_back(slice_take(ar, 1, g.n, std::min(kSliceMaxK, g.N - k0)));
   return f;
 }
 
 void f64_slice_x(sox_handle h, F64Ops &f, const double *X, int n, cudaStream_t s) {
-  if (!f.on) return;
-  slice_rows(X, false, 0, n, 1, 1, f.X, s);
-  for (size_t i = 0; i < f.XT.size(); ++i) slice_rows(X + (long long)i * kSliceMaxK * n, false, 0, 1, n, 1, f.XT[i], s);
-  h->launches += 1 + (long long)f.XT.size();
+  if (f.on_p) slice_rows(X, false, 0, n, 1, 1, f.X, s);
+  for (size_t i = 0; f.on_s && i < f.XT.size(); ++i)
+    slice_rows(X + (long long)i * kSliceMaxK * n, false, 0, 1, n, 1, f.XT[i], s);
+  h->launches += (f.on_p ? 1 : 0) + (f.on_s ? (long long)f.XT.size() : 0);
 }
 
 // FP64 projections G_Rq = X G, G_wP^T = X G^T of bc batches.  For a symmetric G(tau) (real
@@ -103,7 +105,7 @@ void f64_slice_x(sox_handle h, F64Ops &f, const double *X, int n, cudaStream_t s
 Status project_f64(sox_handle h, const F64Ops &f, const double *Gc, const double *X, int N, int n, int bc,
                    const int *symf, double *GR64, double *GW64, Arena scratch, cudaStream_t s) {
   const long long nn = (long long)n * n;
-  if (f.on) {
+  if (f.on_p) {
     SliceOp Gq = slice_take(scratch, bc, n, n), Gw = slice_take(scratch, bc, n, n);
     if (!Gq.p || !Gw.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
     slice_rows(Gc, false, nn, 1, n, bc, Gq, s);
@@ -135,7 +137,7 @@ Status project_f64(sox_handle h, const F64Ops &f, const double *Gc, const double
 Status final_sum_f64(sox_handle h, const F64Ops &f, const double *X, const float *Tm, int N, int n, int bc,
                      double *Sigma, const int *sym, Arena scratch, cudaStream_t s) {
   const long long nn = (long long)n * n;
-  if (!f.on) {
+  if (!f.on_s) {
     launch_backproject_sigma(X, Tm, N, n, bc, Sigma, nn, s, sym);
     return Status::ok();
   }
