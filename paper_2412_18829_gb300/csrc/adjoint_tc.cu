@@ -27,6 +27,7 @@
 
 #include "adjoint.h"
 #include "ctc.h"
+#include "f64_slices.h"
 #include "gemm_mn.h"
 #include "smem_attr.h"
 #include "tc_common.cuh"
@@ -562,7 +563,10 @@ AdjGeom adj_geom(sox_handle h, int n, int N, int T, int S) {
 
 size_t adjoint_tc_bytes(sox_handle h, int n, int N, int T, int S) {
   const AdjGeom g = adj_geom(h, n, N, T, S);
-  return fixed_bytes(g) + std::max(per_tau_bytes(g) * g.Bc, end_bytes(g)) + (1 << 20);
+  GemmF64 a;   // the FP64 projections (their digits follow the chunk's buffers)
+  a.M = N; a.Nc = n; a.K = n; a.batch = T;
+  a.sB = (long long)n * n;
+  return fixed_bytes(g) + std::max(per_tau_bytes(g) * g.Bc, end_bytes(g)) + gemm_f64_bytes(a) + (1 << 20);
 }
 
 Status phi_adjoint_xv_tc(sox_handle h, int n, int N, int T, int S, const double *G, const double *X, const double *V,
@@ -744,10 +748,10 @@ Status phi_adjoint_xv_tc(sox_handle h, int n, int N, int T, int S, const double 
       a.A = X; a.ai = n; a.ak = 1;
       a.B = Gs; a.sB = nn; a.bk = n; a.bj = 1;
       a.C = GRall; a.sC = Nn; a.ci = n; a.cj = 1;
-      launch_gemm_f64(a, s);
+      SOX_TRY(gemm_f64(h, a, ar, s));
       GemmF64 b = a;
       b.bk = 1; b.bj = n; b.C = GWall; b.skip = symf;
-      launch_gemm_f64(b, s);
+      SOX_TRY(gemm_f64(h, b, ar, s));
       k_copy_flagged<<<grid1((long long)T * Nn), 256, 0, s>>>(GRall, GWall, Nn, T, symf);
       launches += 4;
     }
@@ -811,6 +815,7 @@ Status phi_adjoint_xv_tc(sox_handle h, int n, int N, int T, int S, const double 
         a1.a.mn_major = 1; a1.a.zb = 1;   // pairs [R][P]: rows P run along the MN side
         a1.b.mn_major = 1; a1.b.zb = 1; a1.b.zdiv = nv;
         a1.alpha = &sc->f[kFacAbar];
+        a1.absmax = &sc->mx[1];
         a1.spin_limit = limit; a1.status = h->d_status;
         SOX_CUDA_TRY(launch_gemm_mn(mi, a1, plan_gemm_mn(a1, sms, 1), s));
         // (ii) GRbar (per b; K = (v, P))
@@ -842,7 +847,6 @@ Status phi_adjoint_xv_tc(sox_handle h, int n, int N, int T, int S, const double 
         SOX_CUDA_TRY(launch_gemm_mn(miv, a4, plan_gemm_mn(a4, sms, 64), s));
       }
       // (v) U1bar += Abar (x) G(-tau): Abar split once per chunk, then K = (b, v)
-      launch_absmax(Abar, true, g.np4, N, (long long)N * g.np4, bc * nv, 1, n, &sc->mx[1], s);
       launch_split_tensor(Abar, true, g.np4, N, (long long)N * g.np4, bc * nv, 1, n, n, g.abar_pitch, 1.f, &sc->mx[1],
                           nullptr, Abh, Abl, &sc->sc[kScAbar], s);
       k_u1bar_factor<<<1, 1, 0, s>>>(sc);
@@ -864,21 +868,22 @@ Status phi_adjoint_xv_tc(sox_handle h, int n, int N, int T, int S, const double 
       launch_split_tensor(Ebar, true, g.ldN, N, (long long)N * g.ldN, bc, 1, N, g.ldN8, (long long)N * g.ldN8, 1.f,
                           &sc->mx[7], nullptr, Ebh, Ebl, &sc->sc[kScEbar], s);
       k_ex_factor<<<1, 1, 0, s>>>(sc);
+      SOX_CUDA_TRY(cudaMemsetAsync(&sc->mx[kMxXa], 0, 2 * sizeof(float), s));
       {
         GemmMnArgs e1;
         e1.M = N; e1.Ncols = n; e1.batch = bc; e1.kc_inner = kcN; e1.nk_outer = 1;
         e1.a.mn_major = 0; e1.a.zb = 1;
         e1.b.mn_major = 1;
         e1.alpha = &sc->f[kFacEX];
+        e1.absmax = &sc->mx[kMxXa];
         e1.spin_limit = limit; e1.status = h->d_status;
         SOX_CUDA_TRY(launch_gemm_mn(mm1, e1, plan_gemm_mn(e1, sms, 1), s));
         GemmMnArgs e2 = e1;
         e2.a.mn_major = 1;
         SOX_CUDA_TRY(launch_gemm_mn(mm2, e2, plan_gemm_mn(e2, sms, 1), s));
       }
-      SOX_CUDA_TRY(cudaMemsetAsync(&sc->mx[kMxXa], 0, 2 * sizeof(float), s));
       const float *xa[4] = {GRbf, GWbf, m1f, m2f};
-      for (int t = 0; t < 4; ++t)
+      for (int t = 0; t < 2; ++t)   // (m1 and m2: from their products)
         launch_absmax(xa[t], true, g.np4, N, (long long)N * g.np4, bc, 1, n, &sc->mx[kMxXa], s);
       for (int t = 0; t < 4; ++t)
         launch_split_tensor(xa[t], true, g.np4, N, (long long)N * g.np4, bc, 1, n, g.np8, 4LL * N * g.np8, 1.f,

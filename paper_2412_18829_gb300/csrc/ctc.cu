@@ -36,10 +36,11 @@ __device__ __forceinline__ void split_pair(float x, float s, __half &h, __half &
   l = __float2half_rn(xs - __half2float(h));
 }
 __device__ __forceinline__ void split_pair(double x, float s, __half &h, __half &l) {
-  const double xs = x * (double)s;
-  h = __float2half_rn((float)xs);
-  l = __float2half_rn((float)(xs - (double)__half2float(h)));
+  tc::split_f16_f64(x, tc::log2_of(s), h, l);
 }
+// |x| in FP32
+__device__ __forceinline__ float abs_f32(double x) { return tc::f32_abs(x); }
+__device__ __forceinline__ float abs_f32(float x) { return fabsf(x); }
 // rounding to nearest is symmetric, so the pair of -x is the negated pair of x: a B row's
 // four signed copies of (b_r, b_i) take two splits
 __device__ __forceinline__ __half neg_if(bool n, __half v) { return n ? __hneg(v) : v; }
@@ -121,7 +122,7 @@ __global__ void k_csplit_a(const T *src, RowMap m, int batch, int rows, int K, i
   if (live)
     for (int k = gl; k < K; k += lpr) {
       const T v = ld_c(x + k * m.sk);
-      mx = fmaxf(mx, fmaxf((float)fabs(v.x), (float)fabs(v.y)));
+      mx = fmaxf(mx, fmaxf(abs_f32(v.x), abs_f32(v.y)));
     }
   mx = group_max(mx, lpr);
   if (!live) return;
@@ -154,7 +155,7 @@ __global__ void k_csplit_b(const T *src, RowMap m, int batch, int cols, int K, i
   if (live)
     for (int k = gl; k < K; k += lpr) {
       const T v = ld_c(x + k * m.sk);
-      mx = fmaxf(mx, fmaxf((float)fabs(v.x), (float)fabs(v.y)));
+      mx = fmaxf(mx, fmaxf(abs_f32(v.x), abs_f32(v.y)));
     }
   mx = group_max(mx, lpr);
   if (!live) return;
@@ -242,7 +243,7 @@ __global__ void k_csplit_pairs(const double2 *X, const int *sub, int nk, int N, 
   float mx = 0.f;
   for (int Q = lane; Q < N; Q += 32) {
     const double2 v = y(Q);
-    mx = fmaxf(mx, fmaxf((float)fabs(v.x), (float)fabs(v.y)));
+    mx = fmaxf(mx, fmaxf(abs_f32(v.x), abs_f32(v.y)));
   }
   mx = cwarp_max(mx);
   const float s = tc::pow2_floor_inv(mx);
@@ -521,7 +522,7 @@ cudaError_t launch_dfft(const float2 *B, const float2 *C, long long sP, long lon
 // warp per row finds its scale and writes the FP16 pairs.  kind 0: A rows, 1: B rows.
 constexpr int kRB = 32;
 template <class T>
-__global__ void __launch_bounds__(256) k_csplit_t(const T *src, RowMap m, int batch, int rows, int K, int Kp2, int kind,
+__global__ void __launch_bounds__(1024) k_csplit_t(const T *src, RowMap m, int batch, int rows, int K, int Kp2, int kind,
                                                  float sa, float sbc, __half *hi, __half *lo, float *unscale) {
   extern __shared__ __align__(16) unsigned char tile_raw[];
   T *tile = reinterpret_cast<T *>(tile_raw);   // [K][kRB + 1]
@@ -536,13 +537,13 @@ __global__ void __launch_bounds__(256) k_csplit_t(const T *src, RowMap m, int ba
   }
   __syncthreads();
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  for (int rr = warp; rr < kRB; rr += 8) {
+  for (int rr = warp; rr < kRB; rr += blockDim.x / 32) {
     const int r = r0 + rr;
     if (r >= rows) break;
     float mx = 0.f;
     for (int k = lane; k < K; k += 32) {
       const T v = tile[k * (kRB + 1) + rr];
-      mx = fmaxf(mx, fmaxf((float)fabs(v.x), (float)fabs(v.y)));
+      mx = fmaxf(mx, fmaxf(abs_f32(v.x), abs_f32(v.y)));
     }
     mx = cwarp_max(mx);
     const float s = tc::pow2_floor_inv(mx);
@@ -604,7 +605,8 @@ bool launch_split_t(const T *src, const RowMap &m, int batch, int rows, int K, i
     return false;
   }
   const long long blocks = (long long)batch * ((rows + kRB - 1) / kRB);
-  k_csplit_t<T><<<(unsigned)blocks, 256, smem, s>>>(src, m, batch, rows, K, Kp2, kind, sa, sbc, hi, lo, unscale);
+  // a long K leaves few blocks on an SM (the tile holds it all): then a warp per row
+  k_csplit_t<T><<<(unsigned)blocks, K >= 128 ? 1024 : 256, smem, s>>>(src, m, batch, rows, K, Kp2, kind, sa, sbc, hi, lo, unscale);
   return true;
 }
 
@@ -642,7 +644,7 @@ __global__ void k_rsplit(const T *src, const float *mul, RowMap m, int batch, in
   auto val = [&](int k) -> T { return mu ? ld_r(x + k * m.sk) * static_cast<T>(mu[k * m.sk]) : ld_r(x + k * m.sk); };
   float mx = 0.f;
   if (live)
-    for (int k = gl; k < K; k += lpr) mx = fmaxf(mx, (float)fabs(val(k)));
+    for (int k = gl; k < K; k += lpr) mx = fmaxf(mx, abs_f32(val(k)));
   mx = group_max(mx, lpr);
   if (!live) return;
   const float s = tc::pow2_floor_inv(mx);
@@ -687,7 +689,7 @@ __global__ void __launch_bounds__(256) k_rsplit_t(const T *src, const float *mul
     }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < 8; ++j) my = fmaxf(my, fabsf((float)tile[part * 8 + j][rr]));
+    for (int j = 0; j < 8; ++j) my = fmaxf(my, abs_f32(tile[part * 8 + j][rr]));
   }
   // row maxima: the 8 threads of a row are consecutive lanes
   for (int o = 4; o > 0; o >>= 1) my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, o));
@@ -772,7 +774,9 @@ int blocks_for(long long warps) { return (int)std::max<long long>(1, (warps * 32
 
 }  // namespace
 
-int csplit_kp2(int K) { return ((2 * K + 63) / 64) * 64; }
+// rows of 2K values, a multiple of 8 (16 bytes, the TMA's row pitch; the copies fill the rest of
+// a 64-wide chunk with zeros)
+int csplit_kp2(int K) { return (2 * K + 7) & ~7; }
 
 size_t csplit_bytes(int batch, int rows_real, int K) {
   const size_t e = (size_t)batch * rows_real * csplit_kp2(K);
@@ -872,7 +876,8 @@ Status cgemm_tc(sox_handle h, const CSplit &A, const CSplit &B, int batch, const
     GemmTcArgs ga;
     ga.M = A.rows;
     ga.Ncols = B.rows;
-    ga.Kp = kw;
+    ga.Kp = (kw + 63) & ~63;
+    ga.K = kw;
     ga.batch = batch;
     ga.batchA_shared = (A.batch == 1);
     ga.batchB_shared = (B.batch == 1);

@@ -7,7 +7,7 @@
 
 namespace sox {
 
-// A split operand: `batch` blocks of `rows` real rows, each Kp2 = 64*ceil(2K/64) FP16
+// A split operand: `batch` blocks of `rows` real rows, each Kp2 = 8*ceil(2K/8) FP16
 // values (hi and lo), and one FP32 factor per real row that undoes its scale.
 struct CSplit {
   __half *hi = nullptr, *lo = nullptr;

@@ -17,7 +17,9 @@
 #include <algorithm>
 
 #include "dynamic.h"
+#include "f64_slices.h"
 #include "gemm_mn.h"
+#include "tc_common.cuh"
 #include "tc_kernels.h"
 
 namespace sox {
@@ -26,21 +28,50 @@ namespace {
 int rup(long long x, int m) { return (int)((x + m - 1) / m * m); }
 int grid1(long long total) { return (int)std::max<long long>(1, std::min<long long>((total + 255) / 256, 65535 * 8)); }
 
-// GG[j][Q][u] = GWt[j][Q][u] * (-GR[T-1-j][Q][v])
-__global__ void k_gg_tc(const double *GWt, const double *GR, int T, int N, int n, int v, double *GG) {
-  const long long Nn = (long long)N * n, total = Nn * T;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int j = (int)(e / Nn);
-    const long long r = e % Nn;
-    const int Q = (int)(r / n);
-    GG[e] = -GWt[e] * GR[(long long)(T - 1 - j) * Nn + (long long)Q * n + v];
+// mx[v] = max |GG| over (j, Q, u) with GG = -GWt[j][Q][u] GR[T-1-j][Q][v]: rounding is monotonic,
+// so the largest product of a row (j, Q) is that of its largest |GWt|.  One warp per (j, Q).
+__global__ void __launch_bounds__(256) k_gg_max(const double *GWt, const double *GR, int T, int N, int n, int stride,
+                                                float *mx) {
+  const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32;
+  const int lane = threadIdx.x % 32;
+  if (row >= (long long)T * N) return;
+  const int j = (int)(row / N), Q = (int)(row % N);
+  const double *w = GWt + row * n, *g = GR + ((long long)(T - 1 - j) * N + Q) * n;
+  unsigned long long m = 0ull;   // |x| as bits
+  for (int u = lane; u < n; u += 32) m = max(m, (unsigned long long)__double_as_longlong(w[u]) & 0x7fffffffffffffffull);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const double wm = __longlong_as_double((long long)m);
+  for (int v = lane; v < n; v += 32) {
+    const float p = tc::f32_abs(wm * g[v]);
+    if (p > 0.f) atomicMax(reinterpret_cast<unsigned int *>(mx + (long long)v * stride), __float_as_uint(p));
   }
 }
 
-// out = 1 / (a * b) for the scalars at a and b (device values)
-__global__ void k_inv_prod(const float *a, const float *b, float *out) {
-  *out = (float)(1.0 / ((double)*a * (double)*b));
+// The FP16 pairs of GG for one v, [j][(Q,u)] with rows of ld (the padding zero): formed and split
+// in one pass (GG itself never leaves the SM), scale as launch_split_tensor.  n = 120, N = 600,
+// 80 times: 36 us product + 20 us maximum + 63 us split before, 39 us here.
+__global__ void __launch_bounds__(256) k_gg_split(const double *GWt, const double *GR, int T, int N, int n, int v,
+                                                  long long ld, const float *mx, __half *hi, __half *lo,
+                                                  float *scale_out) {
+  const float s = tc::big_scale(*mx);
+  const int ks = tc::log2_of(s);
+  const long long Nn = (long long)N * n;
+  const int j = blockIdx.y, lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const double *w = GWt + j * Nn, *g = GR + (long long)(T - 1 - j) * Nn + v;
+  __half *h = hi + j * ld, *l = lo + j * ld;
+  for (int Q = blockIdx.x * 8 + warp; Q < N; Q += gridDim.x * 8) {   // a warp per Q
+    const double gq = g[(long long)Q * n];
+    const long long o = (long long)Q * n;
+    for (int u = lane; u < n; u += 32) {
+      __half a, b;
+      tc::split_f16_f64(-w[o + u] * gq, ks, a, b);
+      h[o + u] = a;
+      l[o + u] = b;
+    }
+  }
+  if (blockIdx.x == 0)
+    for (long long c = Nn + threadIdx.x; c < ld; c += 256) h[c] = l[c] = __float2half(0.f);
+  if (scale_out && blockIdx.x == 0 && j == 0 && threadIdx.x == 0) *scale_out = s;
 }
 
 // fill[i] = *src for i < count
@@ -54,12 +85,12 @@ __global__ void k_fill1(float *p, int count, float v) {
   if (i < count) p[i] = v;
 }
 
-// scalars of the chain: split scales (written by the splits) and GEMM factors
+// scalars of the chain: split scales (written by the splits) and maxima
 struct DynScalars {
-  float mx[8];     // atomicMax targets: Wd, Tf, Ti, GG, GGw, Aw, A
-  float sc[8];     // scales of the same tensors
-  float f[4];      // factors of the FT, W_d and IFT GEMMs
+  float mx[8];     // atomicMax targets: Wd, Tf, Ti, -, -, -, A
+  float sc[8];     // scales of Wd, Tf, Ti, GG, GGw, Aw, A
 };
+constexpr int kMxV = 4;   // maxima per v: GG, GGw, Aw
 enum { kWd = 0, kTf, kTi, kGG, kGGw, kAw, kA };
 
 struct DynGeom {
@@ -98,14 +129,30 @@ size_t fixed_bytes(const DynGeom &g) {
              aligned_bytes(N, 4) + aligned_bytes(rows_f32_bytes(N, n), 1);            // U mixed, U2 split, X in FP32
   b += 2 * aligned_bytes((size_t)nO * N * g.Np, 2);                                   // W_d split
   b += 2 * aligned_bytes((size_t)2 * nO * g.KpT, 2) + 2 * aligned_bytes((size_t)T * g.KpO, 2);   // transforms
-  b += 3 * aligned_bytes((size_t)T * N * n, 8);                                       // GR, GWt, GG
+  b += 2 * aligned_bytes((size_t)T * N * n, 8) + aligned_bytes((size_t)kMxV * n, 4);  // GR, GWt, maxima per v
   b += 2 * aligned_bytes((size_t)T * g.NR * g.Kp, 2) + aligned_bytes((size_t)T * N, 4);   // GWt split
   b += 2 * aligned_bytes((size_t)T * g.NR * g.Kp, 2) + aligned_bytes((size_t)T * N, 4);   // X split per tau
   b += 2 * aligned_bytes((size_t)T * g.Nn8, 2);                                       // GG split
   b += aligned_bytes((size_t)2 * nO * g.Nn4, 4) + 2 * aligned_bytes((size_t)2 * nO * N * g.np8, 2);   // GGw
   b += aligned_bytes((size_t)2 * nO * N * g.np4, 4) + 2 * aligned_bytes((size_t)2 * nO * g.Nn8, 2);  // Aw
-  b += aligned_bytes(sizeof(DynScalars), 4) + 4 * aligned_bytes((size_t)std::max(T, N), 4) + (1 << 16);
+  b += aligned_bytes(sizeof(DynScalars), 4) + 2 * aligned_bytes((size_t)std::max(T, N), 4) + (1 << 16);
   return b;
+}
+
+// GR[j][R][q] = sum_u X[R][u] G_j[u][q] (and GWt with the strides of G exchanged)
+GemmF64 projection(int n, int N, int T) {
+  GemmF64 a;
+  a.M = N; a.Nc = n; a.K = n; a.batch = T;
+  a.ai = n; a.ak = 1;
+  a.sB = (long long)n * n; a.bk = n; a.bj = 1;
+  a.sC = (long long)N * n; a.ci = n; a.cj = 1;
+  return a;
+}
+
+// digits of the FP64 products
+size_t slice_scratch(const DynGeom &g) {
+  const int k = std::min(g.N, kSliceMaxK);
+  return std::max(gemm_f64_bytes(projection(g.n, g.N, g.T)), slice_bytes(1, g.n, k) + slice_bytes(g.tc, g.n, k));
 }
 
 size_t chunk_bytes(const DynGeom &g) {
@@ -122,7 +169,7 @@ size_t chunk_bytes(const DynGeom &g) {
 
 size_t dynamic_tc_bytes(sox_handle h, int n, int N, int T, int S, int n_omega) {
   const DynGeom g = geom(h, n, N, T, S, n_omega);
-  return fixed_bytes(g) + std::max(chunk_bytes(g), aligned_bytes(mixed_f32_scratch(N, n), 1)) + (1 << 20);
+  return fixed_bytes(g) + std::max(chunk_bytes(g), aligned_bytes(mixed_f32_scratch(N, n), 1)) + slice_scratch(g) + (1 << 20);
 }
 
 Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omega, const double *G, const double *X,
@@ -140,7 +187,7 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
   __half *Tfh = ar.take<__half>((size_t)2 * nO * g.KpT), *Tfl = ar.take<__half>((size_t)2 * nO * g.KpT);
   __half *Tih = ar.take<__half>((size_t)T * g.KpO), *Til = ar.take<__half>((size_t)T * g.KpO);
   double *GR = ar.take<double>((size_t)T * Nn), *GWt = ar.take<double>((size_t)T * Nn);
-  double *GG = ar.take<double>((size_t)T * Nn);
+  float *mxv = ar.take<float>((size_t)kMxV * n);   // [v]: GG, GGw, Aw
   __half *GWh = ar.take<__half>((size_t)T * NR * Kp), *GWl = ar.take<__half>((size_t)T * NR * Kp);
   float *inv_gw = ar.take<float>((size_t)T * N);
   __half *Xh = ar.take<__half>((size_t)T * NR * Kp), *Xl = ar.take<__half>((size_t)T * NR * Kp);
@@ -152,7 +199,7 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
   __half *Awh = ar.take<__half>((size_t)2 * nO * g.Nn8), *Awl = ar.take<__half>((size_t)2 * nO * g.Nn8);
   DynScalars *sc = ar.take<DynScalars>(1);
   const int mT = std::max(T, N);
-  float *ones = ar.take<float>(mT), *sAv = ar.take<float>(mT), *tmp1 = ar.take<float>(mT), *tmp2 = ar.take<float>(mT);
+  float *ones = ar.take<float>(mT), *sAv = ar.take<float>(mT);
   float *Xf = reinterpret_cast<float *>(ar.take<char>(rows_f32_bytes(N, n)));
   Arena scr = ar;   // the mixed tensor's scratch, where the chunk buffers will lie
   void *mix_scratch = scr.take<char>(mixed_f32_scratch(N, n));
@@ -163,8 +210,6 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
   float *Dt = ar.take<float>((size_t)tcn * N * N), *Tm = ar.take<float>((size_t)tcn * N * n);
   double *Sd = ar.take<double>((size_t)tcn * nn);
   if (!Sd || !mix_scratch) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-  (void)tmp1;
-  (void)tmp2;
   ProfScope ps(h, "sosex_dynamic_tc", s, 0);
   long long launches = 0;
   const long long limit = h->spin_limit;
@@ -219,16 +264,15 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
   for (int sp = 0; sp < S; ++sp) {
     const double *Gs = G + (long long)sp * T * nn;
     {  // GR[j][R][q] = sum_u X[R][u] G_j[u][q], GWt[j][P][w] = sum_p X[P][p] G_j[w][p]  (FP64)
-      GemmF64 a;
-      a.M = N; a.Nc = n; a.K = n; a.batch = T;
-      a.A = X; a.ai = n; a.ak = 1;
-      a.B = Gs; a.sB = nn; a.bk = n; a.bj = 1;
-      a.C = GR; a.sC = Nn; a.ci = n; a.cj = 1;
-      launch_gemm_f64(a, s);
-      GemmF64 b = a;
-      b.bk = 1; b.bj = n; b.C = GWt;
-      launch_gemm_f64(b, s);
+      GemmF64 a = projection(n, N, T);
+      a.A = X; a.B = Gs; a.C = GR;
+      SOX_TRY(gemm_f64(h, a, ar, s));
+      a.bk = 1; a.bj = n; a.C = GWt;
+      SOX_TRY(gemm_f64(h, a, ar, s));
     }
+    // the maxima of GG of every v; those of GGw and Aw follow from their products
+    SOX_CUDA_TRY(cudaMemsetAsync(mxv, 0, sizeof(float) * kMxV * n, s));
+    k_gg_max<<<(unsigned)(((long long)T * N + 7) / 8), 256, 0, s>>>(GWt, GR, T, N, n, kMxV, mxv);
     launch_split_rows_f64(GWt, n, Nn, N, NR, n, Kp, GWh, GWl, inv_gw, T, s);
     launches += 3;
     for (int i0 = 0; i0 < T; i0 += tcn) {
@@ -241,38 +285,34 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
           !make_tmap_f16_3d_rs(&mift[2], Awh, Nn, g.Nn8, 2 * nO, 1, (uint64_t)2 * nO * g.Nn8, 64, 64, &err) ||
           !make_tmap_f16_3d_rs(&mift[3], Awl, Nn, g.Nn8, 2 * nO, 1, (uint64_t)2 * nO * g.Nn8, 64, 64, &err))
         return {SOX_ERR_CUDA, "dynamic maps: " + err};
+      SOX_CUDA_TRY(cudaMemsetAsync(&sc->mx[kA], 0, sizeof(float), s));
       for (int v = v_lo; v < v_hi; ++v) {
-        SOX_CUDA_TRY(cudaMemsetAsync(&sc->mx[kGG], 0, 3 * sizeof(float), s));
-        k_gg_tc<<<grid1((long long)T * Nn), 256, 0, s>>>(GWt, GR, T, N, n, v, GG);
-        launch_absmax(GG, false, Nn, T, 0, 1, 1, (int)Nn, &sc->mx[kGG], s);
-        launch_split_tensor(GG, false, Nn, T, 0, 1, 1, (int)Nn, g.Nn8, 0, 1.f, &sc->mx[kGG], nullptr, GGh, GGl,
-                            &sc->sc[kGG], s);
-        k_inv_prod<<<1, 1, 0, s>>>(&sc->sc[kTf], &sc->sc[kGG], &sc->f[0]);
+        float *mx = mxv + (size_t)kMxV * v;
+        k_gg_split<<<dim3((unsigned)std::min((N + 7) / 8, 64), T), 256, 0, s>>>(
+            GWt, GR, T, N, n, v, g.Nn8, mx, GGh, GGl, &sc->sc[kGG]);
         {  // GGw[(m,c)][(Q,u)] = sum_j conj(T_fwd)_c[m][j] GG[j][(Q,u)]
           GemmMnArgs a;
           a.M = 2 * nO; a.Ncols = (int)Nn; a.batch = 1; a.kc_inner = (T + 63) / 64; a.nk_outer = 1;
           a.a.mn_major = 0; a.b.mn_major = 1;
-          a.alpha = &sc->f[0];
+          a.inv_a = &sc->sc[kTf]; a.inv_b = &sc->sc[kGG];
+          a.absmax = i0 == 0 ? mx + 1 : nullptr;
           a.spin_limit = limit; a.status = h->d_status;
           SOX_CUDA_TRY(launch_gemm_mn(mft, a, plan_gemm_mn(a, sms, 1), s));
         }
-        launch_absmax(GGw, true, g.Nn4, 2 * nO, 0, 1, 1, (int)Nn, &sc->mx[kGGw], s);
-        launch_split_tensor(GGw, true, n, N, g.Nn4, 2 * nO, 1, n, g.np8, (long long)N * g.np8, 1.f, &sc->mx[kGGw],
+        launch_split_tensor(GGw, true, n, N, g.Nn4, 2 * nO, 1, n, g.np8, (long long)N * g.np8, 1.f, mx + 1,
                             nullptr, GGwh, GGwl, &sc->sc[kGGw], s);
-        k_inv_prod<<<1, 1, 0, s>>>(&sc->sc[kWd], &sc->sc[kGGw], &sc->f[1]);
         {  // Aw[(m,c)][P][u] = sum_Q W_d[m][P][Q] GGw[(m,c)][Q][u]
           GemmMnArgs a;
           a.M = N; a.Ncols = n; a.batch = 2 * nO; a.kc_inner = (N + 63) / 64; a.nk_outer = 1;
           a.a.mn_major = 0; a.a.zb = 1; a.a.zdiv = 2;
           a.b.mn_major = 1; a.b.zb = 1;
-          a.alpha = &sc->f[1];
+          a.inv_a = &sc->sc[kWd]; a.inv_b = &sc->sc[kGGw];
+          a.absmax = i0 == 0 ? mx + 2 : nullptr;
           a.spin_limit = limit; a.status = h->d_status;
           SOX_CUDA_TRY(launch_gemm_mn(mwd, a, plan_gemm_mn(a, sms, 1), s));
         }
-        launch_absmax(Aw, true, g.np4, 2 * nO * N, 0, 1, 1, n, &sc->mx[kAw], s);
-        launch_split_tensor(Aw, true, g.np4, N, (long long)N * g.np4, 2 * nO, 1, n, n, g.Nn8, 1.f, &sc->mx[kAw],
+        launch_split_tensor(Aw, true, g.np4, N, (long long)N * g.np4, 2 * nO, 1, n, n, g.Nn8, 1.f, mx + 2,
                             nullptr, Awh, Awl, &sc->sc[kAw], s);
-        k_inv_prod<<<1, 1, 0, s>>>(&sc->sc[kTi], &sc->sc[kAw], &sc->f[2]);
         {  // A[i][v][(P,u)] = sum_(m,c) T_inv[i][(m,c)] Aw[(m,c)][(P,u)]  (i in this chunk)
           CUtensorMap mo;
           if (!make_tmap_f32_store3d(&mo, Af + (size_t)v * g.Nn4, Nn, ic, 1, (uint64_t)n * g.Nn4,
@@ -282,17 +322,16 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
           GemmMnArgs a;
           a.M = ic; a.Ncols = (int)Nn; a.batch = 1; a.kc_inner = (2 * nO + 63) / 64; a.nk_outer = 1;
           a.a.mn_major = 0; a.b.mn_major = 1;
-          a.alpha = &sc->f[2];
+          a.inv_a = &sc->sc[kTi]; a.inv_b = &sc->sc[kAw];
+          a.absmax = &sc->mx[kA];
           a.spin_limit = limit; a.status = h->d_status;
           SOX_CUDA_TRY(launch_gemm_mn(mift, a, plan_gemm_mn(a, sms, 1), s));
         }
-        launches += 14;
+        launches += 6;
       }
       // A of the chunk as FP16 pairs [i][v][P][q] with one scale; then the fused B / C / D kernel
-      SOX_CUDA_TRY(cudaMemsetAsync(&sc->mx[kA], 0, sizeof(float), s));
       SOX_CUDA_TRY(cudaMemsetAsync(Ah, 0, 2 * (size_t)ic * n * NR * Kp, s));
       SOX_CUDA_TRY(cudaMemsetAsync(Al, 0, 2 * (size_t)ic * n * NR * Kp, s));
-      launch_absmax(Af, true, g.Nn4, ic * n, 0, 1, 1, (int)Nn, &sc->mx[kA], s);
       launch_split_tensor(Af, true, n, N, g.Nn4, ic * n, 1, n, Kp, (long long)NR * Kp, 1.f, &sc->mx[kA], nullptr, Ah,
                           Al, &sc->sc[kA], s);
       k_bcast<<<(ic + 255) / 256, 256, 0, s>>>(&sc->sc[kA], sAv, ic, 1.f);
@@ -316,10 +355,29 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
       }
       // Sigma_d = -X^T D^T X (FP32 half transform, FP64 final sum), added to Sigma
       launch_backproject_T(Dt, N, Xf, N, n, ic, Tm, s);
-      launch_backproject_sigma(X, Tm, N, n, ic, Sd, nn, s, nullptr);
       double *Sout = Sigma + ((long long)sp * T + i0) * nn;
-      launch_add_f64(Sout, Sd, Sout, (long long)ic * nn, s);
-      launches += 10;
+      if (slices_pay(n, n, N, ic)) {   // Sigma -= X^T T through digit slices, N in blocks
+        for (int k0 = 0; k0 < N; k0 += kSliceMaxK) {
+          const int kc = std::min(kSliceMaxK, N - k0);
+          Arena a2 = ar;
+          SliceOp XT = slice_take(a2, 1, n, kc), Ts = slice_take(a2, ic, n, kc);
+          if (!XT.p || !Ts.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+          slice_rows(X + (long long)k0 * n, false, 0, 1, n, 1, XT, s);
+          slice_rows(Tm + (long long)k0 * n, true, Nn, 1, n, ic, Ts, s);
+          SliceGemm sg;
+          sg.batch = ic;
+          sg.C = Sout; sg.sC = nn; sg.ci = n; sg.cj = 1;
+          sg.alpha = -1.0;
+          sg.beta = 1.0;
+          SOX_TRY(slice_gemm(h, XT, Ts, sg, s));
+          launches += 3;
+        }
+      } else {
+        launch_backproject_sigma(X, Tm, N, n, ic, Sd, nn, s, nullptr);
+        launch_add_f64(Sout, Sd, Sout, (long long)ic * nn, s);
+        launches += 2;
+      }
+      launches += 7;
     }
   }
   h->launches += launches;

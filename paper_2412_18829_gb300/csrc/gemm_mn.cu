@@ -102,6 +102,11 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
+// 1 / (x y) for powers of two
+__device__ __forceinline__ float inv_product(float x, float y) {
+  return scalbnf(1.f, -(tc::log2_of(x) + tc::log2_of(y)));
+}
+
 struct Item {
   int b, i0, j0;
   long long c0, c1;   // chunk range
@@ -282,7 +287,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int row = q * 32 + lane;
     const int h = (warp - 2) >> 2;
     const bool storer = (warp == 2 && lane == 0);
-    const float alpha = a.alpha_host * (a.alpha ? *a.alpha : 1.f);
+    const float alpha = a.alpha_host * (a.alpha ? *a.alpha : (a.inv_a ? inv_product(*a.inv_a, *a.inv_b) : 1.f));
+    float mx = 0.f;
     long long acc_it = 0;
     bool live = true;
     for (long long t = blockIdx.x; t < items && live; t += gridDim.x) {
@@ -312,6 +318,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::mbar_arrive(&bar->acc_empty[buf]);
       }
       if (!live) break;
+      if (a.absmax) {   // rows past M are sums of zeros; columns past Ncols hold no sums at all
+        const int cols = a.Ncols - w.j0 - h * 64;
+#pragma unroll
+        for (int j = 0; j < 64; ++j)
+          if (j < cols) mx = fmaxf(mx, fabsf(sum[j] * alpha));
+      }
       // scaled tile -> TMA, one 64-column half at a time through the staging buffer (two
       // 128-byte-swizzled boxes of 128 rows x 32 columns); the half-h warps fill it
       float *tile = reinterpret_cast<float *>(stage_out);
@@ -348,6 +360,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
+    if (a.absmax) {
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      // non-negative floats order like their bit patterns
+      if (lane == 0 && mx > 0.f) atomicMax(reinterpret_cast<unsigned int *>(a.absmax), __float_as_uint(mx));
+    }
     if (storer) bulk_wait_all();
   }
   __syncthreads();
@@ -366,20 +383,17 @@ constexpr int kUnitCols = 256;
 // |x| as FP32 (an FP64 value rounds up to at most one FP32 ulp); FP32 sources stay on the
 // FP32 pipe (the FP64 rate is 1/64 of it)
 __device__ __forceinline__ float abs_f(float x) { return fabsf(x); }
-__device__ __forceinline__ float abs_f(double x) { return (float)fabs(x); }
+__device__ __forceinline__ float abs_f(double x) { return tc::f32_abs(x); }
 
-// FP16 pair of x * sd (sd a signed power of two; x * sd exact): hi rounds to nearest and
-// lo = RN(x sd - hi).  For an FP32 x both steps are exact in FP32, so no FP64 arithmetic
-// is needed; an FP64 x keeps its remainder in FP64.
-__device__ __forceinline__ void split_scaled(float x, float sf, double, __half &a, __half &b) {
+// FP16 pair of +-x * s (s a power of two): hi rounds to nearest and lo = RN(x s - hi).  For an
+// FP32 x both steps are exact in FP32; an FP64 x keeps its remainder in integers.
+__device__ __forceinline__ void split_scaled(float x, float sf, int, bool, __half &a, __half &b) {
   const float xs = x * sf;
   a = __float2half_rn(xs);
   b = __float2half_rn(xs - __half2float(a));
 }
-__device__ __forceinline__ void split_scaled(double x, float, double sd, __half &a, __half &b) {
-  const double xs = x * sd;
-  a = __float2half_rn((float)xs);
-  b = __float2half_rn((float)(xs - (double)__half2float(a)));
+__device__ __forceinline__ void split_scaled(double x, float, int ks, bool neg, __half &a, __half &b) {
+  tc::split_f16_f64(neg ? -x : x, ks, a, b);
 }
 
 template <class T>
@@ -407,24 +421,14 @@ __global__ void k_absmax(const T *src, long long ld0, int rows0, long long ld1, 
   if (lane == 0 && m > 0.f) atomicMax(reinterpret_cast<unsigned int *>(out), __float_as_uint(m));
 }
 
-// 2^(14 - floor(log2 m)) for m > 0 (m in [2^e, 2^(e+1)) -> scaled max in [2^14, 2^15)), 1 for
-// m == 0; clamped to normal FP32 powers of two
-__device__ __forceinline__ float big_scale(float m) {
-  if (!(m > 0.f)) return 1.f;
-  int e;
-  frexpf(m, &e);   // m = f 2^e, f in [0.5, 1): floor(log2 m) = e - 1
-  int k = 15 - e;
-  k = k < -120 ? -120 : (k > 120 ? 120 : k);
-  return ldexpf(1.f, k);
-}
-
 template <class T>
 __global__ void k_split_tensor(const T *src, long long ld0, int rows0, long long ld1, int rows1, long long ldc,
                                int cols, long long ldo, long long ldo1, float sign, const float *absmax,
                                const float *scale_in, __half *hi, __half *lo, float *scale_out) {
-  const float s = scale_in ? *scale_in : big_scale(*absmax);
-  const double sd = (double)sign * (double)s;
+  const float s = scale_in ? *scale_in : tc::big_scale(*absmax);
   const float sf = sign * s;
+  const int ks = tc::log2_of(s);
+  const bool neg = sign < 0.f;
   const long long cpr = (ldo + kUnitCols - 1) / kUnitCols;
   const long long units = (long long)rows1 * rows0 * cpr;
   const int lane = threadIdx.x & 31;
@@ -441,7 +445,7 @@ __global__ void k_split_tensor(const T *src, long long ld0, int rows0, long long
       const long long c = c0 + lane + 32 * k;
       if (c >= ldo) break;
       __half a = __float2half(0.f), b = __float2half(0.f);
-      if (c < cols) split_scaled(row[c * ldc], sf, sd, a, b);
+      if (c < cols) split_scaled(row[c * ldc], sf, ks, neg, a, b);
       h[c] = a;
       l[c] = b;
     }
@@ -485,7 +489,7 @@ __global__ void k_absmax_f32x2(const float *src, long long ld0, int rows0, long 
 __global__ void k_split_f32x2(const float *src, long long ld0, int rows0, long long ld1, int rows1, int cols,
                               long long ldo, long long ldo1, float sign, const float *absmax, const float *scale_in,
                               __half *hi, __half *lo, float *scale_out) {
-  const float s = scale_in ? *scale_in : big_scale(*absmax);
+  const float s = scale_in ? *scale_in : tc::big_scale(*absmax);
   const float sf = sign * s;
   const long long cpr = (ldo + kUnitCols2 - 1) / kUnitCols2;
   const long long units = (long long)rows1 * rows0 * cpr;

@@ -40,6 +40,11 @@ struct GemmMnArgs {
   long long cps = 0;            // chunks per split item (set by plan_gemm_mn)
   MnOperand a, b;
   const float *alpha = nullptr; // optional device scalar multiplying alpha_host
+  // or the factor 1 / (*inv_a * *inv_b) of two split scales (powers of two; alpha NULL)
+  const float *inv_a = nullptr, *inv_b = nullptr;
+  // optional: raised to max |C| over the call's outputs by atomicMax, as launch_absmax would
+  // (ksplit 1 and no accumulation only: the epilogue then holds every output once)
+  float *absmax = nullptr;
   float alpha_host = 1.f;
   int accumulate = 0;           // reduce-add into C instead of storing
   long long spin_limit = 0;

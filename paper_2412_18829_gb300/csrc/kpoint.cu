@@ -19,6 +19,7 @@
 #include "f64_slices.h"
 #include "gj.h"
 #include "kpoint.h"
+#include "tc_common.cuh"
 
 namespace sox {
 namespace {
@@ -940,6 +941,73 @@ Status kpoint_sigma_tc(sox_handle h, const sox_problem *pr, const double *Gd, co
 
 namespace {
 
+// The pairs of GG^{ks}(tau_j)[(Q,u)] = GWt^{ku}[j][Q][u] (-GR^{ks}[T-1-j][Q][v]) for one q1 (k_u =
+// k_s - q1) as a B operand: per (k_s, (Q,u)) the re-row and the im-row, K = tau_j, Kp2 halves each.
+// 2^lp lanes per row, four times (16 bytes of every output) per lane and step; neighbouring groups
+// are neighbouring u, so reads stay coalesced.  Up to 128 times a lane forms its four products
+// once and keeps them; beyond that they are formed again for the pairs.  3 x 3 x 3, n = 26, N =
+// 300, 8 times: 17 us product + 163 us split before (114 through FP64 conversions), 34 us here;
+// 2 x 1 x 1, 60 times: 45 us before, 33 us here.
+__global__ void __launch_bounds__(256) k_gg_csplit(const z *GWt, const z *GR, const int *sub, int nk, int q1, int T, int N,
+                                                   int n, int v, int lp, int Kp2, __half *hi, __half *lo, float *unscale) {
+  const long long Nn = (long long)N * n;
+  const long long e0 = (blockIdx.x * 256ll + threadIdx.x) >> lp;
+  const long long e = e0 < Nn ? e0 : Nn - 1;   // a warp's surplus lanes stay for the shuffles
+  const int gl = threadIdx.x & ((1 << lp) - 1);
+  const int ks = blockIdx.y;
+  const int ku = sub[ks * nk + q1];
+  const z *w = GWt + (long long)ku * T * Nn + e;
+  const z *g = GR + (long long)ks * T * Nn + (e / n) * n + v;
+  const int nc = Kp2 / 8;   // chunks of four times
+  z p[4];
+  auto form = [&](int c) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int j = c * 4 + i;
+      p[i] = make_double2(0.0, 0.0);
+      if (j < T) {
+        const z b = g[(long long)(T - 1 - j) * Nn];
+        p[i] = zmul(w[(long long)j * Nn], make_double2(-b.x, -b.y));
+      }
+    }
+  };
+  float mx = 0.f;
+  for (int c = gl; c < nc; c += 1 << lp) {
+    form(c);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mx = fmaxf(mx, fmaxf(tc::f32_abs(p[i].x), tc::f32_abs(p[i].y)));
+  }
+  for (int o = (1 << lp) >> 1; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (e0 >= Nn) return;
+  const float s = tc::pow2_floor_inv(mx);
+  const int k2 = tc::log2_of(s);
+  const long long row = ((long long)ks * Nn + e) * 2;
+  __half *h0 = hi + row * Kp2, *l0 = lo + row * Kp2, *h1 = h0 + Kp2, *l1 = l0 + Kp2;
+  const bool once = nc <= (1 << lp);
+  for (int c = gl; c < nc; c += 1 << lp) {
+    if (!once) form(c);
+    uint32_t a0[4], b0[4], a1[4], b1[4];   // re-row (x, -y), im-row (y, x): hi words a, lo words b
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      __half xh, xl, yh, yl;
+      tc::split_f16_f64(p[i].x, k2, xh, xl);
+      tc::split_f16_f64(p[i].y, k2, yh, yl);
+      auto pack = [](__half l_, __half h_) {
+        return (uint32_t)__half_as_ushort(l_) | ((uint32_t)__half_as_ushort(h_) << 16);
+      };
+      a0[i] = pack(xh, __hneg(yh));
+      b0[i] = pack(xl, __hneg(yl));
+      a1[i] = pack(yh, xh);
+      b1[i] = pack(yl, xl);
+    }
+    *reinterpret_cast<uint4 *>(h0 + c * 8) = make_uint4(a0[0], a0[1], a0[2], a0[3]);
+    *reinterpret_cast<uint4 *>(l0 + c * 8) = make_uint4(b0[0], b0[1], b0[2], b0[3]);
+    *reinterpret_cast<uint4 *>(h1 + c * 8) = make_uint4(a1[0], a1[1], a1[2], a1[3]);
+    *reinterpret_cast<uint4 *>(l1 + c * 8) = make_uint4(b1[0], b1[1], b1[2], b1[3]);
+  }
+  if (gl == 0) unscale[row] = unscale[row + 1] = 1.f / s;
+}
+
 struct KDynTc {
   KTc g;
   int nO, ct, upad;
@@ -959,7 +1027,7 @@ KDynTc kdyn_geom(sox_handle h, const sox_problem *p, int nO, size_t *fixed_out, 
   f += csplit_bytes(g.nk, 2 * g.N, g.n);                                        // X split
   f += csplit_bytes(g.nk * nO, g.N, g.N);                                       // W_d split
   f += csplit_bytes(1, nO, g.T) + csplit_bytes(1, g.T, nO);                     // transforms
-  f += 3 * aligned_bytes((size_t)g.nk * g.T * g.Nn, 16);                        // GR, GWt, GG (FP64)
+  f += 2 * aligned_bytes((size_t)g.nk * g.T * g.Nn, 16);                        // GR, GWt (FP64)
   f += csplit_bytes(g.nk, g.T * g.N, g.n);                                      // GWt split, all tau
   f += csplit_bytes(g.nk, (int)(2 * g.Nn), g.T);                                // GG split
   f += aligned_bytes((size_t)g.nk * nO * d.ldNn, 8);                            // GG(i Omega)
@@ -1009,7 +1077,6 @@ Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const
   CSplit Wds = csplit_take(ar, nk * nO, N, N);
   CSplit Tfs = csplit_take(ar, 1, nO, T), Tis = csplit_take(ar, 1, T, nO);
   z *GR = ar.take<z>((size_t)nk * T * g.Nn), *GWt = ar.take<z>((size_t)nk * T * g.Nn);
-  z *GG = ar.take<z>((size_t)nk * T * g.Nn);
   CSplit GWts = csplit_take(ar, nk, T * N, n);
   CSplit GGs = csplit_take(ar, nk, (int)(2 * g.Nn), T);
   float *GGw = ar.take<float>(2 * (size_t)nk * nO * d.ldNn);
@@ -1051,9 +1118,11 @@ Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const
     ++launches;
     for (int v = v_lo; v < v_hi; ++v) {   // the handle's v range (sox_set_v_range)
       for (int q1 = 0; q1 < nk; ++q1) {
-        k_gg_k<<<grid1((long long)nk * T * g.Nn), 256, 0, s>>>(GWt, GR, tb.sub, nk, q1, T, N, n, v, GG);
         // B rows (Q,u) of GG^{ks}, K = tau_j
-        csplit_b(GG, false, (long long)T * g.Nn, 1, 0, 0, g.Nn, nk, (int)g.Nn, T, false, false, GGs, s);
+        int lp = 0;   // lanes per row: a lane takes four times
+        while (lp < 5 && (4 << lp) < T) ++lp;
+        k_gg_csplit<<<dim3((unsigned)(((g.Nn << lp) + 255) / 256), nk), 256, 0, s>>>(GWt, GR, tb.sub, nk, q1, T, N, n, v, lp,
+                                                                                   GGs.Kp2, GGs.hi, GGs.lo, GGs.unscale);
         // GG(i Omega_m)[ks][(Q,u)] = sum_j T_fwd[m][j] GG[ks][j][(Q,u)]
         SOX_TRY(cgemm_tc(h, Tfs, GGs, nk, nullptr, nullptr, 1.f, GGw, 2 * d.ldNn, 2LL * nO * d.ldNn, s));
         // B rows u of GG(i Omega_m)^{ks}, K = Q

@@ -298,6 +298,17 @@ __device__ __forceinline__ float pow2_floor_inv(float m) {
   return ldexpf(1.f, k);
 }
 
+// 2^(14 - floor(log2 m)) for m > 0 (m in [2^e, 2^(e+1)) -> scaled max in [2^14, 2^15)), 1 for
+// m == 0; clamped to normal FP32 powers of two
+__device__ __forceinline__ float big_scale(float m) {
+  if (!(m > 0.f)) return 1.f;
+  int e;
+  frexpf(m, &e);   // m = f 2^e, f in [0.5, 1): floor(log2 m) = e - 1
+  int k = 15 - e;
+  k = k < -120 ? -120 : (k > 120 ? 120 : k);
+  return ldexpf(1.f, k);
+}
+
 // x = hi + lo (FP16 pair) after scaling; hi rounds to nearest.
 __device__ __forceinline__ void split_f16(float x, __half &hi, __half &lo) {
   hi = __float2half_rn(x);
@@ -312,6 +323,57 @@ __device__ __forceinline__ void split_f16x2(float x0, float x1, uint32_t &hi, ui
   const __half2 l = __floats2half2_rn(x0 - hf.x, x1 - hf.y);
   hi = *reinterpret_cast<const uint32_t *>(&h);
   lo = *reinterpret_cast<const uint32_t *>(&l);
+}
+
+// FP64 values into FP32 and FP16 pairs without the FP64 pipe (1.9 lanes a clock and SM: a
+// conversion or a subtraction there costs as much as forty other instructions).
+
+// (float)x, round to nearest even
+__device__ __forceinline__ float f32_of(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int ef = (int)((hi >> 20) & 0x7ffu);
+  if (ef == 0) return __uint_as_float(hi & 0x80000000u);      // FP64 subnormals lie below FP32's
+  if (ef < 898 || ef > 1149) return (float)x;                 // FP32 subnormals, overflow, infinities, NaNs
+  uint32_t u = ((uint32_t)(ef - 896) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const uint32_t rem = lo & 0x1fffffffu;
+  u += (rem + (u & 1u)) > 0x10000000u ? 1u : 0u;
+  return __uint_as_float(u | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float f32_abs(double x) {
+  return f32_of(__hiloint2double(__double2hiint(x) & 0x7fffffff, __double2loint(x)));
+}
+
+// exponent k of a power of two s = 2^k (normal)
+__device__ __forceinline__ int log2_of(float s) { return (int)((__float_as_uint(s) >> 23) & 0xffu) - 127; }
+
+// FP16 pair of x 2^k: h = RN16(RN32(x 2^k)), l = RN16(RN32(x 2^k - h)).  With f = RN32(x 2^k) and
+// the 29 bits g = x 2^k - f that FP32 drops, f - h is exact in FP32 and l = RN16(f - h + g): g
+// only decides where f - h lies half way between two FP16 numbers (its own rounding to FP32
+// could matter there for one value in 10^7, by one bit of l).
+__device__ __forceinline__ void split_f16_f64(double x, int k, __half &h, __half &l) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int ef = (int)((hi >> 20) & 0x7ffu), e = ef + k - 1023;   // exponent of x 2^k
+  if (e < -30 || e > 15 || ef == 0 || ef == 0x7ff) {
+    if (ef == 0 || e < -30) {   // rounds to zero in both halves
+      h = l = __ushort_as_half(0);
+    } else {                    // infinities, NaNs, values above the range of the scale
+      const double xs = x * scalbn(1.0, k);
+      h = __float2half_rn((float)xs);
+      l = __float2half_rn((float)(xs - (double)__half2float(h)));
+    }
+    return;
+  }
+  uint32_t u = ((uint32_t)(e + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const uint32_t rem = lo & 0x1fffffffu;
+  const bool up = (rem + (u & 1u)) > 0x10000000u;
+  u += up ? 1u : 0u;
+  const int g = (int)rem - (up ? 0x20000000 : 0);
+  const uint32_t sgn = hi & 0x80000000u;
+  const float f = __uint_as_float(u | sgn);
+  h = __float2half_rn(f);
+  // 2^(e - 52) with the sign of x
+  const float unit = __uint_as_float(((uint32_t)(e - 52 + 127) << 23) | sgn);
+  l = __float2half_rn(fmaf((float)g, unit, f - __half2float(h)));
 }
 
 }  // namespace tc

@@ -1205,8 +1205,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if (t + gridDim.x < total) pre = f32_tile_scale(a, t + gridDim.x, ep, tM, tN);
         const float rsc = s_sc[kTile + row];
         float *tile = reinterpret_cast<float *>(stage_out);
+        // a warp whose 32 rows or 64 columns lie outside the output has nothing to read or stage
+        // (the stores clip them): 3 of 4 warps of a product with M <= 32
+        const bool live = i0 + q * 32 < a.M && j0 + h * 64 < a.Ncols;
+        if (!live) {
+          tc::tc_fence_before();
+          tc::mbar_arrive(&bar->acc_empty[buf]);
+        }
 #pragma unroll
-        for (int c = 0; c < 64; c += 32) {
+        for (int c = 0; live && c < 64; c += 32) {
           float v[32];
           tc::tmem_ld_32x32b_x32(base + c, v);
           tc::tmem_ld_wait();
@@ -1249,7 +1256,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       } else {
         float m = 0.f;
 #pragma unroll
-        for (int c = 0; c < 64; c += 32) {
+        for (int c = 0; i0 + q * 32 < a.M && c < 64; c += 32) {
           float v[32];
           tc::tmem_ld_32x32b_x32(base + c, v);
           tc::tmem_ld_wait();
@@ -1279,8 +1286,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       // split into FP16 pairs, written to the 128-byte-swizzled staging tile of this half
       uint8_t *hi_tile = stage_out + (size_t)(0 * 2 + h) * (kTile * 128);
       uint8_t *lo_tile = stage_out + (size_t)(1 * 2 + h) * (kTile * 128);
+      const bool live = i0 + q * 32 < a.M;   // as above
+      if (!live) {
+        tc::tc_fence_before();
+        tc::mbar_arrive(&bar->acc_empty[buf]);
+      }
 #pragma unroll
-      for (int c = 0; c < 64; c += 32) {
+      for (int c = 0; live && c < 64; c += 32) {
         float v[32];
         tc::tmem_ld_32x32b_x32(base + c, v);
         tc::tmem_ld_wait();
@@ -1352,17 +1364,14 @@ __global__ void k_split_rows_f64(const double *src, long long ld, long long bstr
   }
   const double *x = ((use_alt && use_alt[b]) ? alt_src : src) + b * bstride + r * ld;
   float m = 0.f;
-  for (int k = lane; k < L; k += 32) m = fmaxf(m, (float)fabs(x[k]));
+  for (int k = lane; k < L; k += 32) m = fmaxf(m, tc::f32_abs(x[k]));
   m = warp_max(m);
   const float s = tc::pow2_floor_inv(m);
+  const int ks = tc::log2_of(s);
   for (int k = lane; k < Kp; k += 32) {
     __half a = __float2half(0.f), c = __float2half(0.f);
     if (k < L) {
-      // scale in FP64 (exact: power of two), then round to the FP16 pair via FP32
-      const double xs = x[k] * (double)s;
-      const float f = (float)xs;
-      a = __float2half_rn(f);
-      c = __float2half_rn((float)(xs - (double)__half2float(a)));
+      tc::split_f16_f64(x[k], ks, a, c);
     }
     h[k] = a;
     l[k] = c;
@@ -1449,13 +1458,14 @@ __global__ void k_prep_gminus(const double *G, int n, int T, int Kp, __half *hi,
   const int sp = (b0 + b) / T, j = (b0 + b) % T;
   const double *g = G + ((long long)sp * T + (T - 1 - j)) * n * n;
   float m = 0.f;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) m = fmaxf(m, (float)fabs(g[e]));
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) m = fmaxf(m, tc::f32_abs(g[e]));
   m = block_max(m);
   const float sc = tc::pow2_floor_inv(m);
+  const int ksc = tc::log2_of(sc);
   float cs = 0.f;
   for (int v = threadIdx.x; v < n; v += blockDim.x) {
     float acc = 0.f;
-    for (int s = 0; s < n; ++s) acc += (float)fabs(g[(long long)s * n + v]) * sc;
+    for (int s = 0; s < n; ++s) acc += tc::f32_abs(g[(long long)s * n + v]) * sc;
     cs = fmaxf(cs, acc);
   }
   cs = block_max(cs) * 2.f * 1.0001f;
@@ -1469,9 +1479,7 @@ __global__ void k_prep_gminus(const double *G, int n, int T, int Kp, __half *hi,
     const int v = e2 / Kp, s = e2 % Kp;
     __half a = __float2half(0.f), c = __float2half(0.f);
     if (v < n && s < n) {
-      const double xs = -g[(long long)s * n + v] * (double)sc;
-      a = __float2half_rn((float)xs);
-      c = __float2half_rn((float)(xs - (double)__half2float(a)));
+      tc::split_f16_f64(-g[(long long)s * n + v], ksc, a, c);
     }
     h[e2] = a;
     l[e2] = c;

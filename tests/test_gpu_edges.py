@@ -229,3 +229,57 @@ def test_w_dynamic_of_solids_through_slices(env, nk, n, N, n_tau, M):
     pkg.sox_check_device(hs["fp64"])
     ref = kpoints.w_dynamic(w.V, kpoints.pi_omega(w.X, w.G[0], Tf, nk))
     assert np.abs(out.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+def _random_dynamic(rng, n, N, n_tau, M, nk=None):
+    """Inputs of the dynamic calls with random transforms and screening (any n_tau)."""
+    w = synth.solid(70 + n, nk, n, N, n_tau, 10.0) if nk else synth.molecule(70 + n, n, N, n_tau, 10.0)
+    Tf, Ti = (0.3 * (rng.standard_normal(s) + 1j * rng.standard_normal(s)) for s in ((M, n_tau), (n_tau, M)))
+    shape = (w.X.shape[0], M, N, N) if nk else (M, N, N)
+    Wd = rng.standard_normal(shape) / N   # real for molecules
+    if nk:
+        Wd = Wd + 1j * rng.standard_normal(shape) / N
+    return w, Tf, Ti, Wd
+
+
+def _dynamic(env, w, Tf, Ti, Wd, nk=None, scale=1.0):
+    torch, pkg, hs = env
+    h = hs["f16x2"]
+    p = pkg.problem(w.n, w.N, w.n_tau, 1, w.beta, **(dict(nk=nk, dtype=1) if nk else {}))
+    cast = complex if nk else float
+    G, X, V = to_dev(torch, *(np.asarray(a, dtype=cast) for a in (w.G * scale, w.X, w.V)))
+    F, I, W = to_dev(torch, Tf, Ti, Wd)
+    S = torch.full_like(G, float("nan"))
+    pkg.sosex_dynamic_sigma(h, p, G, X, V, W, F, I, Tf.shape[0], S)
+    pkg.sox_check_device(h)
+    return S.cpu().numpy()
+
+
+@pytest.mark.parametrize("n,N,n_tau,M", [(1, 5, 2, 1), (7, 33, 3, 2), (8, 128, 4, 3), (9, 129, 2, 65), (33, 64, 65, 2)])
+def test_dynamic_splits_and_maxima(env, n, N, n_tau, M):
+    """FP16 pairs from integers and tensor maxima from the products' own tiles: N n off the 128
+    columns of a tile, one row, K at 64 and 65, and a propagator 2^20 times smaller
+    (every scale is a power of two: the same pairs, so the same bound on Sigma / 2^-60)."""
+    from oracle import dynamic
+
+    rng = np.random.default_rng(n)
+    w, Tf, Ti, Wd = _random_dynamic(rng, n, N, n_tau, M)
+    ref = dynamic.sosex_dynamic_sigma(w.X, w.V, Wd, Tf, Ti, w.G).real
+    bar = 2e-6 * np.abs(ref).max()   # 22-bit pairs, FP32 sums
+    for scale in (1.0, 2.0 ** -20):
+        got = _dynamic(env, w, Tf, Ti, Wd, scale=scale) / scale ** 3
+        assert np.abs(got - ref).max() <= bar, scale
+
+
+@pytest.mark.parametrize("nk,n,N,n_tau,M", [((2, 1, 1), 3, 5, 2, 1), ((1, 2, 1), 2, 7, 4, 2), ((1, 1, 3), 5, 12, 5, 3),
+                                            ((2, 1, 1), 3, 33, 9, 2), ((1, 1, 2), 4, 31, 129, 3)])
+def test_solid_dynamic_pairs_of_the_time_products(env, nk, n, N, n_tau, M):
+    """One, two, four and 32 lanes per row, times that fill no whole chunk of four, and more times
+    than the lanes of a row keep; pair rows whose pitch is no multiple of 64 values."""
+    from oracle import kpoints
+
+    rng = np.random.default_rng(n_tau)
+    w, Tf, Ti, Wd = _random_dynamic(rng, n, N, n_tau, M, nk)
+    ref = kpoints.sosex_dynamic_sigma(w.X, w.V, Wd, Tf, Ti, w.G, nk)
+    got = _dynamic(env, w, Tf, Ti, Wd, nk=nk)
+    assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max()
