@@ -774,9 +774,16 @@ int blocks_for(long long warps) { return (int)std::max<long long>(1, (warps * 32
 
 }  // namespace
 
-// rows of 2K values, a multiple of 8 (16 bytes, the TMA's row pitch; the copies fill the rest of
-// a 64-wide chunk with zeros)
-int csplit_kp2(int K) { return (2 * K + 7) & ~7; }
+// Pitch of a row of 2K values: 8, 16, 32 or a multiple of 64 halves, so that no 64-wide chunk of a
+// row straddles a 128-byte line.  The copy engine takes lines, about one per 2.5 clocks and SM,
+// whatever part of them it needs: rows of 52 values at a pitch of 56 cost two lines each.  Short
+// rows stay short (the copies fill the rest of a chunk with zeros).
+int csplit_kp2(int K) {
+  if (2 * K > 32) return ((2 * K + 63) / 64) * 64;
+  int p = 8;
+  while (p < 2 * K) p *= 2;
+  return p;
+}
 
 size_t csplit_bytes(int batch, int rows_real, int K) {
   const size_t e = (size_t)batch * rows_real * csplit_kp2(K);
@@ -865,10 +872,12 @@ Status cgemm_tc(sox_handle h, const CSplit &A, const CSplit &B, int batch, const
     const int kw = std::min(kKChunk, A.Kp2 - k0);
     CUtensorMap maps[6];
     std::string err;
-    if (!make_tmap_f16_3d_rs(&maps[0], A.hi + k0, kw, A.Kp2, A.rows, A.batch, bsA * A.Kp2, 64, 128, &err) ||
-        !make_tmap_f16_3d_rs(&maps[1], A.lo + k0, kw, A.Kp2, A.rows, A.batch, bsA * A.Kp2, 64, 128, &err) ||
-        !make_tmap_f16_3d_rs(&maps[2], B.hi + k0, kw, B.Kp2, B.rows, B.batch, bsB * B.Kp2, 64, 128, &err) ||
-        !make_tmap_f16_3d_rs(&maps[3], B.lo + k0, kw, B.Kp2, B.rows, B.batch, bsB * B.Kp2, 64, 128, &err))
+    // what a tile does not have is not copied (its rows and columns of the output are clipped)
+    const int ra = std::min(128, (A.rows + 7) & ~7), rb = std::min(128, (B.rows + 7) & ~7);
+    if (!make_tmap_f16_3d_rs(&maps[0], A.hi + k0, kw, A.Kp2, A.rows, A.batch, bsA * A.Kp2, 64, ra, &err) ||
+        !make_tmap_f16_3d_rs(&maps[1], A.lo + k0, kw, A.Kp2, A.rows, A.batch, bsA * A.Kp2, 64, ra, &err) ||
+        !make_tmap_f16_3d_rs(&maps[2], B.hi + k0, kw, B.Kp2, B.rows, B.batch, bsB * B.Kp2, 64, rb, &err) ||
+        !make_tmap_f16_3d_rs(&maps[3], B.lo + k0, kw, B.Kp2, B.rows, B.batch, bsB * B.Kp2, 64, rb, &err))
       return {SOX_ERR_CUDA, "cgemm_tc: " + err};
     if (!make_tmap_f32_store3d(&maps[4], C, B.rows, A.rows, batch, ldc, sCb, &err))
       return {SOX_ERR_CUDA, "cgemm_tc: " + err};
@@ -876,6 +885,8 @@ Status cgemm_tc(sox_handle h, const CSplit &A, const CSplit &B, int batch, const
     GemmTcArgs ga;
     ga.M = A.rows;
     ga.Ncols = B.rows;
+    ga.rows_a = ra;
+    ga.rows_b = rb;
     ga.Kp = (kw + 63) & ~63;
     ga.K = kw;
     ga.batch = batch;

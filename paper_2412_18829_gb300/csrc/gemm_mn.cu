@@ -73,17 +73,6 @@ __device__ __forceinline__ uint64_t op_desc(uint32_t base, int mn, int k16) {
   return mn ? desc_mn_sw128(base + k16 * 2048, kPart / 2) : tc::desc_kmajor_sw128(base + k16 * 32);
 }
 
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool epi_all(bool ok) {
-  int r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 256, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((unsigned)ok)
-      : "memory");
-  return r != 0;
-}
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, const void *src, int x, int y, int z) {
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
@@ -284,9 +273,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp <= 9) {
     // ---------------- epilogue: 8 warps, lane quarter q, 64-column half h ----------------
     const int q = warp & 3;
-    const int row = q * 32 + lane;
     const int h = (warp - 2) >> 2;
-    const bool storer = (warp == 2 && lane == 0);
+    float *own = reinterpret_cast<float *>(stage_out) + (warp - 2) * 1024;   // this warp's box of 4 KB
     const float alpha = a.alpha_host * (a.alpha ? *a.alpha : (a.inv_a ? inv_product(*a.inv_a, *a.inv_b) : 1.f));
     float mx = 0.f;
     long long acc_it = 0;
@@ -300,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int buf = (int)(acc_it & 3);
         const uint32_t aph = (uint32_t)((acc_it >> 2) & 1);
         const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
-        if (!epi_all(got && !*abort)) {
+        if (!__all_sync(0xffffffffu, got && !*abort)) {
           live = false;
           break;
         }
@@ -324,39 +312,30 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < 64; ++j)
           if (j < cols) mx = fmaxf(mx, fabsf(sum[j] * alpha));
       }
-      // scaled tile -> TMA, one 64-column half at a time through the staging buffer (two
-      // 128-byte-swizzled boxes of 128 rows x 32 columns); the half-h warps fill it
-      float *tile = reinterpret_cast<float *>(stage_out);
+      // scaled tile -> TMA: every warp stages and stores its own 32 rows x 32 columns in turn
       const bool add = a.accumulate || a.ksplit > 1;
+      if (w.i0 + q * 32 < a.M) {
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        if (storer) bulk_wait_read();   // the previous stores have read the staging buffer
-        epi_sync();
-        if (h == half) {
-#pragma unroll
-          for (int c = 0; c < 64; c += 32) {
-            float *box = tile + (c / 32) * (kT * 32) + row * 32;
+        for (int c = 0; c < 64; c += 32) {
+          const int x = w.j0 + h * 64 + c;
+          if (x < a.Ncols) {
+            if (lane == 0) bulk_wait_read();   // the previous store has read the box
+            __syncwarp();
 #pragma unroll
             for (int t4 = 0; t4 < 8; ++t4)
-              *reinterpret_cast<float4 *>(box + ((t4 ^ (row & 7)) * 4)) =
+              *reinterpret_cast<float4 *>(own + lane * 32 + ((t4 ^ (lane & 7)) * 4)) =
                   make_float4(sum[c + 4 * t4] * alpha, sum[c + 4 * t4 + 1] * alpha, sum[c + 4 * t4 + 2] * alpha,
                               sum[c + 4 * t4 + 3] * alpha);
-          }
-        }
-        fence_proxy_async_smem();
-        epi_sync();
-        if (storer) {
-#pragma unroll
-          for (int bx = 0; bx < 2; ++bx) {
-            const int x = w.j0 + half * 64 + 32 * bx;
-            if (x < a.Ncols) {
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
               if (add)
-                tma_reduce_add_3d(&tmC, stage_out + (size_t)bx * (kT * 128), x, w.i0, w.b);
+                tma_reduce_add_3d(&tmC, own, x, w.i0 + q * 32, w.b);
               else
-                tma_store_3d(&tmC, stage_out + (size_t)bx * (kT * 128), x, w.i0, w.b);
+                tma_store_3d(&tmC, own, x, w.i0 + q * 32, w.b);
+              bulk_commit();
             }
           }
-          bulk_commit();
         }
       }
     }
@@ -365,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // non-negative floats order like their bit patterns
       if (lane == 0 && mx > 0.f) atomicMax(reinterpret_cast<unsigned int *>(a.absmax), __float_as_uint(mx));
     }
-    if (storer) bulk_wait_all();
+    if (lane == 0) bulk_wait_all();
   }
   __syncthreads();
   if (warp == 1) {

@@ -987,7 +987,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBcdThreads, 1)
 // tile (kStoreSplit: out_scale[b]; kStoreSplitGroup: an exact power of two per
 // group of `group` columns, all of whose rows lie in the tile), splits it into
 // FP16 pairs in swizzled shared memory and writes it with TMA tensor stores into
-// the 4-D output [batch][M][n_groups][group] (box: 128 rows x 64 columns).
+// the 4-D output [batch][M][n_groups][group].  Every epilogue warp stages and stores its own
+// 32 rows x 64 columns (8 KB of the staging buffer), so no warp waits for another one's part of
+// the previous tile; with one 128-row store per tile the stores, two CTA-wide barriers and the
+// next tile's staging ran one after another.  With K of one chunk the epilogue still sets the pace
+// (FP32 output), not the copies or the MMAs: per tile of 128 x 128 it took 3900 clocks, 1500 of them
+// the wait for the next tile's scale behind its batch index, now 2300.  729 x 8 products 300 x 600,
+// K = 52: 1182 -> 664 us (4.25 GB: 6.4 TB/s).
 // ============================================================================
 constexpr int kGStages = 2;
 constexpr int kStageOut = 4 * kTile * 64 * 2;   // hi/lo x two 64-column halves, 64 KB
@@ -1002,7 +1008,11 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, const void 
                : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// all but the last kLeft groups of this thread's stores have read shared memory
+template <int kLeft>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kLeft) : "memory");
+}
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // The split GEMM runs 8 epilogue warps (two per TMEM lane quarter, one per
 // 64-column half): the epilogue, not the MMA, sets its pace.
@@ -1036,48 +1046,79 @@ __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap *map, const 
                "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z)
                : "memory");
 }
-// Output tile t of a GEMM launch: batch b and the tile's first row i0 and column j0.  When
+// Output tiles of a GEMM launch, walked by one CTA: tiles blockIdx.x, + gridDim.x, ...  When
 // every batch shares one B operand (no index table), the column tiles go slowest, then the
 // batches, then the row tiles, so all the tiles that read one B tile run one after another
 // and B leaves DRAM once per launch (the A GEMM of the chain: U_Pqs of up to 0.7 GB read
 // by every (tau, row tile) pair would otherwise be re-read from DRAM for each); otherwise
-// batches slowest, then rows, then columns.
-struct GemmTile {
-  int b, i0, j0;
-};
-__device__ __forceinline__ GemmTile gemm_tile(const GemmTcArgs &a, long long t, int tM, int tN) {
-  GemmTile g;
-  if (a.batchB_shared && !a.idxB) {
-    const long long per_j = (long long)a.batch * tM;
-    const long long j = t / per_j, r = t % per_j;
-    g.b = (int)(r / tM);
-    g.i0 = (int)(r % tM) * kTile;
-    g.j0 = (int)j * kTile;
-  } else {
-    const long long per_b = (long long)tM * tN;
-    const long long r = t % per_b;
-    g.b = (int)(t / per_b);
-    g.i0 = (int)(r / tN) * kTile;
-    g.j0 = (int)(r % tN) * kTile;
+// batches slowest, then rows, then columns.  The position is kept as the digits of the tile number
+// in that order and the grid is added digit by digit: no division per tile.
+struct TileWalk {
+  long long t, total;
+  int d0, d1, d2, r0, r1, s0, s1, s2;   // digits (d0 fastest), radices, the grid's digits
+  bool b_outer;
+  __device__ __forceinline__ TileWalk(const GemmTcArgs &a) {
+    const int tM = (a.M + kTile - 1) / kTile, tN = (a.Ncols + kTile - 1) / kTile;
+    b_outer = !(a.batchB_shared && !a.idxB);
+    r0 = b_outer ? tN : tM;
+    r1 = b_outer ? tM : a.batch;
+    total = (long long)tM * tN * a.batch;
+    t = blockIdx.x;
+    const unsigned per2 = (unsigned)min((long long)r0 * r1, 0x7fffffffll);   // (a grid never reaches a larger one)
+    split(blockIdx.x, per2, d0, d1, d2);
+    split(gridDim.x, per2, s0, s1, s2);
   }
-  return g;
+  __device__ __forceinline__ void split(unsigned x, unsigned per2, int &e0, int &e1, int &e2) const {
+    e2 = (int)(x / per2);
+    x -= (unsigned)e2 * per2;
+    e1 = (int)(x / (unsigned)r0);
+    e0 = (int)(x - (unsigned)e1 * (unsigned)r0);
+  }
+  __device__ __forceinline__ bool valid() const { return t < total; }
+  __device__ __forceinline__ void next() {
+    t += gridDim.x;
+    d0 += s0;
+    d1 += s1;
+    d2 += s2;
+    if (d0 >= r0) { d0 -= r0; ++d1; }
+    if (d1 >= r1) { d1 -= r1; ++d2; }
+  }
+  __device__ __forceinline__ int b() const { return b_outer ? d2 : d1; }
+  __device__ __forceinline__ int i0() const { return (b_outer ? d1 : d0) * kTile; }
+  __device__ __forceinline__ int j0() const { return (b_outer ? d0 : d2) * kTile; }
+};
+// batch coordinates of the operands of the walk's tile
+struct TileZ {
+  int a, b;
+};
+__device__ __forceinline__ TileZ tile_z(const GemmTcArgs &a, const TileWalk &w) {
+  TileZ z{0, 0};
+  if (w.valid()) {
+    z.a = a.idxA ? a.idxA[w.b()] : (a.batchA_shared ? 0 : w.b());
+    z.b = a.idxB ? a.idxB[w.b()] : (a.batchB_shared ? 0 : w.b());
+  }
+  return z;
 }
 
-// kStoreF32 scale of tile t for epilogue thread e: e < 128 the column scale of tile column e,
-// else alpha times the row scale of tile row e - 128
-__device__ __forceinline__ float f32_tile_scale(const GemmTcArgs &a, long long t, int e, int tM, int tN) {
-  const GemmTile g = gemm_tile(a, t, tM, tN);
-  const int b = g.b;
-  if (e < kTile) {
-    const int col = g.j0 + e;
-    if (!a.col_scale || col >= a.Ncols) return 1.f;
-    const int zb = a.idxB ? a.idxB[b] : (a.batchB_shared ? 0 : b);
-    return a.col_scale[zb * a.cs_b + col];
+// kStoreF32 scales of the walk's tile for one epilogue warp (32 rows from r0, 64 columns from
+// c0): alpha times the scale of this lane's row, and the scales of columns lane and lane + 32
+struct TileScales {
+  float row, col[2];
+};
+__device__ __forceinline__ TileScales f32_tile_scales(const GemmTcArgs &a, const TileWalk &w, const TileZ &z, int r0,
+                                                      int c0, int lane) {
+  TileScales s{1.f, {1.f, 1.f}};
+  if (!w.valid()) return s;
+  const int row = w.i0() + r0 + lane;
+  if (a.row_scale && row < a.M) s.row = a.row_scale[z.a * a.rs_b + row];
+  if (a.col_scale) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int col = w.j0() + c0 + lane + 32 * k;
+      if (col < a.Ncols) s.col[k] = a.col_scale[z.b * a.cs_b + col];
+    }
   }
-  const int row = g.i0 + (e - kTile);
-  if (!a.row_scale || row >= a.M) return a.alpha;
-  const int za = a.idxA ? a.idxA[b] : (a.batchA_shared ? 0 : b);
-  return a.alpha * a.row_scale[za * a.rs_b + row];
+  return s;
 }
 
 __device__ __forceinline__ uint32_t pack2(__half a, __half b) {
@@ -1094,9 +1135,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   uint8_t *stage_out = smem + kGStages * kStageBytes;
   Barriers *bar = reinterpret_cast<Barriers *>(stage_out + kStageOut);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int tM = (a.M + kTile - 1) / kTile, tN = (a.Ncols + kTile - 1) / kTile;
-  const long long per_b = (long long)tM * tN;
-  const long long total = per_b * a.batch;
   const int nk = a.Kp / kChunk;
   const int kv = (a.K > 0 && a.K < a.Kp) ? a.K : a.Kp;   // valid K (the rest is zero padding)
 
@@ -1120,22 +1158,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     if (lane == 0) {
       long long it = 0, tt = 0;
       tc::RingPhases ring;
-      for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x, ++tt) {
+      // one A chunk for every tile of the launch stays where the stages' first fills put it
+      const bool fixed_a = nk == 1 && a.M <= kTile && a.batchA_shared && !a.idxA;
+      const uint32_t bytes_a = 2u * a.rows_a * 128, bytes_b = 2u * a.rows_b * 128;
+      TileWalk w(a), wn = w;   // the indexes of the next tile are loaded one tile ahead
+      TileZ zn = tile_z(a, w);
+      for (; w.valid() && !*abort; w.next(), ++tt) {
         const int q = (int)(tt & 1);   // issuer of this tile
-        const GemmTile gt = gemm_tile(a, t, tM, tN);
-        const int b = gt.b, i0 = gt.i0, j0 = gt.j0;
-        const int za = a.idxA ? a.idxA[b] : (a.batchA_shared ? 0 : b);
-        const int zb = a.idxB ? a.idxB[b] : (a.batchB_shared ? 0 : b);
+        const int i0 = w.i0(), j0 = w.j0(), za = zn.a, zb = zn.b;
+        wn.next();
+        zn = tile_z(a, wn);
         for (int kc = 0; kc < nk; ++kc, ++it) {
           const int s = (int)(it % kGStages);
           const uint32_t ph = (uint32_t)((it / kGStages) & 1);
           if (!tc::mbar_wait(&bar->empty[s], ph ^ 1u, a.spin_limit, abort, a.status, 1)) break;
           uint64_t *fb = &bar->full[q][s];
           ring.take(q, s);
-          tc::mbar_arrive_expect_tx(fb, kStageBytes);
+          const bool load_a = !fixed_a || it < kGStages;
+          tc::mbar_arrive_expect_tx(fb, (load_a ? bytes_a : 0u) + bytes_b);
           const int x = kc * kChunk;
-          tc::tma_load_3d(stage_ptr(smem, s, 0), &tmA_hi, fb, x, i0, za);
-          tc::tma_load_3d(stage_ptr(smem, s, 1), &tmA_lo, fb, x, i0, za);
+          if (load_a) {
+            tc::tma_load_3d(stage_ptr(smem, s, 0), &tmA_hi, fb, x, i0, za);
+            tc::tma_load_3d(stage_ptr(smem, s, 1), &tmA_lo, fb, x, i0, za);
+          }
           tc::tma_load_3d(stage_ptr(smem, s, 2), &tmB_hi, fb, x, j0, zb);
           tc::tma_load_3d(stage_ptr(smem, s, 3), &tmB_lo, fb, x, j0, zb);
         }
@@ -1148,7 +1193,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       long long it = 0, acc_it = 0;
       tc::RingPhases ring;   // this issuer's phases on its set, full[my][.]
       bool ok = true;
-      for (long long t = blockIdx.x; t < total && ok && !*abort; t += gridDim.x, ++acc_it) {
+      for (TileWalk w(a); w.valid() && ok && !*abort; w.next(), ++acc_it) {
         if ((acc_it & 1) != my) {   // the other issuer's tile
           it += nk;
           continue;
@@ -1158,13 +1203,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         ok = tc::mbar_wait(&bar->acc_empty[buf], aph ^ 1u, a.spin_limit, abort, a.status, 2);
         if (!ok) break;
         tc::tc_fence_after();
+        // an FP32 output reads only the columns that it has
+        const uint32_t idesc = a.mode == kStoreF32 ? idesc_cols(w.j0(), a.Ncols) : kIdesc;
         const uint32_t acc = tmem + buf * 128;
         for (int kc = 0; kc < nk; ++kc, ++it) {
           const int s = (int)(it % kGStages);
           ok = tc::mbar_wait(&bar->full[my][s], ring.take((int)my, s), a.spin_limit, abort, a.status, 4);
           if (!ok) break;
           tc::tc_fence_after();
-          issue_chunk(acc, stage_ptr(smem, s, 0), kc == 0, chunk_steps(kc, kv));
+          issue_chunk(acc, stage_ptr(smem, s, 0), kc == 0, chunk_steps(kc, kv), idesc);
           tc::mma_commit(&bar->empty[s]);
         }
         if (ok) tc::mma_commit(&bar->acc_full[buf]);
@@ -1177,74 +1224,82 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int q = warp & 3;
     const int row = q * 32 + lane;          // tile row = TMEM lane
     const int h = (warp - 2) >> 2;          // 64-column half of the tile
-    const bool storer = (warp == 2 && lane == 0);
+    uint8_t *own = stage_out + (size_t)(warp - 2) * 8192;   // this warp's part: two boxes of 4 KB
     __shared__ float red[8];
-    __shared__ __align__(16) float s_sc[2 * kTile];   // kStoreF32: column scales, then alpha x row scales
-    const int ep = (warp - 2) * 32 + lane;
-    // the scales of the next tile are loaded one tile ahead (their latency hides behind this one)
-    float pre = (a.mode == kStoreF32 && blockIdx.x < total) ? f32_tile_scale(a, blockIdx.x, ep, tM, tN) : 0.f;
+    __shared__ __align__(16) float s_cs[8][64];   // kStoreF32: the column scales of each warp
+    // The scales of the next tile are loaded one tile ahead and its operands' batch indexes two
+    // tiles ahead (their latencies hide behind those tiles: with the index and the scale loaded
+    // one after the other a third of the kernel was this wait).
+    const bool f32 = a.mode == kStoreF32;
+    TileWalk w(a), w1 = w;
+    w1.next();
+    TileScales pre{};
+    TileZ z1{};
+    if (f32) {
+      pre = f32_tile_scales(a, w, tile_z(a, w), q * 32, h * 64, lane);
+      z1 = tile_z(a, w1);
+    }
     long long acc_it = 0;
-    for (long long t = blockIdx.x; t < total; t += gridDim.x, ++acc_it) {
-      const GemmTile gt = gemm_tile(a, t, tM, tN);
-      const int b = gt.b, i0 = gt.i0, j0 = gt.j0;
+    for (; w.valid(); w.next(), ++acc_it) {
+      const int b = w.b(), i0 = w.i0(), j0 = w.j0();
       const int buf = (int)(acc_it & 1);
       const uint32_t aph = (uint32_t)((acc_it >> 1) & 1);
       const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
-      if (!epi_all(got && !*abort)) break;
+      // only the group maxima need the other warps: there they go on together or not at all
+      if (a.mode == kStoreSplitGroup ? !epi_all(got && !*abort) : !__all_sync(0xffffffffu, got && !*abort)) break;
       tc::tc_fence_after();
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 128 + h * 64;
       const bool row_ok = (i0 + row) < a.M;
+      // a warp whose 32 rows or 64 columns lie outside the output has nothing to read or store
+      const bool live = i0 + q * 32 < a.M && j0 + h * 64 < a.Ncols;
       if (a.mode == kStoreF32) {
-        // scaled FP32 tile in four 128-byte-swizzled boxes of 128 rows x 32 columns, written
-        // (or added, in accumulate mode) by TMA tensor stores; rows >= M and columns >= Ncols
-        // fall outside the tensor map and are not written
-        if (storer) bulk_wait_read();   // the previous tile's stores have read the staging boxes
-        epi_sync();
-        s_sc[ep] = pre;
-        epi_sync();
-        if (t + gridDim.x < total) pre = f32_tile_scale(a, t + gridDim.x, ep, tM, tN);
-        const float rsc = s_sc[kTile + row];
-        float *tile = reinterpret_cast<float *>(stage_out);
-        // a warp whose 32 rows or 64 columns lie outside the output has nothing to read or stage
-        // (the stores clip them): 3 of 4 warps of a product with M <= 32
-        const bool live = i0 + q * 32 < a.M && j0 + h * 64 < a.Ncols;
+        // scaled FP32 in 128-byte-swizzled boxes of 32 rows x 32 columns, written (or added, in
+        // accumulate mode) by TMA tensor stores; rows >= M and columns >= Ncols fall outside the
+        // tensor map and are not written
+        const float rsc = a.alpha * pre.row;
+        if (live) {
+          s_cs[warp - 2][lane] = pre.col[0];
+          s_cs[warp - 2][lane + 32] = pre.col[1];
+          __syncwarp();
+        }
+        pre = f32_tile_scales(a, w1, z1, q * 32, h * 64, lane);
+        w1.next();
+        z1 = tile_z(a, w1);
         if (!live) {
           tc::tc_fence_before();
           tc::mbar_arrive(&bar->acc_empty[buf]);
+          continue;
         }
+        float v[2][32];
+        tc::tmem_ld_32x32b_x32(base, v[0]);
+        tc::tmem_ld_32x32b_x32(base + 32, v[1]);
+        tc::tmem_ld_wait();
+        tc::tc_fence_before();
+        tc::mbar_arrive(&bar->acc_empty[buf]);
 #pragma unroll
-        for (int c = 0; live && c < 64; c += 32) {
-          float v[32];
-          tc::tmem_ld_32x32b_x32(base + c, v);
-          tc::tmem_ld_wait();
-          if (c == 32) {
-            tc::tc_fence_before();
-            tc::mbar_arrive(&bar->acc_empty[buf]);
-          }
-          const int col = h * 64 + c;    // tile column of v[0]; box col / 32 holds v[0..31]
-          float *box = tile + (col / 32) * (kTile * 32) + row * 32;
+        for (int c = 0; c < 2; ++c) {   // two boxes in turn: the store of one runs while the other fills
+          if (lane == 0) bulk_wait_read<1>();
+          __syncwarp();
+          float *box = reinterpret_cast<float *>(own + c * 4096) + lane * 32;
 #pragma unroll
           for (int t4 = 0; t4 < 8; ++t4) {
-            const float4 cs = *reinterpret_cast<const float4 *>(&s_sc[col + 4 * t4]);
-            *reinterpret_cast<float4 *>(box + ((t4 ^ (row & 7)) * 4)) =
-                make_float4(v[4 * t4] * (rsc * cs.x), v[4 * t4 + 1] * (rsc * cs.y), v[4 * t4 + 2] * (rsc * cs.z),
-                            v[4 * t4 + 3] * (rsc * cs.w));
+            const float4 cs = *reinterpret_cast<const float4 *>(&s_cs[warp - 2][c * 32 + 4 * t4]);
+            *reinterpret_cast<float4 *>(box + ((t4 ^ (lane & 7)) * 4)) =
+                make_float4(v[c][4 * t4] * (rsc * cs.x), v[c][4 * t4 + 1] * (rsc * cs.y), v[c][4 * t4 + 2] * (rsc * cs.z),
+                            v[c][4 * t4 + 3] * (rsc * cs.w));
           }
-        }
-        fence_proxy_async_smem();
-        epi_sync();
-        if (storer) {
-#pragma unroll
-          for (int bx = 0; bx < 4; ++bx) {
-            const int x = j0 + 32 * bx;
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            const int x = j0 + h * 64 + 32 * c;
             if (x < a.Ncols) {
               if (a.accumulate)
-                tma_reduce_add_3d(&tmC_hi, stage_out + (size_t)bx * (kTile * 128), x, i0, b);
+                tma_reduce_add_3d(&tmC_hi, own + c * 4096, x, i0 + q * 32, b);
               else
-                tma_store_3d(&tmC_hi, stage_out + (size_t)bx * (kTile * 128), x, i0, b);
+                tma_store_3d(&tmC_hi, own + c * 4096, x, i0 + q * 32, b);
             }
+            bulk_commit();   // (an empty group where the box lies outside: the boxes keep alternating)
           }
-          bulk_commit();
         }
         continue;
       }
@@ -1280,59 +1335,47 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           if (grp < a.n_groups) a.group_scale[(long long)b * a.n_groups + grp] = sc;
         }
       }
-      // the previous tile's TMA stores must have read the staging buffer
-      if (storer) bulk_wait_read();
-      epi_sync();
-      // split into FP16 pairs, written to the 128-byte-swizzled staging tile of this half
-      uint8_t *hi_tile = stage_out + (size_t)(0 * 2 + h) * (kTile * 128);
-      uint8_t *lo_tile = stage_out + (size_t)(1 * 2 + h) * (kTile * 128);
-      const bool live = i0 + q * 32 < a.M;   // as above
       if (!live) {
         tc::tc_fence_before();
         tc::mbar_arrive(&bar->acc_empty[buf]);
+        continue;
       }
+      // split into FP16 pairs: a 128-byte-swizzled box of 32 rows x 64 columns each for hi and lo
+      float v[2][32];
+      tc::tmem_ld_32x32b_x32(base, v[0]);
+      tc::tmem_ld_32x32b_x32(base + 32, v[1]);
+      tc::tmem_ld_wait();
+      tc::tc_fence_before();
+      tc::mbar_arrive(&bar->acc_empty[buf]);
+      if (lane == 0) bulk_wait_read<0>();   // the previous tile's stores have read the boxes
+      __syncwarp();
 #pragma unroll
-      for (int c = 0; live && c < 64; c += 32) {
-        float v[32];
-        tc::tmem_ld_32x32b_x32(base + c, v);
-        tc::tmem_ld_wait();
-        if (c == 32) {  // this half of the accumulator is read: hand it back
-          tc::tc_fence_before();
-          tc::mbar_arrive(&bar->acc_empty[buf]);
+      for (int t16 = 0; t16 < 8; ++t16) {
+        uint32_t ph[4], pl[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int jj = (t16 & 3) * 8 + e * 2;
+          __half h0, l0, h1, l1;
+          tc::split_f16(v[t16 >> 2][jj] * sc, h0, l0);
+          tc::split_f16(v[t16 >> 2][jj + 1] * sc, h1, l1);
+          ph[e] = pack2(h0, h1);
+          pl[e] = pack2(l0, l1);
         }
-#pragma unroll
-        for (int t16 = 0; t16 < 4; ++t16) {
-          uint32_t ph[4], pl[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int jj = t16 * 8 + e * 2;
-            __half h0, l0, h1, l1;
-            tc::split_f16(v[jj] * sc, h0, l0);
-            tc::split_f16(v[jj + 1] * sc, h1, l1);
-            ph[e] = pack2(h0, h1);
-            pl[e] = pack2(l0, l1);
-          }
-          const int chunk = (c / 8 + t16) ^ (row & 7);
-          *reinterpret_cast<uint4 *>(hi_tile + row * 128 + chunk * 16) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-          *reinterpret_cast<uint4 *>(lo_tile + row * 128 + chunk * 16) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
-        }
+        const int chunk = t16 ^ (lane & 7);
+        *reinterpret_cast<uint4 *>(own + lane * 128 + chunk * 16) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
+        *reinterpret_cast<uint4 *>(own + 4096 + lane * 128 + chunk * 16) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
       }
       fence_proxy_async_smem();
-      epi_sync();
-      if (storer) {
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          const int col = j0 + hh * 64;
-          if (col < a.Ncols) {
-            const int grp = col / a.group, x = col % a.group;
-            tma_store_4d(&tmC_hi, stage_out + (size_t)(0 * 2 + hh) * (kTile * 128), x, grp, i0, b);
-            tma_store_4d(&tmC_lo, stage_out + (size_t)(1 * 2 + hh) * (kTile * 128), x, grp, i0, b);
-          }
-        }
+      __syncwarp();
+      if (lane == 0) {
+        const int col = j0 + h * 64;
+        const int grp = col / a.group, x = col % a.group;
+        tma_store_4d(&tmC_hi, own, x, grp, i0 + q * 32, b);
+        tma_store_4d(&tmC_lo, own + 4096, x, grp, i0 + q * 32, b);
         bulk_commit();
       }
     }
-    if (storer) bulk_wait_all();
+    if (lane == 0) bulk_wait_all();
   }
   __syncthreads();
   if (warp == 1) {
@@ -1670,7 +1713,7 @@ bool make_tmap_f16_store4d(CUtensorMap *map, const void *base, uint64_t group, u
   // element (x, grp, row, b) at ((b * rows + row) * n_groups + grp) * group + x
   cuuint64_t dims[4] = {group, n_groups, rows, batch};
   cuuint64_t strides[3] = {group * 2, group * n_groups * 2, group * n_groups * rows * 2};
-  cuuint32_t box[4] = {64, 1, 128, 1};
+  cuuint32_t box[4] = {64, 1, 32, 1};   // the rows of one epilogue warp
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
@@ -1696,10 +1739,11 @@ bool make_tmap_f32_store3d(CUtensorMap *map, const void *base, uint64_t cols, ui
     }
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  // element (x, row, b) at b * batch_stride + row * ld + x; box 32 columns (128 B) x 128 rows
+  // element (x, row, b) at b * batch_stride + row * ld + x; box 32 columns (128 B) x the 32 rows of
+  // one epilogue warp
   cuuint64_t dims[3] = {cols, rows, batch};
   cuuint64_t strides[2] = {ld * 4, batch_stride * 4};
-  cuuint32_t box[3] = {32, 128, 1};
+  cuuint32_t box[3] = {32, 32, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(base), dims, strides, box, estr,
                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,

@@ -50,6 +50,7 @@ struct GemmTcArgs {
   int M = 0, Ncols = 0, Kp = 0, batch = 1;
   int K = 0;   // valid K (operand columns >= K are zero; MMAs stop there); 0 = Kp
   int batchA_shared = 0, batchB_shared = 0;
+  int rows_a = 128, rows_b = 128;   // rows of the operand maps' boxes (a multiple of 8; less for small M, Ncols)
   int mode = kStoreSplit;
   const float *out_scale = nullptr;   // kStoreSplit: one power of two per batch
   // kStoreSplitGroup: columns form groups of `group` (a multiple of 64) whose rows all lie
