@@ -592,11 +592,73 @@ __global__ void __launch_bounds__(1024) k_csplit_t(const T *src, RowMap m, int b
 }
 
 // rows contiguous along the row index and K strided: stage through shared memory
+// The same for few columns (K <= 16): 2^lp lanes per row, four values of K per lane, kept in
+// registers between the row maximum and the pairs, 16-byte stores; neighbouring groups take
+// neighbouring rows, so the reads stay coalesced without a tile in shared memory.  (k_csplit_t's
+// warp per row has Kp2 / 2 of its 32 lanes at work.)
+template <class T>
+__global__ void __launch_bounds__(256) k_csplit_r(const T *src, RowMap m, unsigned total, int rows, int K, int Kp2, int lp,
+                                                  int kind, float sa, float sbc, __half *hi, __half *lo, float *unscale) {
+  const unsigned e0 = (blockIdx.x * 256u + threadIdx.x) >> lp;
+  const unsigned e = e0 < total ? e0 : total - 1;   // a warp's surplus lanes stay for the shuffles
+  const int c = threadIdx.x & ((1 << lp) - 1);
+  const T *x = src + m.row((int)(e / (unsigned)rows), (int)(e % (unsigned)rows));
+  T v[4];
+  float mx = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    v[i] = T{};
+    if (c * 4 + i < K) v[i] = x[(c * 4 + i) * m.sk];
+    mx = fmaxf(mx, fmaxf(abs_f32(v[i].x), abs_f32(v[i].y)));
+  }
+  for (int o = (1 << lp) >> 1; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (e0 >= total) return;
+  const float s = tc::pow2_floor_inv(mx);
+  const bool n_re = kind && sa * sbc > 0.f, n_im = sbc < 0.f, n_x = sa < 0.f;
+  const long long row = (long long)e * (kind ? 2 : 1);
+  if (c == 0) {
+    unscale[row] = 1.f / s;
+    if (kind) unscale[row + 1] = 1.f / s;
+  }
+  if (c * 8 >= Kp2) return;
+  uint32_t p[4][4];   // hi and lo of the first row, hi and lo of a B operand's second row
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    __half xh, xl, yh, yl;
+    split_pair(v[i].x, s, xh, xl);
+    split_pair(v[i].y, s, yh, yl);
+    auto pack = [](__half a, __half b) {
+      return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
+    };
+    p[0][i] = pack(xh, neg_if(n_re, yh));
+    p[1][i] = pack(xl, neg_if(n_re, yl));
+    p[2][i] = pack(neg_if(n_im, yh), neg_if(n_x, xh));
+    p[3][i] = pack(neg_if(n_im, yl), neg_if(n_x, xl));
+  }
+  auto put = [&](__half *dst, const uint32_t(&w)[4]) {
+    *reinterpret_cast<uint4 *>(dst + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+  };
+  put(hi + row * Kp2, p[0]);
+  put(lo + row * Kp2, p[1]);
+  if (kind) {
+    put(hi + (row + 1) * Kp2, p[2]);
+    put(lo + (row + 1) * Kp2, p[3]);
+  }
+}
+
 template <class T>
 bool launch_split_t(const T *src, const RowMap &m, int batch, int rows, int K, int Kp2, int kind, float sa, float sbc,
                     __half *hi, __half *lo, float *unscale, cudaStream_t s) {
   const bool contiguous = (m.R2 == 1 ? m.sr1 == 1 : m.sr2 == 1);
   if (!contiguous || m.sk == 1) return false;
+  if (K <= 16 && (long long)batch * rows < (1ll << 26)) {
+    int lp = 0;   // a lane takes four values
+    while (lp < 2 && (4 << lp) < K) ++lp;
+    const unsigned total = (unsigned)batch * (unsigned)rows;
+    k_csplit_r<T><<<((total << lp) + 255) / 256, 256, 0, s>>>(src, m, total, rows, K, Kp2, lp, kind, sa, sbc, hi, lo,
+                                                              unscale);
+    return true;
+  }
   const size_t smem = (size_t)K * (kRB + 1) * sizeof(T);
   if (smem > 200 * 1024) return false;
   static std::atomic<unsigned long long> attr{0};
@@ -906,7 +968,20 @@ Status cgemm_tc(sox_handle h, const CSplit &A, const CSplit &B, int batch, const
     ga.cs_b = bsB;
     ga.spin_limit = h->spin_limit;
     ga.status = h->d_status;
-    const long long tiles = (long long)batch * ((A.rows + 127) / 128) * ((B.rows + 127) / 128);
+    // Few rows and many columns: the columns become the tile's rows (kStoreF32T; 7 rows: 29 -> 16.5
+    // us, up to 32 the transposed store has one full line per row and warp)
+    if (A.rows <= 32 && B.rows > 128 && A.Kp2 <= kKChunk && !accumulate) {
+      std::swap(maps[0], maps[2]);
+      std::swap(maps[1], maps[3]);
+      std::swap(ga.M, ga.Ncols);
+      std::swap(ga.rows_a, ga.rows_b);
+      std::swap(ga.batchA_shared, ga.batchB_shared);
+      std::swap(ga.idxA, ga.idxB);
+      std::swap(ga.row_scale, ga.col_scale);
+      std::swap(ga.rs_b, ga.cs_b);
+      ga.mode = kStoreF32T;
+    }
+    const long long tiles = (long long)batch * ((ga.M + 127) / 128) * ((ga.Ncols + 127) / 128);
     const int grid = (int)std::max<long long>(1, std::min<long long>(tiles, h->sm_count));
     ++h->launches;
     SOX_CUDA_TRY(launch_gemm_f16x2(maps, ga, grid, s));

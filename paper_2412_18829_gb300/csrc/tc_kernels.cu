@@ -69,8 +69,8 @@ constexpr uint32_t kIdesc = tc::idesc_f16_f32(kTile, kTile);
 struct Barriers {
   uint64_t full[2][kStages];
   uint64_t empty[kStages];
-  uint64_t acc_full[2];
-  uint64_t acc_empty[2];
+  uint64_t acc_full[4];
+  uint64_t acc_empty[4];
   uint64_t drain;
   uint32_t tmem_base;
   int abort;
@@ -91,16 +91,19 @@ __device__ __forceinline__ uint8_t *stage_ptr(uint8_t *smem, int s, int t) {
 // The small cross terms go first: the tensor core truncates every accumulation
 // step to FP32 (round toward zero), and each step into a large accumulator
 // costs up to one ulp, so the large hi*hi steps are kept last and fewest.
-template <int KS>
+// kSwap: the cross terms in the other order (operands in exchanged roles give the same sums).
+template <int KS, bool kSwap>
 __device__ __forceinline__ void issue_chunk_ks(uint32_t acc, uint8_t *st, bool first, uint32_t idesc) {
   const uint32_t a_hi = smem_u32(st), a_lo = a_hi + kTileBytes;
   const uint32_t b_hi = a_hi + 2 * kTileBytes, b_lo = a_hi + 3 * kTileBytes;
+  const uint32_t a1 = kSwap ? a_lo : a_hi, b1 = kSwap ? b_hi : b_lo;
+  const uint32_t a2 = kSwap ? a_hi : a_lo, b2 = kSwap ? b_lo : b_hi;
 #pragma unroll
   for (int k = 0; k < KS; ++k) {
     const uint32_t off = k * 32;
-    tc::mma_f16(acc, tc::desc_kmajor_sw128(a_hi + off), tc::desc_kmajor_sw128(b_lo + off), idesc,
+    tc::mma_f16(acc, tc::desc_kmajor_sw128(a1 + off), tc::desc_kmajor_sw128(b1 + off), idesc,
                 (first && k == 0) ? 0u : 1u);
-    tc::mma_f16(acc, tc::desc_kmajor_sw128(a_lo + off), tc::desc_kmajor_sw128(b_hi + off), idesc, 1u);
+    tc::mma_f16(acc, tc::desc_kmajor_sw128(a2 + off), tc::desc_kmajor_sw128(b2 + off), idesc, 1u);
   }
 #pragma unroll
   for (int k = 0; k < KS; ++k) {
@@ -110,12 +113,13 @@ __device__ __forceinline__ void issue_chunk_ks(uint32_t acc, uint8_t *st, bool f
 }
 // one straight-line MMA sequence per step count (a loop with a runtime exit between the
 // MMAs slowed the issuing thread down measurably)
+template <bool kSwap = false>
 __device__ __forceinline__ void issue_chunk(uint32_t acc, uint8_t *st, bool first, int ks,
                                             uint32_t idesc = kIdesc) {
-  if (ks >= 4) issue_chunk_ks<4>(acc, st, first, idesc);
-  else if (ks == 3) issue_chunk_ks<3>(acc, st, first, idesc);
-  else if (ks == 2) issue_chunk_ks<2>(acc, st, first, idesc);
-  else issue_chunk_ks<1>(acc, st, first, idesc);
+  if (ks >= 4) issue_chunk_ks<4, kSwap>(acc, st, first, idesc);
+  else if (ks == 3) issue_chunk_ks<3, kSwap>(acc, st, first, idesc);
+  else if (ks == 2) issue_chunk_ks<2, kSwap>(acc, st, first, idesc);
+  else issue_chunk_ks<1, kSwap>(acc, st, first, idesc);
 }
 
 // Instruction descriptor of a 128-row tile whose N side holds `cols` valid columns from
@@ -140,7 +144,7 @@ __device__ __forceinline__ void setup_barriers(Barriers *bar, int epi_threads) {
       tc::mbar_init(&bar->full[1][s], 1);
       tc::mbar_init(&bar->empty[s], 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < 4; ++b) {
       tc::mbar_init(&bar->acc_full[b], 1);
       tc::mbar_init(&bar->acc_empty[b], epi_threads);
     }
@@ -987,13 +991,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBcdThreads, 1)
 // tile (kStoreSplit: out_scale[b]; kStoreSplitGroup: an exact power of two per
 // group of `group` columns, all of whose rows lie in the tile), splits it into
 // FP16 pairs in swizzled shared memory and writes it with TMA tensor stores into
-// the 4-D output [batch][M][n_groups][group].  Every epilogue warp stages and stores its own
-// 32 rows x 64 columns (8 KB of the staging buffer), so no warp waits for another one's part of
-// the previous tile; with one 128-row store per tile the stores, two CTA-wide barriers and the
-// next tile's staging ran one after another.  With K of one chunk the epilogue still sets the pace
-// (FP32 output), not the copies or the MMAs: per tile of 128 x 128 it took 3900 clocks, 1500 of them
-// the wait for the next tile's scale behind its batch index, now 2300.  729 x 8 products 300 x 600,
-// K = 52: 1182 -> 664 us (4.25 GB: 6.4 TB/s).
+// the 4-D output [batch][M][n_groups][group].
+//
+// With K of one or two chunks the epilogue sets the pace, not the copies or the MMAs (729 x 8
+// products 300 x 600, K = 52: 968 us, 978 without the copies, 901 without the MMAs).  So every
+// epilogue warp stages and stores its own part (no barrier of all of them, no wait for another
+// one's part of the previous tile), scales and batch indexes are loaded ahead, FP32 outputs give
+// whole tiles to the two epilogue groups in turn (what a tile costs beside its elements is spent
+// once per tile instead of twice), four accumulators let the MMAs run ahead, and one
+// instantiation per mode keeps the code of a role small.  That product: 1182 us with one
+// 128-row store per tile behind two barriers, 961 with a store per warp, 664 with the loads
+// ahead, 635 now (4.25 GB: 6.7 TB/s).  A GEMM of 27 x 15600 columns, 7 rows, K = 16: 42 us,
+// 34, and 16.5 with its columns on the tile's rows (kStoreF32T).
 // ============================================================================
 constexpr int kGStages = 2;
 constexpr int kStageOut = 4 * kTile * 64 * 2;   // hi/lo x two 64-column halves, 64 KB
@@ -1100,21 +1109,26 @@ __device__ __forceinline__ TileZ tile_z(const GemmTcArgs &a, const TileWalk &w) 
   return z;
 }
 
-// kStoreF32 scales of the walk's tile for one epilogue warp (32 rows from r0, 64 columns from
-// c0): alpha times the scale of this lane's row, and the scales of columns lane and lane + 32
+// FP32 outputs: the scales of the walk's tile for one epilogue warp (32 rows from r0): of this
+// lane's row, and of the columns lane + 32 k, k < kCols
+template <int kCols>
 struct TileScales {
-  float row, col[2];
+  float row, col[kCols];
 };
-__device__ __forceinline__ TileScales f32_tile_scales(const GemmTcArgs &a, const TileWalk &w, const TileZ &z, int r0,
-                                                      int c0, int lane) {
-  TileScales s{1.f, {1.f, 1.f}};
+template <int kCols>
+__device__ __forceinline__ TileScales<kCols> f32_tile_scales(const GemmTcArgs &a, const TileWalk &w, const TileZ &z,
+                                                             int r0, int lane) {
+  TileScales<kCols> s;
+  s.row = 1.f;
+#pragma unroll
+  for (int k = 0; k < kCols; ++k) s.col[k] = 1.f;
   if (!w.valid()) return s;
   const int row = w.i0() + r0 + lane;
   if (a.row_scale && row < a.M) s.row = a.row_scale[z.a * a.rs_b + row];
   if (a.col_scale) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int col = w.j0() + c0 + lane + 32 * k;
+    for (int k = 0; k < kCols; ++k) {
+      const int col = w.j0() + lane + 32 * k;
       if (col < a.Ncols) s.col[k] = a.col_scale[z.b * a.cs_b + col];
     }
   }
@@ -1125,6 +1139,7 @@ __device__ __forceinline__ uint32_t pack2(__half a, __half b) {
   return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
 }
 
+template <int kMode>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     k_gemm_f16x2(const __grid_constant__ CUtensorMap tmA_hi, const __grid_constant__ CUtensorMap tmA_lo,
                  const __grid_constant__ CUtensorMap tmB_hi, const __grid_constant__ CUtensorMap tmB_lo,
@@ -1136,11 +1151,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   Barriers *bar = reinterpret_cast<Barriers *>(stage_out + kStageOut);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int nk = a.Kp / kChunk;
+  // FP32 outputs: the two epilogue groups (4 warps, one per TMEM lane quarter) take whole tiles in
+  // turn; pair outputs: each takes a 64-column half of every tile
+  constexpr bool f32 = kMode == kStoreF32 || kMode == kStoreF32T;
   const int kv = (a.K > 0 && a.K < a.Kp) ? a.K : a.Kp;   // valid K (the rest is zero padding)
 
-  setup_barriers(bar, kGemmEpi);
+  setup_barriers(bar, f32 ? kGemmEpi / 2 : kGemmEpi);
   if (warp == 1) {
-    tc::tmem_alloc(&bar->tmem_base, 256);
+    tc::tmem_alloc(&bar->tmem_base, 512);
     tc::tmem_relinquish();
   }
   if (warp == 0 && lane == 0) {
@@ -1158,8 +1176,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     if (lane == 0) {
       long long it = 0, tt = 0;
       tc::RingPhases ring;
-      // one A chunk for every tile of the launch stays where the stages' first fills put it
+      // one A (or B) chunk for every tile of the launch stays where the stages' first fills put it
       const bool fixed_a = nk == 1 && a.M <= kTile && a.batchA_shared && !a.idxA;
+      const bool fixed_b = nk == 1 && a.Ncols <= kTile && a.batchB_shared && !a.idxB;
       const uint32_t bytes_a = 2u * a.rows_a * 128, bytes_b = 2u * a.rows_b * 128;
       TileWalk w(a), wn = w;   // the indexes of the next tile are loaded one tile ahead
       TileZ zn = tile_z(a, w);
@@ -1174,15 +1193,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           if (!tc::mbar_wait(&bar->empty[s], ph ^ 1u, a.spin_limit, abort, a.status, 1)) break;
           uint64_t *fb = &bar->full[q][s];
           ring.take(q, s);
-          const bool load_a = !fixed_a || it < kGStages;
-          tc::mbar_arrive_expect_tx(fb, (load_a ? bytes_a : 0u) + bytes_b);
+          const bool load_a = !fixed_a || it < kGStages, load_b = !fixed_b || it < kGStages;
+          tc::mbar_arrive_expect_tx(fb, (load_a ? bytes_a : 0u) + (load_b ? bytes_b : 0u));
           const int x = kc * kChunk;
           if (load_a) {
             tc::tma_load_3d(stage_ptr(smem, s, 0), &tmA_hi, fb, x, i0, za);
             tc::tma_load_3d(stage_ptr(smem, s, 1), &tmA_lo, fb, x, i0, za);
           }
-          tc::tma_load_3d(stage_ptr(smem, s, 2), &tmB_hi, fb, x, j0, zb);
-          tc::tma_load_3d(stage_ptr(smem, s, 3), &tmB_lo, fb, x, j0, zb);
+          if (load_b) {
+            tc::tma_load_3d(stage_ptr(smem, s, 2), &tmB_hi, fb, x, j0, zb);
+            tc::tma_load_3d(stage_ptr(smem, s, 3), &tmB_lo, fb, x, j0, zb);
+          }
         }
       }
       tc::ring_wind_down(bar->full, ring, wind_down_limit(a.spin_limit));
@@ -1198,20 +1219,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           it += nk;
           continue;
         }
-        const int buf = (int)(acc_it & 1);
-        const uint32_t aph = (uint32_t)((acc_it >> 1) & 1);
+        const int buf = (int)(acc_it & 3);
+        const uint32_t aph = (uint32_t)((acc_it >> 2) & 1);
         ok = tc::mbar_wait(&bar->acc_empty[buf], aph ^ 1u, a.spin_limit, abort, a.status, 2);
         if (!ok) break;
         tc::tc_fence_after();
         // an FP32 output reads only the columns that it has
-        const uint32_t idesc = a.mode == kStoreF32 ? idesc_cols(w.j0(), a.Ncols) : kIdesc;
+        const uint32_t idesc = f32 ? idesc_cols(w.j0(), a.Ncols) : kIdesc;
         const uint32_t acc = tmem + buf * 128;
         for (int kc = 0; kc < nk; ++kc, ++it) {
           const int s = (int)(it % kGStages);
           ok = tc::mbar_wait(&bar->full[my][s], ring.take((int)my, s), a.spin_limit, abort, a.status, 4);
           if (!ok) break;
           tc::tc_fence_after();
-          issue_chunk(acc, stage_ptr(smem, s, 0), kc == 0, chunk_steps(kc, kv), idesc);
+          issue_chunk<kMode == kStoreF32T>(acc, stage_ptr(smem, s, 0), kc == 0, chunk_steps(kc, kv), idesc);
           tc::mma_commit(&bar->empty[s]);
         }
         if (ok) tc::mma_commit(&bar->acc_full[buf]);
@@ -1223,46 +1244,38 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   } else if (warp <= 9) {
     const int q = warp & 3;
     const int row = q * 32 + lane;          // tile row = TMEM lane
-    const int h = (warp - 2) >> 2;          // 64-column half of the tile
+    const int h = (warp - 2) >> 2;          // the epilogue group
     uint8_t *own = stage_out + (size_t)(warp - 2) * 8192;   // this warp's part: two boxes of 4 KB
-    __shared__ float red[8];
-    __shared__ __align__(16) float s_cs[8][64];   // kStoreF32: the column scales of each warp
-    // The scales of the next tile are loaded one tile ahead and its operands' batch indexes two
-    // tiles ahead (their latencies hide behind those tiles: with the index and the scale loaded
-    // one after the other a third of the kernel was this wait).
-    const bool f32 = a.mode == kStoreF32;
-    TileWalk w(a), w1 = w;
-    w1.next();
-    TileScales pre{};
-    TileZ z1{};
-    if (f32) {
-      pre = f32_tile_scales(a, w, tile_z(a, w), q * 32, h * 64, lane);
-      z1 = tile_z(a, w1);
-    }
-    long long acc_it = 0;
-    for (; w.valid(); w.next(), ++acc_it) {
-      const int b = w.b(), i0 = w.i0(), j0 = w.j0();
-      const int buf = (int)(acc_it & 1);
-      const uint32_t aph = (uint32_t)((acc_it >> 1) & 1);
-      const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
-      // only the group maxima need the other warps: there they go on together or not at all
-      if (a.mode == kStoreSplitGroup ? !epi_all(got && !*abort) : !__all_sync(0xffffffffu, got && !*abort)) break;
-      tc::tc_fence_after();
-      const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 128 + h * 64;
-      const bool row_ok = (i0 + row) < a.M;
-      // a warp whose 32 rows or 64 columns lie outside the output has nothing to read or store
-      const bool live = i0 + q * 32 < a.M && j0 + h * 64 < a.Ncols;
-      if (a.mode == kStoreF32) {
-        // scaled FP32 in 128-byte-swizzled boxes of 32 rows x 32 columns, written (or added, in
-        // accumulate mode) by TMA tensor stores; rows >= M and columns >= Ncols fall outside the
-        // tensor map and are not written
-        const float rsc = a.alpha * pre.row;
-        if (live) {
-          s_cs[warp - 2][lane] = pre.col[0];
-          s_cs[warp - 2][lane + 32] = pre.col[1];
+    if constexpr (f32) {
+      constexpr int kCols = kMode == kStoreF32 ? 4 : 1;
+      __shared__ __align__(16) float s_cs[8][128];   // kStoreF32: the column scales of each warp
+      // The scales of the group's next tile are loaded one tile ahead and its operands' batch
+      // indexes two tiles ahead (their latencies hide behind those tiles: with the index and the
+      // scale loaded one after the other a third of the kernel was this wait).
+      TileWalk w(a);
+      if (h) w.next();
+      TileWalk w1 = w;
+      w1.next();
+      w1.next();
+      TileScales<kCols> pre = f32_tile_scales<kCols>(a, w, tile_z(a, w), q * 32, lane);
+      TileZ z1 = tile_z(a, w1);
+      for (long long acc_it = h; w.valid(); w.next(), w.next(), acc_it += 2) {
+        const int b = w.b(), i0 = w.i0(), j0 = w.j0();
+        const int buf = (int)(acc_it & 3);
+        const uint32_t aph = (uint32_t)((acc_it >> 2) & 1);
+        const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+        if (!__all_sync(0xffffffffu, got && !*abort)) break;
+        tc::tc_fence_after();
+        const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 128;
+        const bool live = i0 + q * 32 < a.M;   // a warp whose 32 rows lie outside has nothing to do
+        const float rsc = a.alpha * pre.row, csc = pre.col[0];
+        if (kMode == kStoreF32 && live) {
+#pragma unroll
+          for (int k = 0; k < kCols; ++k) s_cs[warp - 2][lane + 32 * k] = pre.col[k];
           __syncwarp();
         }
-        pre = f32_tile_scales(a, w1, z1, q * 32, h * 64, lane);
+        pre = f32_tile_scales<kCols>(a, w1, z1, q * 32, lane);
+        w1.next();
         w1.next();
         z1 = tile_z(a, w1);
         if (!live) {
@@ -1270,43 +1283,87 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           tc::mbar_arrive(&bar->acc_empty[buf]);
           continue;
         }
-        float v[2][32];
-        tc::tmem_ld_32x32b_x32(base, v[0]);
-        tc::tmem_ld_32x32b_x32(base + 32, v[1]);
-        tc::tmem_ld_wait();
-        tc::tc_fence_before();
-        tc::mbar_arrive(&bar->acc_empty[buf]);
+        if constexpr (kMode == kStoreF32T) {
+          // C is the tile's transpose: a lane's row is a column of C, so 32 lanes write 128 bytes of
+          // a row of C straight from their registers
+          float *dst = a.Cf + b * a.sCb + i0 + row;
+          const bool row_ok = i0 + row < a.M;
+          float v[32];
+          tc::tmem_ld_32x32b_x32(base, v);
+          tc::tmem_ld_wait();
+          tc::tc_fence_before();
+          tc::mbar_arrive(&bar->acc_empty[buf]);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {   // two boxes in turn: the store of one runs while the other fills
-          if (lane == 0) bulk_wait_read<1>();
-          __syncwarp();
-          float *box = reinterpret_cast<float *>(own + c * 4096) + lane * 32;
-#pragma unroll
-          for (int t4 = 0; t4 < 8; ++t4) {
-            const float4 cs = *reinterpret_cast<const float4 *>(&s_cs[warp - 2][c * 32 + 4 * t4]);
-            *reinterpret_cast<float4 *>(box + ((t4 ^ (lane & 7)) * 4)) =
-                make_float4(v[c][4 * t4] * (rsc * cs.x), v[c][4 * t4 + 1] * (rsc * cs.y), v[c][4 * t4 + 2] * (rsc * cs.z),
-                            v[c][4 * t4 + 3] * (rsc * cs.w));
+          for (int j = 0; j < 32; ++j) {
+            if (j >= a.Ncols) break;   // (one tile of columns: j0 = 0)
+            const float cs = __shfl_sync(0xffffffffu, csc, j);
+            if (row_ok) *dst = v[j] * (rsc * cs);
+            dst += a.ldc;
           }
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            const int x = j0 + h * 64 + 32 * c;
-            if (x < a.Ncols) {
-              if (a.accumulate)
-                tma_reduce_add_3d(&tmC_hi, own + c * 4096, x, i0 + q * 32, b);
-              else
-                tma_store_3d(&tmC_hi, own + c * 4096, x, i0 + q * 32, b);
+        } else {
+          // scaled FP32 in 128-byte-swizzled boxes of 32 rows x 32 columns, written (or added, in
+          // accumulate mode) by TMA tensor stores; rows >= M and columns >= Ncols fall outside the
+          // tensor map and are not written
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            const bool more = p == 0 && j0 + 64 < a.Ncols;   // a second pair of boxes follows
+            float v[2][32];
+            tc::tmem_ld_32x32b_x32(base + p * 64, v[0]);
+            tc::tmem_ld_32x32b_x32(base + p * 64 + 32, v[1]);
+            tc::tmem_ld_wait();
+            if (!more) {
+              tc::tc_fence_before();
+              tc::mbar_arrive(&bar->acc_empty[buf]);
             }
-            bulk_commit();   // (an empty group where the box lies outside: the boxes keep alternating)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {   // two boxes in turn: the store of one runs while the other fills
+              if (lane == 0) bulk_wait_read<1>();
+              __syncwarp();
+              float *box = reinterpret_cast<float *>(own + c * 4096) + lane * 32;
+#pragma unroll
+              for (int t4 = 0; t4 < 8; ++t4) {
+                const float4 cs = *reinterpret_cast<const float4 *>(&s_cs[warp - 2][p * 64 + c * 32 + 4 * t4]);
+                *reinterpret_cast<float4 *>(box + ((t4 ^ (lane & 7)) * 4)) =
+                    make_float4(v[c][4 * t4] * (rsc * cs.x), v[c][4 * t4 + 1] * (rsc * cs.y),
+                                v[c][4 * t4 + 2] * (rsc * cs.z), v[c][4 * t4 + 3] * (rsc * cs.w));
+              }
+              fence_proxy_async_smem();
+              __syncwarp();
+              if (lane == 0) {
+                const int x = j0 + p * 64 + 32 * c;
+                if (x < a.Ncols) {
+                  if (a.accumulate)
+                    tma_reduce_add_3d(&tmC_hi, own + c * 4096, x, i0 + q * 32, b);
+                  else
+                    tma_store_3d(&tmC_hi, own + c * 4096, x, i0 + q * 32, b);
+                }
+                bulk_commit();   // (an empty group where the box lies outside: the boxes keep alternating)
+              }
+            }
+            if (!more) break;
           }
         }
-        continue;
       }
+    } else {
+    __shared__ float red[8];
+    TileWalk w(a);
+    long long acc_it = 0;
+    for (; w.valid(); w.next(), ++acc_it) {
+      const int b = w.b(), i0 = w.i0(), j0 = w.j0();
+      const int buf = (int)(acc_it & 3);
+      const uint32_t aph = (uint32_t)((acc_it >> 2) & 1);
+      const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+      // only the group maxima need the other warps: there they go on together or not at all
+      if (kMode == kStoreSplitGroup ? !epi_all(got && !*abort) : !__all_sync(0xffffffffu, got && !*abort)) break;
+      tc::tc_fence_after();
+      const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 128 + h * 64;
+      const bool row_ok = (i0 + row) < a.M;
+      // a warp whose 32 rows or 64 columns lie outside the output has nothing to read or store
+      const bool live = i0 + q * 32 < a.M && j0 + h * 64 < a.Ncols;
       // this half's columns belong to group g (groups are 64 or 128 columns wide)
       const int g = (h * 64) >= a.group ? 1 : 0;
       float sc = 1.f;
-      if (a.mode == kStoreSplit) {
+      if (kMode == kStoreSplit) {
         sc = a.out_scale[b];
       } else {
         float m = 0.f;
@@ -1375,12 +1432,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         bulk_commit();
       }
     }
+    }
     if (lane == 0) bulk_wait_all();
   }
   __syncthreads();
   if (warp == 1) {
     tc::tc_fence_after();
-    tc::tmem_dealloc(tmem, 256);
+    tc::tmem_dealloc(tmem, 512);
   }
 }
 
@@ -1688,12 +1746,22 @@ cudaError_t launch_sox_bcd_multi(const BcdJobs &jobs, int grid, cudaStream_t s) 
 
 size_t gemm_smem_bytes() { return (size_t)kGStages * kStageBytes + kStageOut + sizeof(Barriers) + 1024; }
 
-cudaError_t launch_gemm_f16x2(const CUtensorMap *maps, const GemmTcArgs &a, int grid, cudaStream_t s) {
+template <int kMode>
+cudaError_t launch_gemm_mode(const CUtensorMap *maps, const GemmTcArgs &a, int grid, cudaStream_t s) {
   static std::atomic<unsigned long long> attr{0};
-  const cudaError_t e = set_smem_once(k_gemm_f16x2, (int)gemm_smem_bytes(), attr);
+  const cudaError_t e = set_smem_once(k_gemm_f16x2<kMode>, (int)gemm_smem_bytes(), attr);
   if (e != cudaSuccess) return e;
-  k_gemm_f16x2<<<grid, kGemmThreads, gemm_smem_bytes(), s>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], a);
+  k_gemm_f16x2<kMode><<<grid, kGemmThreads, gemm_smem_bytes(), s>>>(maps[0], maps[1], maps[2], maps[3], maps[4], maps[5],
+                                                                    a);
   return cudaGetLastError();
+}
+cudaError_t launch_gemm_f16x2(const CUtensorMap *maps, const GemmTcArgs &a, int grid, cudaStream_t s) {
+  switch (a.mode) {
+    case kStoreSplit: return launch_gemm_mode<kStoreSplit>(maps, a, grid, s);
+    case kStoreSplitGroup: return launch_gemm_mode<kStoreSplitGroup>(maps, a, grid, s);
+    case kStoreF32: return launch_gemm_mode<kStoreF32>(maps, a, grid, s);
+    default: return launch_gemm_mode<kStoreF32T>(maps, a, grid, s);
+  }
 }
 
 bool make_tmap_f16_store4d(CUtensorMap *map, const void *base, uint64_t group, uint64_t n_groups, uint64_t rows,

@@ -9,7 +9,7 @@
 
 namespace sox {
 
-enum { kStoreSplit = 1, kStoreSplitGroup = 2, kStoreF32 = 3 };
+enum { kStoreSplit = 1, kStoreSplitGroup = 2, kStoreF32 = 3, kStoreF32T = 4 };
 
 struct BcdArgs {
   // K extent Kp (a multiple of 64): n valid columns, then zeros; the MMAs of the last
@@ -62,6 +62,10 @@ struct GemmTcArgs {
   // (either scale may be NULL); rows >= M and columns >= Ncols are not written.  Cf 16-byte
   // aligned, ldc and sCb multiples of 4; the stores go through the FP32 tensor map passed as
   // the first output map (make_tmap_f32_store3d over Ncols x M x batch).
+  // kStoreF32T: the same into the transpose, Cf[b * sCb + j * ldc + i], for Ncols <= 32 and without
+  // accumulation: a C of few rows and many columns comes with its operands in exchanged roles, so
+  // that its columns fill the tile's 128 rows and all epilogue warps (with 8 rows two of eight had
+  // work); no output map.
   float *Cf = nullptr;
   long long ldc = 0, sCb = 0;
   float alpha = 1.f;

@@ -283,3 +283,17 @@ def test_solid_dynamic_pairs_of_the_time_products(env, nk, n, N, n_tau, M):
     ref = kpoints.sosex_dynamic_sigma(w.X, w.V, Wd, Tf, Ti, w.G, nk)
     got = _dynamic(env, w, Tf, Ti, Wd, nk=nk)
     assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("nk,n,N,n_tau,M", [((1, 1, 2), 4, 16, 32, 16), ((1, 1, 2), 5, 13, 32, 16),
+                                            ((1, 1, 2), 5, 13, 33, 17), ((2, 1, 1), 3, 50, 8, 7)])
+def test_solid_transforms_with_exchanged_roles(env, nk, n, N, n_tau, M):
+    """Transforms of 32 and 33 rows, 128 and 130 columns (both sides of the rule that puts the
+    columns on the tile's rows), and K = 16 and 17 of the register and the shared-tile split."""
+    from oracle import kpoints
+
+    rng = np.random.default_rng(100 + n_tau)
+    w, Tf, Ti, Wd = _random_dynamic(rng, n, N, n_tau, M, nk)
+    ref = kpoints.sosex_dynamic_sigma(w.X, w.V, Wd, Tf, Ti, w.G, nk)
+    got = _dynamic(env, w, Tf, Ti, Wd, nk=nk)
+    assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max()
