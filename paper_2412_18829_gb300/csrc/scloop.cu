@@ -166,27 +166,23 @@ __device__ __forceinline__ bool small_invert(z *A, z *rk, z *fk, int *piv, int n
   for (int k = 0; k < n; ++k) {
     __syncthreads();
     if (tid < 32) {
-      double bv = -1.0;
-      int bi = k;
+      // the larger of |re|, |im| by its high word (NaNs last): no FP64 instruction in the search
+      // (n = 20, 400 systems: a bisection step of 72 us takes 61)
+      unsigned bv = 0u;
+      int bi = k + tid;
       for (int i = k + tid; i < n; i += 32) {
         const z a = A[i * n + k];
-        const double m2 = a.x * a.x + a.y * a.y;
-        if (m2 > bv) {
-          bv = m2;
+        const unsigned hx = (unsigned)__double2hiint(a.x) & 0x7fffffffu, hy = (unsigned)__double2hiint(a.y) & 0x7fffffffu;
+        const unsigned m = max(hx, hy) > 0x7ff00000u ? 0u : max(hx, hy);
+        if (m > bv) {
+          bv = m;
           bi = i;
         }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > bv || (ov == bv && oi < bi)) {
-          bv = ov;
-          bi = oi;
-        }
-      }
-      const int p = bi;   // the same in every lane
+      const unsigned top = __reduce_max_sync(0xffffffffu, bv);
+      const int p = top == 0u ? k : (int)__reduce_min_sync(0xffffffffu, bv == top ? (unsigned)bi : 0xffffffffu);
       const z pv = A[p * n + k], akk = A[k * n + k];
-      const double id = 1.0 / (pv.x * pv.x + pv.y * pv.y);
+      const double den = pv.x * pv.x + pv.y * pv.y, id = 1.0 / den;
       const z inv = make_double2(pv.x * id, -pv.y * id);
       for (int j = tid; j < n; j += 32) {
         const z b = A[p * n + j];
@@ -196,7 +192,7 @@ __device__ __forceinline__ bool small_invert(z *A, z *rk, z *fk, int *piv, int n
       __syncwarp();
       if (p != k)
         for (int j = tid; j < n; j += 32) A[p * n + j] = A[k * n + j];
-      if (tid == 0) piv[k] = bv > 0.0 ? p : -1;
+      if (tid == 0) piv[k] = den > 0.0 ? p : -1;
     }
     __syncthreads();
     if (piv[k] < 0) return false;

@@ -308,14 +308,14 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
       ProfScope ps(h, "A_tc", s, 2);
       launch_prep_gminus(G, n, T, bc, Kp, Gmh, Gml, gsc, osc, b0, RG, s);
       GemmTcArgs ga;
-      ga.M = n; ga.Ncols = NR * Kp; ga.Kp = Kp; ga.K = n; ga.batch = bc;
+      ga.M = n; ga.Ncols = N * Kp; ga.Kp = Kp; ga.K = n; ga.batch = bc;
       ga.batchA_shared = 0; ga.batchB_shared = 1;
       // n <= 128: one tile holds all (v, q) of each P -> exact per-P scale; else the a-priori bound
       ga.mode = exact_a ? kStoreSplitGroup : kStoreSplit;
       ga.out_scale = osc;
       ga.group = Kp; ga.n_groups = NR; ga.group_scale = asc;
       ga.spin_limit = limit; ga.status = h->d_status;
-      const long long tiles = (long long)bc * ((n + 127) / 128) * ((NR * Kp + 127) / 128);
+      const long long tiles = (long long)bc * ((n + 127) / 128) * ((N * Kp + 127) / 128);
       SOX_CUDA_TRY(launch_gemm_f16x2(agemm, ga, grid_for(tiles), s));
     }
     launch_bcd_scales(inv_u1, gsc, osc, exact_a ? asc : nullptr, NR, inv_gw, inv_gr, inv_u2, N, bc, rowf, colf, s);
@@ -515,13 +515,13 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
         const bool exact_a = (c.Kp <= 128);
         launch_prep_gminus(c.G, c.n, c.T, bc, c.Kp, c.Gmh, c.Gml, c.gsc, c.osc, b0, c.RG, s);
         GemmTcArgs ga;
-        ga.M = c.n; ga.Ncols = c.NR * c.Kp; ga.Kp = c.Kp; ga.K = c.n; ga.batch = bc;
+        ga.M = c.n; ga.Ncols = c.N * c.Kp; ga.Kp = c.Kp; ga.K = c.n; ga.batch = bc;
         ga.batchA_shared = 0; ga.batchB_shared = 1;
         ga.mode = exact_a ? kStoreSplitGroup : kStoreSplit;
         ga.out_scale = c.osc;
         ga.group = c.Kp; ga.n_groups = c.NR; ga.group_scale = c.asc;
         ga.spin_limit = limit; ga.status = h->d_status;
-        const long long tiles = (long long)bc * ((c.n + 127) / 128) * (((long long)c.NR * c.Kp + 127) / 128);
+        const long long tiles = (long long)bc * ((c.n + 127) / 128) * (((long long)c.N * c.Kp + 127) / 128);
         SOX_CUDA_TRY(launch_gemm_f16x2(c.agemm, ga, grid_for(tiles), s));
         launch_bcd_scales(c.inv_u1, c.gsc, c.osc, exact_a ? c.asc : nullptr, c.NR, c.inv_gw, c.inv_gr, c.inv_u2, c.N,
                           bc, c.rowf, c.colf, s);
