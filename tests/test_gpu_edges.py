@@ -297,3 +297,21 @@ def test_solid_transforms_with_exchanged_roles(env, nk, n, N, n_tau, M):
     ref = kpoints.sosex_dynamic_sigma(w.X, w.V, Wd, Tf, Ti, w.G, nk)
     got = _dynamic(env, w, Tf, Ti, Wd, nk=nk)
     assert np.abs(got - ref).max() <= 2e-6 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("nk", [(4, 1, 1), (1, 5, 1), (1, 3, 4), (2, 1, 3)])
+def test_w_dynamic_mesh_sides(env, nk):
+    """Mesh transforms by butterflies (sides of 2, 3, 4) and by the twiddle matrix, along every axis."""
+    from oracle import kpoints
+
+    torch, pkg, hs = env
+    n, N, n_tau, M = 3, 11, 6, 2
+    w = synth.solid(90, nk, n, N, n_tau, 20.0)
+    _, Tf, _ = synth.bosonic_transforms(w.tau, w.beta, M)
+    p = pkg.problem(n, N, n_tau, 1, w.beta, nk=nk, dtype=1)
+    G, X, V, F = to_dev(torch, *(np.asarray(a, dtype=complex) for a in (w.G, w.X, w.V, Tf)))
+    out = torch.full((w.n_k, 2 * M + 1, N, N), complex(float("nan"), 0.0), dtype=torch.complex128, device="cuda")
+    pkg.sox_w_dynamic(hs["fp64"], p, G, X, V, F, 2 * M + 1, out)
+    pkg.sox_check_device(hs["fp64"])
+    ref = kpoints.w_dynamic(w.V, kpoints.pi_omega(w.X, w.G[0], Tf, nk))
+    assert np.abs(out.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
