@@ -306,6 +306,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc::mbar_arrive(&bar->acc_empty[buf]);
       }
       if (!live) break;
+      if (a.row_scale) {
+        const int i = w.i0 + q * 32 + lane, j0 = w.j0 + h * 64 + lane;
+        const float rs = i < a.M ? a.row_scale[i] : 0.f;
+        const float c0 = j0 < a.Ncols ? a.col_scale[j0] : 0.f, c1 = j0 + 32 < a.Ncols ? a.col_scale[j0 + 32] : 0.f;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          sum[j] *= rs * __shfl_sync(0xffffffffu, c0, j);
+          sum[j + 32] *= rs * __shfl_sync(0xffffffffu, c1, j);
+        }
+      }
       if (a.absmax) {   // rows past M are sums of zeros; columns past Ncols hold no sums at all
         const int cols = a.Ncols - w.j0 - h * 64;
 #pragma unroll

@@ -45,6 +45,8 @@ struct GemmMnArgs {
   // optional: raised to max |C| over the call's outputs by atomicMax, as launch_absmax would
   // (ksplit 1 and no accumulation only: the epilogue then holds every output once)
   float *absmax = nullptr;
+  // optional (batch 1): C(i, j) also times row_scale[i] col_scale[j] (powers of two)
+  const float *row_scale = nullptr, *col_scale = nullptr;
   float alpha_host = 1.f;
   int accumulate = 0;           // reduce-add into C instead of storing
   long long spin_limit = 0;

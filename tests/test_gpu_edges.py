@@ -315,3 +315,19 @@ def test_w_dynamic_mesh_sides(env, nk):
     pkg.sox_check_device(hs["fp64"])
     ref = kpoints.w_dynamic(w.V, kpoints.pi_omega(w.X, w.G[0], Tf, nk))
     assert np.abs(out.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n,N", [(32, 127), (33, 128), (46, 129)])
+def test_split_adjoint_windows_of_k(env, n, N):
+    """K = n^2 of one window (1024), one and a little, two and a little: the products of the
+    adjoint's end in one launch that adds the windows in registers."""
+    from oracle import grid, phi
+    from test_gpu_phi import _grads_with
+
+    torch, pkg, hs = env
+    w = synth.molecule(120 + n, n, N, 3, 3.0)
+    wt = grid.clenshaw_curtis(w.n_tau, w.beta)
+    gX, gV = _grads_with(torch, pkg, hs["f16x2"], w, wt, [1.0])
+    _, _, rX, rV = phi.phi_and_grads(w.X[0], w.V[0], w.G[0, 0], wt)
+    assert np.abs(gX - rX).max() <= 2e-5 * np.abs(rX).max()
+    assert np.abs(gV - rV).max() <= 2e-5 * np.abs(rV).max()
