@@ -48,8 +48,11 @@ __global__ void __launch_bounds__(256) k_gg_max(const double *GWt, const double 
 }
 
 // The FP16 pairs of GG for one v, [j][(Q,u)] with rows of ld (the padding zero): formed and split
-// in one pass (GG itself never leaves the SM), scale as launch_split_tensor.  n = 120, N = 600,
-// 80 times: 36 us product + 20 us maximum + 63 us split before, 39 us here.
+// in one pass (GG itself never leaves the SM), scale as launch_split_tensor.  A warp per Q and
+// step; kVec: two u per lane (16-byte loads, packed stores; n even, so that every row of n is
+// aligned).  n = 120, N = 600, 80 times: 36 us product + 20 us maximum + 63 us split before, 39 us
+// with one u per lane, 27 us with two (92 MB).
+template <bool kVec>
 __global__ void __launch_bounds__(256) k_gg_split(const double *GWt, const double *GR, int T, int N, int n, int v,
                                                   long long ld, const float *mx, __half *hi, __half *lo,
                                                   float *scale_out) {
@@ -59,14 +62,26 @@ __global__ void __launch_bounds__(256) k_gg_split(const double *GWt, const doubl
   const int j = blockIdx.y, lane = threadIdx.x % 32, warp = threadIdx.x / 32;
   const double *w = GWt + j * Nn, *g = GR + (long long)(T - 1 - j) * Nn + v;
   __half *h = hi + j * ld, *l = lo + j * ld;
-  for (int Q = blockIdx.x * 8 + warp; Q < N; Q += gridDim.x * 8) {   // a warp per Q
-    const double gq = g[(long long)Q * n];
+#pragma unroll 2
+  for (int Q = blockIdx.x * 8 + warp; Q < N; Q += gridDim.x * 8) {
+    const double gq = -g[(long long)Q * n];
     const long long o = (long long)Q * n;
-    for (int u = lane; u < n; u += 32) {
-      __half a, b;
-      tc::split_f16_f64(-w[o + u] * gq, ks, a, b);
-      h[o + u] = a;
-      l[o + u] = b;
+    if constexpr (kVec) {
+      for (int u = 2 * lane; u < n; u += 64) {
+        const double2 x = *reinterpret_cast<const double2 *>(w + o + u);
+        __half a0, b0, a1, b1;
+        tc::split_f16_f64(x.x * gq, ks, a0, b0);
+        tc::split_f16_f64(x.y * gq, ks, a1, b1);
+        *reinterpret_cast<__half2 *>(h + o + u) = __halves2half2(a0, a1);
+        *reinterpret_cast<__half2 *>(l + o + u) = __halves2half2(b0, b1);
+      }
+    } else {
+      for (int u = lane; u < n; u += 32) {
+        __half a, b;
+        tc::split_f16_f64(w[o + u] * gq, ks, a, b);
+        h[o + u] = a;
+        l[o + u] = b;
+      }
     }
   }
   if (blockIdx.x == 0)
@@ -288,7 +303,7 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
       SOX_CUDA_TRY(cudaMemsetAsync(&sc->mx[kA], 0, sizeof(float), s));
       for (int v = v_lo; v < v_hi; ++v) {
         float *mx = mxv + (size_t)kMxV * v;
-        k_gg_split<<<dim3((unsigned)std::min((N + 7) / 8, 64), T), 256, 0, s>>>(
+        (n % 2 == 0 ? k_gg_split<true> : k_gg_split<false>)<<<dim3((unsigned)std::min((N + 7) / 8, 64), T), 256, 0, s>>>(
             GWt, GR, T, N, n, v, g.Nn8, mx, GGh, GGl, &sc->sc[kGG]);
         {  // GGw[(m,c)][(Q,u)] = sum_j conj(T_fwd)_c[m][j] GG[j][(Q,u)]
           GemmMnArgs a;

@@ -369,6 +369,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 // k < 8) of one row r = (r1, r0); the index divisions happen once per unit.
 constexpr int kUnitCols = 256;
 
+struct UnitPos {
+  long long r1, r0, c;   // row, and the unit's number along it
+};
+// (32-bit divisions wherever the count allows: with rows of 120 values the 64-bit ones cost about
+// as many instructions as the row)
+__device__ __forceinline__ UnitPos unit_pos(long long u, long long units, long long cpr, int rows0) {
+  if (units <= 0x7fffffffll) {
+    const unsigned r = (unsigned)u / (unsigned)cpr, r1 = r / (unsigned)rows0;
+    return {(long long)r1, (long long)(r - r1 * (unsigned)rows0), (long long)((unsigned)u - r * (unsigned)cpr)};
+  }
+  const long long r = u / cpr;
+  return {r / rows0, r % rows0, u % cpr};
+}
+
 // |x| as FP32 (an FP64 value rounds up to at most one FP32 ulp); FP32 sources stay on the
 // FP32 pipe (the FP64 rate is 1/64 of it)
 __device__ __forceinline__ float abs_f(float x) { return fabsf(x); }
@@ -395,9 +409,9 @@ __global__ void k_absmax(const T *src, long long ld0, int rows0, long long ld1, 
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   float m = 0.f;
   for (long long u = warp0; u < units; u += nwarps) {
-    const long long r = u / cpr;
-    const int c0 = (int)(u % cpr) * kUnitCols;
-    const long long r1 = r / rows0, r0 = r % rows0;
+    const UnitPos up = unit_pos(u, units, cpr, rows0);
+    const int c0 = (int)up.c * kUnitCols;
+    const long long r1 = up.r1, r0 = up.r0;
     const T *row = src + r1 * ld1 + r0 * ld0;
 #pragma unroll
     for (int k = 0; k < kUnitCols / 32; ++k) {
@@ -424,9 +438,9 @@ __global__ void k_split_tensor(const T *src, long long ld0, int rows0, long long
   const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long u = warp0; u < units; u += nwarps) {
-    const long long r = u / cpr;
-    const long long c0 = (u % cpr) * kUnitCols;
-    const long long r1 = r / rows0, r0 = r % rows0;
+    const UnitPos up = unit_pos(u, units, cpr, rows0);
+    const long long c0 = up.c * kUnitCols;
+    const long long r1 = up.r1, r0 = up.r0;
     const T *row = src + r1 * ld1 + r0 * ld0;
     __half *h = hi + r1 * ldo1 + r0 * ldo, *l = lo + r1 * ldo1 + r0 * ldo;
 #pragma unroll
@@ -456,9 +470,9 @@ __global__ void k_absmax_f32x2(const float *src, long long ld0, int rows0, long 
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   float m = 0.f;
   for (long long u = warp0; u < units; u += nwarps) {
-    const long long r = u / cpr;
-    const int c0 = (int)(u % cpr) * kUnitCols2;
-    const long long r1 = r / rows0, r0 = r % rows0;
+    const UnitPos up = unit_pos(u, units, cpr, rows0);
+    const int c0 = (int)up.c * kUnitCols2;
+    const long long r1 = up.r1, r0 = up.r0;
     const float *row = src + r1 * ld1 + r0 * ld0;
 #pragma unroll
     for (int k = 0; k < kUnitCols2 / 64; ++k) {
@@ -486,9 +500,9 @@ __global__ void k_split_f32x2(const float *src, long long ld0, int rows0, long l
   const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
   for (long long u = warp0; u < units; u += nwarps) {
-    const long long r = u / cpr;
-    const long long c0 = (u % cpr) * kUnitCols2;
-    const long long r1 = r / rows0, r0 = r % rows0;
+    const UnitPos up = unit_pos(u, units, cpr, rows0);
+    const long long c0 = up.c * kUnitCols2;
+    const long long r1 = up.r1, r0 = up.r0;
     const float *row = src + r1 * ld1 + r0 * ld0;
     __half *h = hi + r1 * ldo1 + r0 * ldo, *l = lo + r1 * ldo1 + r0 * ldo;
 #pragma unroll
@@ -573,6 +587,12 @@ void launch_absmax(const void *src, bool f32, long long ld0, int rows0, long lon
 void launch_split_tensor(const void *src, bool f32, long long ld0, int rows0, long long ld1, int rows1, long long ldc,
                          int cols, long long ldo, long long ldo1, float sign, const float *absmax,
                          const float *scale_in, __half *hi, __half *lo, float *scale_out, cudaStream_t s) {
+  // rows that follow one another on both sides are one long row (no row is too short for a unit)
+  if (ldc == 1 && rows0 > 1 && ld0 == cols && ldo == cols && (long long)cols * rows0 <= 0x7fffffffll) {
+    cols *= rows0;
+    ld0 = ldo = cols;
+    rows0 = 1;
+  }
   if (f32 && f32x2_ok(src, ld0, ld1, ldc) && (ldo % 2) == 0 && (ldo1 % 2) == 0 &&
       (reinterpret_cast<uintptr_t>(hi) % 4) == 0 && (reinterpret_cast<uintptr_t>(lo) % 4) == 0) {
     const int blocks = blocks_for_units((long long)rows1 * rows0 * ((ldo + kUnitCols2 - 1) / kUnitCols2));
