@@ -347,9 +347,10 @@ __device__ __forceinline__ float f32_abs(double x) {
 __device__ __forceinline__ int log2_of(float s) { return (int)((__float_as_uint(s) >> 23) & 0xffu) - 127; }
 
 // FP16 pair of x 2^k: h = RN16(RN32(x 2^k)), l = RN16(RN32(x 2^k - h)).  With f = RN32(x 2^k) and
-// the 29 bits g = x 2^k - f that FP32 drops, f - h is exact in FP32 and l = RN16(f - h + g): g
-// only decides where f - h lies half way between two FP16 numbers (its own rounding to FP32
-// could matter there for one value in 10^7, by one bit of l).
+// the 29 bits g = x 2^k - f that FP32 drops, f - h is exact in FP32 and l = RN16(RN32(f - h + g)).
+// g has up to 28 bits: it enters with its last four as a sticky bit, far below the rounding of
+// the sum, or rounded by itself where f = h.  (Rounded to FP32 in every case one value in 10^9 came
+// out a bit off, and one value of a long operand shows in the last digits of a whole output row.)
 __device__ __forceinline__ void split_f16_f64(double x, int k, __half &h, __half &l) {
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
   const int ef = (int)((hi >> 20) & 0x7ffu), e = ef + k - 1023;   // exponent of x 2^k
@@ -373,7 +374,9 @@ __device__ __forceinline__ void split_f16_f64(double x, int k, __half &h, __half
   h = __float2half_rn(f);
   // 2^(e - 52) with the sign of x
   const float unit = __uint_as_float(((uint32_t)(e - 52 + 127) << 23) | sgn);
-  l = __float2half_rn(fmaf((float)g, unit, f - __half2float(h)));
+  const float d = f - __half2float(h);
+  const int gs = d == 0.f ? g : ((g & ~15) | ((g & 15) ? 16 : 0));
+  l = __float2half_rn(fmaf((float)gs, unit, d));
 }
 
 }  // namespace tc
