@@ -748,10 +748,10 @@ Status phi_adjoint_xv_tc(sox_handle h, int n, int N, int T, int S, const double 
       a.A = X; a.ai = n; a.ak = 1;
       a.B = Gs; a.sB = nn; a.bk = n; a.bj = 1;
       a.C = GRall; a.sC = Nn; a.ci = n; a.cj = 1;
-      SOX_TRY(gemm_f64(h, a, ar, s));
+      SOX_TRY(gemm_f64(h, a, at, s));   // digits behind the chunk's buffers: those hold padding and osv
       GemmF64 b = a;
       b.bk = 1; b.bj = n; b.C = GWall; b.skip = symf;
-      SOX_TRY(gemm_f64(h, b, ar, s));
+      SOX_TRY(gemm_f64(h, b, at, s));
       k_copy_flagged<<<grid1((long long)T * Nn), 256, 0, s>>>(GRall, GWall, Nn, T, symf);
       launches += 4;
     }
