@@ -314,17 +314,22 @@ __global__ void __launch_bounds__(256) k_gj_block_inverse(const T *Aug, int N, i
   }
 }
 
-// systems per pass: the scratch of a pass stays near 1 GiB
+// bytes of scratch per system of a pass
 size_t per_system(int N, bool cplx) {
   const int c = cplx ? 2 : 1;
   const size_t e = 8 * c;
   return 2 * (size_t)kNb * N * e + kNb * kNb * e + kNb * 4 + slice_bytes(1, kNb, kNb * c) + slice_bytes(1, N, kNb * c) +
          slice_bytes(1, 2 * N * c, kNb * c) + 2048;
 }
+// the most systems of a pass: its scratch stays near 1 GiB.  (Passes are of equal size, so a smaller
+// batch can have larger passes than a larger one: scratch is sized by this, which grows with the batch.)
+size_t most_systems(int N, int batch, bool cplx) {
+  return std::max<size_t>(1, std::min<size_t>(batch, (size_t(1) << 30) / per_system(N, cplx)));
+}
 int pass_systems(int N, int batch, bool cplx) {
-  const size_t most = std::max<size_t>(1, std::min<size_t>(batch, (size_t(1) << 30) / per_system(N, cplx)));
+  const size_t most = most_systems(N, batch, cplx);
   const size_t passes = ((size_t)batch + most - 1) / most;
-  return (int)(((size_t)batch + passes - 1) / passes);   // passes of equal size
+  return (int)(((size_t)batch + passes - 1) / passes);
 }
 
 template <class T>
@@ -407,7 +412,7 @@ Status solve(sox_handle h, T *Aug, int N, int batch, int *info, Arena scratch, c
 bool gj_pays(int N) { return N >= 64; }
 
 size_t gj_bytes(int N, int batch, bool cplx) {
-  return gj_pays(N) ? per_system(N, cplx) * (size_t)pass_systems(N, batch, cplx) : 0;
+  return gj_pays(N) ? per_system(N, cplx) * most_systems(N, batch, cplx) : 0;
 }
 
 Status gj_solve(sox_handle h, double *Aug, int N, int batch, bool cplx, int *info, Arena scratch, cudaStream_t s) {

@@ -31,3 +31,26 @@ def test_adjoint_of_a_long_grid_in_chunks_of_one_time(env, n, N, n_tau, n_spin):
         gX, gV = _grads_with(torch, pkg, h, w, wt, dphi)
     assert np.abs(gX - rX).max() <= 4e-5 * np.abs(rX).max()
     assert np.abs(gV - rV).max() <= 4e-5 * np.abs(rV).max()
+
+
+def _w_dynamic(torch, pkg, h, w, Tf, nk):
+    p = pkg.problem(w.n, w.N, w.n_tau, 1, w.beta, nk=nk, dtype=1)
+    G, X, V, F = to_dev(torch, *(np.asarray(a, dtype=complex) for a in (w.G, w.X, w.V, Tf)))
+    out = torch.full((w.n_k, len(Tf), w.N, w.N), complex(float("nan"), 0.0), dtype=torch.complex128, device="cuda")
+    pkg.sox_w_dynamic(h, p, G, X, V, F, len(Tf), out)
+    pkg.sox_check_device(h)
+    return out
+
+
+@pytest.mark.parametrize("nk,N,n_omega", [((3, 3, 3), 300, 25), ((4, 4, 4), 200, 21)])
+def test_w_dynamic_on_a_handle_made_for_it(env, nk, N, n_omega):
+    """Only half of the +-Omega systems are solved: the scratch that is reserved for all of them has
+    to hold the passes of half of them too.  One frequency against a call of its own."""
+    torch, pkg = env
+    w = synth.solid(131, nk, 3, N, 4, 20.0)
+    _, Tf, _ = synth.bosonic_transforms(w.tau, w.beta, (n_omega - 1) // 2)
+    with pkg.Handle("fp64") as h:
+        out = _w_dynamic(torch, pkg, h, w, Tf, nk)
+    with pkg.Handle("fp64") as h:
+        one = _w_dynamic(torch, pkg, h, w, Tf[2:3], nk)
+    assert float((out[:, 2] - one[:, 0]).abs().max()) <= 1e-10 * float(one.abs().max())
