@@ -314,11 +314,19 @@ __global__ void __launch_bounds__(256) k_gj_block_inverse(const T *Aug, int N, i
   }
 }
 
+// The block's rows, columns k0 + nb ..: Aug = R[b][c][j] (rows of ldr)
+template <class T>
+__global__ void __launch_bounds__(256) k_gj_put_rows(const T *R, long long ldr, int N, int k0, int nb, T *Aug) {
+  const int b = blockIdx.z, c = blockIdx.y;
+  const long long j = blockIdx.x * 256 + threadIdx.x, rest = 2LL * N - k0 - nb;
+  if (j < rest) Aug[((long long)b * N + k0 + c) * 2 * N + k0 + nb + j] = R[((long long)b * kNb + c) * ldr + j];
+}
+
 // bytes of scratch per system of a pass
 size_t per_system(int N, bool cplx) {
   const int c = cplx ? 2 : 1;
   const size_t e = 8 * c;
-  return 2 * (size_t)kNb * N * e + kNb * kNb * e + kNb * 4 + slice_bytes(1, kNb, kNb * c) + slice_bytes(1, N, kNb * c) +
+  return 4 * (size_t)kNb * N * e + kNb * kNb * e + kNb * 4 + slice_bytes(1, kNb, kNb * c) + slice_bytes(1, N, kNb * c) +
          slice_bytes(1, 2 * N * c, kNb * c) + 2048;
 }
 // the most systems of a pass: its scratch stays near 1 GiB.  (Passes are of equal size, so a smaller
@@ -337,7 +345,7 @@ Status solve(sox_handle h, T *Aug, int N, int batch, int *info, Arena scratch, c
   constexpr bool cplx = sizeof(T) == 16;
   constexpr int c = cplx ? 2 : 1;
   T *P = scratch.take<T>((size_t)batch * kNb * N), *F = scratch.take<T>((size_t)batch * N * kNb);
-  T *Inv = scratch.take<T>((size_t)batch * kNb * kNb);
+  T *Inv = scratch.take<T>((size_t)batch * kNb * kNb), *Rs = scratch.take<T>((size_t)batch * kNb * 2 * N);
   int *piv = scratch.take<int>((size_t)batch * kNb);
   if (!piv) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
   static std::atomic<unsigned long long> attr{0};
@@ -371,36 +379,41 @@ Status solve(sox_handle h, T *Aug, int N, int batch, int *info, Arena scratch, c
     k_gj_factor<T><<<dim3((N + 7) / 8, batch), 256, 0, s>>>(Aug, N, k0, nb, F);
     h->launches += 4;
     const int rest = 2 * N - k0 - nb;
-    double *blk = reinterpret_cast<double *>(Aug + (long long)k0 * ld + k0 + nb);
-    double *all = reinterpret_cast<double *>(Aug + k0 + nb);
+    const double *blk = reinterpret_cast<const double *>(Aug + (long long)k0 * ld + k0 + nb);
+    const double *rs = reinterpret_cast<const double *>(Rs);
+    const double *inv = reinterpret_cast<const double *>(Inv), *f = reinterpret_cast<const double *>(F);
     Arena ar = scratch;
     SliceOp I = slice_take(ar, batch, nb, nb * c), Fs = slice_take(ar, batch, N, nb * c),
             R = slice_take(ar, batch, rest * c, nb * c);
     if (!I.p || !Fs.p || !R.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-    const double *inv = reinterpret_cast<const double *>(Inv), *f = reinterpret_cast<const double *>(F);
+    // R = A11^-1 A_blk into scratch (a product may read its sources again until it is done: it may
+    // not write over them), then A -= F R, then R into the block's rows
     SliceGemm g;
     g.batch = batch;
-    g.sC = c * sys; g.ci = c * ld; g.cj = 1;
-    for (int part = 0; part < 2; ++part) {   // R = A11^-1 A_blk in place, then A -= F R
-      if (part == 0) {
-        if (cplx) {
-          slice_complex_a(inv, kNb * kNb, kNb, 1, batch, I, s);
-          slice_complex_a(f, (long long)N * kNb, kNb, 1, batch, Fs, s);
-        } else {
-          slice_rows(inv, false, kNb * kNb, kNb, 1, batch, I, s);
-          slice_rows(f, false, (long long)N * kNb, kNb, 1, batch, Fs, s);
-        }
-      }
-      if (cplx)
-        slice_complex_b(blk, sys, 1, ld, batch, false, false, R, s);
-      else
-        slice_rows(blk, false, sys, 1, ld, batch, R, s);
-      g.C = part == 0 ? blk : all;
-      g.alpha = part == 0 ? 1.0 : -1.0;
-      g.beta = part == 0 ? 0.0 : 1.0;
-      SOX_TRY(slice_gemm(h, part == 0 ? I : Fs, R, g, s));
+    g.C = reinterpret_cast<double *>(Rs);
+    g.sC = c * kNb * ld; g.ci = c * ld; g.cj = 1;
+    if (cplx) {
+      slice_complex_a(inv, kNb * kNb, kNb, 1, batch, I, s);
+      slice_complex_b(blk, sys, 1, ld, batch, false, false, R, s);
+    } else {
+      slice_rows(inv, false, kNb * kNb, kNb, 1, batch, I, s);
+      slice_rows(blk, false, sys, 1, ld, batch, R, s);
     }
-    h->launches += 6;
+    SOX_TRY(slice_gemm(h, I, R, g, s));
+    if (cplx) {
+      slice_complex_a(f, (long long)N * kNb, kNb, 1, batch, Fs, s);
+      slice_complex_b(rs, kNb * ld, 1, ld, batch, false, false, R, s);
+    } else {
+      slice_rows(f, false, (long long)N * kNb, kNb, 1, batch, Fs, s);
+      slice_rows(rs, false, kNb * ld, 1, ld, batch, R, s);
+    }
+    g.C = reinterpret_cast<double *>(Aug + k0 + nb);
+    g.sC = c * sys;
+    g.alpha = -1.0;
+    g.beta = 1.0;
+    SOX_TRY(slice_gemm(h, Fs, R, g, s));
+    k_gj_put_rows<T><<<dim3((rest + 255) / 256, nb, batch), 256, 0, s>>>(Rs, ld, N, k0, nb, Aug);
+    h->launches += 7;
   }
   SOX_CUDA_TRY(cudaGetLastError());
   return Status::ok();
