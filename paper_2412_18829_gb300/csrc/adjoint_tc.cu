@@ -266,7 +266,7 @@ __device__ __forceinline__ void adj_epilogue(PBars *bar, uint32_t tmem, const Ad
   const int tiles_per_b = tP * tP;
   const int row = q * 32 + lane;
   long long acc_it = 0;
-  for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+  for (long long t = blockIdx.x; t < total; t += gridDim.x) {
     const int b = (int)(t / tiles_per_b);
     const int r = (int)(t % tiles_per_b);
     const int P0 = (r / tP) * kT, R0 = (r % tP) * kT;
@@ -293,7 +293,7 @@ __device__ __forceinline__ void adj_epilogue(PBars *bar, uint32_t tmem, const Ad
     for (int v = a.v0; v < a.v1; ++v, ++acc_it) {
       const int buf = (int)(acc_it & 1);
       const uint32_t aph = (uint32_t)((acc_it >> 1) & 1);
-      ok = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+      ok = tc::mbar_wait_warp(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
       if (!ok) break;
       tc::tc_fence_after();
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 256 + col0;

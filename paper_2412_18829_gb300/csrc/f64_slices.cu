@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3, part = (warp - 2) >> 2;
     const int lr = q * 32 + lane;
     long long win = 0;
-    for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < total; t += gridDim.x) {
       const int b = (int)(t / per_b), r = (int)(t % per_b);
       if (a.skip && a.skip[b]) continue;
       const int l = (r % a.tL) * kL + lr, w0 = (r / a.tL) * kW + part * kC;
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = 0; j < kC; ++j) acc[j] = 0;
       bool ok = true;
       for (int w = 0; w < nwin; ++w, ++win) {
-        ok = tc::mbar_wait(&bar->acc_full, (uint32_t)(win & 1), limit, abort, a.status, 8);
+        ok = tc::mbar_wait_warp(&bar->acc_full, (uint32_t)(win & 1), limit, abort, a.status, 8);
         if (!ok) break;
         tc::tc_fence_after();
         read_window<LK, kC, kW>(tmem + ((uint32_t)(q * 32) << 16) + part * kC, bar->acc_empty, lane, acc);
@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3, part = (warp - 2) >> 2;
     const int lr = q * 32 + lane;
     long long win = 0;
-    for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < total; t += gridDim.x) {
       const int b = (int)(t / per_b), r = (int)(t % per_b);
       const int P = (r / a.tR) * kL + lr, R0 = (r % a.tR) * kFW + part * kC;
       double d[kC];
@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int eUl = lane < cols ? a.eU[(long long)v * a.N + R0 + lane] : 0;
         for (int h = 0; h < 2 && ok; ++h)
           for (int w = 0; w < nwin; ++w) {
-            ok = tc::mbar_wait(&bar->acc_full[h], (uint32_t)((win + w) & 1), limit, abort, a.status, 8);
+            ok = tc::mbar_wait_warp(&bar->acc_full[h], (uint32_t)((win + w) & 1), limit, abort, a.status, 8);
             if (!ok) break;
             tc::tc_fence_after();
             const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + h * 256 + part * kC;

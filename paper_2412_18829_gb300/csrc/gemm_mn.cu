@@ -287,8 +287,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (long long w0 = w.c0; w0 < w.c1; w0 += a.window, ++acc_it) {
         const int buf = (int)(acc_it & 3);
         const uint32_t aph = (uint32_t)((acc_it >> 2) & 1);
-        const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
-        if (!__all_sync(0xffffffffu, got && !*abort)) {
+        const bool got = tc::mbar_wait_warp(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+        if (!got) {
           live = false;
           break;
         }

@@ -60,6 +60,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, long l
   return false;
 }
 
+// The same for a whole warp: its lanes go on together or leave together.  (A lane that alone sees
+// the wait run out, or the abort flag, must not leave the others in warp-wide loads, shuffles and
+// barriers.)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, long long limit,
+                                               volatile int *abort, int *status, int code) {
+  const bool got = mbar_wait(bar, parity, limit, abort, status, code);
+  return __all_sync(0xffffffffu, got && !*abort);
+}
+
 // Phase bookkeeping for a stage ring whose full barriers come in two sets, one per MMA
 // issuer (full[q][s]), fed by one TMA producer.  Bit 16q + s of `par` is the parity of the
 // next phase the holder expects on full[q][s]; bit 16q + s of `used` marks a barrier the

@@ -181,7 +181,7 @@ __device__ __forceinline__ void bcd_epilogue(Bar *bar, uint32_t tmem, const BcdA
   const int q = warp & 3;                 // TMEM lane quarter of this warp
   const int row = q * 32 + lane;          // P offset inside the tile
   long long acc_it = 0;
-  for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+  for (long long t = blockIdx.x; t < total; t += gridDim.x) {
     const int b = (int)(t / tiles_per_b);
     const int r = (int)(t % tiles_per_b);
     const int P0 = (r / tP) * kTile, R0 = (r % tP) * kTile;
@@ -192,7 +192,7 @@ __device__ __forceinline__ void bcd_epilogue(Bar *bar, uint32_t tmem, const BcdA
     for (int v = a.v0; v < a.v1; ++v, ++acc_it) {
       const int buf = (int)(acc_it & 1);
       const uint32_t aph = (uint32_t)((acc_it >> 1) & 1);
-      ok = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+      ok = tc::mbar_wait_warp(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
       if (!ok) break;
       tc::tc_fence_after();
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 256;
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kBcdThreads, 1) k_sox_bcd_multi(const __grid_c
     const int q = warp & 3;
     const int row = q * 32 + lane;
     long long acc_it = 0;
-    for (long long t = blockIdx.x; t < total && !*abort; t += gridDim.x) {
+    for (long long t = blockIdx.x; t < total; t += gridDim.x) {
       const MultiTile m = multi_tile(jobs, t);
       const BcdJob &J = jobs.job[m.j];
       float d[kTile];
@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(kBcdThreads, 1) k_sox_bcd_multi(const __grid_c
       for (int v = J.v0; v < J.v1; ++v, ++acc_it) {
         const int buf = (int)(acc_it & 1);
         const uint32_t aph = (uint32_t)((acc_it >> 1) & 1);
-        ok = tc::mbar_wait(&bar->acc_full[buf], aph, limit, abort, jobs.status, 8);
+        ok = tc::mbar_wait_warp(&bar->acc_full[buf], aph, limit, abort, jobs.status, 8);
         if (!ok) break;
         tc::tc_fence_after();
         const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 256;
@@ -932,7 +932,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBcdThreads, 1)
     const int q = warp & 3;                 // TMEM lane quarter of this warp
     const int row = q * 32 + lane;          // P offset inside this CTA's tile
     long long acc_it = 0;
-    for (long long u = pair; u < total && !*abort; u += npairs) {
+    for (long long u = pair; u < total; u += npairs) {
       const int b = (int)(u / units_per_b);
       const int r = (int)(u % units_per_b);
       const int P0 = (2 * (r / tP) + (int)rank) * kTile, R0 = (r % tP) * kTile;
@@ -943,7 +943,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kBcdThreads, 1)
       for (int v = a.v0; v < a.v1; ++v, ++acc_it) {
         const int buf = (int)(acc_it & 1);
         const uint32_t aph = (uint32_t)((acc_it >> 1) & 1);
-        ok = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+        ok = tc::mbar_wait_warp(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
         if (!ok) break;
         tc::tc_fence_after();
         const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 256;
@@ -1263,8 +1263,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const int b = w.b(), i0 = w.i0(), j0 = w.j0();
         const int buf = (int)(acc_it & 3);
         const uint32_t aph = (uint32_t)((acc_it >> 2) & 1);
-        const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
-        if (!__all_sync(0xffffffffu, got && !*abort)) break;
+        const bool got = tc::mbar_wait_warp(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+        if (!got) break;
         tc::tc_fence_after();
         const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 128;
         const bool live = i0 + q * 32 < a.M;   // a warp whose 32 rows lie outside has nothing to do
@@ -1352,9 +1352,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const int b = w.b(), i0 = w.i0(), j0 = w.j0();
       const int buf = (int)(acc_it & 3);
       const uint32_t aph = (uint32_t)((acc_it >> 2) & 1);
-      const bool got = tc::mbar_wait(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
+      const bool got = tc::mbar_wait_warp(&bar->acc_full[buf], aph, a.spin_limit, abort, a.status, 8);
       // only the group maxima need the other warps: there they go on together or not at all
-      if (kMode == kStoreSplitGroup ? !epi_all(got && !*abort) : !__all_sync(0xffffffffu, got && !*abort)) break;
+      if (kMode == kStoreSplitGroup ? !epi_all(got) : !got) break;
       tc::tc_fence_after();
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + buf * 128 + h * 64;
       const bool row_ok = (i0 + row) < a.M;
