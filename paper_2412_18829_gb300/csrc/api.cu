@@ -7,9 +7,9 @@
 #include <vector>
 
 #include "adjoint.h"
+#include "block_lu.h"
 #include "dynamic.h"
 #include "f64_slices.h"
-#include "gj.h"
 #include "internal.h"
 #include "ctc.h"
 #include "kpoint.h"
@@ -802,19 +802,19 @@ int sox_w_static(sox_handle h, const sox_problem *p, const double *V, const doub
     g.ci = 2LL * N; g.cj = 1;
     g.alpha = -1.0; g.beta = 1.0;
     SOX_TRY(call.begin(sox::aligned_bytes((size_t)2 * N * N, 8) + 256 +
-                           std::max(sox::gemm_f64_bytes(g), sox::gj_bytes(N, 1, false)), &ar));
+                           std::max(sox::gemm_f64_bytes(g), sox::lu_bytes(N, 1, false)), &ar));
     double *Aug = ar.take<double>((size_t)2 * N * N);
     int *info = ar.take<int>(4);
     cudaStream_t s = call.stream();
     SOX_CUDA_TRY(cudaMemsetAsync(info, 0, 4 * sizeof(int), s));
     {
-      const bool blocked = sox::gj_pays(N);
+      const bool blocked = sox::lu_pays(N);
       sox::ProfScope ps(h, "w_static_gj", s, blocked ? 3 : 3 + 2 * N);
       sox::launch_gj_init(sV.in, Aug, N, s);
       g.A = sV.in; g.B = sP.in; g.C = Aug;
       SOX_TRY(sox::gemm_f64(h, g, ar, s));
       if (blocked)
-        SOX_TRY(sox::gj_solve(h, Aug, N, 1, false, info, ar, s));
+        SOX_TRY(sox::lu_solve(h, Aug, N, 1, false, info, ar, s));
       else
         for (int k = 0; k < N; ++k) sox::launch_gj_step(Aug, N, k, info, s);
       sox::launch_copy_right_half(Aug, oW.out, N, s);

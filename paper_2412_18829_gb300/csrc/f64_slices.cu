@@ -14,11 +14,22 @@ namespace {
 constexpr int kNonFinite = 1 << 20;
 
 // ------------------------------------------------------------------ slicing
-// Exponent field of x, subnormals counted with the smallest normal exponent.
-__device__ __forceinline__ int exp_field(double x) {
-  const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  return e == 0 ? 1 : e;
+constexpr int kZeroRow = -kNonFinite;   // (a row maximum over nothing)
+// Exponent field of x 2^sh (subnormals with the smallest normal exponent), kNonFinite for infinities
+// and NaNs, kZeroRow for zeros.
+__device__ __forceinline__ int exp_field(double x, int sh) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
+  if (((hi & 0x7fffffff) | __double2loint(x)) == 0) return kZeroRow;
+  return e == 0x7ff ? kNonFinite : max(e, 1) + sh;
 }
+// e_k of a balanced operand (SliceBalance)
+__device__ __forceinline__ int balance(const SliceBalance &bal, int b, int k) {
+  if (!bal.kex) return 0;
+  const int e = bal.kex[(long long)b * bal.stride + k];
+  return e > 0 ? bal.sgn * (e - 1023) : 0;
+}
+// the exponent that is kept for a row of maximum E
+__device__ __forceinline__ int row_exp(int E) { return E == kZeroRow ? 1 : E; }
 // x scaled by the row's exponent as an integer: x = X 2^-55 2^(E - 1022), |X| <= 2^55,
 // rounded to nearest (ties up)
 __device__ __forceinline__ long long fixed55(double x, int E) {
@@ -26,6 +37,7 @@ __device__ __forceinline__ long long fixed55(double x, int E) {
   const int ef = (int)((bits >> 52) & 0x7ff);
   long long m = bits & 0xfffffffffffffll;
   if (ef) m |= 1ll << 52;
+  if (m == 0) return 0;
   const int sh = E - (ef ? ef : 1) - 2;   // m 2^-sh
   if (sh <= 0)
     m <<= -sh;
@@ -62,19 +74,21 @@ __device__ __forceinline__ void digits8(long long (&X)[8], uint4 (&w)[kSlices]) 
 // Rows with contiguous elements (sk == 1): `lpr` lanes per row.
 template <class T>
 __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, long long sr, int rows, int batch,
-                                                    int batch_all, int K, int K8, int lpr, __half *p, int *ex) {
+                                                    int batch_all, int K, int K8, int lpr, SliceBalance bal, __half *p,
+                                                    int *ex) {
   const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long row = g / lpr;
   const int l = (int)(g % lpr);
   const bool live = row < (long long)rows * batch;
-  const T *x = live ? src + (row / rows) * sb + (row % rows) * sr : src;
-  int E = 1;
+  const int b = live ? (int)(row / rows) : 0;
+  const T *x = live ? src + b * sb + (row % rows) * sr : src;
+  int E = kZeroRow;
   if (live)
-    for (int k = l; k < K; k += lpr) E = max(E, exp_field((double)x[k]));
+    for (int k = l; k < K; k += lpr) E = max(E, exp_field((double)x[k], balance(bal, b, k)));
   for (int o = lpr / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
   if (!live) return;
-  const bool fin = E < 0x7ff;
-  if (l == 0) ex[row] = fin ? E : kNonFinite;
+  const bool fin = E < kNonFinite;
+  if (l == 0) ex[row] = row_exp(E);
   const long long plane = (long long)batch_all * rows * K8;
   for (int c = l; c < K8 / 8; c += lpr) {
     long long X[8];
@@ -82,7 +96,7 @@ __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, 
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int k = c * 8 + e;
-      X[e] = (fin && k < K) ? fixed55((double)x[k], E) : 0;
+      X[e] = (fin && k < K) ? fixed55((double)x[k], E - balance(bal, b, k)) : 0;
     }
     digits8(X, w);
 #pragma unroll
@@ -93,28 +107,28 @@ __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, 
 // Rows whose elements lie apart: 32 rows per block, transposed through shared memory.
 template <class T>
 __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, long long sr, long long sk, int rows,
-                                                    int batch_all, int K, int K8, __half *p, int *ex) {
+                                                    int batch_all, int K, int K8, SliceBalance bal, __half *p, int *ex) {
   __shared__ long long sx[64][33];
   __shared__ int se[8][32];
   const int b = blockIdx.y, r0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   const T *x = src + b * sb + (long long)(r0 + tx) * sr;
   const bool in = r0 + tx < rows;
-  int E = 1;
+  int E = kZeroRow;
   if (in)
-    for (int k = ty; k < K; k += 8) E = max(E, exp_field((double)x[k * sk]));
+    for (int k = ty; k < K; k += 8) E = max(E, exp_field((double)x[k * sk], balance(bal, b, k)));
   se[ty][tx] = E;
   __syncthreads();
-  E = 1;
+  E = kZeroRow;
 #pragma unroll
   for (int i = 0; i < 8; ++i) E = max(E, se[i][tx]);
-  const bool fin = E < 0x7ff;
-  if (ty == 0 && in) ex[(long long)b * rows + r0 + tx] = fin ? E : kNonFinite;
+  const bool fin = E < kNonFinite;
+  if (ty == 0 && in) ex[(long long)b * rows + r0 + tx] = row_exp(E);
   const long long plane = (long long)batch_all * rows * K8;
   const int row = threadIdx.x / 8, c8 = threadIdx.x % 8;
   for (int k0 = 0; k0 < K8; k0 += 64) {
     __syncthreads();
     for (int k = ty; k < 64; k += 8)
-      sx[k][tx] = (in && fin && k0 + k < K) ? fixed55((double)x[(k0 + k) * sk], E) : 0;
+      sx[k][tx] = (in && fin && k0 + k < K) ? fixed55((double)x[(k0 + k) * sk], E - balance(bal, b, k0 + k)) : 0;
     __syncthreads();
     if (r0 + row < rows && k0 + c8 * 8 < K8) {
       long long X[8];
@@ -134,38 +148,40 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
 template <int KIND>
 __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long long sb, long long sr, long long sk,
                                                        int rows, int batch_all, int K, int K8, int sa, int sc,
-                                                       __half *p, int *ex) {
+                                                       SliceBalance bal, __half *p, int *ex) {
   __shared__ long long sx[2][32][33];
   __shared__ int se[32];
   const int b = blockIdx.y, r0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   const bool along_k = sk == 1;
   const double2 *x = src + b * sb;
-  if (threadIdx.x < 32) se[threadIdx.x] = 1;
+  if (threadIdx.x < 32) se[threadIdx.x] = kZeroRow;
   __syncthreads();
   if (along_k) {
     for (int r = ty; r < 32; r += 8) {
-      int E = 1;
+      int E = kZeroRow;
       if (r0 + r < rows)
         for (int k = tx; k < K; k += 32) {
           const double2 v = x[(long long)(r0 + r) * sr + k];
-          E = max(E, max(exp_field(v.x), exp_field(v.y)));
+          const int sh = balance(bal, b, k);
+          E = max(E, max(exp_field(v.x, sh), exp_field(v.y, sh)));
         }
       for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
       if (tx == 0) se[r] = E;
     }
   } else {
-    int E = 1;
+    int E = kZeroRow;
     if (r0 + tx < rows)
       for (int k = ty; k < K; k += 8) {
         const double2 v = x[(long long)(r0 + tx) * sr + k * sk];
-        E = max(E, max(exp_field(v.x), exp_field(v.y)));
+        const int sh = balance(bal, b, k);
+        E = max(E, max(exp_field(v.x, sh), exp_field(v.y, sh)));
       }
     atomicMax(&se[tx], E);
   }
   __syncthreads();
   const int nr = KIND == 2 ? 2 : 1;   // real rows per complex row
   if (threadIdx.x < 32 && r0 + tx < rows) {
-    const int e = se[tx] < 0x7ff ? se[tx] : kNonFinite;
+    const int e = row_exp(se[tx]);
     for (int i = 0; i < nr; ++i) ex[((long long)b * rows + r0 + tx) * nr + i] = e;
   }
   const long long plane = (long long)batch_all * rows * nr * K8;
@@ -174,11 +190,12 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
     __syncthreads();
     for (int i = ty; i < 32; i += 8) {
       const int k = along_k ? tx : i, r = along_k ? i : tx, E = se[r];
-      const bool in = r0 + r < rows && k0 + k < K && E < 0x7ff;
+      const bool in = r0 + r < rows && k0 + k < K && E < kNonFinite;
       double2 v = make_double2(0.0, 0.0);
       if (in) v = x[(long long)(r0 + r) * sr + (k0 + k) * sk];
-      sx[0][k][r] = in ? fixed55(v.x, E) : 0;
-      sx[1][k][r] = in ? fixed55(v.y, E) : 0;
+      const int sh = in ? balance(bal, b, k0 + k) : 0;
+      sx[0][k][r] = in ? fixed55(v.x, E - sh) : 0;
+      sx[1][k][r] = in ? fixed55(v.y, E - sh) : 0;
     }
     __syncthreads();
     if (r0 + row < rows && 2 * k0 + c8 * 8 < K8) {
@@ -852,7 +869,7 @@ SliceOp slice_take(Arena &ar, int batch, int rows, int K) {
 }
 
 void slice_rows(const void *src, bool f32, long long sb, long long sr, long long sk, int batch, SliceOp &op,
-                cudaStream_t s) {
+                cudaStream_t s, SliceBalance bal) {
   op.src = src;
   op.f32 = f32;
   op.sb = sb;
@@ -865,32 +882,33 @@ void slice_rows(const void *src, bool f32, long long sb, long long sr, long long
     const long long blocks = ((long long)batch * op.rows * lpr + 255) / 256;
     if (f32)
       k_slice_rows<float><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const float *>(src), sb, sr, op.rows, batch,
-                                                         op.batch, op.K, op.K8, lpr, op.p, op.ex);
+                                                         op.batch, op.K, op.K8, lpr, bal, op.p, op.ex);
     else
       k_slice_rows<double><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const double *>(src), sb, sr, op.rows, batch,
-                                                          op.batch, op.K, op.K8, lpr, op.p, op.ex);
+                                                          op.batch, op.K, op.K8, lpr, bal, op.p, op.ex);
   } else {
     const dim3 grid((op.rows + 31) / 32, batch);
     if (f32)
       k_slice_cols<float><<<grid, 256, 0, s>>>(static_cast<const float *>(src), sb, sr, sk, op.rows, op.batch, op.K,
-                                               op.K8, op.p, op.ex);
+                                               op.K8, bal, op.p, op.ex);
     else
       k_slice_cols<double><<<grid, 256, 0, s>>>(static_cast<const double *>(src), sb, sr, sk, op.rows, op.batch, op.K,
-                                                op.K8, op.p, op.ex);
+                                                op.K8, bal, op.p, op.ex);
   }
 }
 
-void slice_complex_a(const double *src, long long sb, long long sr, long long sk, int batch, SliceOp &op, cudaStream_t s) {
+void slice_complex_a(const double *src, long long sb, long long sr, long long sk, int batch, SliceOp &op, cudaStream_t s,
+                     SliceBalance bal) {
   op.src = src;
   op.sb = sb; op.sr = sr; op.sk = sk;
   op.kind = 1;
   if (batch <= 0 || op.rows <= 0) return;
   k_slice_complex<1><<<dim3((op.rows + 31) / 32, batch), 256, 0, s>>>(
-      reinterpret_cast<const double2 *>(src), sb, sr, sk, op.rows, op.batch, op.K / 2, op.K8, 1, 1, op.p, op.ex);
+      reinterpret_cast<const double2 *>(src), sb, sr, sk, op.rows, op.batch, op.K / 2, op.K8, 1, 1, bal, op.p, op.ex);
 }
 
 void slice_complex_b(const double *src, long long sb, long long sr, long long sk, int batch, bool conjA, bool conjB,
-                     SliceOp &op, cudaStream_t s) {
+                     SliceOp &op, cudaStream_t s, SliceBalance bal) {
   op.src = src;
   op.sb = sb; op.sr = sr; op.sk = sk;
   op.kind = 2;
@@ -899,7 +917,7 @@ void slice_complex_b(const double *src, long long sb, long long sr, long long sk
   if (batch <= 0 || op.rows <= 0) return;
   const int rows = op.rows / 2;
   k_slice_complex<2><<<dim3((rows + 31) / 32, batch), 256, 0, s>>>(
-      reinterpret_cast<const double2 *>(src), sb, sr, sk, rows, op.batch, op.K / 2, op.K8, op.sa, op.sc, op.p, op.ex);
+      reinterpret_cast<const double2 *>(src), sb, sr, sk, rows, op.batch, op.K / 2, op.K8, op.sa, op.sc, bal, op.p, op.ex);
 }
 
 Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceGemm &g, cudaStream_t s) {

@@ -37,15 +37,24 @@ struct SliceOp {
 };
 size_t slice_bytes(long long batch, int rows, int K);
 SliceOp slice_take(Arena &ar, int batch, int rows, int K);
+// Powers of two along the inner index: operand A of a product times 2^e_k, B times 2^-e_k, with e_k from
+// the exponent fields kex[b * stride + k] (0: none) and sgn = 1 for A, -1 for B.  The product is the
+// same; a K index that is large in one operand and small in the other keeps its digits in both.
+struct SliceBalance {
+  const int *kex = nullptr;
+  int stride = 0, sgn = 0;
+};
 // digits of element (b, r, k) = src[b * sb + r * sr + k * sk], FP64 or FP32; `batch` blocks
 // (at most op's)
 void slice_rows(const void *src, bool f32, long long sb, long long sr, long long sk, int batch, SliceOp &op,
-                cudaStream_t s);
+                cudaStream_t s, SliceBalance bal = {});
 
 // The same for complex rows (FP64, interleaved): op taken with rows (A) or 2 rows (B) and 2 K
-void slice_complex_a(const double *src, long long sb, long long sr, long long sk, int batch, SliceOp &op, cudaStream_t s);
+// (bal: over the K complex indices)
+void slice_complex_a(const double *src, long long sb, long long sr, long long sk, int batch, SliceOp &op, cudaStream_t s,
+                     SliceBalance bal = {});
 void slice_complex_b(const double *src, long long sb, long long sr, long long sk, int batch, bool conjA, bool conjB,
-                     SliceOp &op, cudaStream_t s);
+                     SliceOp &op, cudaStream_t s, SliceBalance bal = {});
 
 // C[b](i, j) = alpha sum_k A(b, i, k) B(b, j, k) + beta C[b](i, j); an operand of batch 1 is
 // shared.  Element (i, j) at C + b * sC + i * ci + j * cj.

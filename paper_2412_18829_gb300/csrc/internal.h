@@ -153,7 +153,7 @@ void launch_pi0_reduce(const double *GPQ, const double *w, int N, int n_tau, dou
 
 // Gauss-Jordan on the augmented [K | Bm] (N x 2N, row-major, in place), a column at a time:
 // returns the solution K^-1 Bm in the right half.  piv_info: device int[2].  (Small systems;
-// gj.h has the blocked form.)
+// block_lu.h has the blocked form.)
 void launch_gj_step(double *Aug, int N, int k, int *piv_info, cudaStream_t s);
 void launch_gj_init(const double *V, double *Aug, int N, cudaStream_t s);   // [I | V]
 void launch_copy_right_half(const double *Aug, double *W, int N, cudaStream_t s);

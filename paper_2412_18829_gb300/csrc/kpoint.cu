@@ -15,9 +15,9 @@
 #include <cstring>
 #include <vector>
 
+#include "block_lu.h"
 #include "ctc.h"
 #include "f64_slices.h"
-#include "gj.h"
 #include "kpoint.h"
 #include "tc_common.cuh"
 
@@ -1534,7 +1534,7 @@ size_t w_dynamic_bytes(const sox_problem *p, int n_omega) {
   size_t scratch = std::max(zgemm_bytes(Ni, ni, ni, Ti, true, false), zgemm_bytes(Ni, Ni, ni, Ti, false, true));
   scratch = std::max(scratch, zgemm_bytes(Ni, Ni, Ni, n_omega, true, false));
   scratch = std::max(scratch, aligned_bytes(T * NN, 16) + zgemm_bytes(n_omega, (int)NN, Ti, 1, true, true));
-  if (gj_pays(Ni)) scratch = std::max(scratch, gj_bytes(Ni, (int)nk * n_omega, true));
+  if (lu_pays(Ni)) scratch = std::max(scratch, lu_bytes(Ni, (int)nk * n_omega, true));
   return b + scratch + (1 << 20);
 }
 
@@ -1658,8 +1658,8 @@ Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *
     g.alpha = -1.0; g.beta = 1.0;
     SOX_TRY(zgemm_f64(h, g, ar, s));
   }
-  const bool blocked = gj_pays(N);
-  if (blocked) SOX_TRY(gj_solve(h, reinterpret_cast<double *>(Aug), N, batch, true, info, ar, s));
+  const bool blocked = lu_pays(N);
+  if (blocked) SOX_TRY(lu_solve(h, reinterpret_cast<double *>(Aug), N, batch, true, info, ar, s));
   for (int k = 0; !blocked && k < N; ++k) {
     k_gj_pivot_c<<<batch, 256, 0, s>>>(Aug, N, k, info);
     const int ncols = 2 * N - (k + 1);
