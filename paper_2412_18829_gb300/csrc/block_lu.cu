@@ -229,13 +229,8 @@ __global__ void __launch_bounds__(256) k_lu_inner_update(T *P, int N, int k0, in
 template <class T> __device__ __forceinline__ T one();
 template <> __device__ __forceinline__ double one<double>() { return 1.0; }
 template <> __device__ __forceinline__ z one<z>() { return make_double2(1.0, 0.0); }
-// exponent field of the larger part of a finite value, 0 for zeros, infinities and NaNs
-__device__ __forceinline__ int exponent_of(double a) {
-  const int hi = __double2hiint(a), e = (hi >> 20) & 0x7ff;
-  if (e == 0x7ff || (((hi & 0x7fffffff) | __double2loint(a)) == 0)) return 0;
-  return max(e, 1);
-}
-__device__ __forceinline__ int exponent_of(z a) { return max(exponent_of(a.x), exponent_of(a.y)); }
+__device__ __forceinline__ int exponent_of(double a) { return balance_exponent(a); }
+__device__ __forceinline__ int exponent_of(z a) { return max(balance_exponent(a.x), balance_exponent(a.y)); }
 
 // kex[b][c] = max over the warp's columns of the exponent of row c: what the product that
 // follows balances its inner index by

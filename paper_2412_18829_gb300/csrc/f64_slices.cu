@@ -11,6 +11,15 @@
 namespace sox {
 namespace {
 
+// Digits are fixed point below a row's largest element, so the error of a product goes with the product
+// of the two maxima; FP64 arithmetic errs by the sum S of the element's |a_k b_k|.  An element is
+// taken from the digits only where S is known to be within 2^kSignif of the product of the scales: by
+// its own size, by a k at which both rows are within 2^kBig of their largest (bit masks of the rows), or by
+// the sum of products of 8-bit magnitudes (complex elements count by the larger part).  Any other is
+// summed in FP64 from the sources.  (The checks cost an FP64 bare SOX of n = 80, N = 480, 30 times 4 %,
+// 9.63 -> 9.98 ms, W of the 3 x 3 x 3 solid 7 %, the split-precision calls at most 2 %.)
+constexpr int kBig = 2, kSignif = 2 * kBig + 2;
+
 constexpr int kNonFinite = 1 << 20;
 
 // ------------------------------------------------------------------ slicing
@@ -22,14 +31,20 @@ __device__ __forceinline__ int exp_field(double x, int sh) {
   if (((hi & 0x7fffffff) | __double2loint(x)) == 0) return kZeroRow;
   return e == 0x7ff ? kNonFinite : max(e, 1) + sh;
 }
-// e_k of a balanced operand (SliceBalance)
+// e_k of a balanced operand (SliceBalance; BAL: there is one)
+template <bool BAL>
 __device__ __forceinline__ int balance(const SliceBalance &bal, int b, int k) {
-  if (!bal.kex) return 0;
+  if (!BAL) return 0;
   const int e = bal.kex[(long long)b * bal.stride + k];
-  return e > 0 ? bal.sgn * (e - 1023) : 0;
+  return e > 0 ? (e - 1023) / bal.part : 0;
 }
-// the exponent that is kept for a row of maximum E
-__device__ __forceinline__ int row_exp(int E) { return E == kZeroRow ? 1 : E; }
+// What is kept of a row: its largest exponent E, or that it holds an infinity or a NaN.  The codes of two
+// rows add up field by field.
+constexpr int kCodeBias = 8192, kCodeNonFinite = 1 << 16;
+__device__ __forceinline__ int row_code(int E) {
+  if (E == kZeroRow) E = 1;
+  return E >= kNonFinite ? kCodeBias | kCodeNonFinite : E + kCodeBias;
+}
 // x scaled by the row's exponent as an integer: x = X 2^-55 2^(E - 1022), |X| <= 2^55,
 // rounded to nearest (ties up)
 __device__ __forceinline__ long long fixed55(double x, int E) {
@@ -44,6 +59,57 @@ __device__ __forceinline__ long long fixed55(double x, int E) {
   else
     m = sh > 60 ? 0 : (m + (1ll << (sh - 1))) >> sh;
   return bits < 0 ? -m : m;
+}
+// Eight elements of a row as its epilogue's checks see them: bits for those within 2^kBig of the row's
+// largest and for those that are not zero, and magnitudes in 256ths of the scale, rounded down
+// (negative values by their complement, one unit of the high word short).  pair: complex elements, by
+// the larger part.
+struct Sizes {
+  unsigned big = 0u, nz = 0u;
+  uint2 mag = make_uint2(0u, 0u);
+};
+__device__ __forceinline__ Sizes sizes_of(const long long (&X)[8], unsigned nz, bool pair) {
+  Sizes z;
+  z.nz = nz;
+  unsigned a[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int hi = (int)(X[e] >> 32);
+    a[e] = (unsigned)(hi ^ (hi >> 31));
+  }
+  if (pair) {
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) a[e] = a[e + 1] = max(a[e], a[e + 1]);
+    z.nz |= ((nz & 0x55u) << 1) | ((nz >> 1) & 0x55u);
+  }
+  unsigned *m = &z.mag.x;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    z.big |= a[e] >= (1u << (22 - kBig)) ? 1u << e : 0u;
+    m[e / 4] |= min(a[e] >> 15, 255u) << (8 * (e & 3));
+  }
+  return z;
+}
+// Stores chunk c of a row's masks (two of nw words) and magnitudes (K8 bytes); the four threads of a word
+// are four consecutive lanes that call this together.
+__device__ __forceinline__ void put_sizes(uint32_t *mask, uint8_t *mag, int nw, int K8, int c, const Sizes &z) {
+  const unsigned quad = 0xfu << (threadIdx.x & 28);
+  unsigned x = (z.big | (z.nz << 16)) << (8 * (c & 1));   // two chunks of both masks
+  x |= __shfl_xor_sync(quad, x, 1);
+  const unsigned y = __shfl_xor_sync(quad, x, 2);           // the other two
+  if ((c & 3) == 0) mask[c / 4] = (x & 0xffffu) | (y << 16);
+  if ((c & 3) == 1) mask[nw + c / 4] = (x >> 16) | (y & 0xffff0000u);
+  if (c * 8 < K8) *reinterpret_cast<uint2 *>(mag + c * 8) = z.mag;
+}
+__device__ __forceinline__ unsigned nonzero(double x) {
+  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0 ? 1u : 0u;
+}
+// X with the nonzero flag of its value (which may have rounded to X = 0) at bit 58, for shared memory
+__device__ __forceinline__ long long flagged55(double x, int E) { return fixed55(x, E) + ((long long)nonzero(x) << 58); }
+__device__ __forceinline__ unsigned take_flag(long long &X) {
+  const int hi = (int)(X >> 32), f = (hi + (1 << 25)) >> 26;
+  X -= (long long)f << 58;
+  return (unsigned)f;
 }
 // Balanced base-256 digits of eight values, one 16-byte word of FP16 integers per digit.
 // An integer v in [0, 1023] is the FP16 number 1024 + v with v in its low bits.
@@ -71,11 +137,14 @@ __device__ __forceinline__ void digits8(long long (&X)[8], uint4 (&w)[kSlices]) 
   }
 }
 
+// words of one of a row's two bit masks (near the largest, nonzero; zero beyond K)
+__host__ __device__ inline int mask_words(int K) { return (K + 31) / 32; }
+
 // Rows with contiguous elements (sk == 1): `lpr` lanes per row.
-template <class T>
+template <class T, bool BAL>
 __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, long long sr, int rows, int batch,
                                                     int batch_all, int K, int K8, int lpr, SliceBalance bal, __half *p,
-                                                    int *ex) {
+                                                    int *ex, uint32_t *mask, uint8_t *mag) {
   const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long row = g / lpr;
   const int l = (int)(g % lpr);
@@ -84,20 +153,26 @@ __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, 
   const T *x = live ? src + b * sb + (row % rows) * sr : src;
   int E = kZeroRow;
   if (live)
-    for (int k = l; k < K; k += lpr) E = max(E, exp_field((double)x[k], balance(bal, b, k)));
+    for (int k = l; k < K; k += lpr) E = max(E, exp_field((double)x[k], balance<BAL>(bal, b, k)));
   for (int o = lpr / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
   if (!live) return;
   const bool fin = E < kNonFinite;
-  if (l == 0) ex[row] = row_exp(E);
+  if (l == 0) ex[row] = row_code(E);
   const long long plane = (long long)batch_all * rows * K8;
-  for (int c = l; c < K8 / 8; c += lpr) {
+  const int nw = mask_words(K);
+  for (int c = l; c < nw * 4; c += lpr) {   // (four lanes at least per row: a word's bytes go together)
     long long X[8];
     uint4 w[kSlices];
+    unsigned nz = 0u;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int k = c * 8 + e;
-      X[e] = (fin && k < K) ? fixed55((double)x[k], E - balance(bal, b, k)) : 0;
+      const double v = (fin && k < K) ? (double)x[k] : 0.0;
+      X[e] = fixed55(v, E - (k < K ? balance<BAL>(bal, b, k) : 0));
+      nz |= nonzero(v) << e;
     }
+    put_sizes(mask + row * 2 * nw, mag + row * K8, nw, K8, c, sizes_of(X, nz, false));
+    if (c * 8 >= K8) continue;
     digits8(X, w);
 #pragma unroll
     for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint4 *>(p + s * plane + row * K8 + c * 8) = w[s];
@@ -105,9 +180,10 @@ __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, 
 }
 
 // Rows whose elements lie apart: 32 rows per block, transposed through shared memory.
-template <class T>
+template <class T, bool BAL>
 __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, long long sr, long long sk, int rows,
-                                                    int batch_all, int K, int K8, SliceBalance bal, __half *p, int *ex) {
+                                                    int batch_all, int K, int K8, SliceBalance bal, __half *p, int *ex,
+                                                    uint32_t *mask, uint8_t *mag) {
   __shared__ long long sx[64][33];
   __shared__ int se[8][32];
   const int b = blockIdx.y, r0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
@@ -115,28 +191,35 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
   const bool in = r0 + tx < rows;
   int E = kZeroRow;
   if (in)
-    for (int k = ty; k < K; k += 8) E = max(E, exp_field((double)x[k * sk], balance(bal, b, k)));
+    for (int k = ty; k < K; k += 8) E = max(E, exp_field((double)x[k * sk], balance<BAL>(bal, b, k)));
   se[ty][tx] = E;
   __syncthreads();
-  E = kZeroRow;
 #pragma unroll
   for (int i = 0; i < 8; ++i) E = max(E, se[i][tx]);
   const bool fin = E < kNonFinite;
-  if (ty == 0 && in) ex[(long long)b * rows + r0 + tx] = row_exp(E);
+  if (ty == 0 && in) ex[(long long)b * rows + r0 + tx] = row_code(E);
   const long long plane = (long long)batch_all * rows * K8;
-  const int row = threadIdx.x / 8, c8 = threadIdx.x % 8;
+  const int row = threadIdx.x / 8, c8 = threadIdx.x % 8, nw = mask_words(K);
   for (int k0 = 0; k0 < K8; k0 += 64) {
     __syncthreads();
     for (int k = ty; k < 64; k += 8)
-      sx[k][tx] = (in && fin && k0 + k < K) ? fixed55((double)x[(k0 + k) * sk], E - balance(bal, b, k0 + k)) : 0;
+      sx[k][tx] = (in && fin && k0 + k < K) ? flagged55((double)x[(k0 + k) * sk], E - balance<BAL>(bal, b, k0 + k)) : 0;
     __syncthreads();
-    if (r0 + row < rows && k0 + c8 * 8 < K8) {
+    const int c = k0 / 8 + c8;
+    if (r0 + row < rows && c < nw * 4) {
       long long X[8];
       uint4 w[kSlices];
+      unsigned nz = 0u;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) X[e] = sx[c8 * 8 + e][row];
+      for (int e = 0; e < 8; ++e) {
+        X[e] = sx[c8 * 8 + e][row];
+        nz |= take_flag(X[e]) << e;
+      }
+      const long long r1 = (long long)b * rows + r0 + row;
+      put_sizes(mask + r1 * 2 * nw, mag + r1 * K8, nw, K8, c, sizes_of(X, nz, false));
+      if (c * 8 >= K8) continue;
       digits8(X, w);
-      const long long o = ((long long)b * rows + r0 + row) * K8 + k0 + c8 * 8;
+      const long long o = r1 * K8 + c * 8;
 #pragma unroll
       for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint4 *>(p + s * plane + o) = w[s];
     }
@@ -145,10 +228,10 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
 
 // Complex rows (see SliceOp::kind): 32 rows per block, lanes along the index that is
 // contiguous in memory, a row's eight halves (four complex values) per thread.
-template <int KIND>
+template <int KIND, bool BAL>
 __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long long sb, long long sr, long long sk,
                                                        int rows, int batch_all, int K, int K8, int sa, int sc,
-                                                       SliceBalance bal, __half *p, int *ex) {
+                                                       SliceBalance bal, __half *p, int *ex, uint32_t *mask, uint8_t *mag) {
   __shared__ long long sx[2][32][33];
   __shared__ int se[32];
   const int b = blockIdx.y, r0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
@@ -162,10 +245,10 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
       if (r0 + r < rows)
         for (int k = tx; k < K; k += 32) {
           const double2 v = x[(long long)(r0 + r) * sr + k];
-          const int sh = balance(bal, b, k);
+          const int sh = balance<BAL>(bal, b, k);
           E = max(E, max(exp_field(v.x, sh), exp_field(v.y, sh)));
         }
-      for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+      E = __reduce_max_sync(0xffffffffu, E);
       if (tx == 0) se[r] = E;
     }
   } else {
@@ -173,7 +256,7 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
     if (r0 + tx < rows)
       for (int k = ty; k < K; k += 8) {
         const double2 v = x[(long long)(r0 + tx) * sr + k * sk];
-        const int sh = balance(bal, b, k);
+        const int sh = balance<BAL>(bal, b, k);
         E = max(E, max(exp_field(v.x, sh), exp_field(v.y, sh)));
       }
     atomicMax(&se[tx], E);
@@ -181,11 +264,11 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
   __syncthreads();
   const int nr = KIND == 2 ? 2 : 1;   // real rows per complex row
   if (threadIdx.x < 32 && r0 + tx < rows) {
-    const int e = row_exp(se[tx]);
+    const int e = row_code(se[tx]);
     for (int i = 0; i < nr; ++i) ex[((long long)b * rows + r0 + tx) * nr + i] = e;
   }
   const long long plane = (long long)batch_all * rows * nr * K8;
-  const int row = threadIdx.x / 8, c8 = threadIdx.x % 8;
+  const int row = threadIdx.x / 8, c8 = threadIdx.x % 8, nw = mask_words(2 * K);
   for (int k0 = 0; 2 * k0 < K8; k0 += 32) {
     __syncthreads();
     for (int i = ty; i < 32; i += 8) {
@@ -193,34 +276,46 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
       const bool in = r0 + r < rows && k0 + k < K && E < kNonFinite;
       double2 v = make_double2(0.0, 0.0);
       if (in) v = x[(long long)(r0 + r) * sr + (k0 + k) * sk];
-      const int sh = in ? balance(bal, b, k0 + k) : 0;
-      sx[0][k][r] = in ? fixed55(v.x, E - sh) : 0;
-      sx[1][k][r] = in ? fixed55(v.y, E - sh) : 0;
+      const int sh = in ? balance<BAL>(bal, b, k0 + k) : 0;
+      sx[0][k][r] = in ? flagged55(v.x, E - sh) : 0;
+      sx[1][k][r] = in ? flagged55(v.y, E - sh) : 0;
     }
     __syncthreads();
-    if (r0 + row < rows && 2 * k0 + c8 * 8 < K8) {
-      const long long o = ((long long)b * rows + r0 + row) * nr * K8 + 2 * k0 + c8 * 8;
+    const int c = k0 / 4 + c8;
+    if (r0 + row < rows && c < nw * 4) {
+      const long long r1 = ((long long)b * rows + r0 + row) * nr;
+      long long re[4], im[4];
+      unsigned nz = 0u;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        re[e] = sx[0][c8 * 4 + e][row];
+        im[e] = sx[1][c8 * 4 + e][row];
+        nz |= (take_flag(re[e]) | take_flag(im[e])) << (2 * e);
+      }
+      Sizes sizes;
 #pragma unroll
       for (int i = 0; i < nr; ++i) {
         long long X[8];
         uint4 w[kSlices];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const long long re = sx[0][c8 * 4 + e][row], im = sx[1][c8 * 4 + e][row];
           if (KIND == 1) {
-            X[2 * e] = re;
-            X[2 * e + 1] = im;
+            X[2 * e] = re[e];
+            X[2 * e + 1] = im[e];
           } else if (i == 0) {
-            X[2 * e] = re;
-            X[2 * e + 1] = sa * sc > 0 ? -im : im;
+            X[2 * e] = re[e];
+            X[2 * e + 1] = sa * sc > 0 ? -im[e] : im[e];
           } else {
-            X[2 * e] = sc > 0 ? im : -im;
-            X[2 * e + 1] = sa > 0 ? re : -re;
+            X[2 * e] = sc > 0 ? im[e] : -im[e];
+            X[2 * e + 1] = sa > 0 ? re[e] : -re[e];
           }
         }
+        if (i == 0) sizes = sizes_of(X, nz, true);   // (of both parts: the same for either row)
+        put_sizes(mask + (r1 + i) * 2 * nw, mag + (r1 + i) * K8, nw, K8, c, sizes);
+        if (c * 8 >= K8) continue;
         digits8(X, w);
 #pragma unroll
-        for (int d = 0; d < kSlices; ++d) *reinterpret_cast<uint4 *>(p + d * plane + o + (long long)i * K8) = w[d];
+        for (int d = 0; d < kSlices; ++d) *reinterpret_cast<uint4 *>(p + d * plane + (r1 + i) * K8 + c * 8) = w[d];
       }
     }
   }
@@ -265,6 +360,9 @@ struct Args {
   int nL, nW, K, batch, tL, tW;
   int bL, bW;                // batches of the operands (1: shared)
   const int *eL, *eW;
+  const uint32_t *mL, *mW;   // bit masks, twice mw words a row
+  const uint8_t *gL, *gW;    // magnitudes, kw words a row
+  int mw, kw;
   double *C;
   long long sC, cl, cw;
   double alpha, beta;
@@ -397,30 +495,118 @@ __device__ double plain_at(const Plain &p, long long b, int r, int k) {
   if (!(r & 1)) return (k & 1) ? -p.sa * p.sc * v.y : v.x;
   return (k & 1) ? p.sa * v.x : p.sc * v.y;
 }
-// the element as a chain of FP64 FMAs from the sources (rows with infinities or NaNs)
-__device__ __noinline__ double plain_element(const Args &a, int b, int l, int w) {
+// Elements summed in FP64 from the sources, by a warp whose lanes hold the rows l0 + lane of the lane side
+// and kC columns from w0.  A few: one at a time, the lanes over k.  Many: all columns in one pass over k,
+// which the FP64 pipe bounds as it would a product that never saw digits.
+constexpr int kFew = 32;
+__device__ __noinline__ double plain_element(const Args &a, int b, int l, int w, int lane) {
   double acc = 0.0;
-  for (int k = 0; k < a.K; ++k)
+  for (int k = lane; k < a.K; k += 32)
     acc = fma(plain_at(a.xL, a.bL == 1 ? 0 : b, l, k), plain_at(a.xW, a.bW == 1 ? 0 : b, w, k), acc);
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   return acc;
 }
+template <int C>
+__device__ __noinline__ void plain_block(const Args &a, int b, int l, int w0, double *out) {
+  double acc[C] = {};
+  const bool in = l < a.nL;
+  for (int k = 0; k < a.K; ++k) {
+    const double x = in ? plain_at(a.xL, a.bL == 1 ? 0 : b, l, k) : 0.0;
+#pragma unroll
+    for (int j = 0; j < C; ++j)
+      if (w0 + j < a.nW) acc[j] = fma(x, plain_at(a.xW, a.bW == 1 ? 0 : b, w0 + j, k), acc[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < C; ++j) out[j] = acc[j];
+}
 
-// I 2^x rounded to nearest even, from integer instructions (a 64-bit conversion and a
-// scaling would cost the FP64 pipe more than all products of the element did).  False, and no
-// value, for a row with infinities or NaNs (x then lies beyond any exponent) and for results
-// outside the normal range: those elements are recomputed from the sources.
-__device__ __forceinline__ bool scaled_double(long long I, int x, double &v) {
+// Bit j: |I[j]| below 2^-kSignif of the scales
+template <int LK, int C>
+__device__ __forceinline__ unsigned small_sums(const long long (&I)[C]) {
+  unsigned m = 0u;
+#pragma unroll
+  for (int j = 0; j < C; ++j) {
+    const int hi = (int)(I[j] >> 32);
+    m |= (unsigned)(hi ^ (hi >> 31)) < (1u << (30 - LK - kSignif)) ? 1u << j : 0u;
+  }
+  return m;
+}
+// What the checks read of a row: its masks (two of mw words) and magnitudes (words of four)
+struct RowSizes {
+  const uint32_t *mask, *mag;
+};
+// The columns of `small` whose S may be small too: none where the magnitudes' products sum to 2^-kSignif
+// of the scales, or where no k is nonzero in both rows (an exact zero).  L: the lane's row; W: column
+// `lane`; l0, w0: the first words of their masks.
+__device__ __forceinline__ RowSizes row_sizes(const uint32_t *mask, const uint8_t *mag, long long row, int mw, int kw) {
+  return {mask + row * 2 * mw, reinterpret_cast<const uint32_t *>(mag) + row * kw};
+}
+template <int C>
+__device__ __noinline__ unsigned unsettled_rest(unsigned small, RowSizes L, RowSizes W, int mw, int kw) {
+  unsigned sum[C], some = 0u;
+#pragma unroll
+  for (int j = 0; j < C; ++j) sum[j] = 0u;
+  const uint2 *l = reinterpret_cast<const uint2 *>(L.mag), *w = reinterpret_cast<const uint2 *>(W.mag);
+  constexpr int kStep = 4;   // pairs of words at a time; most columns are settled by the first
+  for (int i = 0; i < kw / 2; i += kStep) {
+    const unsigned any = __reduce_or_sync(0xffffffffu, small);   // columns to look at, the same for all lanes
+    if (any == 0u) return 0u;
+    uint2 x[kStep], y[kStep];
+#pragma unroll
+    for (int t = 0; t < kStep; ++t) {
+      x[t] = i + t < kw / 2 ? l[i + t] : make_uint2(0u, 0u);
+      y[t] = i + t < kw / 2 ? w[i + t] : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+      if (!((any >> j) & 1u)) continue;
+#pragma unroll
+      for (int t = 0; t < kStep; ++t) {
+        sum[j] = __dp4a(x[t].x, __shfl_sync(0xffffffffu, y[t].x, j), sum[j]);
+        sum[j] = __dp4a(x[t].y, __shfl_sync(0xffffffffu, y[t].y, j), sum[j]);
+      }
+      if (sum[j] >= 1u << (16 - kSignif)) small &= ~(1u << j);
+    }
+  }
+  if (!__any_sync(0xffffffffu, small != 0u)) return 0u;
+  for (int i = 0; i < mw; ++i) {
+    const uint32_t l = L.mask[mw + i], w = W.mask[mw + i];
+#pragma unroll
+    for (int j = 0; j < C; ++j) some |= (l & __shfl_sync(0xffffffffu, w, j)) ? 1u << j : 0u;
+  }
+  return small & some;
+}
+template <int C>
+__device__ __forceinline__ unsigned unsettled(unsigned small, RowSizes L, RowSizes W, uint32_t l0, uint32_t w0, int mw,
+                                              int kw) {
+  for (int i = 0; __any_sync(0xffffffffu, small != 0u);) {
+#pragma unroll
+    for (int j = 0; j < C; ++j) small &= (l0 & __shfl_sync(0xffffffffu, w0, j)) ? ~(1u << j) : ~0u;
+    if (++i == mw) break;
+    l0 = L.mask[i];
+    w0 = W.mask[i];
+  }
+  return __any_sync(0xffffffffu, small != 0u) ? unsettled_rest<C>(small, L, W, mw, kw) : 0u;
+}
+
+// I 2^x rounded to nearest even, x from the codes of the two rows, by integer instructions (a 64-bit
+// conversion and a scaling would cost the FP64 pipe more than all products of the element did).
+// False, and no value, for infinities or NaNs in a row and for a result outside the normal range:
+// those elements are summed from the sources.
+template <int LK>
+__device__ __forceinline__ bool scaled_double(long long I, int code, double &v) {
   const unsigned long long u = I < 0 ? 0ull - (unsigned long long)I : (unsigned long long)I;
   const int lz = __clzll((long long)(u | 1));
   const unsigned long long m = u << lz;
   unsigned long long r = m >> 11;
   const unsigned rem = (unsigned)m & 0x7ffu;
   r += (rem + (unsigned)(r & 1)) > 0x400u ? 1u : 0u;
+  const int x = (code & 0xffff) - 2 * kCodeBias - 2044 - (62 - LK);
   const int eb = 63 - lz + x + 1023;   // biased exponent of the leading bit
   const unsigned long long b =
       ((unsigned long long)(eb - 1) << 52) + r + (I < 0 ? 0x8000000000000000ull : 0ull);
   v = I == 0 ? 0.0 : __longlong_as_double((long long)b);
-  return I == 0 ? x < kNonFinite / 2 : (unsigned)(eb - 1) <= 2044u;
+  return code < kCodeNonFinite && (I == 0 || (unsigned)(eb - 1) <= 2044u);
 }
 
 // What happens to an element on its way out: +-v, C +- v, or alpha v + beta C.  A template
@@ -538,6 +724,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       // exponents of this lane's row and of column w0 + lane (handed round by shuffles)
       const int eL = l < a.nL ? a.eL[(a.bL == 1 ? 0LL : (long long)b * a.nL) + l] : 0;
       const int eWl = lane < kC && w0 + lane < a.nW ? a.eW[(a.bW == 1 ? 0LL : (long long)b * a.nW) + w0 + lane] : 0;
+      const RowSizes sL = row_sizes(a.mL, a.gL, (a.bL == 1 ? 0LL : (long long)b * a.nL) + min(l, a.nL - 1), a.mw, a.kw);
+      const RowSizes sW =
+          row_sizes(a.mW, a.gW, (a.bW == 1 ? 0LL : (long long)b * a.nW) + min(w0 + lane % kC, a.nW - 1), a.mw, a.kw);
+      const uint32_t mL0 = sL.mask[0], mW0 = sW.mask[0];
       long long acc[kC];
 #pragma unroll
       for (int j = 0; j < kC; ++j) acc[j] = 0;
@@ -553,7 +743,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       double *Cm = a.C + b * a.sC + w0 * a.cl + l * a.cw;   // mirror image
       const bool mir = a.mirror && a.mirror[b];
       const long long sign = a.alpha < 0.0 ? (long long)0x8000000000000000ull : 0ll;
-      unsigned odd = 0u;   // columns to recompute from the sources
+      const int live = l < a.nL ? min(kC, a.nW - w0) : 0;
+      // columns to sum from the sources
+      unsigned odd = unsettled<kC>(small_sums<LK>(acc) & (live > 0 ? (1u << live) - 1u : 0u), sL, sW, mL0, mW0, a.mw, a.kw);
       constexpr int kH = 8;   // C is read eight columns at a time, all loads before the first store
 #pragma unroll
       for (int j0 = 0; j0 < kC; j0 += kH) {
@@ -567,7 +759,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int j = j0 + i, w = w0 + j;
           const int eW = __shfl_sync(0xffffffffu, eWl, j);
           double v;
-          const bool fine = scaled_double(acc[j], eL + eW - 2044 - (62 - LK), v);
+          const bool fine = scaled_double<LK>(acc[j], eL + eW, v) && !((odd >> j) & 1u);
           if (l < a.nL && w < a.nW) {
             if (fine) {
               v = out_value<OUT>(v, sign, old[i], a.alpha, a.beta);
@@ -584,14 +776,30 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      while (odd) {
-        const int j = __ffs((int)odd) - 1, w = w0 + j;
-        odd &= odd - 1;
-        double v = a.alpha * plain_element(a, b, l, w);
+      const int left = __reduce_add_sync(0xffffffffu, __popc(odd));
+      if (left == 0) continue;
+      auto put = [&](int j, double x) {
+        const int w = w0 + j;
+        double v = a.alpha * x;
         if (a.beta != 0.0) v = fma(a.beta, C[j * a.cw], v);
         const int ib = (a.lane_is_row ? l : w) / 32, jb = (a.lane_is_row ? w : l) / 32;
         if (!mir || ib <= jb) C[j * a.cw] = v;
         if (mir && ib < jb) Cm[j * a.cl] = v;
+      };
+      if (left > kFew) {
+        double x[kC];
+        plain_block<kC>(a, b, l, w0, x);
+        for (int j = 0; j < kC; ++j)
+          if ((odd >> j) & 1u) put(j, x[j]);
+        continue;
+      }
+      for (unsigned who; (who = __ballot_sync(0xffffffffu, odd != 0u)) != 0u;) {
+        const int from = __ffs((int)who) - 1, j = __shfl_sync(0xffffffffu, __ffs((int)odd) - 1, from);
+        const double x = plain_element(a, b, l - lane + from, w0 + j, lane);
+        if (lane == from) {
+          put(j, x);
+          odd &= odd - 1;
+        }
       }
     }
   }
@@ -626,6 +834,9 @@ struct FBars {
 struct FArgs {
   int n, N, batch, v0, v1, tP, tR;
   const int *eA, *eGR, *eGW, *eU;   // [b][v][P], [b][R], [b][P], [v][R]
+  const uint32_t *mA, *mGR, *mGW, *mU;
+  const uint8_t *gA, *gGR, *gGW, *gU;
+  int mw, kw;
   double *D;
   long long sD;
   // sources, for rows with infinities or NaNs: A[b][v][P][q], GR[b][R][q], GW[b][P][w], U2[R][v][w]
@@ -635,10 +846,45 @@ struct FArgs {
   int *status;
 };
 
-__device__ __noinline__ double plain_row_dot(const double *x, const double *y, int n) {
-  double acc = 0.0;
-  for (int k = 0; k < n; ++k) acc = fma(x[k], y[k], acc);
-  return acc;
+// the same two ways as plain_element and plain_block, for B_v and C_v at once (contiguous sources)
+__device__ __forceinline__ void plain_rows(const FArgs &a, int b, int v, int P, int R, const double *(&x)[4]) {
+  x[0] = a.xA + (((long long)b * a.nv + v) * a.N + P) * a.n;
+  x[1] = a.xGR + ((long long)b * a.N + R) * a.n;
+  x[2] = a.xGW + ((long long)b * a.N + P) * a.n;
+  x[3] = a.xU + ((long long)R * a.nv + v) * a.n;
+}
+__device__ __noinline__ double2 plain_bc(const FArgs &a, int b, int v, int P, int R, int lane) {
+  const double *x[4];
+  plain_rows(a, b, v, P, R, x);
+  double2 s = make_double2(0.0, 0.0);
+  for (int k = lane; k < a.n; k += 32) {
+    s.x = fma(x[0][k], x[1][k], s.x);
+    s.y = fma(x[2][k], x[3][k], s.y);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+  }
+  return s;
+}
+template <int C>
+__device__ __noinline__ void plain_bc_block(const FArgs &a, int b, int v, int P, int R0, double2 *out) {
+  double2 s[C];
+  const double *x[4];
+#pragma unroll
+  for (int j = 0; j < C; ++j) s[j] = make_double2(0.0, 0.0);
+  plain_rows(a, b, v, min(P, a.N - 1), 0, x);
+  for (int k = 0; k < a.n; ++k) {
+    const double p = x[0][k], q = x[2][k];
+#pragma unroll
+    for (int j = 0; j < C; ++j)
+      if (R0 + j < a.N) {
+        s[j].x = fma(p, x[1][(long long)(R0 + j) * a.n + k], s[j].x);
+        s[j].y = fma(q, x[3][(long long)(R0 + j) * a.nv * a.n + k], s[j].y);
+      }
+  }
+#pragma unroll
+  for (int j = 0; j < C; ++j) out[j] = s[j];
 }
 
 template <int LK>
@@ -759,6 +1005,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int cols = min(kC, a.N - R0);   // columns of this warp inside the tile (<= 0: none)
       const int eW = in ? a.eGW[(long long)b * a.N + P] : 0;
       const int eRl = lane < cols ? a.eGR[(long long)b * a.N + R0 + lane] : 0;
+      const unsigned live = in && cols > 0 ? (1u << cols) - 1u : 0u;
+      const int Pm = min(P, a.N - 1), Rm = min(R0 + lane % kC, a.N - 1);   // rows of the masks
+      const RowSizes sR = row_sizes(a.mGR, a.gGR, (long long)b * a.N + Rm, a.mw, a.kw);
+      const RowSizes sW = row_sizes(a.mGW, a.gGW, (long long)b * a.N + Pm, a.mw, a.kw);
+      const uint32_t mR0 = sR.mask[0], mW0 = sW.mask[0];
       bool ok = true;
       for (int v = a.v0; v < a.v1 && ok; ++v) {
         long long ib[kC], ic[kC];
@@ -766,6 +1017,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < kC; ++j) ib[j] = ic[j] = 0;
         const int eA = in ? a.eA[((long long)b * a.nv + v) * a.N + P] : 0;
         const int eUl = lane < cols ? a.eU[(long long)v * a.N + R0 + lane] : 0;
+        const RowSizes sA = row_sizes(a.mA, a.gA, ((long long)b * a.nv + v) * a.N + Pm, a.mw, a.kw);
+        const RowSizes sU = row_sizes(a.mU, a.gU, (long long)v * a.N + Rm, a.mw, a.kw);
+        const uint32_t mA0 = sA.mask[0], mU0 = sU.mask[0];
         for (int h = 0; h < 2 && ok; ++h)
           for (int w = 0; w < nwin; ++w) {
             ok = tc::mbar_wait_warp(&bar->acc_full[h], (uint32_t)((win + w) & 1), limit, abort, a.status, 8);
@@ -779,27 +1033,36 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         win += nwin;
         if (!ok) break;
-        unsigned odd = 0u;   // columns to recompute from the sources
+        // columns to sum from the sources
+        unsigned odd = unsettled<kC>(small_sums<LK>(ib) & live, sA, sR, mA0, mR0, a.mw, a.kw) |
+                       unsettled<kC>(small_sums<LK>(ic) & live, sW, sU, mW0, mU0, a.mw, a.kw);
 #pragma unroll
         for (int j = 0; j < kC; ++j) {
           const int eR = __shfl_sync(0xffffffffu, eRl, j), eU = __shfl_sync(0xffffffffu, eUl, j);
           double bv, cv;
-          const bool fb = scaled_double(ib[j], eA + eR - 2044 - (62 - LK), bv);
-          const bool fc = scaled_double(ic[j], eW + eU - 2044 - (62 - LK), cv);
-          if (fb && fc)
+          const bool fb = scaled_double<LK>(ib[j], eA + eR, bv);
+          const bool fc = scaled_double<LK>(ic[j], eW + eU, cv);
+          if (!(fb && fc))
+            odd |= live & (1u << j);
+          else if (!((odd >> j) & 1u))
             d[j] = fma(bv, cv, d[j]);
-          else
-            odd |= 1u << j;
         }
-        if (odd && in) {
+        const int left = __reduce_add_sync(0xffffffffu, __popc(odd));
+        if (left > kFew) {
+          double2 x[kC];
+          plain_bc_block<kC>(a, b, v, P, R0, x);
 #pragma unroll
           for (int j = 0; j < kC; ++j)
-            if (((odd >> j) & 1u) && j < cols)
-              d[j] = fma(plain_row_dot(a.xA + (((long long)b * a.nv + v) * a.N + P) * a.n,
-                                       a.xGR + ((long long)b * a.N + R0 + j) * a.n, a.n),
-                         plain_row_dot(a.xGW + ((long long)b * a.N + P) * a.n,
-                                       a.xU + ((long long)(R0 + j) * a.nv + v) * a.n, a.n),
-                         d[j]);
+            if ((odd >> j) & 1u) d[j] = fma(x[j].x, x[j].y, d[j]);
+        } else if (left > 0) {
+          for (unsigned who; (who = __ballot_sync(0xffffffffu, odd != 0u)) != 0u;) {
+            const int from = __ffs((int)who) - 1, at = __shfl_sync(0xffffffffu, __ffs((int)odd) - 1, from);
+            const double2 x = plain_bc(a, b, v, P - lane + from, R0 + at, lane);
+#pragma unroll
+            for (int j = 0; j < kC; ++j)
+              if (lane == from && j == at) d[j] = fma(x.x, x.y, d[j]);
+            if (lane == from) odd &= odd - 1;
+          }
         }
       }
       if (!ok) break;
@@ -853,7 +1116,8 @@ inline size_t al(size_t b) { return (b + 255) & ~size_t(255); }
 }  // namespace
 
 size_t slice_bytes(long long batch, int rows, int K) {
-  return al((size_t)kSlices * batch * rows * round8(K) * 2) + al((size_t)batch * rows * 4);
+  return al((size_t)kSlices * batch * rows * round8(K) * 2) + al((size_t)batch * rows * 4) +
+         al((size_t)batch * rows * 2 * mask_words(K) * 4) + al((size_t)batch * rows * round8(K));
 }
 
 SliceOp slice_take(Arena &ar, int batch, int rows, int K) {
@@ -864,7 +1128,9 @@ SliceOp slice_take(Arena &ar, int batch, int rows, int K) {
   op.K8 = round8(K);
   op.p = ar.take<__half>((size_t)kSlices * batch * rows * op.K8);
   op.ex = ar.take<int>((size_t)batch * rows);
-  if (!op.ex) op.p = nullptr;
+  op.mask = ar.take<uint32_t>((size_t)batch * rows * 2 * mask_words(K));
+  op.mag = ar.take<uint8_t>((size_t)batch * rows * op.K8);
+  if (!op.mag) op.p = nullptr;
   return op;
 }
 
@@ -876,25 +1142,27 @@ void slice_rows(const void *src, bool f32, long long sb, long long sr, long long
   op.sr = sr;
   op.sk = sk;
   if (batch <= 0 || op.rows <= 0) return;
-  if (sk == 1) {
-    int lpr = 4;
-    while (lpr < 32 && lpr * 8 < op.K8) lpr *= 2;
-    const long long blocks = ((long long)batch * op.rows * lpr + 255) / 256;
-    if (f32)
-      k_slice_rows<float><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const float *>(src), sb, sr, op.rows, batch,
-                                                         op.batch, op.K, op.K8, lpr, bal, op.p, op.ex);
-    else
-      k_slice_rows<double><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const double *>(src), sb, sr, op.rows, batch,
-                                                          op.batch, op.K, op.K8, lpr, bal, op.p, op.ex);
-  } else {
-    const dim3 grid((op.rows + 31) / 32, batch);
-    if (f32)
-      k_slice_cols<float><<<grid, 256, 0, s>>>(static_cast<const float *>(src), sb, sr, sk, op.rows, op.batch, op.K,
-                                               op.K8, bal, op.p, op.ex);
-    else
-      k_slice_cols<double><<<grid, 256, 0, s>>>(static_cast<const double *>(src), sb, sr, sk, op.rows, op.batch, op.K,
-                                                op.K8, bal, op.p, op.ex);
-  }
+  auto go = [&](auto t, auto bl) {
+    using T = decltype(t);
+    constexpr bool BAL = decltype(bl)::value;
+    const T *x = static_cast<const T *>(src);
+    if (sk == 1) {
+      int lpr = 4;
+      while (lpr < 32 && lpr * 8 < op.K8) lpr *= 2;
+      const long long blocks = ((long long)batch * op.rows * lpr + 255) / 256;
+      k_slice_rows<T, BAL><<<(unsigned)blocks, 256, 0, s>>>(x, sb, sr, op.rows, batch, op.batch, op.K, op.K8, lpr, bal, op.p,
+                                                            op.ex, op.mask, op.mag);
+    } else {
+      k_slice_cols<T, BAL><<<dim3((op.rows + 31) / 32, batch), 256, 0, s>>>(x, sb, sr, sk, op.rows, op.batch, op.K, op.K8,
+                                                                            bal, op.p, op.ex, op.mask, op.mag);
+    }
+  };
+  if (f32)
+    go(float{}, std::false_type{});   // (no FP32 operand is balanced)
+  else if (bal.kex)
+    go(double{}, std::true_type{});
+  else
+    go(double{}, std::false_type{});
 }
 
 void slice_complex_a(const double *src, long long sb, long long sr, long long sk, int batch, SliceOp &op, cudaStream_t s,
@@ -903,8 +1171,9 @@ void slice_complex_a(const double *src, long long sb, long long sr, long long sk
   op.sb = sb; op.sr = sr; op.sk = sk;
   op.kind = 1;
   if (batch <= 0 || op.rows <= 0) return;
-  k_slice_complex<1><<<dim3((op.rows + 31) / 32, batch), 256, 0, s>>>(
-      reinterpret_cast<const double2 *>(src), sb, sr, sk, op.rows, op.batch, op.K / 2, op.K8, 1, 1, bal, op.p, op.ex);
+  auto *k = bal.kex ? k_slice_complex<1, true> : k_slice_complex<1, false>;
+  k<<<dim3((op.rows + 31) / 32, batch), 256, 0, s>>>(reinterpret_cast<const double2 *>(src), sb, sr, sk, op.rows, op.batch,
+                                                     op.K / 2, op.K8, 1, 1, bal, op.p, op.ex, op.mask, op.mag);
 }
 
 void slice_complex_b(const double *src, long long sb, long long sr, long long sk, int batch, bool conjA, bool conjB,
@@ -916,8 +1185,9 @@ void slice_complex_b(const double *src, long long sb, long long sr, long long sk
   op.sc = conjB ? -1 : 1;
   if (batch <= 0 || op.rows <= 0) return;
   const int rows = op.rows / 2;
-  k_slice_complex<2><<<dim3((rows + 31) / 32, batch), 256, 0, s>>>(
-      reinterpret_cast<const double2 *>(src), sb, sr, sk, rows, op.batch, op.K / 2, op.K8, op.sa, op.sc, bal, op.p, op.ex);
+  auto *k = bal.kex ? k_slice_complex<2, true> : k_slice_complex<2, false>;
+  k<<<dim3((rows + 31) / 32, batch), 256, 0, s>>>(reinterpret_cast<const double2 *>(src), sb, sr, sk, rows, op.batch,
+                                                  op.K / 2, op.K8, op.sa, op.sc, bal, op.p, op.ex, op.mask, op.mag);
 }
 
 Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceGemm &g, cudaStream_t s) {
@@ -937,6 +1207,10 @@ Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceG
   a.tW = (W.rows + kW - 1) / kW;
   a.bL = L.batch; a.bW = W.batch;
   a.eL = L.ex; a.eW = W.ex;
+  a.mL = L.mask; a.mW = W.mask;
+  a.gL = L.mag; a.gW = W.mag;
+  a.mw = mask_words(A.K);
+  a.kw = A.K8 / 4;
   a.C = g.C; a.sC = g.sC;
   a.cl = lane_a ? g.ci : g.cj;
   a.cw = lane_a ? g.cj : g.ci;
@@ -983,6 +1257,10 @@ Status slice_bcd(sox_handle h, const SliceOp &A, const SliceOp &GR, const SliceO
   a.tP = (N + kL - 1) / kL;
   a.tR = (N + kFW - 1) / kFW;
   a.eA = A.ex; a.eGR = GR.ex; a.eGW = GW.ex; a.eU = U2.ex;
+  a.mA = A.mask; a.mGR = GR.mask; a.mGW = GW.mask; a.mU = U2.mask;
+  a.gA = A.mag; a.gGR = GR.mag; a.gGW = GW.mag; a.gU = U2.mag;
+  a.mw = mask_words(n);
+  a.kw = A.K8 / 4;
   a.D = D; a.sD = sD;
   a.xA = static_cast<const double *>(A.src);
   a.xGR = static_cast<const double *>(GR.src);

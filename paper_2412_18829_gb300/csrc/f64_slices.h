@@ -2,11 +2,13 @@
 //
 // Each row of an operand (its K elements) is scaled by a power of two and written as seven
 // 8-bit signed digits, x = 2^e sum_i d_i 2^-(8 i + 7), |d_i| <= 128, each digit an FP16
-// integer.  Digit products d_i d_j are exact in the tensor core, and so are their FP32 sums
-// over 128 elements (at most 7 * 128 * 2^14 < 2^24).  Products with equal i + j share one
-// accumulator; i + j <= 7 are kept (34 of 49).  The eight sums are added as 64-bit integers
-// and rounded to FP64 once.  What is dropped lies below 2^-63 of (row maximum x column
-// maximum) per term, so the result is closer to the exact sum than a chain of FP64 FMAs.
+// integer: fixed point to 2^-55 of the row's largest element.  Digit products d_i d_j are exact in the
+// tensor core, and so are their FP32 sums over 128 elements (at most 7 * 128 * 2^14 < 2^24).  Products
+// with equal i + j share one accumulator; i + j <= 7 are kept (34 of 49).  The eight sums are added as
+// 64-bit integers and rounded to FP64 once.  An element's error is below (1.1 K + 9) 2^-54 of the product
+// of the two rows' largest elements: for rows of similar elements less than a chain of FP64 FMAs makes.
+// Elements whose terms may all be far smaller than that product (their magnitudes' sum S below 2^-6 of
+// it) are summed in FP64 from the sources, so the error is also below (1.1 K + 9) 2^-48 S.
 // This is the Ozaki splitting (error-free transformation of a matrix product into exact
 // lower-precision ones; Ozaki, Ogita, Oishi and Rump, 2012), with the digits on the K-major
 // operand layout of tcgen05.
@@ -20,12 +22,14 @@ namespace sox {
 constexpr int kSlices = 7;
 
 // A sliced operand: `batch` blocks of `rows` rows of K elements, digit s of (b, r, k) at
-// p[((s * batch + b) * rows + r) * K8 + k]; ex[b * rows + r] the row's exponent (kNonFinite:
-// the row holds an infinity or a NaN).  src and its strides stay readable until the products
-// that use the operand are done.
+// p[((s * batch + b) * rows + r) * K8 + k]; ex[b * rows + r] the row's exponent
+// (f64_slices.cu, row_code), mask and mag the elements' sizes within it.  src stays readable,
+// and unchanged, until the products that use the operand are done: they sum some elements from it.
 struct SliceOp {
   __half *p = nullptr;
   int *ex = nullptr;
+  uint32_t *mask = nullptr;
+  uint8_t *mag = nullptr;
   int batch = 0, rows = 0, K = 0, K8 = 0;
   const void *src = nullptr;
   bool f32 = false;
@@ -37,13 +41,22 @@ struct SliceOp {
 };
 size_t slice_bytes(long long batch, int rows, int K);
 SliceOp slice_take(Arena &ar, int batch, int rows, int K);
-// Powers of two along the inner index: operand A of a product times 2^e_k, B times 2^-e_k, with e_k from
-// the exponent fields kex[b * stride + k] (0: none) and sgn = 1 for A, -1 for B.  The product is the
-// same; a K index that is large in one operand and small in the other keeps its digits in both.
+// Powers of two along the inner index: operand A of a product times 2^e_k, B times 2^-e_k, with e_k =
+// (kex[b * stride + k] - 1023) / part from exponent fields (0: none); part > 0 for A, the negative for
+// B.  The product is the same; a K index that is large in one operand and small in the other keeps its
+// digits in both.  kex holds B's largest exponents: part 1 where A's elements fall as B's rise (rows of a
+// factored system), 2 where they do not depend on them (the range is then shared).
 struct SliceBalance {
   const int *kex = nullptr;
-  int stride = 0, sgn = 0;
+  int stride = 0, part = 1;
 };
+// what goes into kex: the exponent field of a finite value, 0 for zeros, infinities and NaNs (the
+// greatest one along index k of B, by atomicMax on zeroed memory)
+__device__ __forceinline__ int balance_exponent(double a) {
+  const int hi = __double2hiint(a), e = (hi >> 20) & 0x7ff;
+  if (e == 0x7ff || (((hi & 0x7fffffff) | __double2loint(a)) == 0)) return 0;
+  return max(e, 1);
+}
 // digits of element (b, r, k) = src[b * sb + r * sr + k * sk], FP64 or FP32; `batch` blocks
 // (at most op's)
 void slice_rows(const void *src, bool f32, long long sb, long long sr, long long sk, int batch, SliceOp &op,

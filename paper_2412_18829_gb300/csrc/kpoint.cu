@@ -41,6 +41,7 @@ struct ZGemm {
   const z *B; long long sB, bk, bj; const long long *offB; int conjB;
   z *C; long long sC, ci, cj; const long long *offC;
   double alpha, beta;
+  const int *kex;   // optional: exponents along k that the digits are balanced by (f64_slices.h)
 };
 
 __global__ void __launch_bounds__(NT) k_zgemm(ZGemm g) {
@@ -148,15 +149,17 @@ Status zgemm_f64(sox_handle h, const ZGemm &g, Arena scratch, cudaStream_t s) {
   for (int k0 = 0; k0 < g.K; k0 += p.k)
     for (int b0 = 0; b0 < g.batch; b0 += p.nb) {
       const int k = std::min(p.k, g.K - k0), nb = std::min(p.nb, g.batch - b0);
+      const SliceBalance up{g.kex ? g.kex + k0 : nullptr, 0, 2}, down{up.kex, 0, -2};
       Arena ar = scratch;
       SliceOp A = slice_take(ar, p.sharedA ? 1 : nb, g.M, 2 * k);
       if (!A.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-      slice_complex_a(d(g.A + b0 * g.sA + k0 * g.ak), g.sA, g.ai, g.ak, A.batch, A, s);
+      slice_complex_a(d(g.A + b0 * g.sA + k0 * g.ak), g.sA, g.ai, g.ak, A.batch, A, s, up);
       for (int j0 = 0; j0 < g.Nc; j0 += p.rows) {
         Arena br = ar;
         SliceOp B = slice_take(br, p.sharedB ? 1 : nb, 2 * std::min(p.rows, g.Nc - j0), 2 * k);
         if (!B.p) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-        slice_complex_b(d(g.B + b0 * g.sB + k0 * g.bk + j0 * g.bj), g.sB, g.bj, g.bk, B.batch, g.conjA, g.conjB, B, s);
+        slice_complex_b(d(g.B + b0 * g.sB + k0 * g.bk + j0 * g.bj), g.sB, g.bj, g.bk, B.batch, g.conjA, g.conjB, B, s,
+                        down);
         SliceGemm sg;
         sg.C = reinterpret_cast<double *>(g.C + b0 * g.sC + j0);
         sg.sC = 2 * g.sC; sg.ci = 2 * g.ci; sg.cj = 1;
@@ -1329,8 +1332,10 @@ __global__ void __launch_bounds__(256) k_bubble_reduce(const z *Ah, const z *Tf,
 }
 
 // Pr[j][P][Q] = Ah[m][j][P][Q] Ah[-m][T-1-j][Q][P] for one m: 32 x 32 tiles, the transposed
-// partner through shared memory.  The sum over j with the transform is then one product.
-__global__ void __launch_bounds__(256) k_bubble_pairs(const z *Am, const z *Bm, int N, int T, z *Pr) {
+// partner through shared memory.  The sum over j with the transform is then one product; kex[j] is
+// raised to the largest exponent of Pr[j], which spans many powers of two over the times while the
+// transform's rows do not.
+__global__ void __launch_bounds__(256) k_bubble_pairs(const z *Am, const z *Bm, int N, int T, z *Pr, int *kex) {
   __shared__ z tb[32][33];
   const int j = blockIdx.z, P0 = blockIdx.y * 32, Q0 = blockIdx.x * 32;
   const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
@@ -1339,13 +1344,18 @@ __global__ void __launch_bounds__(256) k_bubble_pairs(const z *Am, const z *Bm, 
   for (int r = ty; r < 32; r += 8)
     if (Q0 + r < N && P0 + tx < N) tb[r][tx] = Bj[(long long)(Q0 + r) * N + P0 + tx];   // tb[Q][P]
   __syncthreads();
+  int top = 0;
   for (int r = ty; r < 32; r += 8) {
     const int P = P0 + r, Q = Q0 + tx;
     if (P < N && Q < N) {
       const long long e = (long long)j * NN + (long long)P * N + Q;
-      Pr[e] = zmul(Am[e], tb[tx][r]);
+      const z v = zmul(Am[e], tb[tx][r]);
+      Pr[e] = v;
+      top = max(top, max(balance_exponent(v.x), balance_exponent(v.y)));
     }
   }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (tx == 0 && top > 0) atomicMax(kex + j, top);
 }
 
 // molecules: Pi(i Omega) <- (Re Pi + Re Pi^T) / 2 in place, per frequency
@@ -1533,7 +1543,7 @@ size_t w_dynamic_bytes(const sox_problem *p, int n_omega) {
   // scratch of the products, the bubble's pairs (one m at a time) and the solve
   size_t scratch = std::max(zgemm_bytes(Ni, ni, ni, Ti, true, false), zgemm_bytes(Ni, Ni, ni, Ti, false, true));
   scratch = std::max(scratch, zgemm_bytes(Ni, Ni, Ni, n_omega, true, false));
-  scratch = std::max(scratch, aligned_bytes(T * NN, 16) + zgemm_bytes(n_omega, (int)NN, Ti, 1, true, true));
+  scratch = std::max(scratch, aligned_bytes(T * NN, 16) + aligned_bytes(nk * T, 4) + zgemm_bytes(n_omega, (int)NN, Ti, 1, true, true));
   if (lu_pays(Ni)) scratch = std::max(scratch, lu_bytes(Ni, (int)nk * n_omega, true));
   return b + scratch + (1 << 20);
 }
@@ -1626,16 +1636,19 @@ Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *
       // transform on the FP64 pipe inside the reduction 47 ms
       Arena pa = ar;
       z *Pr = pa.take<z>((size_t)T * NN);
-      if (!Pr) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+      int *kex = pa.take<int>((size_t)nk * T);
+      if (!kex) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
+      SOX_CUDA_TRY(cudaMemsetAsync(kex, 0, sizeof(int) * (size_t)nk * T, s));
       for (int m = 0; m < nk; ++m) {
         k_bubble_pairs<<<dim3((N + 31) / 32, (N + 31) / 32, T), 256, 0, s>>>(
-            Ah + (long long)m * T * NN, Ah + (long long)h_neg[m] * T * NN, N, T, Pr);
+            Ah + (long long)m * T * NN, Ah + (long long)h_neg[m] * T * NN, N, T, Pr, kex + (size_t)m * T);
         ZGemm f = zg();   // H[m][o] += alpha sum_j T_fwd[o][j] Pr[j]
         f.M = ns; f.Nc = (int)NN; f.K = T;
         f.A = Tf; f.ai = T; f.ak = 1;
         f.B = Pr; f.bk = NN; f.bj = 1;
         f.C = H + (long long)m * nO * NN; f.ci = NN; f.cj = 1;
         f.alpha = -1.0 / ((double)nk * nk); f.beta = 1.0;
+        f.kex = kex + (size_t)m * T;
         SOX_TRY(zgemm_f64(h, f, pa, s));
       }
       launches += 2 * nk + 3;

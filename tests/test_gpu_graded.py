@@ -3,6 +3,8 @@ accuracy relative to the sum of the magnitudes of an element's terms, not to the
 import numpy as np
 import pytest
 
+import synth
+from oracle import sox as osox
 from gpu_common import pkg_built, to_dev, torch_cuda
 
 pytestmark = pytest.mark.gpu
@@ -83,3 +85,82 @@ def test_w_static_of_subnormal_values(env, N):
     pkg.sox_check_device(h)
     bound = 8 * N * np.linalg.cond(K.astype(float)) * (2.0 ** -53 * np.abs(ref).max() + LD(2.0) ** -1074)
     assert (np.abs(W.cpu().numpy() - ref) <= bound).all()
+
+
+@pytest.mark.parametrize("nk,n,N", [((2, 1, 1), 5, 97), ((1, 1, 3), 4, 130)])
+def test_w_dynamic_of_a_graded_basis(env, nk, n, N):
+    """Rows of X times D and V between D^-2 and D^-2, D powers of two: the bubble has two factors of X per
+    index, so W is D^-2 W D^-2, to the bound of the ungraded call (1e-10 of the largest)."""
+    torch, pkg, h = env
+    rng = np.random.default_rng(N)
+    w = synth.solid(140, nk, n, N, 6, 20.0)
+    _, Tf, _ = synth.bosonic_transforms(w.tau, w.beta, 2)
+    p = pkg.problem(n, N, w.n_tau, 1, w.beta, nk=nk, dtype=1)
+    d = np.exp2(rng.integers(-4, 5, N).astype(float))
+    dd = (d[:, None] * d[None, :]) ** 2
+    res = []
+    for X, V in ((w.X, w.V), (w.X * d[:, None], w.V / dd)):
+        Gd, Xd, Vd, F = to_dev(torch, *(np.asarray(a, dtype=complex) for a in (w.G, X, V, Tf)))
+        out = torch.full((w.n_k, 5, N, N), complex(float("nan"), 0.0), dtype=torch.complex128, device="cuda")
+        pkg.sox_w_dynamic(h, p, Gd, Xd, Vd, F, 5, out)
+        pkg.sox_check_device(h)
+        res.append(out.cpu().numpy())
+    got = res[1] * dd
+    assert np.abs(got - res[0]).max() <= 1e-10 * np.abs(res[0]).max()
+
+
+def _digits(K):
+    """A digit product is good to (1.1 K + 9) 2^-54 of the product of the maxima, and an element whose
+    terms' magnitudes do not sum to 2^-6 of it is not taken from one: its error by that sum."""
+    return (1.1 * K + 9) * 2.0 ** -48
+
+
+@pytest.mark.parametrize("n,N,nb", [(2, 130, 3000), (33, 127, 120), (64, 65, 64), (130, 129, 6)])
+@pytest.mark.parametrize("form", ["rows", "both", "diagonal"])
+def test_projections_of_graded_rows(env, n, N, nb, form):
+    """Rows of X that fall off over 200 powers of two, against G that is dense, falls off the other way
+    or is diagonal: every element to the bound of a digit product by the sum of its terms' magnitudes
+    (G_PQ: of two products)."""
+    torch, pkg, h = env
+    rng = np.random.default_rng(n + N)
+    G, X = rng.standard_normal((nb, n, n)), rng.standard_normal((N, n))
+    X *= np.exp2(-rng.integers(0, 200, size=(N, n)).astype(float))
+    if form == "both":
+        f = np.exp2(-100.0 * np.arange(n) / max(n - 1, 1))
+        X = rng.standard_normal((N, n)) * f
+        G = G * f[::-1, None]
+    if form == "diagonal":
+        G = np.eye(n) * rng.standard_normal((nb, 1, n))
+    p = pkg.problem(n, N, nb, 1, 10.0)
+    Gd, Xd = to_dev(torch, G[None, None], X[None])
+    out = [torch.full(s, float("nan"), dtype=torch.float64, device="cuda")
+           for s in ((1, 1, nb, N, n), (1, 1, nb, n, N), (1, 1, nb, N, N))]
+    pkg.thc_project_G(h, p, Gd, Xd, *out)
+    pkg.sox_check_device(h)
+    for b in {0, nb // 2, nb - 1}:
+        g, x = G[b].astype(LD), X.astype(LD)
+        gr, gw, gq = (o[0, 0, b].cpu().numpy() for o in out)
+        ag, ax = np.abs(g), np.abs(x)
+        assert (np.abs(gr - x @ g) <= _digits(n) * (ax @ ag) + 1e-320).all()
+        assert (np.abs(gw - g @ x.T) <= _digits(n) * (ag @ ax.T) + 1e-320).all()
+        assert (np.abs(gq - x @ g @ x.T) <= 2.1 * _digits(n) * (ax @ ag @ ax.T) + 1e-320).all()
+
+
+def test_fp64_sigma_of_graded_orbitals(env):
+    """Orbital columns of X over 2^60 and G between the inverse factors: Sigma (r, t) carries the columns'
+    factors, and keeps its digits in the smallest of them (five chained products of at most N
+    terms, each to its bound by the magnitudes)."""
+    torch, pkg, h = env
+    n, N, T = 33, 160, 4
+    w = synth.molecule(150, n, N, T, 10.0)
+    f = np.exp2(np.round(np.linspace(0, 60, n)))
+    X, G = w.X / f, w.G * (f[:, None] * f[None, :])
+    p = pkg.problem(n, N, T, 1, w.beta)
+    Gd, Xd, Vd = to_dev(torch, G, X, w.V)
+    S = torch.full_like(Gd, float("nan"))
+    pkg.sox_sigma(h, p, Gd, Xd, Vd, S)
+    pkg.sox_check_device(h)
+    ref = osox.sox_sigma(w.X, w.V, w.G).real
+    mag = np.abs(osox.sox_sigma(np.abs(w.X), np.abs(w.V), np.abs(w.G)).real)
+    got = S.cpu().numpy() * (f[:, None] * f[None, :])
+    assert (np.abs(got - ref) <= 5 * _digits(N) * mag).all()
