@@ -48,6 +48,9 @@ __device__ __forceinline__ z recip(z a) {
   const double d = 1.0 / (a.x * a.x + a.y * a.y);
   return make_double2(a.x * d, -a.y * d);
 }
+// whether recip has a number to divide by (a modulus whose square underflows is none)
+__device__ __forceinline__ bool divisible(double) { return true; }
+__device__ __forceinline__ bool divisible(z a) { return a.x * a.x + a.y * a.y > 0.0; }
 template <class T> __device__ __forceinline__ T zero();
 template <> __device__ __forceinline__ double zero<double>() { return 0.0; }
 template <> __device__ __forceinline__ z zero<z>() { return make_double2(0.0, 0.0); }
@@ -132,15 +135,15 @@ __global__ void __launch_bounds__(kPanelThreads) k_lu_factor(T *P, int N, int k0
         }
         urow[tid] = v;
       }
-      if (tid == 0) {
-        s_p = best > 0 ? p : -1;
-        piv[(long long)b * kNb + j0 + c] = r0 + (best > 0 ? p : c);
-      }
+      if (tid == 0) piv[(long long)b * kNb + j0 + c] = r0 + (best > 0 ? p : c);
       __syncwarp();
-      if (tid == 0) s_inv = recip(urow[c]);
+      if (tid == 0) {
+        s_p = best > 0 && divisible(urow[c]) ? p : -1;
+        s_inv = recip(urow[c]);
+      }
     }
     __syncthreads();
-    if (s_p < 0) {   // a zero column (or NaNs): uniform for the block
+    if (s_p < 0) {   // a zero column (or NaNs, or no number to divide by): uniform for the block
       if (tid == 0) atomicExch(&info[1], 1);
       for (int c2 = c + 1 + tid; c2 < nc; c2 += kPanelThreads) piv[(long long)b * kNb + j0 + c2] = r0 + c2;
       break;

@@ -164,3 +164,23 @@ def test_fp64_sigma_of_graded_orbitals(env):
     mag = np.abs(osox.sox_sigma(np.abs(w.X), np.abs(w.V), np.abs(w.G)).real)
     got = S.cpu().numpy() * (f[:, None] * f[None, :])
     assert (np.abs(got - ref) <= 5 * _digits(N) * mag).all()
+
+
+@pytest.mark.parametrize("N", [40, 64])
+def test_w_dynamic_reports_a_system_whose_pivots_underflow(env, N):
+    """The last pivot of 1 - V Pi is 1e-200: the square of its modulus is no number to divide by, and the
+    call says so (below and above the rule of the block solve)."""
+    torch, pkg, h = env
+    G = np.zeros((1, 1, 2, N, N), complex)
+    G[..., range(N), range(N)] = 0.5
+    p, q = N - 2, N - 1   # Pi = G(0) o G(1)^T: 1 on the diagonal, 1e-200 and 1/4 beside it
+    G[..., p, p] = G[..., q, q] = 1.0
+    G[0, 0, 0, p, q] = G[0, 0, 1, q, p] = 1e-100
+    G[0, 0, 0, q, p] = G[0, 0, 1, p, q] = 0.5
+    p = pkg.problem(N, N, 2, 1, 10.0, nk=(1, 1, 1), dtype=1)
+    Gd, Xd, Vd, F = to_dev(torch, G, np.eye(N, dtype=complex)[None], np.eye(N, dtype=complex)[None],
+                           np.array([[-1.0 + 0j, 0.0]]))
+    out = torch.empty(1, 1, N, N, dtype=torch.complex128, device="cuda")
+    with pytest.raises(pkg.SoxError) as e:
+        pkg.sox_w_dynamic(h, p, Gd, Xd, Vd, F, 1, out)
+    assert e.value.code == 1
