@@ -566,7 +566,7 @@ size_t adjoint_tc_bytes(sox_handle h, int n, int N, int T, int S) {
   GemmF64 a;   // the FP64 projections (their digits follow the chunk's buffers)
   a.M = N; a.Nc = n; a.K = n; a.batch = T;
   a.sB = (long long)n * n;
-  return fixed_bytes(g) + std::max(per_tau_bytes(g) * g.Bc, end_bytes(g)) + gemm_f64_bytes(a) + (1 << 20);
+  return fixed_bytes(g) + std::max(per_tau_bytes(g) * g.Bc, end_bytes(g)) + gemm_f64_bytes(h, a) + (1 << 20);
 }
 
 Status phi_adjoint_xv_tc(sox_handle h, int n, int N, int T, int S, const double *G, const double *X, const double *V,

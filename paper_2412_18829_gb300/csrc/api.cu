@@ -226,7 +226,7 @@ Fp64Plan fp64_plan(sox_handle h, const Dims &d, bool two_slots) {
   p.c = tau_chunk(h, d, per_tau, fixed);
   const Fp64Gemms f = fp64_gemms(d, p.c);
   size_t scratch = 0;
-  for (const GemmF64 *g : {&f.mix, &f.gr, &f.gw, &f.A, &f.T, &f.S}) scratch = std::max(scratch, sox::gemm_f64_bytes(*g));
+  for (const GemmF64 *g : {&f.mix, &f.gr, &f.gw, &f.A, &f.T, &f.S}) scratch = std::max(scratch, sox::gemm_f64_bytes(h, *g));
   p.bytes = fixed + sox::aligned_bytes(std::max<size_t>(Nn2 * p.c, Nn2), 8) +
             4 * sox::aligned_bytes((size_t)p.c * d.N * std::max(d.n, d.N), 8) + scratch;
   if (p.slices) p.bytes += sox::slice_bytes((long long)d.n * p.c, d.N, d.n) + 2 * sox::slice_bytes(p.c, d.N, d.n);
@@ -617,9 +617,9 @@ int thc_project_G(sox_handle h, const sox_problem *p, const double *G, const dou
     q.sA = (long long)d.N * d.n; q.ai = d.n; q.ak = 1;
     q.bk = 1; q.bj = d.n;
     q.sC = (long long)d.N * d.N; q.ci = d.N; q.cj = 1;
-    size_t scratch = sox::gemm_f64_bytes(g);
-    if (G_wP) scratch = std::max(scratch, sox::gemm_f64_bytes(w));
-    if (G_PQ) scratch = std::max(scratch, sox::gemm_f64_bytes(q));
+    size_t scratch = sox::gemm_f64_bytes(h, g);
+    if (G_wP) scratch = std::max(scratch, sox::gemm_f64_bytes(h, w));
+    if (G_PQ) scratch = std::max(scratch, sox::gemm_f64_bytes(h, q));
     Arena ar;
     SOX_TRY(call.begin((G_PQ && !G_Rq ? sox::aligned_bytes(nb * d.N * d.n, 8) : 0) + scratch, &ar));
     double *gr = oR.out ? oR.out : (G_PQ ? ar.take<double>(nb * d.N * d.n) : nullptr);
@@ -762,7 +762,7 @@ int sox_pi0(sox_handle h, const sox_problem *p, const double *G, const double *X
     q.sC = (long long)d.N * d.N; q.ci = d.N; q.cj = 1;
     Arena ar;
     SOX_TRY(call.begin(sox::aligned_bytes(gpq, 8) + sox::aligned_bytes(gr, 8) +
-                           std::max(sox::gemm_f64_bytes(g), sox::gemm_f64_bytes(q)), &ar));
+                           std::max(sox::gemm_f64_bytes(h, g), sox::gemm_f64_bytes(h, q)), &ar));
     double *GPQ = ar.take<double>(gpq);
     double *GR = ar.take<double>(gr);
     cudaStream_t s = call.stream();
@@ -802,7 +802,7 @@ int sox_w_static(sox_handle h, const sox_problem *p, const double *V, const doub
     g.ci = 2LL * N; g.cj = 1;
     g.alpha = -1.0; g.beta = 1.0;
     SOX_TRY(call.begin(sox::aligned_bytes((size_t)2 * N * N, 8) + 256 +
-                           std::max(sox::gemm_f64_bytes(g), sox::lu_bytes(N, 1, false)), &ar));
+                           std::max(sox::gemm_f64_bytes(h, g), sox::lu_bytes(h, N, 1, false)), &ar));
     double *Aug = ar.take<double>((size_t)2 * N * N);
     int *info = ar.take<int>(4);
     cudaStream_t s = call.stream();
@@ -969,7 +969,7 @@ int sox_w_dynamic(sox_handle h, const sox_problem *p, const double *G, const dou
     SOX_TRY(call.input(T_fwd, 2 * (size_t)n_omega * p->n_tau, &sF));
     SOX_TRY(call.output(Wd, c * nk * n_omega * NN, &oW));
     Arena ar;
-    SOX_TRY(call.begin(sox::w_dynamic_bytes(p, n_omega), &ar));
+    SOX_TRY(call.begin(sox::w_dynamic_bytes(h, p, n_omega), &ar));
     SOX_TRY(sox::w_dynamic(h, p, n_omega, sG.in, sX.in, sV.in, sF.in, oW.out, ar, call.stream()));
     return call.end();
   }();

@@ -336,13 +336,13 @@ size_t per_system(int N, bool cplx) {
   return (size_t)kNb * N * 8 * c + kNb * 4 + (size_t)2 * blocks_of(N) * kNb * 4 + slice_bytes(1, N, kNb * c) +
          slice_bytes(1, 2 * N * c, kNb * c) + 2048;
 }
-// the most systems of a pass: its scratch stays near 1 GiB.  (Passes are of equal size, so a smaller
+// the most systems of a pass: its scratch stays below slice_pass_bytes (one system at least).  (Passes are of equal size, so a smaller
 // batch can have larger passes than a larger one: scratch is sized by this, which grows with the batch.)
-size_t most_systems(int N, int batch, bool cplx) {
-  return std::max<size_t>(1, std::min<size_t>(batch, (size_t(1) << 30) / per_system(N, cplx)));
+size_t most_systems(sox_handle h, int N, int batch, bool cplx) {
+  return std::max<size_t>(1, std::min<size_t>(batch, slice_pass_bytes(h) / per_system(N, cplx)));
 }
-int pass_systems(int N, int batch, bool cplx) {
-  const size_t most = most_systems(N, batch, cplx);
+int pass_systems(sox_handle h, int N, int batch, bool cplx) {
+  const size_t most = most_systems(h, N, batch, cplx);
   const size_t passes = ((size_t)batch + most - 1) / most;
   return (int)(((size_t)batch + passes - 1) / passes);
 }
@@ -439,12 +439,12 @@ Status solve(sox_handle h, T *Aug, int N, int batch, int *info, Arena scratch, c
 // Below, two launches per column cost less than the twenty of a block.
 bool lu_pays(int N) { return N >= 64; }
 
-size_t lu_bytes(int N, int batch, bool cplx) {
-  return lu_pays(N) ? per_system(N, cplx) * most_systems(N, batch, cplx) : 0;
+size_t lu_bytes(sox_handle h, int N, int batch, bool cplx) {
+  return lu_pays(N) ? per_system(N, cplx) * most_systems(h, N, batch, cplx) : 0;
 }
 
 Status lu_solve(sox_handle h, double *Aug, int N, int batch, bool cplx, int *info, Arena scratch, cudaStream_t s) {
-  const int per = pass_systems(N, batch, cplx);
+  const int per = pass_systems(h, N, batch, cplx);
   for (int b0 = 0; b0 < batch; b0 += per) {
     const int nb = std::min(per, batch - b0);
     if (cplx)

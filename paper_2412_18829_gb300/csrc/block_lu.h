@@ -9,7 +9,7 @@ namespace sox {
 // lu_pays: whether the blocked form is the faster one; scratch: lu_bytes, of this or of any larger
 // batch.
 bool lu_pays(int N);
-size_t lu_bytes(int N, int batch, bool cplx);
+size_t lu_bytes(sox_handle h, int N, int batch, bool cplx);
 Status lu_solve(sox_handle h, double *Aug, int N, int batch, bool cplx, int *info, Arena scratch, cudaStream_t s);
 
 }  // namespace sox

@@ -165,9 +165,9 @@ GemmF64 projection(int n, int N, int T) {
 }
 
 // digits of the FP64 products
-size_t slice_scratch(const DynGeom &g) {
+size_t slice_scratch(sox_handle h, const DynGeom &g) {
   const int k = std::min(g.N, kSliceMaxK);
-  return std::max(gemm_f64_bytes(projection(g.n, g.N, g.T)), slice_bytes(1, g.n, k) + slice_bytes(g.tc, g.n, k));
+  return std::max(gemm_f64_bytes(h, projection(g.n, g.N, g.T)), slice_bytes(1, g.n, k) + slice_bytes(g.tc, g.n, k));
 }
 
 size_t chunk_bytes(const DynGeom &g) {
@@ -184,7 +184,7 @@ size_t chunk_bytes(const DynGeom &g) {
 
 size_t dynamic_tc_bytes(sox_handle h, int n, int N, int T, int S, int n_omega) {
   const DynGeom g = geom(h, n, N, T, S, n_omega);
-  return fixed_bytes(g) + std::max(chunk_bytes(g), aligned_bytes(mixed_f32_scratch(N, n), 1)) + slice_scratch(g) + (1 << 20);
+  return fixed_bytes(g) + std::max(chunk_bytes(g), aligned_bytes(mixed_f32_scratch(N, n), 1)) + slice_scratch(h, g) + (1 << 20);
 }
 
 Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omega, const double *G, const double *X,

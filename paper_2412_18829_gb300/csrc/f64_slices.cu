@@ -1292,30 +1292,30 @@ bool slices_pay(long long M, long long N, long long K, long long batch) {
 }
 
 namespace {
-// A product runs in passes whose digits stay below kPassBytes per operand: over batches, and
+// A product runs in passes whose digits stay below slice_pass_bytes per operand: over batches, and
 // over the columns of a single large one.
-constexpr size_t kPassBytes = size_t(1) << 30;
 struct Passes {
   bool sharedA, sharedB;   // one block for every batch
   int k, nb, rows;         // K, batches and columns of a pass
 };
-Passes passes_of(const GemmF64 &g) {
+Passes passes_of(sox_handle h, const GemmF64 &g) {
+  const size_t most = slice_pass_bytes(h);
   Passes p;
   p.sharedA = g.batch == 1 || g.sA == 0;
   p.sharedB = g.batch == 1 || g.sB == 0;
   p.k = std::min(g.K, kSliceMaxK);
   const size_t per = std::max(p.sharedA ? 0 : slice_bytes(1, g.M, p.k), p.sharedB ? 0 : slice_bytes(1, g.Nc, p.k));
-  p.nb = per == 0 ? g.batch : (int)std::max<size_t>(1, std::min<size_t>(g.batch, kPassBytes / per));
+  p.nb = per == 0 ? g.batch : (int)std::max<size_t>(1, std::min<size_t>(g.batch, most / per));
   const size_t row = slice_bytes(1, 1024, p.k) / 1024 + 1;
-  p.rows = (int)std::max<size_t>(1024, std::min<size_t>(g.Nc, kPassBytes / row / (p.sharedB ? 1 : p.nb)));
+  p.rows = (int)std::max<size_t>(1024, std::min<size_t>(g.Nc, most / row / (p.sharedB ? 1 : p.nb)));
   p.rows = std::min(p.rows, g.Nc);
   return p;
 }
 }  // namespace
 
-size_t gemm_f64_bytes(const GemmF64 &g) {
+size_t gemm_f64_bytes(sox_handle h, const GemmF64 &g) {
   if (!slices_pay(g.M, g.Nc, g.K, g.batch)) return 0;
-  const Passes p = passes_of(g);
+  const Passes p = passes_of(h, g);
   return slice_bytes(p.sharedA ? 1 : p.nb, g.M, p.k) + slice_bytes(p.sharedB ? 1 : p.nb, p.rows, p.k);
 }
 
@@ -1325,7 +1325,7 @@ Status gemm_f64(sox_handle h, const GemmF64 &g, Arena scratch, cudaStream_t s) {
     launch_gemm_f64(g, s);
     return Status::ok();
   }
-  const Passes p = passes_of(g);
+  const Passes p = passes_of(h, g);
   for (int k0 = 0; k0 < g.K; k0 += p.k)
     for (int b0 = 0; b0 < g.batch; b0 += p.nb) {
       const int k = std::min(p.k, g.K - k0), nb = std::min(p.nb, g.batch - b0);

@@ -94,8 +94,14 @@ Status slice_bcd(sox_handle h, const SliceOp &A, const SliceOp &GR, const SliceO
 bool slices_pay(long long M, long long N, long long K, long long batch);
 
 // Any GemmF64 through slices (operands sliced into `scratch`, K in blocks of kSliceMaxK), or
-// on the FP64 pipe where slices_pay says so.  gemm_f64_bytes: the scratch it needs (0 without).
-size_t gemm_f64_bytes(const GemmF64 &g);
+// on the FP64 pipe where slices_pay says so, in passes over batches and columns whose digits stay below
+// slice_pass_bytes per operand (one batch and 1024 columns at least).  gemm_f64_bytes: the scratch it
+// needs (0 without).
+inline size_t slice_pass_bytes(const sox_context *h) {   // the handle's limit, 1 GiB at most
+  const size_t most = size_t(1) << 30, b = chunk_budget(h, most);
+  return b < most ? b : most;
+}
+size_t gemm_f64_bytes(sox_handle h, const GemmF64 &g);
 Status gemm_f64(sox_handle h, const GemmF64 &g, Arena scratch, cudaStream_t s);
 
 }  // namespace sox

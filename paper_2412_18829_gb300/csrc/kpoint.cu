@@ -114,28 +114,28 @@ void zgemm(const ZGemm &g, cudaStream_t s) {
 
 // The complex product through digit slices (f64_slices.h) as one real one: rows of A
 // interleaved, each row of B as its re-row and its im-row, K doubled.  For contiguous C rows
-// (cj = 1), batches at fixed strides; the digits of a pass stay below a GiB per operand.
+// (cj = 1), batches at fixed strides, in passes as gemm_f64.
 struct ZPasses {
   bool sharedA, sharedB;
   int k, nb, rows;   // K, batches and columns (complex) of a pass
 };
-ZPasses zpasses(int M, int Nc, int K, int batch, bool sharedA, bool sharedB) {
-  constexpr size_t kPass = size_t(1) << 30;
+ZPasses zpasses(sox_handle h, int M, int Nc, int K, int batch, bool sharedA, bool sharedB) {
+  const size_t most = slice_pass_bytes(h);
   ZPasses p;
   p.sharedA = sharedA;
   p.sharedB = sharedB;
   p.k = std::min(K, kSliceMaxK / 2);
   const size_t per = std::max(sharedA ? 0 : slice_bytes(1, M, 2 * p.k), sharedB ? 0 : slice_bytes(1, 2 * Nc, 2 * p.k));
-  p.nb = per == 0 ? batch : (int)std::max<size_t>(1, std::min<size_t>(batch, kPass / per));
+  p.nb = per == 0 ? batch : (int)std::max<size_t>(1, std::min<size_t>(batch, most / per));
   const size_t row = slice_bytes(1, 1024, 2 * p.k) / 512 + 1;
-  p.rows = (int)std::max<size_t>(1024, std::min<size_t>(Nc, kPass / row / (sharedB ? 1 : p.nb)));
+  p.rows = (int)std::max<size_t>(1024, std::min<size_t>(Nc, most / row / (sharedB ? 1 : p.nb)));
   p.rows = std::min(p.rows, Nc);
   return p;
 }
 bool zslices_pay(int M, int Nc, int K, long long batch) { return slices_pay(M, 2LL * Nc, 2LL * K, batch); }
-size_t zgemm_bytes(int M, int Nc, int K, int batch, bool sharedA, bool sharedB) {
+size_t zgemm_bytes(sox_handle h, int M, int Nc, int K, int batch, bool sharedA, bool sharedB) {
   if (!zslices_pay(M, Nc, K, batch)) return 0;
-  const ZPasses p = zpasses(M, Nc, K, batch, sharedA || batch == 1, sharedB || batch == 1);
+  const ZPasses p = zpasses(h, M, Nc, K, batch, sharedA || batch == 1, sharedB || batch == 1);
   return slice_bytes(p.sharedA ? 1 : p.nb, M, 2 * p.k) + slice_bytes(p.sharedB ? 1 : p.nb, 2 * p.rows, 2 * p.k);
 }
 Status zgemm_f64(sox_handle h, const ZGemm &g, Arena scratch, cudaStream_t s) {
@@ -144,7 +144,7 @@ Status zgemm_f64(sox_handle h, const ZGemm &g, Arena scratch, cudaStream_t s) {
     zgemm(g, s);
     return Status::ok();
   }
-  const ZPasses p = zpasses(g.M, g.Nc, g.K, g.batch, g.sA == 0 || g.batch == 1, g.sB == 0 || g.batch == 1);
+  const ZPasses p = zpasses(h, g.M, g.Nc, g.K, g.batch, g.sA == 0 || g.batch == 1, g.sB == 0 || g.batch == 1);
   auto d = [](const z *x) { return reinterpret_cast<const double *>(x); };
   for (int k0 = 0; k0 < g.K; k0 += p.k)
     for (int b0 = 0; b0 < g.batch; b0 += p.nb) {
@@ -773,10 +773,10 @@ KGemms k_gemms(const KTc &g, int cc) {
   f.out.sC = g.nn; f.out.ci = g.n; f.out.cj = 1;
   return f;
 }
-size_t k_gemms_bytes(const KTc &g, int cc) {
-  size_t b = zgemm_bytes(g.N, g.n, g.n, cc, true, false);
-  b = std::max(b, zgemm_bytes(g.N, g.n, g.N, cc, false, true));
-  return std::max(b, zgemm_bytes(g.n, g.n, g.N, cc, true, false));
+size_t k_gemms_bytes(sox_handle h, const KTc &g, int cc) {
+  size_t b = zgemm_bytes(h, g.N, g.n, g.n, cc, true, false);
+  b = std::max(b, zgemm_bytes(h, g.N, g.n, g.N, cc, false, true));
+  return std::max(b, zgemm_bytes(h, g.n, g.n, g.N, cc, true, false));
 }
 
 // GR and GWt ([k][cc][N][n]) of tau points t0 .. t0 + cc - 1 for every k
@@ -837,7 +837,7 @@ KStatTc kstat_plan(sox_handle h, const KTc &g, bool two) {
   KStatTc p;
   long long c = budget > fixed ? (long long)((budget - fixed) / one) : 1;
   p.ct = (int)std::max<long long>(1, std::min<long long>(c, g.T));
-  p.bytes = fixed + per(p.ct) + k_gemms_bytes(g, p.ct) + (1 << 20);
+  p.bytes = fixed + per(p.ct) + k_gemms_bytes(h, g, p.ct) + (1 << 20);
   return p;
 }
 
@@ -1055,7 +1055,7 @@ KDynTc kdyn_geom(sox_handle h, const sox_problem *p, int nO, size_t *fixed_out, 
 size_t kpoint_dynamic_tc_bytes(sox_handle h, const sox_problem *p, int n_omega) {
   size_t f = 0, per_t = 0;
   const KDynTc d = kdyn_geom(h, p, n_omega, &f, &per_t);
-  return f + per_t * d.ct + std::max(k_gemms_bytes(d.g, d.ct), k_gemms_bytes(d.g, d.g.T)) + (1 << 20);
+  return f + per_t * d.ct + std::max(k_gemms_bytes(h, d.g, d.ct), k_gemms_bytes(h, d.g, d.g.T)) + (1 << 20);
 }
 
 Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const double *Gd, const double *Xd,
@@ -1528,7 +1528,7 @@ void mesh_dft(z *buf, long long inner, long long kstride, const int nk3[3], int 
 
 }  // namespace
 
-size_t w_dynamic_bytes(const sox_problem *p, int n_omega) {
+size_t w_dynamic_bytes(sox_handle h, const sox_problem *p, int n_omega) {
   const size_t nk = (size_t)p->nk[0] * p->nk[1] * p->nk[2];
   const size_t N = p->N, n = p->n, T = p->n_tau, NN = N * N;
   size_t b = 0;
@@ -1541,10 +1541,10 @@ size_t w_dynamic_bytes(const sox_problem *p, int n_omega) {
   b += aligned_bytes(nk, 4) + aligned_bytes(4, 4) + aligned_bytes(2, 8);
   const int Ni = p->N, ni = p->n, Ti = p->n_tau;
   // scratch of the products, the bubble's pairs (one m at a time) and the solve
-  size_t scratch = std::max(zgemm_bytes(Ni, ni, ni, Ti, true, false), zgemm_bytes(Ni, Ni, ni, Ti, false, true));
-  scratch = std::max(scratch, zgemm_bytes(Ni, Ni, Ni, n_omega, true, false));
-  scratch = std::max(scratch, aligned_bytes(T * NN, 16) + aligned_bytes(nk * T, 4) + zgemm_bytes(n_omega, (int)NN, Ti, 1, true, true));
-  if (lu_pays(Ni)) scratch = std::max(scratch, lu_bytes(Ni, (int)nk * n_omega, true));
+  size_t scratch = std::max(zgemm_bytes(h, Ni, ni, ni, Ti, true, false), zgemm_bytes(h, Ni, Ni, ni, Ti, false, true));
+  scratch = std::max(scratch, zgemm_bytes(h, Ni, Ni, Ni, n_omega, true, false));
+  scratch = std::max(scratch, aligned_bytes(T * NN, 16) + aligned_bytes(nk * T, 4) + zgemm_bytes(h, n_omega, (int)NN, Ti, 1, true, true));
+  if (lu_pays(Ni)) scratch = std::max(scratch, lu_bytes(h, Ni, (int)nk * n_omega, true));
   return b + scratch + (1 << 20);
 }
 

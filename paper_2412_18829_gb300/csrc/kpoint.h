@@ -25,7 +25,7 @@ Status kpoint_dynamic_add_f64(sox_handle h, const sox_problem *p, int n_omega, c
 // frequencies for every transfer q (molecules: the mesh 1x1x1, real data, real W_d
 // [n_omega][N][N]; solids: complex W_d [n_q][n_omega][N][N]); device inputs in the
 // library layouts, T_fwd [n_omega][n_tau] complex.  Synchronises s (reads the singular flag).
-size_t w_dynamic_bytes(const sox_problem *p, int n_omega);
+size_t w_dynamic_bytes(sox_handle h, const sox_problem *p, int n_omega);
 Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *G, const double *X, const double *V,
                  const double *T_fwd, double *Wd, Arena &ar, cudaStream_t s);
 }  // namespace sox

@@ -54,3 +54,52 @@ def test_w_dynamic_on_a_handle_made_for_it(env, nk, N, n_omega):
     with pkg.Handle("fp64") as h:
         one = _w_dynamic(torch, pkg, h, w, Tf[2:3], nk)
     assert float((out[:, 2] - one[:, 0]).abs().max()) <= 1e-10 * float(one.abs().max())
+
+
+def _free(torch):
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_digits_of_a_product_stay_within_the_limit(env):
+    """G_Rq, G_wP and G_PQ of 1024 times: the digits of the last product's operands take 0.5 GB at once,
+    passes of 64 MB with that limit, and the same numbers either way."""
+    torch, pkg = env
+    n, N, T = 64, 512, 1024
+    rng = np.random.default_rng(5)
+    p = pkg.problem(n, N, T, 1, 10.0)
+    G, X = to_dev(torch, rng.standard_normal((1, 1, T, n, n)), rng.standard_normal((1, N, n)))
+    outs, used = [], []
+    for limit in (0, 64 << 20):
+        out = [torch.full(s, float("nan"), dtype=torch.float64, device="cuda")
+               for s in ((1, 1, T, N, n), (1, 1, T, n, N), (1, 1, T, N, N))]
+        with pkg.Handle("fp64", workspace_limit=limit) as h:
+            before = _free(torch)
+            pkg.thc_project_G(h, p, G, X, *out)
+            used.append(before - _free(torch))
+            pkg.sox_check_device(h)
+        outs.append(out)
+    assert all(bool((a == b).all()) for a, b in zip(*outs))
+    assert used[0] >= 400 << 20 and used[1] <= 160 << 20   # two operands of a pass
+
+
+@pytest.mark.parametrize("case", ["solve", "columns"])
+def test_passes_of_the_solve_give_the_same_numbers(env, case):
+    """One system (or 1024 columns) per pass against all at once."""
+    torch, pkg = env
+    res = []
+    if case == "solve":
+        w = synth.solid(132, (2, 2, 1), 3, 70, 4, 20.0)
+        _, Tf, _ = synth.bosonic_transforms(w.tau, w.beta, 3)
+        for limit in (0, 1):
+            with pkg.Handle("fp64", workspace_limit=limit) as h:
+                res.append(_w_dynamic(torch, pkg, h, w, Tf, w.nk))
+    else:
+        N, rng = 1100, np.random.default_rng(6)
+        V, Pi = to_dev(torch, *(rng.standard_normal((N, N)) / np.sqrt(N) for _ in range(2)))
+        for limit in (0, 1):
+            with pkg.Handle("fp64", workspace_limit=limit) as h:
+                res.append(torch.empty_like(V))
+                pkg.sox_w_static(h, pkg.problem(2, N, 2, 1, 10.0), V, Pi, res[-1])
+                pkg.sox_check_device(h)
+    assert bool((res[0] == res[1]).all())
