@@ -1360,13 +1360,13 @@ int sox_iw_to_tau(sox_handle h, const sox_problem *p, int n_w, const double *ome
     SOX_TRY(call.input(tails, 3 * S * nn, &sT));
     SOX_TRY(call.input(tau, (size_t)n_t, &st_));
     SOX_TRY(call.output(G_tau, S * n_t * nn, &oG));
-    const size_t scratch = sox::iw_to_tau_bytes(n_w, n_t);
+    const size_t scratch = sox::iw_to_tau_bytes(h, n_w, n_t);
     Arena ar;
     SOX_TRY(call.begin(scratch, &ar));
     void *phases = ar.take<char>(scratch);
     if (!phases) return {SOX_ERR_OOM, "workspace too small (internal sizing error)"};
-    sox::ProfScope ps(h, "iw_to_tau", call.stream(), 2);
-    sox::launch_iw_to_tau(sG.in, sw.in, n_w, sT.in, st_.in, n_t, p->n, p->n_spin, p->beta, phases, oG.out,
+    sox::ProfScope ps(h, "iw_to_tau", call.stream(), 0);
+    sox::launch_iw_to_tau(h, sG.in, sw.in, n_w, sT.in, st_.in, n_t, p->n, p->n_spin, p->beta, phases, oG.out,
                           call.stream());
     SOX_CUDA_TRY(cudaGetLastError());
     return call.end();

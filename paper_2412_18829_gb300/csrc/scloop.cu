@@ -350,7 +350,7 @@ __global__ void k_tails(const double *F, double mu, const double *Sig_tau, int n
   }
 }
 
-// (cos, sin)(w tau_t) for every time and frequency, [n_w][n_t8] with the times padded to 8
+// (cos, sin)(w tau_t) for every frequency and a block of times, [n_w][n_t8], the times padded to 8
 __global__ void k_phases(const double *omegas, int n_w, const double *tau, int n_t, int n_t8, z *ph) {
   const long long total = (long long)n_w * n_t8;
   for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
@@ -369,7 +369,7 @@ __global__ void k_phases(const double *omegas, int n_w, const double *tau, int n
 // A block holds 32 matrix elements and 8 times; 8 warps share the frequencies.  The phases
 // come from a table (a sincos per element, time and frequency took 20 times the sums).
 __global__ void __launch_bounds__(256) k_iw_to_tau(const z *Giw, const double *omegas, int n_w, const double *tails,
-                                                   const double *tau, const z *ph, int n_t, int n_t8, int n,
+                                                   const double *tau, const z *ph, int n_t, int n_t8, int n_all, int n,
                                                    double beta, double *Gtau) {
   __shared__ double red[8][8][33];
   const long long nn = (long long)n * n;
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(256) k_iw_to_tau(const z *Giw, const double *o
 #pragma unroll
   for (int i = 0; i < 8; ++i) a += red[i][warp][lane];
   const double tt = tau[t];
-  Gtau[((long long)s * n_t + t) * nn + e] =
+  Gtau[((long long)s * n_all + t) * nn + e] =
       a / beta - 0.5 * c1 + 0.25 * (2.0 * tt - beta) * c2 + 0.25 * tt * (beta - tt) * c3;
 }
 
@@ -643,16 +643,30 @@ void launch_green_tails(const double *F, double mu, const double *Sigma_tau, int
   k_tails<<<grid_of((long long)n * n * n_spin), 256, 0, s>>>(F, mu, Sigma_tau, n, T, n_spin, tails);
 }
 
-size_t iw_to_tau_bytes(int n_w, int n_t) { return aligned_bytes((size_t)n_w * ((n_t + 7) / 8 * 8), 16); }
+// Times of a block of phases: as many groups of eight as 64 MB (or the handle's limit) hold, one at least
+// (then 128 bytes per frequency, no more than G(i w) itself from n = 3 on).
+int iw_to_tau_block(sox_handle h, int n_w, int n_t) {
+  const size_t most = std::min(size_t(64) << 20, chunk_budget(h, size_t(64) << 20));
+  const long long groups = std::max<long long>(1, (long long)(most / ((size_t)n_w * 8 * sizeof(z))));
+  return (int)std::min<long long>(8 * groups, (n_t + 7) / 8 * 8);
+}
+size_t iw_to_tau_bytes(sox_handle h, int n_w, int n_t) {
+  return aligned_bytes((size_t)n_w * iw_to_tau_block(h, n_w, n_t), sizeof(z));
+}
 
-void launch_iw_to_tau(const double *G_iw, const double *omegas, int n_w, const double *tails, const double *tau,
-                      int n_t, int n, int n_spin, double beta, void *scratch, double *G_tau, cudaStream_t s) {
+void launch_iw_to_tau(sox_handle h, const double *G_iw, const double *omegas, int n_w, const double *tails,
+                      const double *tau, int n_t, int n, int n_spin, double beta, void *scratch, double *G_tau,
+                      cudaStream_t s) {
   z *ph = static_cast<z *>(scratch);
-  const int n_t8 = (n_t + 7) / 8 * 8;
-  k_phases<<<grid_of((long long)n_w * n_t8), 256, 0, s>>>(omegas, n_w, tau, n_t, n_t8, ph);
-  const dim3 grid((unsigned)(((long long)n * n + 31) / 32), n_t8 / 8, n_spin);
-  k_iw_to_tau<<<grid, 256, 0, s>>>(reinterpret_cast<const z *>(G_iw), omegas, n_w, tails, tau, ph, n_t, n_t8, n, beta,
-                                   G_tau);
+  const int block = iw_to_tau_block(h, n_w, n_t);
+  const long long nn = (long long)n * n;
+  for (int t0 = 0; t0 < n_t; t0 += block) {
+    const int nt = std::min(block, n_t - t0), nt8 = (nt + 7) / 8 * 8;
+    k_phases<<<grid_of((long long)n_w * nt8), 256, 0, s>>>(omegas, n_w, tau + t0, nt, nt8, ph);
+    k_iw_to_tau<<<dim3((unsigned)((nn + 31) / 32), nt8 / 8, n_spin), 256, 0, s>>>(
+        reinterpret_cast<const z *>(G_iw), omegas, n_w, tails, tau + t0, ph, nt, nt8, n_t, n, beta, G_tau + t0 * nn);
+    h->launches += 2;
+  }
 }
 
 void launch_tau_to_iw(const double *Tw, const double *F_tau, int n_w, int T, int n, int n_spin, double *F_iw,

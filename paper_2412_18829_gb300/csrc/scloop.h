@@ -21,9 +21,10 @@ Status mu_bisect(sox_handle h, int n, int T, int n_w, int n_spin, const double *
 void launch_green_tails(const double *F, double mu, const double *Sigma_tau, int n, int T, int n_spin, double *tails,
                         cudaStream_t s);
 // scratch: iw_to_tau_bytes on the device
-size_t iw_to_tau_bytes(int n_w, int n_t);
-void launch_iw_to_tau(const double *G_iw, const double *omegas, int n_w, const double *tails, const double *tau,
-                      int n_t, int n, int n_spin, double beta, void *scratch, double *G_tau, cudaStream_t s);
+size_t iw_to_tau_bytes(sox_handle h, int n_w, int n_t);
+void launch_iw_to_tau(sox_handle h, const double *G_iw, const double *omegas, int n_w, const double *tails,
+                      const double *tau, int n_t, int n, int n_spin, double beta, void *scratch, double *G_tau,
+                      cudaStream_t s);
 void launch_tau_to_iw(const double *Tw, const double *F_tau, int n_w, int T, int n, int n_spin, double *F_iw,
                       cudaStream_t s);
 // count[0] = sum_s Tr gamma^s with gamma = -G(beta^-)^T

@@ -103,3 +103,28 @@ def test_passes_of_the_solve_give_the_same_numbers(env, case):
                 pkg.sox_w_static(h, pkg.problem(2, N, 2, 1, 10.0), V, Pi, res[-1])
                 pkg.sox_check_device(h)
     assert bool((res[0] == res[1]).all())
+
+
+@pytest.mark.parametrize("n_t", [1, 8, 37])
+def test_iw_to_tau_in_blocks_of_times(env, n_t):
+    """8192 frequencies and 4096 times would be 0.5 GB of phases: 64 MB are taken.  In blocks of eight times
+    (the smallest limit) the numbers are those of one block."""
+    torch, pkg = env
+    n, n_w, rng = 3, 8192, np.random.default_rng(7)
+    om = (2 * np.arange(-n_w // 2, n_w // 2) + 1) * np.pi / 5.0
+    tau = np.sort(rng.uniform(0, 5.0, 4096))
+    G = rng.standard_normal((2, n_w, n, n)) + 1j * rng.standard_normal((2, n_w, n, n))
+    Gd, tails, omd, td = to_dev(torch, G, rng.standard_normal((2, 3, n, n)), om, tau)
+    p = pkg.problem(n, 4, 8, 2, 5.0)
+    with pkg.Handle("fp64") as h:
+        before = _free(torch)
+        out = torch.empty(2, 4096, n, n, dtype=torch.float64, device="cuda")
+        pkg.sox_iw_to_tau(h, p, omd, Gd, tails, td, out)
+        assert before - _free(torch) <= 80 << 20
+        few = torch.empty(2, n_t, n, n, dtype=torch.float64, device="cuda")
+        pkg.sox_iw_to_tau(h, p, omd, Gd, tails, td[:n_t].contiguous(), few)
+    with pkg.Handle("fp64", workspace_limit=1) as h:
+        one = torch.empty_like(few)
+        pkg.sox_iw_to_tau(h, p, omd, Gd, tails, td[:n_t].contiguous(), one)
+        pkg.sox_check_device(h)
+    assert bool((few == out[:, :n_t]).all()) and bool((one == few).all())
