@@ -350,7 +350,18 @@ Status run_sigma_complex(sox_handle h, const sox_problem *p, const double *G, co
   SOX_TRY(call.output(Sigma, 2 * (size_t)p->n_spin * nk * p->n_tau * nn, &sS));
   Arena ar;
   if (h->precision == SOX_PREC_F16X2) {
-    SOX_TRY(call.begin(sox::kpoint_tc_bytes(h, p, !same), &ar));
+    // all times of a chunk at once are faster, but one time's buffers are enough: without a limit of
+    // the caller's the default budget gives way to the memory that there is
+    Status st = call.begin(sox::kpoint_tc_bytes(h, p, !same), &ar);
+    while (st.code == SOX_ERR_OOM && !h->ws_limit && h->solid_fit != 1) {
+      const size_t fit = (h->solid_fit ? h->solid_fit : sox::kSolidBudget) / 2;
+      h->solid_fit = fit >= size_t(256) << 20 ? fit : 1;
+      st = call.begin(sox::kpoint_tc_bytes(h, p, !same), &ar);
+    }
+    if (!st.good()) {
+      h->solid_fit = 0;
+      return st;
+    }
     SOX_TRY(sox::kpoint_sigma_tc(h, p, sG.in, sX.in, s1.in, same ? s1.in : s2.in, sS.out, ar, call.stream()));
     return call.end();
   }

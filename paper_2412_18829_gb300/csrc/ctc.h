@@ -68,6 +68,7 @@ Status kpoint_D_f32(const float *B, const float *C, long long sP, long long sI, 
                     const int mesh[3], long long NN, int ct, int i0, long long sDi, double *D, cudaStream_t s);
 
 // Split-precision forms of the momentum-resolved chain (handle precision SOX_PREC_F16X2).
+constexpr size_t kSolidBudget = size_t(24) << 30;   // its chunk budget by default
 size_t kpoint_tc_bytes(sox_handle h, const sox_problem *p, bool two);
 Status kpoint_sigma_tc(sox_handle h, const sox_problem *p, const double *G, const double *X, const double *U1,
                        const double *U2, double *Sigma, Arena &ar, cudaStream_t s);

@@ -18,6 +18,7 @@ struct sox_context {
   int precision = SOX_PREC_FP64;
   long long spin_limit = 0;
   size_t ws_limit = 0;       // chunk budget override (sox_options.workspace_limit), 0 = defaults
+  size_t solid_fit = 0;      // the static solid chain's default budget once a larger workspace could not be had
   void *ws = nullptr;        // device workspace
   size_t ws_bytes = 0;
   void *aux = nullptr;       // second device buffer: partial results of composed entry points

@@ -128,3 +128,26 @@ def test_iw_to_tau_in_blocks_of_times(env, n_t):
         pkg.sox_iw_to_tau(h, p, omd, Gd, tails, td[:n_t].contiguous(), one)
         pkg.sox_check_device(h)
     assert bool((few == out[:, :n_t]).all()) and bool((one == few).all())
+
+
+def test_static_solid_takes_the_memory_there_is(env):
+    """A chunk of all 30 times would take 1.9 GB, one time 0.2 GB: with 1 GB left on the device the call
+    runs, in smaller chunks and to the same numbers."""
+    torch, pkg = env
+    w = synth.solid(133, (2, 2, 1), 26, 300, 30, 100.0)
+    p = pkg.problem(w.n, w.N, w.n_tau, 1, w.beta, nk=w.nk, dtype=1)
+    G, X, V = to_dev(torch, w.G, w.X, w.V)
+    S = [torch.full_like(G, complex("nan")) for _ in range(2)]
+    with pkg.Handle("f16x2") as h:
+        pkg.sox_sigma(h, p, G, X, V, S[0])
+        pkg.sox_check_device(h)
+    torch.cuda.empty_cache()
+    fill = torch.empty(_free(torch) - (1 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        with pkg.Handle("f16x2") as h:
+            pkg.sox_sigma(h, p, G, X, V, S[1])
+            pkg.sox_check_device(h)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert bool((S[0] == S[1]).all())
