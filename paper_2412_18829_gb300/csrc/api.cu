@@ -215,7 +215,7 @@ struct Fp64Plan {
 };
 Fp64Plan fp64_plan(sox_handle h, const Dims &d, bool two_slots) {
   Fp64Plan p;
-  p.slices = sox::slices_pay(d.N, d.N, d.nn() / 2, d.T);   // 2 n^2 per tile; ten launches more
+  p.slices = sox::slices_pay(h, d.N, d.N, d.nn() / 2, d.T);   // 2 n^2 per tile; ten launches more
   const size_t Nn2 = (size_t)d.N * d.nn();
   size_t fixed = sox::aligned_bytes(Nn2, 8) * (two_slots ? 2 : 1);
   size_t per_tau = 8 * (Nn2 + 3 * (size_t)d.N * d.n + (size_t)d.N * d.N) + 1024;

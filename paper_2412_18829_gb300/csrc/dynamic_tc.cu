@@ -235,7 +235,7 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
   // ---- set-up: U2 = mixed tensor of V (per-P scale), W_d and the transforms (per tensor)
   SOX_CUDA_TRY(cudaMemsetAsync(sc, 0, sizeof(DynScalars), s));
   launch_rows_f32(X, N, n, Xf, s);
-  launch_mixed_f32(V, X, N, n, Kp, Um, mix_scratch, s);
+  launch_mixed_f32(h->sm_count, V, X, N, n, Kp, Um, mix_scratch, s);
   launch_split_mixed(Um, N, NR, n, Kp, nullptr, nullptr, U2h, U2l, inv_u2, s);
   launch_absmax(Wd, false, N, nO * N, 0, 1, 1, N, &sc->mx[kWd], s);
   launch_split_tensor(Wd, false, N, nO * N, 0, 1, 1, N, g.Np, 0, 1.f, &sc->mx[kWd], nullptr, Wh, Wl, &sc->sc[kWd], s);
@@ -369,9 +369,9 @@ Status dynamic_sigma_add_tc(sox_handle h, int n, int N, int T, int S, int n_omeg
         SOX_CUDA_TRY(launch_sox_bcd_tc(m, ba, grid, s, Kp <= 128 ? kBcdResident : kBcdStreamed));
       }
       // Sigma_d = -X^T D^T X (FP32 half transform, FP64 final sum), added to Sigma
-      launch_backproject_T(Dt, N, Xf, N, n, ic, Tm, s);
+      launch_backproject_T(h->sm_count, Dt, N, Xf, N, n, ic, Tm, s);
       double *Sout = Sigma + ((long long)sp * T + i0) * nn;
-      if (slices_pay(n, n, N, ic)) {   // Sigma -= X^T T through digit slices, N in blocks
+      if (slices_pay(h, n, n, N, ic)) {   // Sigma -= X^T T through digit slices, N in blocks
         for (int k0 = 0; k0 < N; k0 += kSliceMaxK) {
           const int kc = std::min(kSliceMaxK, N - k0);
           Arena a2 = ar;

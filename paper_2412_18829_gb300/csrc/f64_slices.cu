@@ -1283,12 +1283,14 @@ Status slice_bcd(sox_handle h, const SliceOp &A, const SliceOp &GR, const SliceO
   return Status::ok();
 }
 
-// On the FP64 pipe a 64 x 64 tile takes 1.05 us of its SM per k (1.9 FMA a clock), whatever
-// part of it is valid; through slices a product of that size takes about 20 us, most of it
-// the three launches.  (26 x 26 x 300, complex, 4 batches: 1.3 ms against 0.02 ms.)
-bool slices_pay(long long M, long long N, long long K, long long batch) {
+// On the FP64 pipe a wave of 64 x 64 tiles takes 1.05 us per k (1.9 FMA a clock and SM), whatever
+// part of it is valid; through slices a small product takes about 20 us, most of it the three launches.
+// Both ways, us per product at K and waves of 152 tiles: 16 x 1 7 and 19; 20 x 1 14 and 20; 32 x 1
+// 21 and 20; 40 x 1 42 and 22; 64 x 1 72 and 24; 80 x 4 331 and 32; 16 x 8 (600 batches of 128 x 16:
+// tiles a quarter full) 39 and 47.
+bool slices_pay(const sox_context *h, long long M, long long N, long long K, long long batch) {
   const double tiles = (double)((M + 63) / 64) * (double)((N + 63) / 64) * (double)batch;
-  return (double)K * std::ceil(tiles / 152.0) >= 40.0;
+  return (double)K * std::ceil(tiles / h->sm_count) >= 40.0;
 }
 
 namespace {
@@ -1314,14 +1316,14 @@ Passes passes_of(sox_handle h, const GemmF64 &g) {
 }  // namespace
 
 size_t gemm_f64_bytes(sox_handle h, const GemmF64 &g) {
-  if (!slices_pay(g.M, g.Nc, g.K, g.batch)) return 0;
+  if (!slices_pay(h, g.M, g.Nc, g.K, g.batch)) return 0;
   const Passes p = passes_of(h, g);
   return slice_bytes(p.sharedA ? 1 : p.nb, g.M, p.k) + slice_bytes(p.sharedB ? 1 : p.nb, p.rows, p.k);
 }
 
 Status gemm_f64(sox_handle h, const GemmF64 &g, Arena scratch, cudaStream_t s) {
   if (g.M <= 0 || g.Nc <= 0 || g.batch <= 0) return Status::ok();
-  if (!h || !slices_pay(g.M, g.Nc, g.K, g.batch)) {
+  if (!slices_pay(h, g.M, g.Nc, g.K, g.batch)) {
     launch_gemm_f64(g, s);
     return Status::ok();
   }

@@ -90,8 +90,8 @@ Status slice_gemm(sox_handle h, const SliceOp &A, const SliceOp &B, const SliceG
 Status slice_bcd(sox_handle h, const SliceOp &A, const SliceOp &GR, const SliceOp &GW, const SliceOp &U2, int n, int N,
                  int batch, int v0, int v1, double *D, long long sD, cudaStream_t s);
 
-// Whether a product of these sizes is faster through slices than on the FP64 pipe.
-bool slices_pay(long long M, long long N, long long K, long long batch);
+// Whether a product of these sizes is faster through slices than on the FP64 pipe of the handle's device.
+bool slices_pay(const sox_context *h, long long M, long long N, long long K, long long batch);
 
 // Any GemmF64 through slices (operands sliced into `scratch`, K in blocks of kSliceMaxK), or
 // on the FP64 pipe where slices_pay says so, in passes over batches and columns whose digits stay below

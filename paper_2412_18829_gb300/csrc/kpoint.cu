@@ -132,15 +132,15 @@ ZPasses zpasses(sox_handle h, int M, int Nc, int K, int batch, bool sharedA, boo
   p.rows = std::min(p.rows, Nc);
   return p;
 }
-bool zslices_pay(int M, int Nc, int K, long long batch) { return slices_pay(M, 2LL * Nc, 2LL * K, batch); }
+bool zslices_pay(sox_handle h, int M, int Nc, int K, long long batch) { return slices_pay(h, M, 2LL * Nc, 2LL * K, batch); }
 size_t zgemm_bytes(sox_handle h, int M, int Nc, int K, int batch, bool sharedA, bool sharedB) {
-  if (!zslices_pay(M, Nc, K, batch)) return 0;
+  if (!zslices_pay(h, M, Nc, K, batch)) return 0;
   const ZPasses p = zpasses(h, M, Nc, K, batch, sharedA || batch == 1, sharedB || batch == 1);
   return slice_bytes(p.sharedA ? 1 : p.nb, M, 2 * p.k) + slice_bytes(p.sharedB ? 1 : p.nb, 2 * p.rows, 2 * p.k);
 }
 Status zgemm_f64(sox_handle h, const ZGemm &g, Arena scratch, cudaStream_t s) {
   if (g.M <= 0 || g.Nc <= 0 || g.batch <= 0) return Status::ok();
-  if (g.offA || g.offB || g.offC || g.cj != 1 || !zslices_pay(g.M, g.Nc, g.K, g.batch)) {
+  if (g.offA || g.offB || g.offC || g.cj != 1 || !zslices_pay(h, g.M, g.Nc, g.K, g.batch)) {
     zgemm(g, s);
     return Status::ok();
   }
@@ -1632,7 +1632,7 @@ Status w_dynamic(sox_handle h, const sox_problem *p, int n_omega, const double *
       launches += 2;
     }
     mesh_dft(Ah, (long long)T * NN, (long long)T * NN, nk3, -1, s);   // A-hat(m) = sum_k w^{-m.k} A_k
-    if (zslices_pay(ns, (int)NN, T, 1)) {
+    if (zslices_pay(h, ns, (int)NN, T, 1)) {
       // 3 x 3 x 3, N = 300, 60 times, 30 frequencies: pairs, digits and a product per m 15 ms, the
       // transform on the FP64 pipe inside the reduction 47 ms
       Arena pa = ar;

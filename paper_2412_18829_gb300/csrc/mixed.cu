@@ -214,7 +214,7 @@ size_t mixed_f32_scratch(int N, int n) {
   return vt + (size_t)N * pair_tiles(n) * sg::kBN * 4;
 }
 
-void launch_mixed_f32(const double *V, const double *X, int N, int n, int Kp, float *U, void *scratch,
+void launch_mixed_f32(int sms, const double *V, const double *X, int N, int n, int Kp, float *U, void *scratch,
                       cudaStream_t s) {
   const int ldv = round4(N), tiles = pair_tiles(n), ncols = tiles * sg::kBN;
   float *VT = static_cast<float *>(scratch);
@@ -222,7 +222,7 @@ void launch_mixed_f32(const double *V, const double *X, int N, int n, int Kp, fl
   k_transpose_f32<<<dim3((N + 31) / 32, (N + 31) / 32), 256, 0, s>>>(V, N, ldv, VT);
   k_pair_columns<<<dim3(tiles, std::min(N, 64)), 128, 0, s>>>(X, N, n, ncols, Y);
   // 64-row tiles while 128-row tiles would leave SMs idle (fewer than two tiles per SM)
-  if ((long long)((N + 127) / 128) * tiles < 2 * 152)
+  if ((long long)((N + 127) / 128) * tiles < 2LL * sms)
     k_mixed_f32<64><<<dim3((N + 63) / 64, tiles), sg::kThreads, 0, s>>>(VT, ldv, Y, ncols, N, n, Kp, U);
   else
     k_mixed_f32<128><<<dim3((N + 127) / 128, tiles), sg::kThreads, 0, s>>>(VT, ldv, Y, ncols, N, n, Kp, U);
@@ -235,10 +235,10 @@ void launch_rows_f32(const double *X, int N, int n, float *Xf, cudaStream_t s) {
   k_rows_f32<<<(int)std::min<long long>((total + 255) / 256, 65535), 256, 0, s>>>(X, N, n, round4(n), Xf);
 }
 
-void launch_backproject_T(const float *Dt, long long ldD, const float *Xf, int N, int n, int batch, float *T,
+void launch_backproject_T(int sms, const float *Dt, long long ldD, const float *Xf, int N, int n, int batch, float *T,
                           cudaStream_t s) {
   const int tn = (n + sg::kBN - 1) / sg::kBN;
-  if ((long long)((N + 127) / 128) * tn * batch < 2 * 152)
+  if ((long long)((N + 127) / 128) * tn * batch < 2LL * sms)
     k_backproject_T<64><<<dim3(tn, (N + 63) / 64, batch), sg::kThreads, 0, s>>>(Dt, ldD, Xf, round4(n), N, n, T);
   else
     k_backproject_T<128><<<dim3(tn, (N + 127) / 128, batch), sg::kThreads, 0, s>>>(Dt, ldD, Xf, round4(n), N, n, T);

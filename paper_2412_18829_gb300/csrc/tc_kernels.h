@@ -113,7 +113,7 @@ void launch_split_rows_f64(const double *src, long long ld, long long bstride, i
 // not written).  scratch: mixed_f32_scratch bytes, 256-byte aligned, free again after the call
 // on the stream (mixed.cu).
 size_t mixed_f32_scratch(int N, int n);
-void launch_mixed_f32(const double *V, const double *X, int N, int n, int Kp, float *U, void *scratch,
+void launch_mixed_f32(int sms, const double *V, const double *X, int N, int n, int Kp, float *U, void *scratch,
                       cudaStream_t s);
 void launch_split_mixed(const float *U, int N, int NR, int n, int Kp, __half *u1_hi, __half *u1_lo,
                         __half *u2_hi, __half *u2_lo, float *inv_scale, cudaStream_t s);
@@ -129,7 +129,7 @@ size_t rows_f32_bytes(int N, int n);
 void launch_rows_f32(const double *X, int N, int n, float *Xf, cudaStream_t s);
 // Back-projection helpers: the half transform T = Dt X (FP32, mixed.cu) and the final sum
 // (FP64, tc_kernels.cu)
-void launch_backproject_T(const float *Dt, long long ldD, const float *Xf, int N, int n, int batch, float *T,
+void launch_backproject_T(int sms, const float *Dt, long long ldD, const float *Xf, int N, int n, int batch, float *T,
                           cudaStream_t s);
 // sym (optional, per batch): when set, Sigma[b] is symmetric and only the upper
 // block triangle is computed, then mirrored

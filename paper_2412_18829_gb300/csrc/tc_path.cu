@@ -72,8 +72,8 @@ Geometry geometry(sox_handle h, int n, int N, int T, int S, bool two) {
   long long c = (long long)(chunk_budget(h, kChunkBudget) / std::max<size_t>(g.per_b_bytes, 1));
   c = std::max<long long>(1, std::min<long long>(c, (long long)T * S));
   g.Bc = (int)c;
-  g.slices_p = slices_pay(N, n, n, (long long)T * S);
-  g.slices_s = slices_pay(n, n, N, (long long)T * S);
+  g.slices_p = slices_pay(h, N, n, n, (long long)T * S);
+  g.slices_s = slices_pay(h, n, n, N, (long long)T * S);
   return g;
 }
 
@@ -263,7 +263,7 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
     f64_slice_x(h, f64, X, n, s);
     const double *src[2] = {U1, U2};
     for (int k = 0; k < (two ? 2 : 1); ++k) {
-      launch_mixed_f32(src[k], X, N, n, Kp, Uf, mix_scratch, s);
+      launch_mixed_f32(h->sm_count, src[k], X, N, n, Kp, Uf, mix_scratch, s);
       const bool slot1 = (k == 0), slot2 = two ? (k == 1) : true;
       launch_split_mixed(Uf, N, NR, n, Kp, slot1 ? U1h : nullptr, slot1 ? U1l : nullptr, slot2 ? U2h : nullptr,
                          slot2 ? U2l : nullptr, slot1 ? inv_u1 : inv_u2, s);
@@ -336,7 +336,7 @@ Status tc_sigma(sox_handle h, int n, int N, int T, int S, const double *G, const
     }
     {  // back-projection to orbitals
       ProfScope ps(h, "backproject", s, 2);
-      launch_backproject_T(Dt, N, Xf, N, n, bc, Tm, s);
+      launch_backproject_T(h->sm_count, Dt, N, Xf, N, n, bc, Tm, s);
       // bare SOX with a symmetric G(tau) has a symmetric Sigma(tau)
       // (a partial v range breaks that symmetry: then every block is computed)
       SOX_TRY(final_sum_f64(h, f64, X, Tm, N, n, bc, Sigma + (long long)b0 * n * n,
@@ -486,7 +486,7 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
     for (Inst &c : in) {
       launch_rows_f32(c.X, c.N, c.n, c.Xf, s);
       f64_slice_x(h, c.f64, c.X, c.n, s);
-      launch_mixed_f32(c.V, c.X, c.N, c.n, c.Kp, c.Uf, c.mix_scratch, s);
+      launch_mixed_f32(h->sm_count, c.V, c.X, c.N, c.n, c.Kp, c.Uf, c.mix_scratch, s);
       launch_split_mixed(c.Uf, c.N, c.NR, c.n, c.Kp, c.U1h, c.U1l, c.U2h, c.U2l, c.inv_u1, s);
     }
   }
@@ -566,7 +566,7 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
       const int B = c.S * c.T, b0 = k * c.Bc, bc = std::min(c.Bc, B - b0);
       if (bc <= 0) continue;
       ProfScope ps(h, "backproject", s, 2);
-      launch_backproject_T(c.Dt, c.N, c.Xf, c.N, c.n, bc, c.Tm, s);
+      launch_backproject_T(h->sm_count, c.Dt, c.N, c.Xf, c.N, c.n, bc, c.Tm, s);
       SOX_TRY(final_sum_f64(h, c.f64, c.X, c.Tm, c.N, c.n, bc, c.Sigma + (long long)b0 * c.n * c.n,
                             v_range_is_full(h, c.n) ? c.symf : nullptr, c.scratch, s));
     }
