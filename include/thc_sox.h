@@ -64,9 +64,26 @@ extern "C" {
 #define SOX_ERR_TIMEOUT 6      /* a device-side wait hit its iteration cap     */
 
 /* arithmetic of the contractions (projections, back-projection, Phi: FP64) */
-#define SOX_PREC_FP64 0   /* every step in FP64 on CUDA cores (reference path)          */
+#define SOX_PREC_FP64 0   /* every step to FP64 accuracy (reference path; see below)     */
 #define SOX_PREC_F16X2 1  /* B/C/A/U contractions as 2-piece FP16 splits with per-row
                              power-of-two scaling on tcgen05 tensor cores, FP32 accumulate */
+
+/* FP64 steps, on either kind of handle.  Small products, solids' FP64 chain, the FP64 adjoint
+ * and the FP64 part of dynamic SOSEX for molecules run on the CUDA cores' FP64 units.  Where
+ * it is faster, a product runs on the tensor cores as exact products of 8-bit digits of its
+ * operands (the projections and thc_project_G, orbital sums, sox_pi0, the products and the
+ * solve of sox_w_static and sox_w_dynamic, A, B and C of bare and static SOX on an
+ * SOX_PREC_FP64 handle, the adjoint's projections).  Two things follow for the caller:
+ * - Those kernels wait on hardware barriers with a bounded number of tries, so results of an
+ *   SOX_PREC_FP64 handle, too, are valid only once sox_check_device has returned SOX_OK.
+ * - Digits are fixed point below a row's largest element.  An element of such a product of K
+ *   terms is off by less than (1.1 K + 9) 2^-54 of the product of the largest elements of its
+ *   two rows: less than a chain of FP64 operations makes for rows of similar elements.  It is
+ *   also off by less than (1.1 K + 9) 2^-48 of the sum of the magnitudes of its own terms
+ *   (complex terms: of their larger parts): a chain of FP64 operations would stay within K 2^-53
+ *   of that sum, up to 2^5 less where an element's terms are far below the largest ones.
+ * The route of a product depends on the sizes of the whole call (n_tau and n_spin included), so
+ * a call on part of the times can differ from the whole call in the last bits. */
 
 #define SOX_REAL64 0
 #define SOX_COMPLEX128 1
@@ -89,7 +106,12 @@ typedef struct {
                           * batch).  A chunk of one tau
                           * point (or one v) is used even when it exceeds the
                           * limit; fixed-size tensors (mixed tensors, the D
-                          * array of the dynamic paths) are not counted.      */
+                          * array of the dynamic paths) are not counted.  The
+                          * digits of FP64 products (two operands of a pass, and
+                          * the solve's scratch) come on top, each within the
+                          * limit and within 1 GiB.  Without a limit the static
+                          * chain of solids takes less than its default where
+                          * less device memory is free.                       */
   int no_autotune;      /* 0: on the first call for a new shape, the split path
                          * times its fused-kernel variants on the call's own
                          * data (one extra launch each, a host synchronisation)
@@ -133,8 +155,9 @@ SOX_API int sox_profile_enable(sox_handle h, int enable);
 SOX_API int sox_profile_read(sox_handle h, const char *kernel, long long *launches, double *ms);
 
 /* Synchronise the handle's device and report device-side wait failures:
- * SOX_ERR_TIMEOUT if any kernel of an earlier call on this handle gave up a
- * bounded wait (its results are then invalid; the status is cleared). */
+ * SOX_ERR_TIMEOUT if any kernel of an earlier call on this handle, of either
+ * precision, gave up a bounded wait (its results are then invalid; the status is
+ * cleared). */
 SOX_API int sox_check_device(sox_handle h);
 
 /* Partial builds for a split over GPUs (no paper passage: the partition of Sec. II C's
@@ -235,8 +258,8 @@ SOX_API int sox_pi0(sox_handle h, const sox_problem *p, const double *G, const d
             const double *w, double *Pi0, void *stream);
 
 /* Screened interaction W0 = V^1/2 (1 - V^1/2 Pi V^1/2)^-1 V^1/2, computed as
- * the equal (1 - V Pi)^-1 V by Gauss-Jordan elimination with partial
- * pivoting in FP64.  Pi is the total polarisability [N][N] (sum the spin
+ * the equal (1 - V Pi)^-1 V by elimination with partial pivoting in FP64 (by
+ * blocks from N = 64 on).  Pi is the total polarisability [N][N] (sum the spin
  * blocks of sox_pi0 first if desired).  Returns SOX_ERR_INVALID_ARG for a
  * singular system. */
 SOX_API int sox_w_static(sox_handle h, const sox_problem *p, const double *V, const double *Pi,
@@ -255,8 +278,8 @@ SOX_API int phi_sox(sox_handle h, const sox_problem *p, const double *G, const d
  *   dV[0][P][Q]       = sum_s dphi[s] dPhi_s/dV_PQ
  * with respect to the unsymmetrised entries.  Any of dG, dX, dV may be NULL.
  * dG follows from Sigma by the identity above (computed in the handle's
- * precision); dX and dV come from a reverse pass through the THC chain in FP64
- * that recomputes B_v and C_v per tau chunk instead of storing them. */
+ * precision); dX and dV come from a reverse pass through the THC chain in the handle's
+ * precision that recomputes B_v and C_v per tau chunk instead of storing them. */
 SOX_API int phi_sox_backward(sox_handle h, const sox_problem *p, const double *G, const double *X,
                      const double *V, const double *w, const double *dphi, double *dG,
                      double *dX, double *dV, void *stream);
@@ -279,7 +302,7 @@ SOX_API int phi_sox_grad_G(sox_handle h, const sox_problem *p, const double *Sig
  * Wd [n_omega][N][N] real: W(i Omega_m) - v, real and even in Omega for a real
  * molecule; T_fwd [n_omega][n_tau] and T_inv [n_tau][n_omega] complex
  * (interleaved).  The transform pair is the caller's (the paper uses sparse-ir,
- * Sec. II C).  SOX(v, v) runs in the handle's precision, Sigma_d in FP64 with v in
+ * Sec. II C).  SOX(v, v) and Sigma_d run in the handle's precision, Sigma_d with v in
  * the outer loop (GG, transform, W_d product, inverse transform, then the fused
  * B/C/D kernel with X in place of G_Rq).
  * Solids (dtype SOX_COMPLEX128, any k-mesh; Sec. II C with momenta): Wd is
@@ -309,7 +332,7 @@ SOX_API int sosex_dynamic_sigma(sox_handle h, const sox_problem *p, const double
  *   Pi^q(tau_j)_PQ = 1/N_k sum_k G^PQ_{k+q}(tau_j) G^QP_k(-tau_j),  G^PQ_k = X^k G^k X^k^H,
  * and Wd [n_q][n_omega][N][N] complex, the layout sosex_dynamic_sigma reads.
  * T_fwd [n_omega][n_tau] complex (interleaved).  FP64 throughout; the solve is
- * Gauss-Jordan with partial pivoting batched over (q, m).  When the rows of T_fwd pair
+ * elimination with partial pivoting batched over (q, m), by blocks from N = 64 on.  When the rows of T_fwd pair
  * up as +-Omega (row n_omega-1-m the conjugate of row m) and G is Hermitian (a real
  * molecule: the pairs suffice), Wd(-Omega) = Wd(Omega)^H and only m < (n_omega+1)/2 is
  * solved.  Synchronises `stream`.
