@@ -375,7 +375,7 @@ BatchGeo batch_geometry(sox_handle h, int count, const int *n, const int *N, con
   bg.Bc.assign(count, 1);
   size_t fixed = 0;
   for (int i = 0; i < count; ++i) {
-    g[i] = geometry(nullptr, n[i], N[i], T[i], S[i], false);
+    g[i] = geometry(h, n[i], N[i], T[i], S[i], false);
     B[i] = (long long)T[i] * S[i];
     bg.Bc[i] = (int)B[i];
     fixed += g[i].fixed_bytes + 64 * 1024;
@@ -430,7 +430,7 @@ Status tc_sigma_batch(sox_handle h, int count, const int *n, const int *N, const
   std::string err;
   for (int i = 0; i < count; ++i) {
     Inst &c = in[i];
-    const Geometry g = geometry(nullptr, n[i], N[i], T[i], S[i], false);
+    const Geometry g = geometry(h, n[i], N[i], T[i], S[i], false);
     c.n = n[i]; c.N = N[i]; c.T = T[i]; c.S = S[i];
     c.Kp = g.Kp; c.NR = g.NR; c.RG = g.RG; c.Bc = bg.Bc[i];
     c.G = G[i]; c.X = X[i]; c.V = V[i]; c.Sigma = Sigma[i];
