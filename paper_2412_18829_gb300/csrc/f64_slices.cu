@@ -14,11 +14,13 @@ namespace {
 // Digits are fixed point below a row's largest element, so the error of a product goes with the product
 // of the two maxima; FP64 arithmetic errs by the sum S of the element's |a_k b_k|.  An element is
 // taken from the digits only where S is known to be within 2^kSignif of the product of the scales: by
-// its own size, by a k at which both rows are within 2^kBig of their largest (bit masks of the rows), or by
+// kShared k at least where both rows hold elements within 2^kNear of their largest (the rows' counts of
+// such elements mostly show it, one test per tile; else bit masks of the rows do), by its own size, or by
 // the sum of products of 8-bit magnitudes (complex elements count by the larger part).  Any other is
-// summed in FP64 from the sources.  (The checks cost an FP64 bare SOX of n = 80, N = 480, 30 times 4 %,
-// 9.63 -> 9.98 ms, W of the 3 x 3 x 3 solid 7 %, the split-precision calls at most 2 %.)
-constexpr int kBig = 2, kSignif = 2 * kBig + 2;
+// summed in FP64 from the sources.  (The checks cost an FP64 bare SOX of n = 80, N = 480, 30 times 2 %,
+// 9.61 -> 9.82 ms, W of the 3 x 3 x 3 solid 2 %, the split-precision calls at most 2 %.)
+constexpr int kNear = 3, kShared = 4, kSignif = 6;
+static_assert(kShared << kSignif == 1 << (2 * kNear + 2), "kShared products of two such elements");
 
 constexpr int kNonFinite = 1 << 20;
 
@@ -38,13 +40,14 @@ __device__ __forceinline__ int balance(const SliceBalance &bal, int b, int k) {
   const int e = bal.kex[(long long)b * bal.stride + k];
   return e > 0 ? (e - 1023) / bal.part : 0;
 }
-// What is kept of a row: its largest exponent E, or that it holds an infinity or a NaN.  The codes of two
-// rows add up field by field.
-constexpr int kCodeBias = 8192, kCodeNonFinite = 1 << 16;
-__device__ __forceinline__ int row_code(int E) {
+// What is kept of a row: its largest exponent E and how many elements are within 2^kNear of the largest,
+// or that it holds an infinity or a NaN.  The codes of two rows add up field by field.
+constexpr int kCodeBias = 8192, kCodeNonFinite = 1 << 29;
+__device__ __forceinline__ int row_code(int E, int near) {
   if (E == kZeroRow) E = 1;
-  return E >= kNonFinite ? kCodeBias | kCodeNonFinite : E + kCodeBias;
+  return E >= kNonFinite ? kCodeBias | kCodeNonFinite : (E + kCodeBias) | (near << 16);
 }
+__device__ __forceinline__ int code_near(int code) { return (code >> 16) & 0xfff; }
 // x scaled by the row's exponent as an integer: x = X 2^-55 2^(E - 1022), |X| <= 2^55,
 // rounded to nearest (ties up)
 __device__ __forceinline__ long long fixed55(double x, int E) {
@@ -60,12 +63,12 @@ __device__ __forceinline__ long long fixed55(double x, int E) {
     m = sh > 60 ? 0 : (m + (1ll << (sh - 1))) >> sh;
   return bits < 0 ? -m : m;
 }
-// Eight elements of a row as its epilogue's checks see them: bits for those within 2^kBig of the row's
+// Eight elements of a row as its epilogue's checks see them: bits for those within 2^kNear of the row's
 // largest and for those that are not zero, and magnitudes in 256ths of the scale, rounded down
 // (negative values by their complement, one unit of the high word short).  pair: complex elements, by
 // the larger part.
 struct Sizes {
-  unsigned big = 0u, nz = 0u;
+  unsigned near = 0u, nz = 0u;
   uint2 mag = make_uint2(0u, 0u);
 };
 __device__ __forceinline__ Sizes sizes_of(const long long (&X)[8], unsigned nz, bool pair) {
@@ -85,7 +88,7 @@ __device__ __forceinline__ Sizes sizes_of(const long long (&X)[8], unsigned nz, 
   unsigned *m = &z.mag.x;
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
-    z.big |= a[e] >= (1u << (22 - kBig)) ? 1u << e : 0u;
+    z.near |= a[e] >= (1u << (22 - kNear)) ? 1u << e : 0u;
     m[e / 4] |= min(a[e] >> 15, 255u) << (8 * (e & 3));
   }
   return z;
@@ -94,7 +97,7 @@ __device__ __forceinline__ Sizes sizes_of(const long long (&X)[8], unsigned nz, 
 // are four consecutive lanes that call this together.
 __device__ __forceinline__ void put_sizes(uint32_t *mask, uint8_t *mag, int nw, int K8, int c, const Sizes &z) {
   const unsigned quad = 0xfu << (threadIdx.x & 28);
-  unsigned x = (z.big | (z.nz << 16)) << (8 * (c & 1));   // two chunks of both masks
+  unsigned x = (z.near | (z.nz << 16)) << (8 * (c & 1));   // two chunks of both masks
   x |= __shfl_xor_sync(quad, x, 1);
   const unsigned y = __shfl_xor_sync(quad, x, 2);           // the other two
   if ((c & 3) == 0) mask[c / 4] = (x & 0xffffu) | (y << 16);
@@ -157,9 +160,9 @@ __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, 
   for (int o = lpr / 2; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
   if (!live) return;
   const bool fin = E < kNonFinite;
-  if (l == 0) ex[row] = row_code(E);
   const long long plane = (long long)batch_all * rows * K8;
   const int nw = mask_words(K);
+  int near = 0;
   for (int c = l; c < nw * 4; c += lpr) {   // (four lanes at least per row: a word's bytes go together)
     long long X[8];
     uint4 w[kSlices];
@@ -171,12 +174,17 @@ __global__ void __launch_bounds__(256) k_slice_rows(const T *src, long long sb, 
       X[e] = fixed55(v, E - (k < K ? balance<BAL>(bal, b, k) : 0));
       nz |= nonzero(v) << e;
     }
-    put_sizes(mask + row * 2 * nw, mag + row * K8, nw, K8, c, sizes_of(X, nz, false));
+    const Sizes z = sizes_of(X, nz, false);
+    near += __popc(z.near);
+    put_sizes(mask + row * 2 * nw, mag + row * K8, nw, K8, c, z);
     if (c * 8 >= K8) continue;
     digits8(X, w);
 #pragma unroll
     for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint4 *>(p + s * plane + row * K8 + c * 8) = w[s];
   }
+  const unsigned group = lpr == 32 ? 0xffffffffu : ((1u << lpr) - 1u) << (threadIdx.x % 32 / lpr * lpr);
+  for (int o = lpr / 2; o > 0; o >>= 1) near += __shfl_xor_sync(group, near, o);
+  if (l == 0) ex[row] = row_code(E, near);
 }
 
 // Rows whose elements lie apart: 32 rows per block, transposed through shared memory.
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
                                                     int batch_all, int K, int K8, SliceBalance bal, __half *p, int *ex,
                                                     uint32_t *mask, uint8_t *mag) {
   __shared__ long long sx[64][33];
-  __shared__ int se[8][32];
+  __shared__ int se[8][32], sE[32];
   const int b = blockIdx.y, r0 = blockIdx.x * 32, tx = threadIdx.x % 32, ty = threadIdx.x / 32;
   const T *x = src + b * sb + (long long)(r0 + tx) * sr;
   const bool in = r0 + tx < rows;
@@ -197,9 +205,10 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
 #pragma unroll
   for (int i = 0; i < 8; ++i) E = max(E, se[i][tx]);
   const bool fin = E < kNonFinite;
-  if (ty == 0 && in) ex[(long long)b * rows + r0 + tx] = row_code(E);
+  if (ty == 0) sE[tx] = E;
   const long long plane = (long long)batch_all * rows * K8;
   const int row = threadIdx.x / 8, c8 = threadIdx.x % 8, nw = mask_words(K);
+  int near = 0;
   for (int k0 = 0; k0 < K8; k0 += 64) {
     __syncthreads();
     for (int k = ty; k < 64; k += 8)
@@ -216,7 +225,9 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
         nz |= take_flag(X[e]) << e;
       }
       const long long r1 = (long long)b * rows + r0 + row;
-      put_sizes(mask + r1 * 2 * nw, mag + r1 * K8, nw, K8, c, sizes_of(X, nz, false));
+      const Sizes z = sizes_of(X, nz, false);
+      near += __popc(z.near);
+      put_sizes(mask + r1 * 2 * nw, mag + r1 * K8, nw, K8, c, z);
       if (c * 8 >= K8) continue;
       digits8(X, w);
       const long long o = r1 * K8 + c * 8;
@@ -224,6 +235,9 @@ __global__ void __launch_bounds__(256) k_slice_cols(const T *src, long long sb, 
       for (int s = 0; s < kSlices; ++s) *reinterpret_cast<uint4 *>(p + s * plane + o) = w[s];
     }
   }
+  if (r0 + row >= rows) return;
+  for (int o = 4; o > 0; o >>= 1) near += __shfl_xor_sync(0xffu << (threadIdx.x & 24), near, o);
+  if (c8 == 0) ex[(long long)b * rows + r0 + row] = row_code(sE[row], near);
 }
 
 // Complex rows (see SliceOp::kind): 32 rows per block, lanes along the index that is
@@ -263,12 +277,9 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
   }
   __syncthreads();
   const int nr = KIND == 2 ? 2 : 1;   // real rows per complex row
-  if (threadIdx.x < 32 && r0 + tx < rows) {
-    const int e = row_code(se[tx]);
-    for (int i = 0; i < nr; ++i) ex[((long long)b * rows + r0 + tx) * nr + i] = e;
-  }
   const long long plane = (long long)batch_all * rows * nr * K8;
   const int row = threadIdx.x / 8, c8 = threadIdx.x % 8, nw = mask_words(2 * K);
+  int near = 0;
   for (int k0 = 0; 2 * k0 < K8; k0 += 32) {
     __syncthreads();
     for (int i = ty; i < 32; i += 8) {
@@ -310,7 +321,10 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
             X[2 * e + 1] = sa > 0 ? re[e] : -re[e];
           }
         }
-        if (i == 0) sizes = sizes_of(X, nz, true);   // (of both parts: the same for either row)
+        if (i == 0) {   // (of both parts: the same for either row)
+          sizes = sizes_of(X, nz, true);
+          near += __popc(sizes.near);
+        }
         put_sizes(mask + (r1 + i) * 2 * nw, mag + (r1 + i) * K8, nw, K8, c, sizes);
         if (c * 8 >= K8) continue;
         digits8(X, w);
@@ -319,6 +333,9 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
       }
     }
   }
+  if (r0 + row >= rows) return;
+  for (int o = 4; o > 0; o >>= 1) near += __shfl_xor_sync(0xffu << (threadIdx.x & 24), near, o);
+  if (c8 < nr) ex[((long long)b * rows + r0 + row) * nr + c8] = row_code(se[row], near);
 }
 
 // ------------------------------------------------------------------ product
@@ -535,11 +552,24 @@ __device__ __forceinline__ unsigned small_sums(const long long (&I)[C]) {
 struct RowSizes {
   const uint32_t *mask, *mag;
 };
-// The columns of `small` whose S may be small too: none where the magnitudes' products sum to 2^-kSignif
-// of the scales, or where no k is nonzero in both rows (an exact zero).  L: the lane's row; W: column
-// `lane`; l0, w0: the first words of their masks.
 __device__ __forceinline__ RowSizes row_sizes(const uint32_t *mask, const uint8_t *mag, long long row, int mw, int kw) {
   return {mask + row * 2 * mw, reinterpret_cast<const uint32_t *>(mag) + row * kw};
+}
+// Whether every pair of the warp's rows and columns has kShared elements at least within 2^kNear of the
+// largest of both: `near` of the lane's row plus the columns' smallest, of K.
+__device__ __forceinline__ bool all_settled(int near, bool in, int least, int K) {
+  return __all_sync(0xffffffffu, !in || near + least >= K + kShared);
+}
+// The columns of `small` whose S may be small too (unsettled): none that share kShared k near both
+// largest elements, none where the magnitudes' products sum to 2^-kSignif of the scales, and none where no k
+// is nonzero in both rows (an exact zero).  L: the lane's row; W: column `lane`.
+// Where that does not hold for all: the columns of `small` for which the lane's own pair misses it
+template <int C>
+__device__ __forceinline__ unsigned missed_counts(unsigned small, int near, int code_w, int K) {
+#pragma unroll
+  for (int j = 0; j < C; ++j)
+    small &= near + code_near(__shfl_sync(0xffffffffu, code_w, j)) >= K + kShared ? ~(1u << j) : ~0u;
+  return small;
 }
 template <int C>
 __device__ __noinline__ unsigned unsettled_rest(unsigned small, RowSizes L, RowSizes W, int mw, int kw) {
@@ -576,17 +606,23 @@ __device__ __noinline__ unsigned unsettled_rest(unsigned small, RowSizes L, RowS
   }
   return small & some;
 }
+// (Not inlined: a call costs about 2 us of the warp, most of it code that is not in the cache, but one
+// in hundreds of tiles makes it.)
 template <int C>
-__device__ __forceinline__ unsigned unsettled(unsigned small, RowSizes L, RowSizes W, uint32_t l0, uint32_t w0, int mw,
-                                              int kw) {
-  for (int i = 0; __any_sync(0xffffffffu, small != 0u);) {
+__device__ __noinline__ unsigned unsettled(unsigned small, RowSizes L, RowSizes W, int mw, int kw) {
+  int both[C];
 #pragma unroll
-    for (int j = 0; j < C; ++j) small &= (l0 & __shfl_sync(0xffffffffu, w0, j)) ? ~(1u << j) : ~0u;
-    if (++i == mw) break;
-    l0 = L.mask[i];
-    w0 = W.mask[i];
+  for (int j = 0; j < C; ++j) both[j] = 0;
+  for (int i = 0; i < mw; ++i) {
+    const uint32_t l = L.mask[i], w = W.mask[i];
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+      both[j] += __popc(l & __shfl_sync(0xffffffffu, w, j));
+      small &= both[j] >= kShared ? ~(1u << j) : ~0u;
+    }
+    if (!__any_sync(0xffffffffu, small != 0u)) return 0u;
   }
-  return __any_sync(0xffffffffu, small != 0u) ? unsettled_rest<C>(small, L, W, mw, kw) : 0u;
+  return unsettled_rest<C>(small, L, W, mw, kw);
 }
 
 // I 2^x rounded to nearest even, x from the codes of the two rows, by integer instructions (a 64-bit
@@ -727,7 +763,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       const RowSizes sL = row_sizes(a.mL, a.gL, (a.bL == 1 ? 0LL : (long long)b * a.nL) + min(l, a.nL - 1), a.mw, a.kw);
       const RowSizes sW =
           row_sizes(a.mW, a.gW, (a.bW == 1 ? 0LL : (long long)b * a.nW) + min(w0 + lane % kC, a.nW - 1), a.mw, a.kw);
-      const uint32_t mL0 = sL.mask[0], mW0 = sW.mask[0];
       long long acc[kC];
 #pragma unroll
       for (int j = 0; j < kC; ++j) acc[j] = 0;
@@ -744,8 +779,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool mir = a.mirror && a.mirror[b];
       const long long sign = a.alpha < 0.0 ? (long long)0x8000000000000000ull : 0ll;
       const int live = l < a.nL ? min(kC, a.nW - w0) : 0;
-      // columns to sum from the sources
-      unsigned odd = unsettled<kC>(small_sums<LK>(acc) & (live > 0 ? (1u << live) - 1u : 0u), sL, sW, mL0, mW0, a.mw, a.kw);
+      const int least = (int)__reduce_min_sync(0xffffffffu, lane < kC && w0 + lane < a.nW ? code_near(eWl) : 0xffff);
+      unsigned odd = 0u;   // columns to sum from the sources
+      if (!all_settled(code_near(eL), l < a.nL, least, a.K)) {
+        odd = missed_counts<kC>(small_sums<LK>(acc) & (live > 0 ? (1u << live) - 1u : 0u), code_near(eL), eWl, a.K);
+        if (__any_sync(0xffffffffu, odd != 0u)) odd = unsettled<kC>(odd, sL, sW, a.mw, a.kw);
+      }
       constexpr int kH = 8;   // C is read eight columns at a time, all loads before the first store
 #pragma unroll
       for (int j0 = 0; j0 < kC; j0 += kH) {
@@ -1007,9 +1046,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int eRl = lane < cols ? a.eGR[(long long)b * a.N + R0 + lane] : 0;
       const unsigned live = in && cols > 0 ? (1u << cols) - 1u : 0u;
       const int Pm = min(P, a.N - 1), Rm = min(R0 + lane % kC, a.N - 1);   // rows of the masks
+      const int leastR = (int)__reduce_min_sync(0xffffffffu, lane < cols ? code_near(eRl) : 0xffff);
       const RowSizes sR = row_sizes(a.mGR, a.gGR, (long long)b * a.N + Rm, a.mw, a.kw);
       const RowSizes sW = row_sizes(a.mGW, a.gGW, (long long)b * a.N + Pm, a.mw, a.kw);
-      const uint32_t mR0 = sR.mask[0], mW0 = sW.mask[0];
       bool ok = true;
       for (int v = a.v0; v < a.v1 && ok; ++v) {
         long long ib[kC], ic[kC];
@@ -1019,7 +1058,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int eUl = lane < cols ? a.eU[(long long)v * a.N + R0 + lane] : 0;
         const RowSizes sA = row_sizes(a.mA, a.gA, ((long long)b * a.nv + v) * a.N + Pm, a.mw, a.kw);
         const RowSizes sU = row_sizes(a.mU, a.gU, (long long)v * a.N + Rm, a.mw, a.kw);
-        const uint32_t mA0 = sA.mask[0], mU0 = sU.mask[0];
         for (int h = 0; h < 2 && ok; ++h)
           for (int w = 0; w < nwin; ++w) {
             ok = tc::mbar_wait_warp(&bar->acc_full[h], (uint32_t)((win + w) & 1), limit, abort, a.status, 8);
@@ -1033,9 +1071,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         win += nwin;
         if (!ok) break;
-        // columns to sum from the sources
-        unsigned odd = unsettled<kC>(small_sums<LK>(ib) & live, sA, sR, mA0, mR0, a.mw, a.kw) |
-                       unsettled<kC>(small_sums<LK>(ic) & live, sW, sU, mW0, mU0, a.mw, a.kw);
+        unsigned odd = 0u;   // columns to sum from the sources
+        if (!all_settled(code_near(eA), in, leastR, a.n)) {
+          odd = missed_counts<kC>(small_sums<LK>(ib) & live, code_near(eA), eRl, a.n);
+          if (__any_sync(0xffffffffu, odd != 0u)) odd = unsettled<kC>(odd, sA, sR, a.mw, a.kw);
+        }
+        const int leastU = (int)__reduce_min_sync(0xffffffffu, lane < cols ? code_near(eUl) : 0xffff);
+        if (!all_settled(code_near(eW), in, leastU, a.n)) {
+          unsigned oc = missed_counts<kC>(small_sums<LK>(ic) & live, code_near(eW), eUl, a.n);
+          if (__any_sync(0xffffffffu, oc != 0u)) oc = unsettled<kC>(oc, sW, sU, a.mw, a.kw);
+          odd |= oc;
+        }
 #pragma unroll
         for (int j = 0; j < kC; ++j) {
           const int eR = __shfl_sync(0xffffffffu, eRl, j), eU = __shfl_sync(0xffffffffu, eUl, j);
