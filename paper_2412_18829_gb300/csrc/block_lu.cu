@@ -248,39 +248,78 @@ __device__ __forceinline__ void row_exponents(const T (&x)[kNb], bool live, int 
   if (mine > 0) atomicMax(kex + threadIdx.x % 32, mine);
 }
 
+// The block's row exchanges as one permutation, found by a warp: block row c takes the content of row
+// src[c], and the rows out[t] below the block that of the block's rows out_src[t], t < count (a row
+// below the block only ever receives what was in the block: contents move down at a later exchange, but
+// what came up stays).  Lane c follows block row c, and the t-th row below.
+__device__ __forceinline__ void exchanges(const int *piv, int k0, int nb, int lane, int *src, int *out, int *out_src,
+                                          int *count) {
+  int cont = k0 + lane, row = -1, rcont = -1, n = 0;
+  const int mine = lane < nb ? piv[lane] : 0;
+  for (int c = 0; c < nb; ++c) {
+    const int p = __shfl_sync(0xffffffffu, mine, c), cc = __shfl_sync(0xffffffffu, cont, c);
+    int up;
+    if (p < k0 + nb) {
+      up = __shfl_sync(0xffffffffu, cont, p - k0);
+      if (lane == p - k0) cont = cc;
+    } else {
+      const unsigned has = __ballot_sync(0xffffffffu, row == p);
+      const int t = has ? __ffs((int)has) - 1 : n;
+      up = has ? __shfl_sync(0xffffffffu, rcont, t) : p;
+      if (lane == t) {
+        row = p;
+        rcont = cc;
+      }
+      n += has ? 0 : 1;
+    }
+    if (lane == c) cont = up;
+  }
+  src[lane] = cont;
+  out[lane] = row;
+  out_src[lane] = rcont;
+  if (lane == 0) *count = n;
+}
+
 // The block's row exchanges on columns k0 + nb .. 2N - 1 of [K | B] and U12 = L11^-1 A12 by forward
 // substitution, one thread per column; U11 into its place in K (the first block of a system).
 // Bound by the FP64 pipe (kNb^2 / 2 multiply-adds per column): 810 complex systems of N = 300, ten
-// steps, 13.8 ms for 6.8e9 real ones.
+// steps, 13.8 ms for 6.8e9 real ones.  A single system has few columns and waits for memory instead: the
+// exchanges are one permutation, so that its loads do not wait for one another.
 template <class T>
 __global__ void __launch_bounds__(128) k_lu_lower(T *Aug, int N, int k0, int nb, const T *P, const int *piv, int *kex) {
   __shared__ T L[kNb][kNb];   // L[c][i], i > c
-  __shared__ int sp[kNb];
+  __shared__ int src[kNb], out[kNb], out_src[kNb], count;
   const int b = blockIdx.y, tid = threadIdx.x;
   const long long ld = 2LL * N, j = k0 + nb + (long long)blockIdx.x * blockDim.x + tid;
   T *A = Aug + (long long)b * N * ld;
   const T *Pb = P + (long long)b * kNb * N + k0;
+  if (tid < 32) exchanges(piv + (long long)b * kNb, k0, nb, tid, src, out, out_src, &count);
+#pragma unroll 8
   for (int e = tid; e < kNb * kNb; e += blockDim.x) {
     const int c = e / kNb, i = e % kNb;
-    const T v = (c < nb && i < nb) ? Pb[(long long)c * N + i] : zero<T>();
-    L[c][i] = v;
-    if (blockIdx.x == 0 && i <= c && c < nb) A[(k0 + i) * ld + k0 + c] = v;
+    L[c][i] = (c < nb && i < nb) ? Pb[(long long)c * N + i] : zero<T>();
   }
-  for (int c = tid; c < nb; c += blockDim.x) sp[c] = piv[(long long)b * kNb + c];
   __syncthreads();
+  if (blockIdx.x == 0)
+    for (int e = tid; e < nb * kNb; e += blockDim.x) {
+      const int c = e / kNb, i = e % kNb;
+      if (i <= c) A[(k0 + i) * ld + k0 + c] = L[c][i];
+    }
   const bool live = j < ld;
   T x[kNb];
+#pragma unroll
+  for (int c = 0; c < kNb; ++c) x[c] = (live && c < nb) ? A[src[c] * ld + j] : zero<T>();
   if (live) {
-    for (int c = 0; c < nb; ++c) {
-      const int p = sp[c];
-      if (p == k0 + c) continue;
-      const T v = A[p * ld + j], w = A[(k0 + c) * ld + j];
-      A[p * ld + j] = w;
-      A[(k0 + c) * ld + j] = v;
+    for (int t0 = 0; t0 < count; t0 += 8) {   // (the block's rows are still as they were)
+      T v[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (t0 + t < count) v[t] = A[out_src[t0 + t] * ld + j];
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+        if (t0 + t < count) A[out[t0 + t] * ld + j] = v[t];
     }
   }
-#pragma unroll
-  for (int c = 0; c < kNb; ++c) x[c] = (live && c < nb) ? A[(k0 + c) * ld + j] : zero<T>();
 #pragma unroll
   for (int c = 0; c < kNb; ++c)
 #pragma unroll
@@ -302,13 +341,13 @@ __global__ void __launch_bounds__(128) k_lu_upper(T *Aug, int N, int k0, int nb,
   const int b = blockIdx.y, tid = threadIdx.x;
   const long long ld = 2LL * N, j = N + (long long)blockIdx.x * blockDim.x + tid;
   T *A = Aug + (long long)b * N * ld;
+#pragma unroll 8
   for (int e = tid; e < kNb * kNb; e += blockDim.x) {
     const int i = e / kNb, c = e % kNb;
-    const bool in = i <= c && c < nb;
-    const T v = in ? A[(k0 + i) * ld + k0 + c] : zero<T>();
-    U[c][i] = v;
-    if (i == c) inv[c] = in ? recip(v) : one<T>();
+    U[c][i] = (i <= c && c < nb) ? A[(k0 + i) * ld + k0 + c] : zero<T>();
   }
+  __syncthreads();
+  if (tid < kNb) inv[tid] = tid < nb ? recip(U[tid][tid]) : one<T>();
   __syncthreads();
   const bool live = j < ld;
   T x[kNb];
