@@ -592,7 +592,6 @@ __global__ void __launch_bounds__(1024) k_csplit_t(const T *src, RowMap m, int b
   }
 }
 
-// rows contiguous along the row index and K strided: stage through shared memory
 // The same for few columns (K <= 16): 2^lp lanes per row, four values of K per lane, kept in
 // registers between the row maximum and the pairs, 16-byte stores; neighbouring groups take
 // neighbouring rows, so the reads stay coalesced without a tile in shared memory.  (k_csplit_t's
@@ -647,6 +646,8 @@ __global__ void __launch_bounds__(256) k_csplit_r(const T *src, RowMap m, unsign
   }
 }
 
+// Rows contiguous along the row index and K strided: through registers (k_csplit_r) or shared memory
+// (k_csplit_t); false where neither serves.
 template <class T>
 bool launch_split_t(const T *src, const RowMap &m, int batch, int rows, int K, int Kp2, int kind, float sa, float sbc,
                     __half *hi, __half *lo, float *unscale, cudaStream_t s) {

@@ -7,8 +7,9 @@
 
 namespace sox {
 
-// A split operand: `batch` blocks of `rows` real rows, each Kp2 = 8*ceil(2K/8) FP16
-// values (hi and lo), and one FP32 factor per real row that undoes its scale.
+// A split operand: `batch` blocks of `rows` real rows, each Kp2 = csplit_kp2(K) FP16 values (hi and
+// lo; 8, 16, 32 or a multiple of 64 that holds 2K), and one FP32 factor per real row that undoes its
+// scale.
 struct CSplit {
   __half *hi = nullptr, *lo = nullptr;
   float *unscale = nullptr;

@@ -345,8 +345,9 @@ __global__ void __launch_bounds__(256) k_slice_complex(const double2 *src, long 
 // read out; each sum's columns are handed back as soon as they are read, so the next window's
 // first products run while the later sums are still being read.
 // Bound by the MMAs (34 of 128 x 64 x 16 per 16 of K) and, at K <= 128, by reading the sums
-// out in equal parts; the FP64 pipe (1.6 FMA a clock and SM) sees no instruction of it.
-// n = 120, N = 600, 160 batches: projections 2.84 ms on the FP64 pipe, 0.22 ms here with the
+// out in equal parts; the FP64 pipe (1.6 FMA a clock and SM) sees the elements that are
+// summed from the sources, and no other.
+// n = 120, N = 600, 160 batches: projections 2.84 ms on the FP64 pipe, 0.26 ms here with the
 // slicing; final sum (K = 600) 1.74 -> 0.29 ms.  n = 250, N = 2000, 12 times: X G X^T 27.9 -> 1.7 ms.
 constexpr int kL = 128, kW = 64, kKc = 32, kWin = 4;   // kWin chunks per window
 constexpr int kLBytes = kL * kKc * 2, kWBytes = kW * kKc * 2;
@@ -855,7 +856,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // TMEM columns, so one is read out while the other accumulates.  The two products become
 // FP64 numbers with their own scales and D sums their product over v in FP64 registers.
 // Per (tile, v) 14 MMAs (34 digit products each for B_v and C_v) per 16 of n; the FP64 pipe
-// sees one FMA per element and v.  n = 80, N = 480, 30 times: 172.9 ms on the FP64 pipe, 7.4 ms
+// sees one FMA per element and v.  n = 80, N = 480, 30 times: 172.9 ms on the FP64 pipe, 7.5 ms
 // here (tensor pipe 41 % busy; the copies of the digits into shared memory set the pace).
 constexpr int kFW = 32;
 constexpr int kFWBytes = kFW * kKc * 2;

@@ -1189,7 +1189,7 @@ Status kpoint_dynamic_tc(sox_handle h, const sox_problem *pr, int n_omega, const
 // A_k (one in-place DFT of the projections over k), its transform is the pointwise product
 // A-hat_{tau_j}(m)[P][Q] A-hat_{tau_{T-1-j}}(-m)[Q][P] (G(-tau_j) = -G(tau_{T-1-j})), so
 // the bubble of every q costs one pass over the projections and an inverse DFT over m.
-// FP64 throughout; the solve is Gauss-Jordan with partial pivoting, batched over (q, o).
+// FP64 throughout; the solve is elimination with partial pivoting, batched over (q, o).
 namespace {
 
 constexpr int kMaxSide = 8;

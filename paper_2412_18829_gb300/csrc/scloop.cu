@@ -124,10 +124,10 @@ __global__ void k_right_half(const z *Aug, int n, long long batch, z *G) {
 // block per (spin, frequency), with no augmented matrix in global memory.  Bound by the FP64
 // pipe (n^3 complex multiply-adds per system) and the chain of n pivots.  n = 20, 400
 // frequencies: 63 us for an inverse (162 us for the augmented elimination in global memory
-// with its build and copy); a bisection step for mu 72 us in one launch (before: seven
+// with its build and copy); a bisection step for mu 61 us in one launch (before: seven
 // launches and two host round trips, 0.8 ms).
 // ---------------------------------------------------------------------------------------
-constexpr int kSmallN = 110;        // n^2 + 3 n complex values and the pivots stay below 200 KB
+constexpr int kSmallN = 110;        // n^2 + 2 n complex values and the pivots stay below 200 KB
 constexpr int kSmallThreads = 128;
 size_t small_smem(int n) { return sizeof(z) * ((size_t)n * n + 2 * (size_t)n) + sizeof(int) * (size_t)n + 16; }
 
