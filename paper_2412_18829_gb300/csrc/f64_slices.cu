@@ -527,12 +527,26 @@ __device__ __noinline__ double plain_element(const Args &a, int b, int l, int w,
 template <int C>
 __device__ __noinline__ void plain_block(const Args &a, int b, int l, int w0, double *out) {
   double acc[C] = {};
+  const int bl = a.bL == 1 ? 0 : b, bw = a.bW == 1 ? 0 : b, cols = min(C, a.nW - w0);
   const bool in = l < a.nL;
-  for (int k = 0; k < a.K; ++k) {
-    const double x = in ? plain_at(a.xL, a.bL == 1 ? 0 : b, l, k) : 0.0;
+  const Plain &L = a.xL, &W = a.xW;
+  if (L.kind == 0 && W.kind == 0 && !L.f32 && !W.f32) {   // real FP64 rows: no index arithmetic per element
+    const double *x = static_cast<const double *>(L.x) + bl * L.sb + min(l, a.nL - 1) * L.sr;
+    const double *y = static_cast<const double *>(W.x) + bw * W.sb + w0 * W.sr;
+#pragma unroll 2
+    for (int k = 0; k < a.K; ++k, x += L.sk, y += W.sk) {
+      const double v = *x;
 #pragma unroll
-    for (int j = 0; j < C; ++j)
-      if (w0 + j < a.nW) acc[j] = fma(x, plain_at(a.xW, a.bW == 1 ? 0 : b, w0 + j, k), acc[j]);
+      for (int j = 0; j < C; ++j)
+        if (j < cols) acc[j] = fma(v, y[j * W.sr], acc[j]);
+    }
+  } else {
+    for (int k = 0; k < a.K; ++k) {
+      const double x = in ? plain_at(L, bl, l, k) : 0.0;
+#pragma unroll
+      for (int j = 0; j < C; ++j)
+        if (j < cols) acc[j] = fma(x, plain_at(W, bw, w0 + j, k), acc[j]);
+    }
   }
 #pragma unroll
   for (int j = 0; j < C; ++j) out[j] = acc[j];
